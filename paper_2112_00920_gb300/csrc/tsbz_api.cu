@@ -437,6 +437,8 @@ template <typename T> int run_observe(tsbz_ctx* ctx, int fin_mode) {
         launch_bra_tc(L, ctx->psi, ctx->Pa, 1, ctx->stream);
       else if (sep)
         launch_bra_sep(L, ctx->psi, ctx->Pa, 1, 1, ctx->stream);
+      else if (ctx->precision == TSBZ_FP64 && launch_pa64(L, ctx->psi, ctx->Pa, ctx->stream))
+        ;
       else if (ctx->precision == TSBZ_FP32 &&
                launch_bra_slab(L, ctx->psi, ctx->Pa, 1, 1, ctx->stream, p_next ? ctx->P : nullptr))
         wrote_p = p_next && hc.dev.use_proj;
@@ -444,8 +446,8 @@ template <typename T> int run_observe(tsbz_ctx* ctx, int fin_mode) {
         launch_bra<T>(L, ctx->psi, ctx->Pa, 1, 1, ctx->stream);
       ev_stop(ctx);
       if (hc.dev.use_proj) ++ctx->launches;
+      hc.p_by_obs = wrote_p;
     }
-    hc.p_by_obs = wrote_p;
     ev_start(ctx, FAM_OBS);
     if (!(sep && launch_observe_fused(L, ctx->psi, ctx->rho_part, ctx->jk_part, ctx->nrm_part, ctx->stream)) &&
         !(ctx->precision != TSBZ_FP64 &&
@@ -510,8 +512,9 @@ int run_step_tc(tsbz_ctx* ctx) {
 
 // The four Taylor stages of every cell (after the field launch): psi advances by
 // dt * ctx->dt_scale.  fresh_p: the projections of psi are recomputed first
-// (else they are taken from P when the last step left them there).
-template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_allowed) {
+// (else they are taken from P when the last step left them there).  want_pa: the
+// current is evaluated on the resulting psi (ETRS needs it after its last half step only).
+template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_allowed, bool want_pa) {
   void* srcs[4] = {ctx->psi, ctx->tA, ctx->tB, ctx->tA};
   void* dsts[4] = {ctx->tA, ctx->tB, ctx->tA, nullptr};
   for (auto& hc : ctx->cells) {
@@ -546,6 +549,21 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
         ++ctx->launches;
       }
       continue;
+    }
+    if (ctx->precision == TSBZ_FP64) {
+      // 8^3 and 16^3 grids: the whole step in one launch
+      const bool carried = !fresh_p && ctx->p_next_valid && hc.p_by_obs;
+      const bool same_next = want_pa && same_next_allowed && cell_field_const(ctx, hc);
+      ev_start(ctx, FAM_STAGE);
+      const bool whole = launch_step64(L, ctx->psi, ctx->P, ctx->Pa, carried ? 0 : 1, want_pa ? 1 : 0,
+                                       same_next ? 1 : 0, ctx->stream);
+      ev_stop(ctx);
+      hc.pa_by_stage = whole && want_pa;
+      if (whole) {
+        hc.p_by_obs = same_next && hc.dev.use_proj;
+        ++ctx->launches;
+        continue;
+      }
     }
     // single precision on 32-point rows: variant 0 is the slab z-march stage, the
     // point-parallel stage takes the variants after it
@@ -584,7 +602,7 @@ template <typename T> int run_step_etrs(tsbz_ctx* ctx) {
   // predictor: the Taylor-4 step, then rho~ and v~_eff (no current, step unchanged)
   ctx->dt_scale = 1.0;
   run_field<T>(ctx, TSBZ_FIELD_STEP);
-  if ((rc = run_stages<T>(ctx, true, 0))) return rc;
+  if ((rc = run_stages<T>(ctx, true, 0, false))) return rc;
   run_observe<T>(ctx, TSBZ_FIN_RHO);
   run_hxc<T>(ctx);
   launch_veff_keep_t<T>(ctx->d_subs, ctx->d_cells, ns, 1, ctx->stream);   // v_eff(t_n) back, v~_eff kept
@@ -593,11 +611,11 @@ template <typename T> int run_step_etrs(tsbz_ctx* ctx) {
   // the two half steps
   ctx->dt_scale = 0.5;
   run_field<T>(ctx, TSBZ_FIELD_AT_NOW);
-  if ((rc = run_stages<T>(ctx, true, 0))) return rc;
+  if ((rc = run_stages<T>(ctx, true, 0, false))) return rc;
   launch_veff_keep_t<T>(ctx->d_subs, ctx->d_cells, ns, 1, ctx->stream);   // v~_eff in place
   ++ctx->launches;
   run_field<T>(ctx, TSBZ_FIELD_AT_NEXT);
-  if ((rc = run_stages<T>(ctx, true, 0))) return rc;
+  if ((rc = run_stages<T>(ctx, true, 0, true))) return rc;
   ctx->dt_scale = 1.0;
   run_observe<T>(ctx, TSBZ_FIN_STEP);
   run_hxc<T>(ctx);
@@ -609,7 +627,7 @@ template <typename T> int run_step(tsbz_ctx* ctx) {
   if (ctx->precision == TSBZ_FP32_TC) return run_step_tc(ctx);
   if (ctx->propagator == TSBZ_PROP_ETRS) return run_step_etrs<T>(ctx);
   run_field<T>(ctx, TSBZ_FIELD_STEP);
-  int rc = run_stages<T>(ctx, false, 1);
+  int rc = run_stages<T>(ctx, false, 1, true);
   if (rc) return rc;
   run_observe<T>(ctx, TSBZ_FIN_STEP);
   run_hxc<T>(ctx);
@@ -767,7 +785,8 @@ int sync_and_check(tsbz_ctx* ctx) {
 //     stage with CUDA-core projections;
 //   point-parallel path (FP64, and FP32 on shapes without a z-march kernel):
 //     bands per staged projection chunk 8 (0), 4 (1), 16 (2, when its shared
-//     memory fits);
+//     memory fits); FP64 on 8^3 and 16^3 grids takes the whole step in one
+//     launch as variant 0;
 //   FP32 on grids with 32-point rows (slab_supported): 0 slab z-march stage,
 //     then the point-parallel stage with 4 (1), 16 (2, when it fits) or 8 (3)
 //     bands per chunk;
@@ -1073,12 +1092,13 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
     c.pbox = db;
     c.pbox_ok = ok ? 1 : 0;
   }
-  // z groups: atoms with bit-identical z rows of the float factor tables
+  // z groups: atoms with bit-identical z rows of the factor tables
   const int nm_z = c.nmax;
   auto same_z = [&](int a, int b) {
     for (int i = 0; i < nm_z; ++i) {
       const size_t ia = (size_t)(a * 3 + 2) * nm_z + i, ib = (size_t)(b * 3 + 2) * nm_z + i;
       if (g1f[ia] != g1f[ib] || d1f[ia] != d1f[ib]) return false;
+      if (ctx->precision == TSBZ_FP64 && (g1[ia] != g1[ib] || d1[ia] != d1[ib])) return false;
     }
     return true;
   };
@@ -1131,6 +1151,36 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
     for (int g = c.n_zg; g < 8; ++g) c.zg_rep[g] = 0;
   }
   const int nn[3] = {c.n1, c.n2, c.n3};
+  c.hz = d->a[2] / d->n[2];
+  for (int g = 0; g < 8; ++g) {
+    c.zg_k0[g] = 0.0;
+    c.zg_brk[g] = c.n3;
+    if (g >= c.n_zg) continue;
+    // offsets before the box is applied, as in the projector tables
+    const double f = hc.atoms[3 * c.zg_rep[g] + 2];
+    auto image = [&](int z) { return std::floor((z - f * c.n3 + c.n3 / 2.0) / c.n3); };
+    c.zg_k0[g] = (-f * c.n3 - c.n3 * image(0)) * c.hz;
+    for (int z = 1; z < c.n3 && c.zg_brk[g] == c.n3; ++z)
+      if (image(z) != image(0)) c.zg_brk[g] = z;
+  }
+  {
+    std::vector<double> ks(6 * (size_t)c.nmax, 0.0);
+    for (int ax = 0; ax < 3; ++ax)
+      for (int k = 0; k < nn[ax]; ++k) {
+        double lap = c.lapw[ax][0], grd = 0.0;
+        for (int m = 1; m <= c.nd; ++m) {
+          const double th = 2.0 * 3.14159265358979323846 * ((k * m) % nn[ax]) / nn[ax];
+          lap += 2.0 * c.lapw[ax][m] * std::cos(th);
+          grd += 2.0 * c.gradw[ax][m] * std::sin(th);
+        }
+        ks[(2 * ax) * (size_t)c.nmax + k] = -0.5 * lap;
+        ks[(2 * ax + 1) * (size_t)c.nmax + k] = grd;
+      }
+    double* kd = nullptr;
+    if ((rc = dalloc_t(ctx, ks.size(), &kd))) return rc;
+    CK(cudaMemcpy(kd, ks.data(), sizeof(double) * ks.size(), cudaMemcpyHostToDevice));
+    c.ksym = kd;
+  }
   for (int ax = 0; ax < 3; ++ax) {
     std::vector<double2> tw(nn[ax]);
     for (int m = 0; m < nn[ax]; ++m) {
@@ -1566,6 +1616,10 @@ int tsbz_ground_state(tsbz_ctx* ctx, int max_iter, double tol, int degree, doubl
   auto apply = [&](HostCell& hc, const double* filt, void* in, void* out, void* prev) {
     ctx->d_filt = filt;
     LaunchSet L = make_set(ctx, hc);
+    if (!prev && launch_filter64(L, in, out, filt, filt, 1, ctx->stream)) {
+      ++ctx->launches;
+      return;
+    }
     launch_bra<double>(L, in, ctx->P, 0, 0, ctx->stream);
     launch_stage<double>(L, in, out, prev, ctx->P, 0, ctx->stream);
     ctx->launches += 2;
@@ -1688,14 +1742,26 @@ int tsbz_ground_state(tsbz_ctx* ctx, int max_iter, double tol, int degree, doubl
     CK(cudaMemcpyAsync(dfa, fa.data(), sizeof(double) * fa.size(), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaMemcpyAsync(dfb, fb.data(), sizeof(double) * fb.size(), cudaMemcpyHostToDevice, ctx->stream));
     // Chebyshev filter of the block: Y_1 = (h - c)/e Y_0, Y_{j+1} = 2 (h - c)/e Y_j - Y_{j-1}
+    // (the degree - 1 last steps rotate the buffers; a cell whose bands run the whole
+    // recurrence in one launch writes the buffer the others end in)
     void* buf[3] = {ctx->psi, ctx->tA, ctx->tB};
     int prev = 0, cur = 1;
-    for (auto& hc : ctx->cells)
-      if (!hc.unit_ids.empty()) apply(hc, dfa, buf[0], buf[1], nullptr);
+    std::vector<char> whole(ctx->cells.size(), 0);
+    for (size_t i = 0; i < ctx->cells.size(); ++i) {
+      HostCell& hc = ctx->cells[i];
+      if (hc.unit_ids.empty()) continue;
+      if (launch_filter64(make_set(ctx, hc), buf[0], buf[degree % 3], dfa, dfb, degree, ctx->stream)) {
+        whole[i] = 1;
+        ++ctx->launches;
+      } else {
+        apply(hc, dfa, buf[0], buf[1], nullptr);
+      }
+    }
     for (int j = 1; j < degree; ++j) {
       const int next = 3 - prev - cur;
-      for (auto& hc : ctx->cells)
-        if (!hc.unit_ids.empty()) apply(hc, dfb, buf[cur], buf[next], buf[prev]);
+      for (size_t i = 0; i < ctx->cells.size(); ++i)
+        if (!ctx->cells[i].unit_ids.empty() && !whole[i])
+          apply(ctx->cells[i], dfb, buf[cur], buf[next], buf[prev]);
       prev = cur;
       cur = next;
     }

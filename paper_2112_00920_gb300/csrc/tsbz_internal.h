@@ -64,6 +64,14 @@ struct CellDev {
   int zg_rep[8];      // first atom of group g
   int zg_off[9];      // members of group g: zg_mem[zg_off[g] .. zg_off[g + 1])
   int zg_mem[8];
+  // minimal-image displacement of group g along z: zg_k0 + z hz for the planes
+  // z < zg_brk, one cell edge less from there on (zg_brk = n3: no jump)
+  int zg_brk[8];
+  double zg_k0[8];
+  double hz;
+  // kinetic symbol per axis: [3][2][nmax], row 0 the eigenvalues of -1/2 lap_FD on
+  // exp(2 pi i k j / n), row 1 those of -i grad_FD (times q in h)
+  const double* ksym;
   // the same grouping for cells of up to 64 atoms in at most 8 groups (the slab
   // stage of 32-point rows; zs_n = 0 when the cell has more groups or atoms)
   int zs_n;
@@ -206,6 +214,18 @@ bool launch_observe_slab(const LaunchSet& L, const void* psi, double* rho_part, 
 // pnext, if given with with_d, also receives Pa's first-weight entries as P.
 bool launch_bra_slab(const LaunchSet& L, const void* src, void* out, int with_d, int use_obs, void* stream,
                      void* pnext = nullptr);
+
+// Double precision on 8^3 and 16^3 grids (tsbz_step64.cu), variant 0 of such cells;
+// false (nothing launched) otherwise.  launch_step64: the whole time step; fresh_p:
+// the projections of psi are formed first (else taken from P); want_pa: those of the
+// current go to Pa, and with same_next those of the next step to P.
+bool step64_supported(const CellDev& c);
+bool launch_step64(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
+                   void* stream);
+bool launch_pa64(const LaunchSet& L, const void* src, void* Pa, void* stream);
+// the whole Chebyshev recurrence of the ground-state solver (degree 1: fa h + fa1)
+bool launch_filter64(const LaunchSet& L, const void* in, void* out, const double* fa, const double* fb, int degree,
+                     void* stream);
 
 bool sep_supported(const CellDev& c);
 int sep_variants(const CellDev& c);   // kernel variants of the single-precision path on this cell
