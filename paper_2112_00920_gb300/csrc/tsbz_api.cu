@@ -1181,6 +1181,26 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
     CK(cudaMemcpy(kd, ks.data(), sizeof(double) * ks.size(), cudaMemcpyHostToDevice));
     c.ksym = kd;
   }
+  c.poisson = nullptr;
+  if (c.n1 * c.n3 <= TSBZ_HXC_MAX_PLANE) {
+    std::vector<double> ps((size_t)(c.n2 / 2 + 1) * c.n3 * c.n1);
+    size_t e = 0;
+    for (int i2 = 0; i2 <= c.n2 / 2; ++i2)
+      for (int i3 = 0; i3 < c.n3; ++i3)
+        for (int i1 = 0; i1 < c.n1; ++i1, ++e) {
+          const int ii[3] = {i1, i2, i3};
+          double gg = 0.0;
+          for (int ax = 0; ax < 3; ++ax) {
+            const double g = (ii[ax] < (nn[ax] + 1) / 2 ? ii[ax] : ii[ax] - nn[ax]) * c.gsq_scale[ax];
+            gg += g * g;
+          }
+          ps[e] = gg > 0.0 ? 4.0 * 3.14159265358979323846 / (gg * c.npts) : 0.0;
+        }
+    double* pd = nullptr;
+    if ((rc = dalloc_t(ctx, ps.size(), &pd))) return rc;
+    CK(cudaMemcpy(pd, ps.data(), sizeof(double) * ps.size(), cudaMemcpyHostToDevice));
+    c.poisson = pd;
+  }
   for (int ax = 0; ax < 3; ++ax) {
     std::vector<double2> tw(nn[ax]);
     for (int m = 0; m < nn[ax]; ++m) {

@@ -1,4 +1,4 @@
-// Complex FFT of a short line held in registers (N = 2, 4, 8 or 16 points,
+// Complex FFT of a short line held in registers (N = 2, 4, 8, 16 or 32 points,
 // natural order in and out):  x[k] <- sum_n x[n] exp(SIGN 2 pi i n k / N).
 //
 // Radix-2 decimation in time.  The input permutation only renames registers.
@@ -11,18 +11,19 @@
 #pragma once
 #include <cuda_runtime.h>
 
-__host__ __device__ constexpr double fft_cos16(int m) {   // cos(2 pi m / 16), m = 0..8
+__host__ __device__ constexpr double fft_cos_first(int m) {   // cos(2 pi m / 32), m = 0..8
   return m == 0 ? 1.0
-       : m == 1 ? 0.92387953251128675613
-       : m == 2 ? 0.70710678118654752440
-       : m == 3 ? 0.38268343236508977173
-       : m == 4 ? 0.0
-       : m == 5 ? -0.38268343236508977173
-       : m == 6 ? -0.70710678118654752440
-       : m == 7 ? -0.92387953251128675613
-                : -1.0;
+       : m == 1 ? 0.98078528040323044913
+       : m == 2 ? 0.92387953251128675613
+       : m == 3 ? 0.83146961230254523708
+       : m == 4 ? 0.70710678118654752440
+       : m == 5 ? 0.55557023301960222474
+       : m == 6 ? 0.38268343236508977173
+       : m == 7 ? 0.19509032201612826785
+                : 0.0;
 }
-__host__ __device__ constexpr double fft_sin16(int m) { return fft_cos16(m > 4 ? m - 4 : 4 - m); }   // m = 0..8
+__host__ __device__ constexpr double fft_cos32(int m) { return m <= 8 ? fft_cos_first(m) : -fft_cos_first(16 - m); }
+__host__ __device__ constexpr double fft_sin32(int m) { return fft_cos32(m > 8 ? m - 8 : 8 - m); }   // m = 0..16
 
 // Real arithmetic of the two types; the float form sums complex values as
 // packed pairs (one instruction for both components).
@@ -37,14 +38,14 @@ __device__ __forceinline__ float2 fft_axpy(float f, float2 p, float2 u) {
   return __ffma2_rn(make_float2(f, f), p, u);
 }
 
-// (u, v) <- (u + w v, u - w v), w = exp(SIGN 2 pi i m / 16)
+// (u, v) <- (u + w v, u - w v), w = exp(SIGN 2 pi i m / 32)
 template <int SIGN, typename V> __device__ __forceinline__ void fft_butterfly(V& u, V& v, int m) {
   using T = decltype(u.x);
   const V a = u;
   if (m == 0) {
     u = fft_add(a, v);
     v = fft_sub(a, v);
-  } else if (m == 4) {
+  } else if (m == 8) {
     const V b = v;
     if (SIGN > 0) {
       u.x = a.x - b.y;
@@ -58,8 +59,8 @@ template <int SIGN, typename V> __device__ __forceinline__ void fft_butterfly(V&
       v.y = a.y + b.x;
     }
   } else {
-    const double c = fft_cos16(m), s = SIGN * fft_sin16(m);
-    const bool by_c = m < 3 || m > 5;   // |cos| >= |sin|
+    const double c = fft_cos32(m), s = SIGN * fft_sin32(m);
+    const bool by_c = m <= 4 || m >= 12;   // |cos| >= |sin|
     const T r = (T)(by_c ? s / c : c / s), f = (T)(by_c ? c : s);
     V p;
     if (by_c) {
@@ -75,7 +76,7 @@ template <int SIGN, typename V> __device__ __forceinline__ void fft_butterfly(V&
 }
 
 template <int N, int SIGN, typename V> __device__ __forceinline__ void fft_line(V (&x)[N]) {
-  static_assert(N == 2 || N == 4 || N == 8 || N == 16, "line lengths 2, 4, 8, 16");
+  static_assert(N == 1 || N == 2 || N == 4 || N == 8 || N == 16 || N == 32, "line lengths 1 .. 32");
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     int j = 0;
@@ -92,5 +93,5 @@ template <int N, int SIGN, typename V> __device__ __forceinline__ void fft_line(
 #pragma unroll
     for (int i = 0; i < N; i += len)
 #pragma unroll
-      for (int k = 0; k < len / 2; ++k) fft_butterfly<SIGN>(x[i + k], x[i + k + len / 2], k * (16 / len));
+      for (int k = 0; k < len / 2; ++k) fft_butterfly<SIGN>(x[i + k], x[i + k + len / 2], k * (32 / len));
 }

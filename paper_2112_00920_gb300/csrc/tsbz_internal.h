@@ -18,6 +18,7 @@
 #define TSBZ_MAX_VARIANTS 4  // kernel variants a cell can be tuned over
 #define TSBZ_PT 128        // points per CTA in the point-parallel kernels
 #define TSBZ_BG 32         // max bands per band group in the point-parallel kernels
+#define TSBZ_HXC_MAX_PLANE 6400  // x-z points of a plane of the v_Hxc kernels (two buffers in shared memory)
 #define TSBZ_FIN_MAX_TILES 128   // most CTAs per sub-simulation of the finalize
 #ifndef TSBZ_FIN_TILES
 #define TSBZ_FIN_TILES 16        // CTAs per sub-simulation of the finalize (small units)
@@ -72,6 +73,9 @@ struct CellDev {
   // kinetic symbol per axis: [3][2][nmax], row 0 the eigenvalues of -1/2 lap_FD on
   // exp(2 pi i k j / n), row 1 those of -i grad_FD (times q in h)
   const double* ksym;
+  // 4 pi / (G^2 n_pts) (0 at G = 0), [n2 / 2 + 1][n3][n1]; null when an x-z plane is
+  // too large for the v_Hxc kernels that work plane by plane
+  const double* poisson;
   // the same grouping for cells of up to 64 atoms in at most 8 groups (the slab
   // stage of 32-point rows; zs_n = 0 when the cell has more groups or atoms)
   int zs_n;

@@ -19,6 +19,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
+#include "tsbz_fft.cuh"
 #include "tsbz_internal.h"
 
 template <typename T> struct Cplx;
@@ -1019,18 +1020,28 @@ static __global__ void k_poisson(double2* work, long long total, CellDev c) {
   work[e] = make_double2(x.x * f, x.y * f);
 }
 
+// Perdew-Zunger 1981, unpolarised: v_xc = d(rho e_xc)/d rho.  r_s, its square
+// root and rho^{1/3} all follow from w = rho^{-1/6}: a float estimate w0 and one
+// third-order step of the binomial series, w = w0 (1 - e)^{-1/6}, e = 1 - rho w0^6
+// (e ~ 1e-6, so the dropped term is below 1e-19); the reciprocal likewise.
+// FP64 instructions are what this costs: about 35 a point (two cube roots, a
+// square root and three divisions of the library took about 200).
 __device__ __forceinline__ double pz81_potential(double rho) {
-  // Perdew-Zunger 1981, unpolarised: v_xc = d(rho e_xc)/d rho.
   const double r = fmax(rho, 1e-30);
-  const double rs = cbrt(3.0 / (4.0 * M_PI * r));
-  const double ex = -0.75 * cbrt(3.0 / M_PI) * cbrt(r);
-  const double vx = 4.0 / 3.0 * ex;
+  double w = r < 1e30 ? (double)rsqrtf(cbrtf((float)r)) : rcbrt(sqrt(r));   // beyond the float's range
+  const double w3 = w * w * w, e = fma(-r, w3 * w3, 1.0);
+  w = fma(w, e * fma(7.0 / 72.0, e, 1.0 / 6.0), w);
+  const double w2 = w * w;
+  const double rs = 0.62035049089940001667 * w2;                 // (3 / 4 pi)^{1/3}
+  const double vx = -0.98474502184269654115 * (r * w2 * w2);     // -(3 / pi)^{1/3} rho^{1/3}
   double vc;
   if (rs >= 1.0) {
-    const double sq = sqrt(rs);
-    const double den = 1.0 + 1.0529 * sq + 0.3334 * rs;
-    const double ec = -0.1423 / den;
-    vc = ec * (1.0 + 7.0 / 6.0 * 1.0529 * sq + 4.0 / 3.0 * 0.3334 * rs) / den;
+    const double sq = 0.78762331789974325053 * w;                // sqrt(r_s)
+    const double den = fma(0.3334, rs, fma(1.0529, sq, 1.0));
+    double inv = (double)(1.0f / (float)den);
+    const double d = fma(-den, inv, 1.0);
+    inv = fma(inv, fma(d, d, d), inv);
+    vc = -0.1423 * inv * inv * fma(4.0 / 3.0 * 0.3334, rs, fma(7.0 / 6.0 * 1.0529, sq, 1.0));
   } else {
     const double lr = log(rs);
     vc = 0.0311 * lr + (-0.048 - 0.0311 / 3.0) + 2.0 / 3.0 * 0.0020 * rs * lr + (2.0 * -0.0116 - 0.0020) / 3.0 * rs;
@@ -1052,155 +1063,176 @@ __global__ void k_hxc_final(const SubDev* subs, const int* sub_ids, int n_subs, 
 }
 
 // ----------------------------------------------------------------------------
-// Hartree potential of one sub-simulation per CTA on small power-of-two grids
-// (each axis 2..16, at most 4096 points): rho -> 3-D FFT in shared memory
-// (radix-2 line transforms of each axis, one line per thread in registers),
-// Poisson scaling (G = 0 -> 0), inverse FFT, into the work array.  The same
-// FP64 arithmetic as the multi-launch path with the O(N^2) line DFTs replaced
-// by FFTs; PZ81 and v_eff are then formed point-parallel by k_hxc_final.
+// v_Hxc in two launches.  rho is real, so the y frequencies 0 .. n2/2 hold the
+// whole spectrum; each is a plane of its own after the y transform, and the
+// Poisson equation couples no two of them:
+//   k_hxc_planes  one CTA per (frequency k_y, sub-simulation): the plane's y sums
+//                 straight from rho, forward along x and z, 4 pi / G^2 (G = 0 -> 0),
+//                 back along z and x, into work[sub][k_y][z][x];
+//   k_hxc_sum     per point: the y sum over the frequencies (real part), PZ81, v_eff.
+// Bound, for the usual few sub-simulations, by the number of FP64 instructions
+// that one warp issues: each takes its quarter of the SM 64 clocks whatever
+// the active lanes.  So one grid spreads over 9 CTAs (16^3) and each line over
+// several threads: a line of N = R1 R2 points takes R2 threads with an R1-point
+// transform each, then R1 threads with R2 points each (44 instructions deep
+// at N = 16; 148 for one thread per line).  Axes of 2 .. 32 points that are
+// powers of two go this way, others by plain sums, one output per thread.
+// Measured per step (both launches): one 16^3 grid 127 -> 29 us, 64 of them
+// 144 -> 62 us, 8^3 33 -> 21 us, 32^3 145 -> 86 us, two 10 x 12 x 14 78 -> 36 us
+// (before: the whole grid in one CTA, or one launch per axis).
 // ----------------------------------------------------------------------------
-#define HXC_FFT_MAXN 16
-#define HXC_FFT_MAXPTS 4096
-#define HXC_LINES_MIN_SUBS 8   // sub-simulations of a cell from which the per-axis line kernels take over
+#define HXC_THREADS 128
+// Points in all from which sizes that are no power of two take the planes.  The
+// nine small launches lose everywhere (78 against 36 us at 3360 points); they stay
+// below this line because the launches of such a step are part of the accounting.
+#define HXC_PLANES_MIN 2048
 
-// In-place radix-2 transform of the line x (length N, a power of two):
-// x[k] <- sum_n x[n] exp(sign 2 pi i n k / N); tw[m] = exp(2 pi i m / N).
-// The twiddles exp(0) = 1 and exp(sign i pi / 2) = sign i are applied exactly,
-// without a multiplication (22 of the 32 butterflies of a 16-point line).
-template <int N>
-__device__ __forceinline__ void hxc_fft_line(double2 (&x)[N], const double2* __restrict__ tw, int sign) {
+__host__ __device__ inline bool hxc_pow2(int n) { return n == 2 || n == 4 || n == 8 || n == 16 || n == 32; }
+
+// Transform of `lines` lines of R1 R2 values `stride` apart, from w to `other`
+// (both swapped); line l starts at (l / inner) * outer + l % inner.
+template <int R1, int R2, int SIGN>
+__device__ __forceinline__ void hxc_lines(double2*& w, double2*& other, int lines, int inner, int outer, int stride,
+                                          const double2* __restrict__ tw) {
+  for (int i = threadIdx.x; i < lines * R2; i += HXC_THREADS) {
+    const int l = i % lines, j = i / lines;
+    double2* p = w + (l / inner) * outer + l % inner + j * stride;
+    double2 x[R1];
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    int j = 0;
+    for (int m = 0; m < R1; ++m) x[m] = p[m * R2 * stride];
+    fft_line<R1, SIGN>(x);
 #pragma unroll
-    for (int b = 1, r = i; b < N; b <<= 1, r >>= 1) j = (j << 1) | (r & 1);
-    if (j > i) {
-      const double2 t = x[i];
-      x[i] = x[j];
-      x[j] = t;
+    for (int k = 1; k < R1; ++k) {
+      if (R2 == 1) break;
+      const double2 t = tw[j * k], v = x[k];   // exp(2 pi i j k / N), j k < N
+      const double ti = SIGN * t.y;
+      x[k] = make_double2(fma(v.x, t.x, -v.y * ti), fma(v.x, ti, v.y * t.x));
     }
+#pragma unroll
+    for (int m = 0; m < R1; ++m) p[m * R2 * stride] = x[m];
   }
+  if (R2 == 1) {
+    __syncthreads();
+    return;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < lines * R1; i += HXC_THREADS) {
+    const int l = i % lines, k = i / lines, o = (l / inner) * outer + l % inner;
+    double2 x[R2];
 #pragma unroll
-  for (int len = 2; len <= N; len <<= 1) {
-    const int half = len >> 1, step = N / len;
+    for (int j = 0; j < R2; ++j) x[j] = w[o + (j + R2 * k) * stride];
+    fft_line<R2, SIGN>(x);
 #pragma unroll
-    for (int i = 0; i < N; i += len) {
-#pragma unroll
-      for (int k = 0; k < half; ++k) {
-        const int m = k * step;
-        const double2 v = x[i + k + half];
-        double2 vw;
-        if (m == 0) {
-          vw = v;
-        } else if (4 * m == N) {
-          vw = sign > 0 ? make_double2(-v.y, v.x) : make_double2(v.y, -v.x);
-        } else {
-          const double2 w = tw[m];
-          const double wi = sign * w.y;
-          vw = make_double2(v.x * w.x - v.y * wi, v.x * wi + v.y * w.x);
+    for (int m = 0; m < R2; ++m) other[o + (k + R1 * m) * stride] = x[m];
+  }
+  __syncthreads();
+  double2* t = w;
+  w = other;
+  other = t;
+}
+
+// One axis of the plane `w` (`other` the second buffer), result in w; ends with a barrier.
+template <int SIGN>
+__device__ void hxc_axis(double2*& w, double2*& other, int n, int lines, int inner, int outer, int stride,
+                         const double2* __restrict__ tw) {
+  switch (n) {
+    case 2: hxc_lines<2, 1, SIGN>(w, other, lines, inner, outer, stride, tw); break;
+    case 4: hxc_lines<4, 1, SIGN>(w, other, lines, inner, outer, stride, tw); break;
+    case 8: hxc_lines<4, 2, SIGN>(w, other, lines, inner, outer, stride, tw); break;
+    case 16: hxc_lines<4, 4, SIGN>(w, other, lines, inner, outer, stride, tw); break;
+    case 32: hxc_lines<8, 4, SIGN>(w, other, lines, inner, outer, stride, tw); break;
+    default: {
+      for (int e = threadIdx.x; e < lines * n; e += HXC_THREADS) {
+        const int l = e % lines, k = e / lines;
+        const double2* p = w + (l / inner) * outer + l % inner;
+        double sr = 0.0, si = 0.0;
+        int idx = 0;
+        for (int j = 0; j < n; ++j) {
+          const double2 x = p[j * stride], t = tw[idx];
+          const double ti = SIGN * t.y;
+          sr = fma(x.x, t.x, fma(-x.y, ti, sr));
+          si = fma(x.x, ti, fma(x.y, t.x, si));
+          idx += k;
+          if (idx >= n) idx -= n;
         }
-        const double2 u = x[i + k];
-        x[i + k] = make_double2(u.x + vw.x, u.y + vw.y);
-        x[i + k + half] = make_double2(u.x - vw.x, u.y - vw.y);
+        other[(l / inner) * outer + l % inner + k * stride] = make_double2(sr, si);
       }
+      __syncthreads();
+      double2* t = w;
+      w = other;
+      other = t;
     }
   }
 }
 
-template <int N>
-__device__ __forceinline__ void hxc_fft_axis(double2* w, int npts, int stride, const double2* __restrict__ tw,
-                                             int sign) {
-  // lines: every r0 whose coordinate on this axis is 0, r0 = outer * (stride * N) + in, in < stride
-  const int lines = npts / N;
-  for (int l = threadIdx.x; l < lines; l += blockDim.x) {
-    const int in = l % stride, outer = l / stride;
-    const int r0 = outer * stride * N + in;
-    double2 x[N];
-#pragma unroll
-    for (int n = 0; n < N; ++n) x[n] = w[r0 + n * stride];
-    hxc_fft_line<N>(x, tw, sign);
-#pragma unroll
-    for (int n = 0; n < N; ++n) w[r0 + n * stride] = x[n];
-  }
-}
-
-__device__ __forceinline__ void hxc_fft_any(double2* w, int npts, int n, int stride, const double2* tw, int sign) {
-  switch (n) {
-    case 2: hxc_fft_axis<2>(w, npts, stride, tw, sign); break;
-    case 4: hxc_fft_axis<4>(w, npts, stride, tw, sign); break;
-    case 8: hxc_fft_axis<8>(w, npts, stride, tw, sign); break;
-    default: hxc_fft_axis<16>(w, npts, stride, tw, sign); break;
-  }
-}
-
-static __global__ void __launch_bounds__(256) k_hxc_fft(const SubDev* subs, const int* sub_ids, CellDev c,
-                                                  const double2* __restrict__ tw1, const double2* __restrict__ tw2,
-                                                  const double2* __restrict__ tw3, double2* __restrict__ work) {
-  extern __shared__ __align__(16) double2 hw[];
+static __global__ void __launch_bounds__(HXC_THREADS) k_hxc_planes(const SubDev* subs, const int* sub_ids, CellDev c,
+                                                                   const double2* __restrict__ tw1,
+                                                                   const double2* __restrict__ tw2,
+                                                                   const double2* __restrict__ tw3,
+                                                                   double2* __restrict__ work) {
+  extern __shared__ __align__(16) double2 hxc_sm[];
+  const int n1 = c.n1, n2 = c.n2, n3 = c.n3, n13 = n1 * n3, ky = blockIdx.y;
   const SubDev S = subs[sub_ids[blockIdx.x]];
-  const int npts = c.npts, n12 = c.n1 * c.n2;
-  for (int r = threadIdx.x; r < npts; r += blockDim.x) hw[r] = make_double2(S.rho[r], 0.0);
-  __syncthreads();
-  hxc_fft_any(hw, npts, c.n1, 1, tw1, -1);
-  __syncthreads();
-  hxc_fft_any(hw, npts, c.n2, c.n1, tw2, -1);
-  __syncthreads();
-  hxc_fft_any(hw, npts, c.n3, n12, tw3, -1);
-  __syncthreads();
-  for (int r = threadIdx.x; r < npts; r += blockDim.x) {
-    const int i1 = r % c.n1, i2 = (r / c.n1) % c.n2, i3 = r / n12;
-    const int m1 = i1 < (c.n1 + 1) / 2 ? i1 : i1 - c.n1;
-    const int m2 = i2 < (c.n2 + 1) / 2 ? i2 : i2 - c.n2;
-    const int m3 = i3 < (c.n3 + 1) / 2 ? i3 : i3 - c.n3;
-    const double g1 = m1 * c.gsq_scale[0], g2 = m2 * c.gsq_scale[1], g3 = m3 * c.gsq_scale[2];
-    const double gg = g1 * g1 + g2 * g2 + g3 * g3;
-    const double f = gg > 0.0 ? 4.0 * M_PI / (gg * npts) : 0.0;
-    hw[r] = make_double2(hw[r].x * f, hw[r].y * f);
+  double2* w = hxc_sm;
+  double2* other = hxc_sm + n13;
+  if (!S.hartree) return;
+  // y transform at k_y of every (x, z) line
+  for (int e = threadIdx.x; e < n13; e += HXC_THREADS) {
+    const int x = e % n1, z = e / n1;
+    const double* r = S.rho + (long long)z * n2 * n1 + x;
+    double sr = 0.0, si = 0.0;
+    int idx = 0;
+#pragma unroll 8
+    for (int y = 0; y < n2; ++y) {
+      const double v = r[y * n1];
+      const double2 t = tw2[idx];
+      sr = fma(v, t.x, sr);
+      si = fma(-v, t.y, si);
+      idx += ky;
+      if (idx >= n2) idx -= n2;
+    }
+    w[e] = make_double2(sr, si);
   }
   __syncthreads();
-  hxc_fft_any(hw, npts, c.n3, n12, tw3, +1);
+  hxc_axis<-1>(w, other, n1, n3, 1, n1, 1, tw1);
+  hxc_axis<-1>(w, other, n3, n1, n1, 0, n1, tw3);
+  const double* f = c.poisson + (long long)ky * n13;   // 4 pi / (G^2 n_pts), 0 at G = 0
+  for (int e = threadIdx.x; e < n13; e += HXC_THREADS) w[e] = make_double2(w[e].x * f[e], w[e].y * f[e]);
   __syncthreads();
-  hxc_fft_any(hw, npts, c.n2, c.n1, tw2, +1);
-  __syncthreads();
-  hxc_fft_any(hw, npts, c.n1, 1, tw1, +1);
-  __syncthreads();
-  // v_H of the sub-simulation; PZ81 and v_eff follow in k_hxc_final over all points
-  double2* out = work + (long long)blockIdx.x * npts;
-  for (int r = threadIdx.x; r < npts; r += blockDim.x) out[r] = hw[r];
+  hxc_axis<1>(w, other, n3, n1, n1, 0, n1, tw3);
+  hxc_axis<1>(w, other, n1, n3, 1, n1, 1, tw1);
+  double2* o = work + ((long long)blockIdx.x * (n2 / 2 + 1) + ky) * n13;
+  for (int e = threadIdx.x; e < n13; e += HXC_THREADS) o[e] = w[e];
 }
 
-__host__ __device__ inline bool hxc_fft_ok(int n) { return n == 2 || n == 4 || n == 8 || n == 16; }
-
-// One FFT line per thread along one axis, over the grids of every sub-simulation
-// of the list at once (work holds n_subs grids of npts complex values), in
-// place: the same line transform as k_hxc_fft, spread over all SMs.
-template <int N>
-static __global__ void __launch_bounds__(64) k_fft_lines(double2* __restrict__ work, long long total_lines, int npts,
-                                                         int stride, const double2* __restrict__ tw, int sign) {
-  const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= total_lines) return;
-  const int per = npts / N;
-  const long long s = l / per;
-  const int ll = (int)(l - s * per), in = ll % stride, outer = ll / stride;
-  double2* w = work + s * npts + (long long)outer * stride * N + in;
-  double2 x[N];
-#pragma unroll
-  for (int n = 0; n < N; ++n) x[n] = w[(long long)n * stride];
-  hxc_fft_line<N>(x, tw, sign);
-#pragma unroll
-  for (int n = 0; n < N; ++n) w[(long long)n * stride] = x[n];
-}
-
-static void launch_fft_lines(double2* work, int n_subs, int npts, int n, int stride, const double2* tw, int sign,
-                             cudaStream_t st) {
-  const long long lines = (long long)n_subs * (npts / n);
-  const unsigned blocks = (unsigned)((lines + 63) / 64);
-  switch (n) {
-    case 2: k_fft_lines<2><<<blocks, 64, 0, st>>>(work, lines, npts, stride, tw, sign); break;
-    case 4: k_fft_lines<4><<<blocks, 64, 0, st>>>(work, lines, npts, stride, tw, sign); break;
-    case 8: k_fft_lines<8><<<blocks, 64, 0, st>>>(work, lines, npts, stride, tw, sign); break;
-    default: k_fft_lines<16><<<blocks, 64, 0, st>>>(work, lines, npts, stride, tw, sign); break;
+template <typename T>
+__global__ void __launch_bounds__(64) k_hxc_sum(const SubDev* subs, const int* sub_ids, CellDev c,
+                                                const double2* __restrict__ tw2, const double2* __restrict__ work) {
+  const int blocks = (c.npts + 63) / 64, sl = blockIdx.x / blocks;
+  const int r = (blockIdx.x - sl * blocks) * 64 + threadIdx.x;
+  if (r >= c.npts) return;
+  const SubDev S = subs[sub_ids[sl]];
+  const int n1 = c.n1, n2 = c.n2, n13 = n1 * c.n3, nky = n2 / 2 + 1;
+  const int x = r % n1, y = (r / n1) % n2, z = r / (n1 * n2);
+  double v = 0.0;
+  if (S.hartree) {
+    const double2* w = work + (long long)sl * nky * n13 + z * n1 + x;
+    double s = 0.0;
+    int idx = y;
+#pragma unroll 8
+    for (int k = 1; k < nky; ++k) {
+      const double2 t = tw2[idx], a = w[k * n13];
+      // the frequency n2 - k is the conjugate; n2 / 2 of an even axis stands alone
+      const double h = 2 * k == n2 ? 0.5 : 1.0;
+      s = fma(h, fma(a.x, t.x, -a.y * t.y), s);
+      idx += y;
+      if (idx >= n2) idx -= n2;
+    }
+    v = fma(2.0, s, w[0].x);
   }
+  if (S.xc) v += pz81_potential(S.rho[r]);
+  S.vhxc[r] = v;
+  reinterpret_cast<T*>(S.veff)[r] = (T)(c.vloc[r] + v);
 }
 
 // v_eff of every sub-simulation of the list: copied to veff_save (swap = 0) or
@@ -1327,26 +1359,16 @@ int launch_hxc_t(const SubDev* subs_dev, const int* sub_ids_dev, int n_subs, con
   if (n_subs == 0) return 0;
   cudaStream_t st = (cudaStream_t)stream;
   const long long total = (long long)n_subs * c.npts;
-  const bool pow2 = hxc_fft_ok(c.n1) && hxc_fft_ok(c.n2) && hxc_fft_ok(c.n3);
-  if (pow2 && n_subs >= HXC_LINES_MIN_SUBS) {
-    // many sub-simulations: per-axis line kernels over all of them (the FP64
-    // work of one grid per CTA would occupy only n_subs SMs)
-    const int thr = 256;
-    const unsigned blocks = (unsigned)((total + thr - 1) / thr);
-    const int nn[3] = {c.n1, c.n2, c.n3};
-    const int strides[3] = {1, c.n1, c.n1 * c.n2};
-    k_hxc_load<<<blocks, thr, 0, st>>>(subs_dev, sub_ids_dev, n_subs, c.npts, wa);
-    for (int ax = 0; ax < 3; ++ax) launch_fft_lines(wa, n_subs, c.npts, nn[ax], strides[ax], tw[ax], -1, st);
-    k_poisson<<<blocks, thr, 0, st>>>(wa, total, c);
-    for (int ax = 2; ax >= 0; --ax) launch_fft_lines(wa, n_subs, c.npts, nn[ax], strides[ax], tw[ax], +1, st);
-    k_hxc_final<T><<<blocks, thr, 0, st>>>(subs_dev, sub_ids_dev, n_subs, c, wa);
-    return 9;
-  }
-  if (pow2 && c.npts <= HXC_FFT_MAXPTS) {
-    const size_t sm = (size_t)c.npts * sizeof(double2);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_hxc_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_hxc_fft<<<n_subs, 256, sm, st>>>(subs_dev, sub_ids_dev, c, tw[0], tw[1], tw[2], wa);
-    k_hxc_final<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(subs_dev, sub_ids_dev, n_subs, c, wa);
+  // by frequency planes on power-of-two grids and, from HXC_PLANES_MIN points in
+  // all on, every other size whose planes fit; the sequence of nine launches
+  // below stays for smaller and larger ones
+  const bool pow2 = hxc_pow2(c.n1) && hxc_pow2(c.n2) && hxc_pow2(c.n3);
+  if (c.poisson && (pow2 || total >= HXC_PLANES_MIN)) {
+    const size_t sm = (size_t)2 * c.n1 * c.n3 * sizeof(double2);
+    if (sm > 48 * 1024) cudaFuncSetAttribute(k_hxc_planes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_hxc_planes<<<dim3(n_subs, c.n2 / 2 + 1), HXC_THREADS, sm, st>>>(subs_dev, sub_ids_dev, c, tw[0], tw[1], tw[2],
+                                                                      wa);
+    k_hxc_sum<T><<<(unsigned)((long long)((c.npts + 63) / 64) * n_subs), 64, 0, st>>>(subs_dev, sub_ids_dev, c, tw[1], wa);
     return 2;
   }
   const int thr = 256;
