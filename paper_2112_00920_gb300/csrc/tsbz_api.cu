@@ -226,6 +226,34 @@ LaunchSet make_set(tsbz_ctx* ctx, HostCell& hc) {
   return L;
 }
 
+// Point tiles and band groups of a cell's observation kernel.  With few units the
+// bands are split further, until about the CTAs that the GPU holds at once are
+// there (two per SM of the fused form, three of the slab form, and of the
+// point-parallel form two, each already a warp per quarter of an SM); not more,
+// which would begin a second wave (256 units: 116 us in one, 143 us in two).
+void plan_observe(const tsbz_ctx* ctx, CellDev& c, long long n_units) {
+  const bool single = ctx->precision == TSBZ_FP32;
+  int tiles = c.n_tiles, most = TSBZ_BG, least = 1;
+  long long want = 304;
+  if (single && observe_fused_ok(c)) {
+    tiles = 1;
+    most = c.n_bands;
+    least = 2;
+  } else if (ctx->precision != TSBZ_FP64 && observe_zf_ok(c)) {
+    c.n_otiles = 1;
+    return;
+  } else if (single && observe_slab_tiles(c)) {
+    tiles = observe_slab_tiles(c);
+    least = 2;
+    want = 456;
+  }
+  const long long groups = std::max<long long>(1, want / (n_units * tiles));
+  const long long bg = (c.n_bands + groups - 1) / groups;
+  c.n_otiles = tiles;
+  c.obs_bg = (int)std::min<long long>(std::max<long long>(bg, least), most);
+  c.n_bgroups = (c.n_bands + c.obs_bg - 1) / c.obs_bg;
+}
+
 int layout(tsbz_ctx* ctx) {
   if (ctx->laid_out) return TSBZ_OK;
   if (ctx->subs.empty()) return set_err(ctx, TSBZ_ESTATE, "no sub-simulation added");
@@ -239,10 +267,16 @@ int layout(tsbz_ctx* ctx) {
     hc.hxc_subs.clear();
     ph_stride = std::max<long long>(ph_stride, (long long)hc.dev.n_atoms * 3 * hc.dev.nmax);
   }
-  // finalize tiles: TSBZ_FIN_TILES per sub-simulation; with units that take a whole CTA
-  // each, as many as the largest such sub-simulation has k-points (at most
-  // TSBZ_FIN_MAX_TILES)
-  int fin_units = TSBZ_FIN_TILES;
+  {
+    std::vector<long long> cell_units(ctx->cells.size(), 0);
+    for (auto& hs : ctx->subs) cell_units[hs.cell] += hs.n_k;
+    for (size_t i = 0; i < ctx->cells.size(); ++i)
+      if (cell_units[i]) plan_observe(ctx, ctx->cells[i].dev, cell_units[i]);
+  }
+  // finalize tiles: about two CTAs per SM over all sub-simulations, at least
+  // TSBZ_FIN_TILES each; with units that take a whole CTA each, as many as the largest
+  // such sub-simulation has k-points (at most TSBZ_FIN_MAX_TILES)
+  int fin_units = std::max(TSBZ_FIN_TILES, 304 / (int)std::min<size_t>(ctx->subs.size(), 304));
   for (size_t s = 0; s < ctx->subs.size(); ++s)
     if (fin_wide(ctx->cells[ctx->subs[s].cell].dev)) fin_units = std::max(fin_units, ctx->subs[s].n_k);
   ctx->fin_tiles = std::min(TSBZ_FIN_MAX_TILES, fin_units);
@@ -265,8 +299,8 @@ int layout(tsbz_ctx* ctx) {
       p_e += (long long)c.n_bands * c.n_proj;
       pa_e += 4LL * c.n_bands * c.n_proj;
       rho_e += (long long)c.n_bgroups * c.npts;
-      jk_e += 3LL * c.n_tiles * c.n_bgroups;
-      nrm_e += (long long)c.n_tiles * c.n_bands;
+      jk_e += 3LL * c.n_otiles * c.n_bgroups;
+      nrm_e += (long long)c.n_otiles * c.n_bands;
       hc.unit_ids.push_back((int)units.size());
       ctx->unit_psi_off.push_back(U.psi_off);
       units.push_back(U);
@@ -343,6 +377,8 @@ int layout(tsbz_ctx* ctx) {
     d.vhxc = hs.vhxc;
     d.veff = hs.veff;
     d.norms = hs.norms;
+    d.inv_nk = 1.0 / hs.n_k;
+    d.j_scale = -1.0 / (c.omega * hs.n_k);
     d.step = ctx->d_steps + s;
     d.status = ctx->d_status + s;
     d.active = ctx->d_active + s;
@@ -979,6 +1015,8 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
   c.n_bands = d->n_bands;
   c.nd = d->fd_nd;
   c.n_tiles = (c.npts + TSBZ_PT - 1) / TSBZ_PT;
+  c.n_otiles = c.n_tiles;
+  c.obs_bg = TSBZ_BG;
   c.n_bgroups = (c.n_bands + TSBZ_BG - 1) / TSBZ_BG;
   c.omega = d->a[0] * d->a[1] * d->a[2];
   c.dv = c.omega / (double)npts;

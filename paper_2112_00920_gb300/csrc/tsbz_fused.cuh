@@ -1220,7 +1220,7 @@ __global__ void __launch_bounds__(FS_NP, 2) k_pa_fused(LaunchSet L, const float2
 }
 
 // ----------------------------------------------------------------------------
-// Observation pass on 16^3 grids: one CTA per unit, bands in turn through a
+// Observation pass on 16^3 grids: one CTA per (unit, band group), the group's bands in turn through a
 // ring of FO_SLOTS band buffers filled by bulk copies.  A slot's "full"
 // mbarrier completes when its band has landed, its "empty" mbarrier when all
 // warps are done with it; thread 0 refills a slot once it is empty, so warps
@@ -1231,8 +1231,9 @@ __global__ void __launch_bounds__(FS_NP, 2) k_pa_fused(LaunchSet L, const float2
 // per thread sum Re(u* (-i grad u)) (FP32 within a band; over bands again as a
 // two-sum float pair, so that GB300's narrow FP64 pipe is left alone) and
 // per band sum |u|^2 (per-warp partials, added over warps in order at the
-// end).  The unit's sums go to point tile 0 of the partial buffers and zeros to
-// the other tiles.
+// end).  Point tile 0 of the partial buffers is the only one.  The band groups
+// (CellDev::obs_bg) fill the GPU when there are few units: 8 units of 16 bands,
+// 37 -> 17 us with two bands a group.
 // ----------------------------------------------------------------------------
 #define FO_SLOTS 3
 #define FO_MAXB 128   // bands of the per-warp norm table
@@ -1266,8 +1267,9 @@ __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const f
   const int tid = threadIdx.x, col = tid, lane = tid & 31, warp = tid >> 5;
   const int n_warps = (int)(blockDim.x >> 5);
   const int ix = col & (N - 1), iy = col / N;
-  const int nb = c.n_bands;
-  const float2* src = psi + U.psi_off;
+  const int grp = blockIdx.y, b0 = grp * c.obs_bg;
+  const int nb = min(c.obs_bg, c.n_bands - b0);   // bands of the group
+  const float2* src = psi + U.psi_off + (long long)b0 * FS_NPTS;
   volatile int* fail = &sm.fail;
   if (tid == 0) {
     for (int k = 0; k < FO_SLOTS; ++k) {
@@ -1374,7 +1376,8 @@ __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const f
     return;
   }
 #pragma unroll
-  for (int z = 0; z < N; ++z) rho_part[U.rho_off + (long long)z * NP + col] = c.occ * ((double)rho[z] + (double)rho_e[z]);
+  for (int z = 0; z < N; ++z)
+    rho_part[U.rho_off + (long long)grp * FS_NPTS + z * NP + col] = c.occ * ((double)rho[z] + (double)rho_e[z]);
   double jx = (double)js[0] + (double)je[0], jy = (double)js[1] + (double)je[1], jz = (double)js[2] + (double)je[2];
   for (int off = 16; off > 0; off >>= 1) {
     jx += __shfl_xor_sync(0xffffffffu, jx, off);
@@ -1390,13 +1393,11 @@ __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const f
   if (tid < 3) {
     double sum = 0.0;
     for (int w = 0; w < n_warps; ++w) sum += sm.redj[w][tid];
-    jk_part[U.jk_off + tid] = sum;
+    jk_part[U.jk_off + 3 * grp + tid] = sum;
   }
   for (int b = tid; b < nb; b += blockDim.x) {
     double sum = 0.0;
     for (int w = 0; w < n_warps; ++w) sum += (double)sm.nrm[w][b];
-    nrm_part[U.nrm_off + b] = sum;
+    nrm_part[U.nrm_off + b0 + b] = sum;
   }
-  for (int i = tid; i < 3 * (c.n_tiles - 1); i += blockDim.x) jk_part[U.jk_off + 3 + i] = 0.0;
-  for (int i = tid; i < c.n_bands * (c.n_tiles - 1); i += blockDim.x) nrm_part[U.nrm_off + c.n_bands + i] = 0.0;
 }

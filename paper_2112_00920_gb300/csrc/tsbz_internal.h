@@ -6,7 +6,7 @@
 //   P           : complex T, [unit][band][n_proj]          projections <beta~_j|t_b>
 //   Pa          : complex T, [unit][band][n_proj][4]        <beta~_j|u>, <d_a beta~_j|u>
 //   rho_part    : double,    [unit][band group][n_pts]      sum_b occ |u_b(r)|^2
-//   jk_part     : double,    [unit][tile][band group][3]    sum occ Re(u* (-i grad) u)
+//   jk_part     : double,    [unit][tile][band group][3]    sum Re(u* (-i grad) u)
 //   nrm_part    : double,    [unit][tile][band]             sum_r |u_b(r)|^2 per tile
 //   per sub-simulation: rho, v_hxc, v_eff (T), J history, J(0-), norms, step.
 #pragma once
@@ -29,7 +29,10 @@ struct CellDev {
   int n_atoms, n_proj, n_bands;
   int nd;
   int n_tiles;       // ceil(npts / TSBZ_PT)
-  int n_bgroups;     // ceil(n_bands / TSBZ_BG)
+  // partial sums of the observation kernel that the cell takes (set with the layout):
+  int n_otiles;      // point tiles per unit
+  int obs_bg;        // bands per band group
+  int n_bgroups;     // ceil(n_bands / obs_bg)
   int use_proj;
   double dv, omega, occ;
   double lapw[3][TSBZ_MAX_ND + 1];   // c_m / h_ax^2 (m = 0..nd)
@@ -86,7 +89,7 @@ struct CellDev {
 // Whether the finalize spreads one unit over a whole CTA (units with many
 // bands x projectors) rather than over one warp.
 __host__ __device__ inline bool fin_wide(const CellDev& c) {
-  return (long long)c.n_bands * (c.n_proj + c.n_tiles) > 4096;
+  return (long long)c.n_bands * (c.n_proj + c.n_otiles) > 4096;
 }
 
 struct UnitDev {
@@ -116,6 +119,7 @@ struct SubDev {
   double* vhxc;        // [npts]
   void* veff;          // [npts] in T
   double* norms;       // [n_k][n_bands]
+  double inv_nk, j_scale;   // 1 / n_k, -1 / (Omega n_k)
   int* step;           // steps done
   int* status;         // non-zero: non-finite current seen
   int* active;         // 1 while the sub-simulation advances in the current step
@@ -164,6 +168,13 @@ __device__ __forceinline__ bool unit_active(const LaunchSet& L, int u) {
   return *L.subs[L.units[u].sub].active != 0;
 }
 #endif
+
+// Which observation kernel a cell takes, in the order they are asked: the fused 16^3
+// form and the slab form (TSBZ_FP32), the 2.5-D form (both single-precision modes),
+// else the point-parallel one.  The slab form says its point tiles (0: not taken).
+bool observe_fused_ok(const CellDev& c);
+bool observe_zf_ok(const CellDev& c);
+int observe_slab_tiles(const CellDev& c);
 
 // Launchers (templated on the real type in tsbz_kernels.cuh, instantiated per precision).
 template <typename T> void launch_field(const LaunchSet& L, int mode, void* stream);

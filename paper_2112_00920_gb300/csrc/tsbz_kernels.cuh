@@ -56,12 +56,14 @@ template <> struct Tab<double> {
   static __device__ __forceinline__ const double* d1(const CellDev& c) { return c.d1; }
   static __device__ __forceinline__ const double* pnorm(const CellDev& c) { return c.pnorm; }
   static __device__ __forceinline__ const double* wkb(const CellDev& c) { return c.wkb; }
+  static __device__ __forceinline__ const double* ekb(const CellDev& c) { return c.ekb; }
 };
 template <> struct Tab<float> {
   static __device__ __forceinline__ const float* g1(const CellDev& c) { return c.g1f; }
   static __device__ __forceinline__ const float* d1(const CellDev& c) { return c.d1f; }
   static __device__ __forceinline__ const float* pnorm(const CellDev& c) { return c.pnormf; }
   static __device__ __forceinline__ const float* wkb(const CellDev& c) { return c.wkbf; }
+  static __device__ __forceinline__ const float* ekb(const CellDev& c) { return c.ekbf; }
 };
 
 // ----------------------------------------------------------------------------
@@ -736,7 +738,7 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
   const CellDev& c = L.cell;
   if (threadIdx.x < 3 * (TSBZ_MAX_ND + 1)) {
     const int ax = threadIdx.x / (TSBZ_MAX_ND + 1), mm = threadIdx.x % (TSBZ_MAX_ND + 1);
-    gw[ax][mm] = (T)c.gradw[ax][mm];
+    gw[ax][mm] = (T)(2.0 * c.gradw[ax][mm]);   // the correlation form's factor 2
   }
   __syncthreads();
   const int u = L.unit_ids[blockIdx.y];
@@ -748,8 +750,8 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
   const int pp = valid ? p : 0;
   const int ix = pp % c.n1, iy = (pp / c.n1) % c.n2, iz = pp / (c.n1 * c.n2);
   const int n12 = c.n1 * c.n2;
-  const int b_begin = grp * TSBZ_BG;
-  const int b_end = min(c.n_bands, b_begin + TSBZ_BG);
+  const int b_begin = grp * c.obs_bg;
+  const int b_end = min(c.n_bands, b_begin + c.obs_bg);
   T rho = (T)0, jx = (T)0, jy = (T)0, jz = (T)0;
   for (int b = b_begin; b < b_end; ++b) {
     T n2 = (T)0;
@@ -758,20 +760,18 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
       const V ce = tb[pp];
       n2 = ce.x * ce.x + ce.y * ce.y;
       rho += n2;
-      T cx = (T)0, cy = (T)0, cz = (T)0;
+      // v = sum_m w_m u(r + m e_ax) per axis, then Im(conj(u) v) = u_r v_i - u_i v_r
+      const V zero = cmk<V>((T)0, (T)0);
+      V vx = zero, vy = zero, vz = zero;
       const int rowb = iz * n12 + iy * c.n1;
       for (int mm = 1; mm <= c.nd; ++mm) {
-        const V xu = tb[rowb + wrap_idx(ix + mm, c.n1)];
-        const V yu = tb[iz * n12 + wrap_idx(iy + mm, c.n2) * c.n1 + ix];
-        const V zu = tb[wrap_idx(iz + mm, c.n3) * n12 + iy * c.n1 + ix];
-        // Im(conj(u) v) = u_r v_i - u_i v_r
-        cx += gw[0][mm] * (ce.x * xu.y - ce.y * xu.x);
-        cy += gw[1][mm] * (ce.x * yu.y - ce.y * yu.x);
-        cz += gw[2][mm] * (ce.x * zu.y - ce.y * zu.x);
+        rfma(vx, gw[0][mm], tb[rowb + wrap_idx(ix + mm, c.n1)]);
+        rfma(vy, gw[1][mm], tb[iz * n12 + wrap_idx(iy + mm, c.n2) * c.n1 + ix]);
+        rfma(vz, gw[2][mm], tb[wrap_idx(iz + mm, c.n3) * n12 + iy * c.n1 + ix]);
       }
-      jx += (T)2 * cx;
-      jy += (T)2 * cy;
-      jz += (T)2 * cz;
+      jx += ce.x * vx.y - ce.y * vx.x;
+      jy += ce.x * vy.y - ce.y * vy.x;
+      jz += ce.x * vz.y - ce.y * vz.x;
     }
     red_n[b - b_begin][threadIdx.x] = n2;
   }
@@ -807,168 +807,145 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
 // finalize: n_tiles CTAs per sub-simulation.  rho (Eq. 3), norms, and the current
 // J = -(1/(Omega N_k)) sum_k sum_b occ [ dV Re<u|-i grad u> + q |u|^2
 //                                        + 2 sum_j E_j Im(conj(c_j) a_j) ]   (Eqs. 5-6)
-// summed in a fixed order.  The inputs are
-// read-only here and disjoint from the outputs (restrict), so that the loads of
-// a thread's chain of units and bands are issued ahead of the sums and stores.
+// summed in a fixed order.  Bound by latency: a chain of FP64 instructions (64
+// clocks each on a quarter of an SM) and dependent loads, over little data.  So
+// every sum is spread over threads first and reduced once:
+//  - density: the tile's points over the lanes and, when the tile has fewer points
+//    than threads, the (unit, band group) terms over FIN_THREADS / points parts,
+//    added in part order;
+//  - norms, current: tiles take units; a unit is shared by one warp, or by the
+//    whole CTA when its projections are many (fin_wide) or there are no more
+//    units than tiles.  Each thread adds its own bands, partials and projectors
+//    of all its units; one reduction per CTA follows, and the CTA that finishes
+//    last adds the tiles' currents, writes J and advances the step.
+// Measured per step: 8 k-points at 16^3 31 -> 13 us (FP32), two subgrids of 512
+// k-points 155 -> 33 us, 64 of 64 k-points 109 -> 71 us; with one warp and 16 tiles
+// for each unit and a shuffle sum per band before.
 // ----------------------------------------------------------------------------
+#define FIN_THREADS 256
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_finalize(const SubDev* __restrict__ subs, const UnitDev* __restrict__ units,
-                                                  const CellDev* __restrict__ cells, const double* __restrict__ q_obs,
-                                                  const typename Cplx<T>::type* __restrict__ Pa,
-                                                  const double* __restrict__ rho_part,
-                                                  const double* __restrict__ jk_part,
-                                                  const double* __restrict__ nrm_part, const int* __restrict__ mask,
-                                                  int mode) {
+__global__ void __launch_bounds__(FIN_THREADS) k_finalize(
+    const SubDev* __restrict__ subs, const UnitDev* __restrict__ units, const CellDev* __restrict__ cells,
+    const double* __restrict__ q_obs, const typename Cplx<T>::type* __restrict__ Pa,
+    const double* __restrict__ rho_part, const double* __restrict__ jk_part, const double* __restrict__ nrm_part,
+    const int* __restrict__ mask, int mode) {
   using V = typename Cplx<T>::type;
-  const int s = blockIdx.x;
+  __shared__ double red[3][FIN_THREADS];
+  __shared__ int last;
+  const int s = blockIdx.x, tid = threadIdx.x;
   const SubDev S = subs[s];
   if ((mode == TSBZ_FIN_STEP || mode == TSBZ_FIN_RHO) && !*S.active) return;   // budget spent: nothing of this step
-  const CellDev c = cells[S.cell];
-  // density: point tile blockIdx.y of the sub-simulation (fixed k and band-group order per point)
-  const double inv_nk = 1.0 / S.n_k;
-  const int chunk = (c.npts + (int)gridDim.y - 1) / (int)gridDim.y;
-  const int r_end = min(c.npts, ((int)blockIdx.y + 1) * chunk);
-  // the units of a sub-simulation are consecutive, n_bgroups * npts doubles apart
-  const double* rho_s = rho_part + units[S.unit0].rho_off;
-  const long long ustride = (long long)c.n_bgroups * c.npts;
-  for (int r = (int)blockIdx.y * chunk + threadIdx.x; r < r_end; r += blockDim.x) {
-    double acc = 0.0;
-    if (c.n_bgroups == 1) {
-#pragma unroll 8
-      for (int kl = 0; kl < S.n_k; ++kl) acc += rho_s[kl * ustride + r];
-    } else {
-      for (int kl = 0; kl < S.n_k; ++kl)
-        for (int g = 0; g < c.n_bgroups; ++g) acc += rho_s[kl * ustride + (long long)g * c.npts + r];
-    }
-    S.rho[r] = acc * inv_nk;
-  }
-  // current and norms of the units kl = tile + ntile j.  Small units (few
-  // bands x projectors): warp w of the CTA takes every n_warps-th of them, lanes
-  // share a unit.  Large units: the CTA takes them one at a time over all its
-  // threads (warp w takes the band norms w, w + n_warps, ...).  Either way the
-  // partial sums are added in a fixed order (lanes, warps in order, units in
-  // increasing kl); the CTA that finishes last adds the tiles' partial currents
-  // in tile order, writes J and advances the step.
+  const CellDev& c = cells[S.cell];
   const int tile = blockIdx.y, ntile = gridDim.y;
+  const int npts = c.npts, ngrp = c.n_bgroups, n_k = S.n_k;
+  {
+    const int chunk = (npts + ntile - 1) / ntile, r0 = tile * chunk, r1 = min(npts, r0 + chunk);
+    // parts of the (unit, group) terms: the units of a sub-simulation are consecutive,
+    // ngrp * npts doubles apart, so term i starts at i * npts
+    int pts = 32;
+    while (pts < chunk && pts < FIN_THREADS) pts <<= 1;
+    const int parts = FIN_THREADS / pts, part = tid / pts, terms = n_k * ngrp;
+    const double* rho_s = rho_part + units[S.unit0].rho_off;
+    for (int b = r0; b < r1; b += pts) {
+      const int r = b + (tid & (pts - 1));
+      double acc = 0.0;
+      if (r < r1) {
+#pragma unroll 8
+        for (int i = part; i < terms; i += parts) acc += rho_s[(long long)i * npts + r];
+      }
+      if (parts > 1) {
+        __syncthreads();
+        red[0][tid] = acc;
+        __syncthreads();
+        if (part == 0)
+          for (int k = 1; k < parts; ++k) acc += red[0][k * pts + tid];
+      }
+      if (part == 0 && r < r1) S.rho[r] = acc * S.inv_nk;
+    }
+  }
   const int step = *S.step;
   const bool write_j = mode != TSBZ_FIN_RHO &&
                        ((mode == TSBZ_FIN_STEP) || (mask != nullptr && mask[s] != 0 &&
                                                     (mode == TSBZ_FIN_J0MINUS || step == 0)));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = (int)(blockDim.x >> 5);
-  const bool wide = fin_wide(c);
+  const int warp = tid >> 5, lane = tid & 31, n_warps = FIN_THREADS / 32;
+  const bool wide = fin_wide(c) || n_k <= ntile;
   const int u_first = wide ? tile : tile + ntile * warp, u_step = wide ? ntile : ntile * n_warps;
-  const int b_first = wide ? warp : 0, b_step = wide ? n_warps : 1;
-  const int e_first = wide ? (int)threadIdx.x : lane, e_step = wide ? (int)blockDim.x : 32;
-  __shared__ double red[8][4];
-  double jw[3] = {0.0, 0.0, 0.0};   // this warp's units (small), thread 0: this CTA's units (large)
-  for (int kl = u_first; kl < S.n_k; kl += u_step) {
-    const UnitDev U = units[S.unit0 + kl];
+  const int e_first = wide ? tid : lane, e_step = wide ? FIN_THREADS : 32;
+  double v[3] = {0.0, 0.0, 0.0};   // this thread's share of sum occ <u|pi|u> / occ
+  for (int kl = u_first; kl < n_k; kl += u_step) {
     const int u = S.unit0 + kl;
-    double jk[3] = {0.0, 0.0, 0.0}, jn[3] = {0.0, 0.0, 0.0}, nsum = 0.0;
-#pragma unroll 4
-    for (int b = b_first; b < c.n_bands; b += b_step) {
+    const UnitDev U = units[u];
+    double nsum = 0.0, jk[3] = {0.0, 0.0, 0.0};
+    for (int b = e_first; b < c.n_bands; b += e_step) {
       double nb = 0.0;
-      for (int t = lane; t < c.n_tiles; t += 32) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
-      for (int off = 16; off > 0; off >>= 1) nb += __shfl_xor_sync(0xffffffffu, nb, off);
+#pragma unroll 8
+      for (int t = 0; t < c.n_otiles; ++t) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
       nb *= c.dv;
-      if (lane == 0) S.norms[kl * c.n_bands + b] = nb;
-      nsum += nb;  // identical in every lane
+      S.norms[kl * c.n_bands + b] = nb;
+      nsum += nb;
     }
-    for (int i = e_first; i < c.n_tiles * c.n_bgroups; i += e_step)
+    for (int i = e_first; i < c.n_otiles * ngrp; i += e_step)
+#pragma unroll
       for (int ax = 0; ax < 3; ++ax) jk[ax] += jk_part[U.jk_off + 3LL * i + ax];
-    if (c.use_proj) {
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) v[ax] = fma(c.dv, jk[ax], fma(q_obs[3 * u + ax], nsum, v[ax]));
+    if (c.use_proj && mode != TSBZ_FIN_RHO) {
+      // single-precision projections: each thread forms and sums its own terms in
+      // FP32 (the terms carry the projections' own ~1e-6 relative error) and
+      // converts the sum once
       const int np = c.n_proj;
-      if constexpr (sizeof(T) == sizeof(float)) {
-        // single-precision projections: each thread forms and sums its own terms
-        // in FP32 (the terms carry the projections' own ~1e-6 relative error) and
-        // converts the sum once; the FP64 pipe of this GPU is ~1/64 of the FP32 one
-        float jf[3] = {0.f, 0.f, 0.f};
+      T jf[3] = {(T)0, (T)0, (T)0};
 #pragma unroll 4
-        for (int i = e_first; i < c.n_bands * np; i += e_step) {
-          const int j = i % np;
-          const V* pr = Pa + U.pa_off + 4LL * i;
-          const float ar = pr[0].x, ai = pr[0].y;
-          const float e2 = 2.0f * c.ekbf[j];
-          for (int ax = 0; ax < 3; ++ax) {
-            // Im(conj(c) a) = c_r a_i - c_i a_r
-            const float cr = pr[1 + ax].x, ci = pr[1 + ax].y;
-            jf[ax] = __fmaf_rn(e2, __fmaf_rn(cr, ai, -ci * ar), jf[ax]);
-          }
-        }
-        for (int ax = 0; ax < 3; ++ax) jn[ax] = (double)jf[ax];
-      } else {
-#pragma unroll 4
-        for (int i = e_first; i < c.n_bands * np; i += e_step) {
-          const int j = i % np;
-          const V* pr = Pa + U.pa_off + 4LL * i;
-          const double ar = pr[0].x, ai = pr[0].y;
-          const double e2 = 2.0 * c.ekb[j];
-          for (int ax = 0; ax < 3; ++ax) {
-            // Im(conj(c) a) = c_r a_i - c_i a_r
-            const double cr = pr[1 + ax].x, ci = pr[1 + ax].y;
-            jn[ax] += e2 * (cr * ai - ci * ar);
-          }
+      for (int i = e_first; i < c.n_bands * np; i += e_step) {
+        const V* pr = Pa + U.pa_off + 4LL * i;
+        const V a = pr[0];
+        const T e2 = (T)2 * Tab<T>::ekb(c)[i % np];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+          const V cj = pr[1 + ax];   // Im(conj(c) a) = c_r a_i - c_i a_r
+          jf[ax] = fma(e2, fma(cj.x, a.y, -cj.y * a.x), jf[ax]);
         }
       }
+#pragma unroll
+      for (int ax = 0; ax < 3; ++ax) v[ax] += (double)jf[ax];
     }
-    double v[3];
-    for (int ax = 0; ax < 3; ++ax) {
-      v[ax] = c.dv * jk[ax] + jn[ax];
-      for (int off = 16; off > 0; off >>= 1) v[ax] += __shfl_xor_sync(0xffffffffu, v[ax], off);
-    }
-    if (!wide) {
-      for (int ax = 0; ax < 3; ++ax) jw[ax] += c.occ * (v[ax] + q_obs[3 * u + ax] * nsum);
-      continue;
-    }
+  }
+  if (mode == TSBZ_FIN_RHO) return;   // no current, step unchanged
+  // one warp per axis: the threads' shares, then, in the CTA that is last, the tiles'
+  __syncthreads();
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) red[ax][tid] = v[ax];
+  __syncthreads();
+  if (warp < 3) {
+    double t = 0.0;
+#pragma unroll
+    for (int k = 0; k < n_warps; ++k) t += red[warp][lane + 32 * k];
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
     if (lane == 0) {
-      for (int ax = 0; ax < 3; ++ax) red[warp][ax] = v[ax];
-      red[warp][3] = nsum;
+      S.jtile[3 * tile + warp] = t;
+      __threadfence();
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double sum[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int w = 0; w < n_warps; ++w)
-        for (int k = 0; k < 4; ++k) sum[k] += red[w][k];
-      for (int ax = 0; ax < 3; ++ax) jw[ax] += c.occ * (sum[ax] + q_obs[3 * u + ax] * sum[3]);
-    }
-    __syncthreads();
-  }
-  if (!wide) {
-    // the warps' sums in warp order
-    if (lane == 0)
-      for (int ax = 0; ax < 3; ++ax) red[warp][ax] = jw[ax];
-    __syncthreads();
-    if (threadIdx.x == 0)
-      for (int ax = 0; ax < 3; ++ax) {
-        double t = 0.0;
-        for (int w = 0; w < n_warps; ++w) t += red[w][ax];
-        jw[ax] = t;
-      }
-  }
-  __shared__ int last;
-  if (threadIdx.x == 0) {
-    for (int ax = 0; ax < 3; ++ax) S.jtile[3 * tile + ax] = jw[ax];
-    __threadfence();
-    last = atomicAdd(S.jcount, 1) == ntile - 1;
   }
   __syncthreads();
-  if (!last || threadIdx.x != 0) return;
+  if (tid == 0) last = atomicAdd(S.jcount, 1) == ntile - 1;
+  __syncthreads();
+  if (!last || warp >= 3) return;
   __threadfence();
-  double J[3];
-  bool finite = true;
-  for (int ax = 0; ax < 3; ++ax) {
-    double t = 0.0;
-    for (int y = 0; y < ntile; ++y) t += __ldcg(S.jtile + 3 * y + ax);
-    J[ax] = -t / (c.omega * S.n_k);
-    finite = finite && isfinite(J[ax]);
-  }
-  *S.jcount = 0;
-  if (!finite) *S.status |= 1;
+  double t = 0.0;
+  for (int y = lane; y < ntile; y += 32) t += __ldcg(S.jtile + 3 * y + warp);
+  for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+  if (lane != 0) return;
+  const double J = t * (c.occ * S.j_scale);
+  if (!isfinite(J)) atomicOr(S.status, 1);
   if (write_j) {
     double* dst = (mode == TSBZ_FIN_J0MINUS) ? S.J0m : (mode == TSBZ_FIN_J0PLUS ? S.J : S.J + 3LL * (step + 1));
-    for (int ax = 0; ax < 3; ++ax) dst[ax] = J[ax];
+    dst[warp] = J;
   }
-  if (mode == TSBZ_FIN_STEP) *S.step = step + 1;
+  if (warp == 0) {
+    *S.jcount = 0;
+    if (mode == TSBZ_FIN_STEP) *S.step = step + 1;
+  }
 }
 
 // ----------------------------------------------------------------------------
@@ -1349,7 +1326,7 @@ void launch_finalize_t(const SubDev* subs, int n_subs, const UnitDev* units, con
   if (n_subs == 0) return;
   // n_tiles (16 .. TSBZ_FIN_MAX_TILES) tiles per sub-simulation: density points, and units for the
   // current and the norms
-  k_finalize<T><<<dim3(n_subs, n_tiles), 256, 0, (cudaStream_t)stream>>>(subs, units, cells_dev, q_obs, (const V*)Pa,
+  k_finalize<T><<<dim3(n_subs, n_tiles), FIN_THREADS, 0, (cudaStream_t)stream>>>(subs, units, cells_dev, q_obs, (const V*)Pa,
                                                                          rho_part, jk_part, nrm_part, mask, mode);
 }
 

@@ -186,16 +186,20 @@ bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int sam
   return true;
 }
 
+bool observe_fused_ok(const CellDev& c) {
+  return sep_supported(c) && c.n1 == 16 && c.n2 == 16 && c.n3 == 16 && c.n_bands <= FO_MAXB;
+}
+
 bool launch_observe_fused(const LaunchSet& L, const void* psi, double* rho_part, double* jk_part, double* nrm_part,
                           void* stream) {
   const CellDev& c = L.cell;
-  if (L.n_units == 0 || c.n1 != 16 || c.n2 != 16 || c.n3 != 16 || c.n_bands > FO_MAXB) return false;
+  if (L.n_units == 0 || !observe_fused_ok(c)) return false;
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_observe_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FoSmem));
     attr = true;
   }
-  k_observe_fused<<<L.n_units, FS_NP, sizeof(FoSmem), (cudaStream_t)stream>>>(L, (const float2*)psi, rho_part,
+  k_observe_fused<<<dim3(L.n_units, c.n_bgroups), FS_NP, sizeof(FoSmem), (cudaStream_t)stream>>>(L, (const float2*)psi, rho_part,
                                                                               jk_part, nrm_part);
   return true;
 }

@@ -496,8 +496,8 @@ __global__ void __launch_bounds__(SL_T) k_bra_slab(LaunchSet L, const float2* __
 }
 
 // ----------------------------------------------------------------------------
-// Observation on the slab layout: one CTA per (unit, band group of TSBZ_BG
-// bands, slab of 8 rows, block of SO_ZP planes), one thread per column of the
+// Observation on the slab layout: one CTA per (unit, band group of at most
+// TSBZ_BG bands, slab of 8 rows, block of SO_ZP planes), one thread per column of the
 // slab.  The bands of the group stream through a ring of plane slabs (the
 // slab's rows and the next 4 rows, periodic in y; the block's planes and the
 // next 4, periodic in z) filled by bulk copies in one continuous sequence
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(SL_T) k_bra_slab(LaunchSet L, const float2* __
 // the norm.  The density sums over the group's bands in float per point, as the
 // point-parallel form does; the current sums over bands with two-sums.
 // Outputs: rho_part of the group on the block's points, jk_part and nrm_part of
-// point tile slab * (n3 / SO_ZP) + block (zeros in the tiles beyond them).
+// point tile slab * (n3 / SO_ZP) + block.
 // ----------------------------------------------------------------------------
 #define SO_RY (SL_SY + SL_ND)          // staged rows: the slab's and 4 forward
 #define SO_PL (SO_RY * SL_N1)
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(SL_T, 3) k_observe_slab(LaunchSet L, const flo
   const UnitDev U = L.units[u];
   const SubDev S = L.subs[U.sub];
   const int tid = threadIdx.x, ix = tid & (SL_N1 - 1), ry = tid / SL_N1, lane = tid & 31, warp = tid >> 5;
-  const int b0 = grp * TSBZ_BG, nbg = min(TSBZ_BG, c.n_bands - b0);
+  const int b0 = grp * c.obs_bg, nbg = min(c.obs_bg, c.n_bands - b0);
   const float2* gbase = psi + U.psi_off + (long long)b0 * npts;
   const long long qend = (long long)nbg * np;   // sequence elements of the group
   if (tid == 0) {
@@ -685,17 +685,6 @@ __global__ void __launch_bounds__(SL_T, 3) k_observe_slab(LaunchSet L, const flo
     for (int w = 0; w < SL_T / 32; ++w) sum += (double)sm.nrm[w][bl];
     nrm_part[U.nrm_off + (long long)pt * c.n_bands + b0 + bl] = sum;
   }
-  // tiles beyond the kernel's hold nothing of this group
-  if (pt == 0) {
-    for (int i = tid; i < (c.n_tiles - n_pt) * 3; i += SL_T) {
-      const int t = n_pt + i / 3, ax = i - (i / 3) * 3;
-      jk_part[U.jk_off + ((long long)t * c.n_bgroups + grp) * 3 + ax] = 0.0;
-    }
-    for (int i = tid; i < (c.n_tiles - n_pt) * nbg; i += SL_T) {
-      const int t = n_pt + i / nbg, bl = i - (i / nbg) * nbg;
-      nrm_part[U.nrm_off + (long long)t * c.n_bands + b0 + bl] = 0.0;
-    }
-  }
 }
 
 }  // namespace
@@ -766,11 +755,15 @@ bool launch_bra_slab(const LaunchSet& L, const void* src, void* out, int with_d,
   return true;
 }
 
+int observe_slab_tiles(const CellDev& c) {
+  return slab_supported(c) && c.n3 % SO_ZP == 0 ? (c.n2 / SL_SY) * (c.n3 / SO_ZP) : 0;
+}
+
 bool launch_observe_slab(const LaunchSet& L, const void* psi, double* rho_part, double* jk_part, double* nrm_part,
                          void* stream) {
   const CellDev& c = L.cell;
-  const int n_pt = (c.n2 / SL_SY) * (c.n3 / SO_ZP);
-  if (!slab_supported(c) || c.n3 % SO_ZP != 0 || c.n_tiles < n_pt) return false;
+  const int n_pt = observe_slab_tiles(c);
+  if (n_pt == 0) return false;
   if (L.n_units == 0) return true;
   const size_t smem = sizeof(SoSmem);
   cudaFuncSetAttribute(k_observe_slab, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

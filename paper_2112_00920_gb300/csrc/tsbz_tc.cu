@@ -70,10 +70,12 @@ void launch_stage_v(const LaunchSet& L, const void* tin, void* tout, void* psi, 
                                                                       (float2*)psi, (const float2*)V, m);
 }
 
+bool observe_zf_ok(const CellDev& c) { return c.n3 == 16 && c.n1 <= 16 && c.n2 <= 16 && c.n_bgroups == 1; }
+
 bool launch_observe_zf(const LaunchSet& L, const void* psi, double* rho_part, double* jk_part, double* nrm_part,
                        void* stream) {
   const int n12 = L.cell.n1 * L.cell.n2;
-  if (L.cell.n3 != 16 || L.cell.n1 > 16 || L.cell.n2 > 16 || L.cell.n_bgroups != 1 || L.n_units == 0) return false;
+  if (!observe_zf_ok(L.cell) || L.n_units == 0) return false;
   const int threads = ((n12 + 31) / 32) * 32;
   k_observe_zf<16><<<L.n_units, threads, 0, (cudaStream_t)stream>>>(L, (const float2*)psi, rho_part, jk_part,
                                                                     nrm_part);

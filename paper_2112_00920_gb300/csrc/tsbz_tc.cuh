@@ -621,8 +621,7 @@ __global__ void __launch_bounds__(ZB_NP, VP ? 2 : 3) k_stage_zb(LaunchSet L, con
 // per unit, one thread per (x, y) column; bands outer, z-march inner.  Per
 // column and plane it accumulates occ sum_b |u|^2 (rho) over the bands, and
 // per thread sum Re(u* (-i grad u)) and per band sum |u|^2 (block-reduced per
-// band).  The unit's sums are written to point tile 0 of the partial
-// buffers and zeros to the other tiles, which the finalize kernel adds.
+// band).  Point tile 0 of the partial buffers is the only one.
 // ----------------------------------------------------------------------------
 template <int NZ>
 __global__ void __launch_bounds__(256) k_observe_zf(LaunchSet L, const float2* __restrict__ psi,
@@ -717,8 +716,4 @@ __global__ void __launch_bounds__(256) k_observe_zf(LaunchSet L, const float2* _
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += redj[w][threadIdx.x];
     jk_part[U.jk_off + threadIdx.x] = sum;
   }
-  // zeros for the other point tiles of the partial layout
-  for (int i = threadIdx.x; i < 3 * (c.n_tiles - 1); i += blockDim.x) jk_part[U.jk_off + 3 + i] = 0.0;
-  for (int i = threadIdx.x; i < c.n_bands * (c.n_tiles - 1); i += blockDim.x)
-    nrm_part[U.nrm_off + c.n_bands + i] = 0.0;
 }
