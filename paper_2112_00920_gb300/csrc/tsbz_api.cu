@@ -569,10 +569,11 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
       }
       const int same_next = (same_next_allowed && cell_field_const(ctx, hc)) ? 1 : 0;
       ev_start(ctx, FAM_STAGE);
-      const bool whole = launch_step_fused(L, ctx->psi, ctx->P, ctx->Pa, same_next, ctx->stream);
+      const bool whole = launch_step_fused(L, ctx->psi, ctx->P, ctx->Pa, same_next, want_pa ? 1 : 0,
+                                           ctx->stream);
       ev_stop(ctx);
       if (whole) {
-        hc.pa_by_stage = true;
+        hc.pa_by_stage = want_pa;
         ++ctx->launches;
         continue;
       }
@@ -1020,6 +1021,7 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
   c.n_bgroups = (c.n_bands + TSBZ_BG - 1) / TSBZ_BG;
   c.omega = d->a[0] * d->a[1] * d->a[2];
   c.dv = c.omega / (double)npts;
+  c.dvf = (float)c.dv;
   c.occ = d->occ;
   double cw[TSBZ_MAX_ND + 1], dw[TSBZ_MAX_ND + 1];
   tsbz::fd_weights(d->fd_nd, cw, dw);
@@ -1218,6 +1220,11 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
     if ((rc = dalloc_t(ctx, ks.size(), &kd))) return rc;
     CK(cudaMemcpy(kd, ks.data(), sizeof(double) * ks.size(), cudaMemcpyHostToDevice));
     c.ksym = kd;
+    const std::vector<float> ksf = to_f(ks);
+    float* kf = nullptr;
+    if ((rc = dalloc_t(ctx, ksf.size(), &kf))) return rc;
+    CK(cudaMemcpy(kf, ksf.data(), sizeof(float) * ksf.size(), cudaMemcpyHostToDevice));
+    c.ksymf = kf;
   }
   c.poisson = nullptr;
   if (c.n1 * c.n3 <= TSBZ_HXC_MAX_PLANE) {

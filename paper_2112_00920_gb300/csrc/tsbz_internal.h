@@ -49,6 +49,7 @@ struct CellDev {
   const double* wkb;    // [n_proj]            pnorm_j * E_j
   const double* vloc;   // [npts]
   // the same tables in float for the single-precision kernels
+  float dvf;
   const float* g1f;
   const float* d1f;
   const float* pnormf;
@@ -76,6 +77,7 @@ struct CellDev {
   // kinetic symbol per axis: [3][2][nmax], row 0 the eigenvalues of -1/2 lap_FD on
   // exp(2 pi i k j / n), row 1 those of -i grad_FD (times q in h)
   const double* ksym;
+  const float* ksymf;
   // 4 pi / (G^2 n_pts) (0 at G = 0), [n2 / 2 + 1][n3][n1]; null when an x-z plane is
   // too large for the v_Hxc kernels that work plane by plane
   const double* poisson;
@@ -246,7 +248,8 @@ bool sep_supported(const CellDev& c);
 int sep_variants(const CellDev& c);   // kernel variants of the single-precision path on this cell
 // The whole time step of every unit in one launch (16^3 cells with z groups,
 // variant 0); false when the cell takes the per-stage kernels.
-bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int same_next, void* stream);
+// want_pa: the projections of the current (and of the next step) follow from psi.
+bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int same_next, int want_pa, void* stream);
 void launch_bra_sep(const LaunchSet& L, const void* src, void* out, int with_d, int use_obs, void* stream);
 // stage 4 on the bulk-staged path also writes P (next step) and Pa; returns whether it did
 // same_next: the field is constant, so at m = 4 the next step's projections come from the current's sums

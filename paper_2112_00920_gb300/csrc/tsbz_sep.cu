@@ -2,6 +2,7 @@
 #include "tsbz_internal.h"
 #include "tsbz_sep.cuh"
 #include "tsbz_fused.cuh"
+#include "tsbz_step32.cuh"
 
 // The 16^3 fused kernels run their z contractions per z group when the cell's
 // atoms occupy at most 4 distinct z tables with at most two atoms each (NZU = 4),
@@ -63,39 +64,34 @@ void launch_bra_sep(const LaunchSet& L, const void* src, void* out, int with_d, 
     // the projections the 16^3 fused stage leaves are formed by the same pass
     static bool attr = false;
     if (!attr) {
-      fs_attr(k_bra_fused<4, true>, sizeof(FsSmem));
-      fs_attr(k_bra_fused<4, false>, sizeof(FsSmem));
-      fs_attr(k_bra_fused<SEP_NA, false>, sizeof(FsSmem));
+      fs_attr(k_project_fft<false>, sizeof(FxSmem));
+      fs_attr(k_bra_fused<4>, sizeof(FsSmem));
+      fs_attr(k_bra_fused<SEP_NA>, sizeof(FsSmem));
       attr = true;
     }
     if (fs_grouped(c) && fs_umma(L))
-      k_bra_fused<4, true><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src,
-                                                                                (float2*)out);
+      k_project_fft<false><<<grid, FX_NP, sizeof(FxSmem), (cudaStream_t)stream>>>(L, (const float2*)src, (float2*)out);
     else if (fs_grouped(c))
-      k_bra_fused<4, false><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src,
-                                                                                 (float2*)out);
+      k_bra_fused<4><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src, (float2*)out);
     else
-      k_bra_fused<SEP_NA, false><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src,
-                                                                                        (float2*)out);
+      k_bra_fused<SEP_NA><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src, (float2*)out);
     return;
   }
   if (stage_kind(L) <= 1 && with_d && use_obs && fs_cube16(c)) {
     // the current's projections by the second-order pass of the fused stage 4
     static bool attr_pa = false;
     if (!attr_pa) {
-      fs_attr(k_pa_fused<4, true>, sizeof(FsSmem));
-      fs_attr(k_pa_fused<4, false>, sizeof(FsSmem));
-      fs_attr(k_pa_fused<SEP_NA, false>, sizeof(FsSmem));
+      fs_attr(k_project_fft<true>, sizeof(FxSmem));
+      fs_attr(k_pa_fused<4>, sizeof(FsSmem));
+      fs_attr(k_pa_fused<SEP_NA>, sizeof(FsSmem));
       attr_pa = true;
     }
     if (fs_grouped(c) && fs_umma(L))
-      k_pa_fused<4, true><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src, (float2*)out);
+      k_project_fft<true><<<grid, FX_NP, sizeof(FxSmem), (cudaStream_t)stream>>>(L, (const float2*)src, (float2*)out);
     else if (fs_grouped(c))
-      k_pa_fused<4, false><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src,
-                                                                                (float2*)out);
+      k_pa_fused<4><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src, (float2*)out);
     else
-      k_pa_fused<SEP_NA, false><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src,
-                                                                                       (float2*)out);
+      k_pa_fused<SEP_NA><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (const float2*)src, (float2*)out);
     return;
   }
   const unsigned thr = sep_threads(L.cell);
@@ -168,21 +164,21 @@ bool launch_stage_sep(const LaunchSet& L, const void* tin, void* tout, void* psi
   return false;
 }
 
-bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int same_next, void* stream) {
+bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int same_next, int want_pa, void* stream) {
   if (L.n_units == 0 || stage_kind(L) != 0) return false;
   static bool attr = false;
   if (!attr) {
-    fs_attr(k_step_fused<4, true>, sizeof(FsSmem));
-    fs_attr(k_step_fused<4, false>, sizeof(FsSmem));
+    fs_attr(k_step_fft, sizeof(FxSmem));
+    fs_attr(k_step_fused<4>, sizeof(FsSmem));
     attr = true;
   }
   const unsigned grid = (unsigned)L.n_units * (unsigned)L.cell.n_bands;
   if (fs_umma(L))
-    k_step_fused<4, true><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P,
-                                                                                (float2*)Pa, same_next);
+    k_step_fft<<<grid, FX_NP, sizeof(FxSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P, (float2*)Pa,
+                                                                      same_next, want_pa);
   else
-    k_step_fused<4, false><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P,
-                                                                                 (float2*)Pa, same_next);
+    k_step_fused<4><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P, (float2*)Pa,
+                                                                           same_next);
   return true;
 }
 
