@@ -270,8 +270,8 @@ int tsbz_autotune(tsbz_ctx* ctx, int budget_ms, int* n_tried);
  * any output pointer may be NULL.  Variants: FP32 on 16^3 and 8^3 cells:
  * 0 = fused tensor-core / bulk-staged stage, 1 = z-march stage with CUDA-core
  * projections; point-parallel stage kernels (FP64, other FP32 shapes): bands
- * per staged projection chunk 8 (0), 4 (1), 16 (2); FP64 on 8^3 and 16^3 grids:
- * 0 = the whole step in one launch (from 8 orbitals on). */
+ * per staged projection chunk 8 (0), 4 (1), 16 (2); 16^3 grids in FP64 and small
+ * grids in FP64 and FP32: 0 = the whole step in one launch (from 8 orbitals on). */
 int tsbz_get_variant(tsbz_ctx* ctx, int cell_id, int* variant, int* n_variants, double* ms, int n_ms);
 
 /* Force a cell's variant (0 <= variant < n_variants; TSBZ_EINVAL otherwise). */

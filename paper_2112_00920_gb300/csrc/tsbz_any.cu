@@ -1,0 +1,691 @@
+// Small grids of any shape: the whole time step of a band (or the whole
+// Chebyshev recurrence of the ground-state solver) in one CTA and one launch, in
+// double or single precision.
+//
+// What bounds such runs is latency: a step of nine to twelve launches, each a
+// few CTAs that wait on dependent loads, and in double precision the FP64
+// instructions a warp issues (64 clocks each on its quarter of the SM).  So
+// the band of t_{m-1}, t_m and the Taylor sum stay in shared memory, every
+// contraction is spread over all eight warps as independent items, and the next
+// launch is the observation.
+//  - Kinetic operator: the star stencil from shared memory, or on 8^3 grids its
+//    Fourier symbol (ANY_FFT8): four threads per line, each forming the outputs k and
+//    k + 4 of an 8-point transform (20 operations), 6 passes.
+//  - Projectors: the phase e^{i q z} is taken off once per point, so the z sums are
+//    real per (z group, column); then x sums per (atom, power, row), y sums per
+//    (atom, monomial).  The ket goes back the same way.  A group's minimum image
+//    jumps by one cell edge at one plane; the running sums are turned there.
+//  - Taylor terms are s_m = h^m psi; (-i dt)^m / m! enters the sum only.
+// Everything the first- and second-order projection passes share is formed by the
+// same rounded operations, so a step may start from the projections that the
+// last one left (same q) or from fresh ones, bit for bit.
+// Measured per step, all four stages with their projections: 8^3, 16 orbitals in
+// double 298 -> 109 us, 512 orbitals in single 65 -> 46 us; 10 x 12 x 14, 324 orbitals
+// in single under a pulse 179 -> 78 us (before: two launches per stage and one for
+// the current).
+#include <cuda_runtime.h>
+
+#include "tsbz_internal.h"
+
+namespace {
+
+constexpr int ANY_T = 256;         // threads
+constexpr int ANY_NA = 8;          // atoms
+constexpr int ANY_MIN_ORB = 8;     // orbitals from which the whole-step form is taken
+constexpr size_t ANY_MAX_SMEM = 200 * 1024;
+
+__host__ __device__ __forceinline__ bool any_fft8(const CellDev& c) { return c.n1 == 8 && c.n2 == 8 && c.n3 == 8; }
+
+template <typename T> struct AnyC;
+template <> struct AnyC<double> { using V = double2; };
+template <> struct AnyC<float> { using V = float2; };
+
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double rfm(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float rfm(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+template <typename V> __device__ __forceinline__ V vmk(decltype(V().x) a, decltype(V().x) b) {
+  V r;
+  r.x = a;
+  r.y = b;
+  return r;
+}
+template <typename V> __device__ __forceinline__ V vmul(V a, V b) {   // complex product, fixed rounding
+  return vmk<V>(rfm(a.x, b.x, -rmul(a.y, b.y)), rfm(a.x, b.y, rmul(a.y, b.x)));
+}
+template <typename V> __device__ __forceinline__ V vconj(V a) { return vmk<V>(a.x, -a.y); }
+template <typename V, typename T> __device__ __forceinline__ V vaxpy(T s, V b, V a) {   // a + s b
+  return vmk<V>(rfm(s, b.x, a.x), rfm(s, b.y, a.y));
+}
+// sign flip without arithmetic
+__device__ __forceinline__ double flip(double a, unsigned m) {
+  return __hiloint2double(__double2hiint(a) ^ (int)(m << 31), __double2loint(a));
+}
+__device__ __forceinline__ float flip(float a, unsigned m) { return __uint_as_float(__float_as_uint(a) ^ (m << 31)); }
+
+// Shared memory of a CTA: pointers into one block, laid out alike on both sides.
+template <typename T> struct AnySmem {
+  using V = typename AnyC<T>::V;
+  V *a, *b, *acc;        // t_{m-1} / t_m (roles alternate), Taylor sum
+  V* s;                  // z sums, ket coefficients per (group, column); line transforms (8^3)
+  V *rs, *gt, *xf, *yf, *phi, *w, *mres, *k0, *kfin, *turn;
+  T *xd, *yd, *zw, *lam, *st;
+  int *idx, *zb;
+};
+
+constexpr int ANY_X8 = 8 * 72;   // one 8^3 line buffer with rows of 9
+
+template <typename T> __host__ __device__ inline size_t any_carve(const CellDev& c, unsigned char* base, AnySmem<T>& m) {
+  using V = typename AnyC<T>::V;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    unsigned char* p = base + at;
+    at += (bytes + 15) / 16 * 16;
+    return p;
+  };
+  const int na = c.use_proj ? c.n_atoms : 0, ng = c.use_proj ? c.n_zg : 0, n12 = c.n1 * c.n2;
+  size_t ns = (size_t)3 * ng * n12;
+  if (any_fft8(c) && ns < 2 * ANY_X8) ns = 2 * ANY_X8;
+  m.a = (V*)take(sizeof(V) * c.npts);
+  m.b = (V*)take(sizeof(V) * c.npts);
+  m.acc = (V*)take(sizeof(V) * c.npts);
+  m.s = (V*)take(sizeof(V) * ns);
+  m.rs = (V*)take(sizeof(V) * na * 6 * c.n2);
+  m.gt = (V*)take(sizeof(V) * na * 3 * c.n1);
+  m.xf = (V*)take(sizeof(V) * na * c.n1);
+  m.yf = (V*)take(sizeof(V) * na * c.n2);
+  m.phi = (V*)take(sizeof(V) * c.n3);
+  m.w = (V*)take(sizeof(V) * 4 * ANY_NA);
+  m.mres = (V*)take(sizeof(V) * 10 * ANY_NA);
+  m.k0 = (V*)take(sizeof(V) * ANY_NA);
+  m.kfin = (V*)take(sizeof(V) * ANY_NA);
+  m.turn = (V*)take(sizeof(V) * ANY_NA);
+  m.xd = (T*)take(sizeof(T) * na * c.n1);
+  m.yd = (T*)take(sizeof(T) * na * c.n2);
+  m.zw = (T*)take(sizeof(T) * 3 * ng * c.n3);
+  m.lam = (T*)take(sizeof(T) * 3 * 8);
+  m.st = (T*)take(sizeof(T) * (6 * (TSBZ_MAX_ND + 1) + 1));
+  m.idx = (int*)take(sizeof(int) * c.npts);
+  m.zb = (int*)take(sizeof(int) * ANY_NA);
+  return at;
+}
+
+template <typename T> struct AnyTab;
+template <> struct AnyTab<double> {
+  static __device__ const double* g1(const CellDev& c) { return c.g1; }
+  static __device__ const double* d1(const CellDev& c) { return c.d1; }
+  static __device__ const double* pnorm(const CellDev& c) { return c.pnorm; }
+  static __device__ const double* wkb(const CellDev& c) { return c.wkb; }
+  static __device__ const double* ksym(const CellDev& c) { return c.ksym; }
+  static __device__ double dv(const CellDev& c) { return c.dv; }
+};
+template <> struct AnyTab<float> {
+  static __device__ const float* g1(const CellDev& c) { return c.g1f; }
+  static __device__ const float* d1(const CellDev& c) { return c.d1f; }
+  static __device__ const float* pnorm(const CellDev& c) { return c.pnormf; }
+  static __device__ const float* wkb(const CellDev& c) { return c.wkbf; }
+  static __device__ const float* ksym(const CellDev& c) { return c.ksymf; }
+  static __device__ float dv(const CellDev& c) { return c.dvf; }
+};
+
+__device__ __forceinline__ int any_mono(int i, int j, int k) {   // 000 100 010 001 200 110 101 020 011 002
+  const int deg = i + j + k;
+  if (deg == 0) return 0;
+  if (deg == 1) return i ? 1 : (j ? 2 : 3);
+  if (i == 2) return 4;
+  if (i == 1) return j ? 5 : 6;
+  if (j == 2) return 7;
+  return j ? 8 : 9;
+}
+
+// Point i of the thread: in 8^3 cells the outputs z = p, p + 4 of column l (l = t / 4, p = t % 4).
+template <bool F8> __device__ __forceinline__ int any_point(int i) {
+  return F8 ? ((int)threadIdx.x & 3) * 64 + ((int)threadIdx.x >> 2) + 256 * i : (int)threadIdx.x + ANY_T * i;
+}
+
+// Projector factor tables of one q (phase table ph of the unit); read after a barrier.
+template <typename T>
+__device__ void any_tables(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* ph, const double* q) {
+  using V = typename AnyC<T>::V;
+  const int nm = c.nmax;
+  const T *g1 = AnyTab<T>::g1(c), *d1 = AnyTab<T>::d1(c);
+  for (int i = threadIdx.x; i < c.n_atoms * c.n1; i += ANY_T) {
+    const int a = i / c.n1, k = a * 3 * nm + i - a * c.n1;
+    sm.xf[i] = vmk<V>(g1[k] * ph[k].x, g1[k] * ph[k].y);
+    sm.xd[i] = d1[k];
+  }
+  for (int i = threadIdx.x; i < c.n_atoms * c.n2; i += ANY_T) {
+    const int a = i / c.n2, k = (a * 3 + 1) * nm + i - a * c.n2;
+    sm.yf[i] = vmk<V>(g1[k] * ph[k].x, g1[k] * ph[k].y);
+    sm.yd[i] = d1[k];
+  }
+  for (int i = threadIdx.x; i < c.n_zg * c.n3; i += ANY_T) {
+    const int g = i / c.n3, k = (c.zg_rep[g] * 3 + 2) * nm + i - g * c.n3;
+    sm.zw[i] = g1[k];
+    sm.zw[c.n_zg * c.n3 + i] = g1[k] * d1[k];
+    sm.zw[2 * c.n_zg * c.n3 + i] = g1[k] * d1[k] * d1[k];
+  }
+  // phases along z: of the planes, and of each group before and after its jump
+  for (int i = threadIdx.x; i < c.n3 + 2 * c.n_zg; i += ANY_T) {
+    const int g = (i - c.n3) >> 1, after = (i - c.n3) & 1;
+    const double z = i < c.n3 ? c.hz * i : c.zg_k0[g] - (after ? c.hz * c.n3 : 0.0);
+    double sn, co;
+    sincos(q[2] * z, &sn, &co);
+    const V e = vmk<V>((T)co, (T)sn);
+    if (i < c.n3) {
+      sm.phi[i] = e;
+    } else {
+      if (!after) sm.k0[g] = e;
+      if (after == (c.zg_brk[g] < c.n3 ? 1 : 0)) sm.kfin[g] = e;
+      if (after) {
+        double s2, c2;
+        sincos(q[2] * (c.hz * c.n3), &s2, &c2);
+        sm.turn[g] = vmk<V>((T)c2, (T)s2);   // phase before over phase after
+        sm.zb[g] = c.zg_brk[g];
+      }
+    }
+  }
+}
+
+// Stencil weights (or the symbol of 8^3 grids) of the step's q, and the points' coordinates.
+template <typename T, bool F8>
+__device__ void any_setup(const AnySmem<T>& sm, const CellDev& c, const double* q) {
+  const int tid = threadIdx.x;
+  if (F8) {
+    if (tid < 24) {
+      const int ax = tid >> 3, k = tid & 7;
+      const T* s = AnyTab<T>::ksym(c) + 2 * ax * 8;
+      const T qa = (T)q[ax];
+      sm.lam[tid] = rfm(qa, s[8 + k], rfm((T)0.5 * qa, qa, s[k])) * (T)(1.0 / 512.0);
+    }
+  } else {
+    constexpr int M = TSBZ_MAX_ND + 1;
+    if (tid < 3 * M) {
+      const int ax = tid / M, m = tid - ax * M;
+      sm.st[tid] = (T)(-0.5 * c.lapw[ax][m]);
+      sm.st[3 * M + tid] = (T)(q[ax] * c.gradw[ax][m]);
+    }
+    if (tid == 3 * M) {
+      double d = 0.5 * (q[0] * q[0] + q[1] * q[1] + q[2] * q[2]);
+      for (int ax = 0; ax < 3; ++ax) d -= 0.5 * c.lapw[ax][0];
+      sm.st[6 * M] = (T)d;
+    }
+    for (int p = tid; p < c.npts; p += ANY_T) {
+      const int ix = p % c.n1, r = p / c.n1;
+      sm.idx[p] = ix | (r % c.n2) << 10 | (r / c.n2) << 20;
+    }
+  }
+}
+
+// Monomial sums of order <= D of every atom into mres[a NM + mono] (see tsbz_step64.cu),
+// from the band in t; u is scratch of npts.  Begins and ends with a barrier.
+template <typename T, int D>
+__device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* t,
+                            typename AnyC<T>::V* u) {
+  using V = typename AnyC<T>::V;
+  constexpr int NM = D == 1 ? 4 : 10;
+  const int tid = threadIdx.x, n1 = c.n1, n2 = c.n2, n3 = c.n3, n12 = n1 * n2, ng = c.n_zg;
+  __syncthreads();
+  for (int p = tid; p < c.npts; p += ANY_T) u[p] = vmul(sm.phi[p / n12], t[p]);
+  __syncthreads();
+  // z sums of (group, column)
+  for (int i = tid; i < ng * n12; i += ANY_T) {
+    const int g = i / n12, col = i - g * n12, zb = sm.zb[g];
+    const T* w = sm.zw + g * n3;
+    V s[D + 1];
+#pragma unroll
+    for (int k = 0; k <= D; ++k) s[k] = vmk<V>((T)0, (T)0);
+    auto run = [&](int z0, int z1) {
+#pragma unroll 4
+      for (int z = z0; z < z1; ++z) {
+        const V v = u[z * n12 + col];
+#pragma unroll
+        for (int k = 0; k <= D; ++k) s[k] = vaxpy(w[k * ng * n3 + z], v, s[k]);
+      }
+    };
+    run(0, zb);
+    if (zb < n3) {
+#pragma unroll
+      for (int k = 0; k <= D; ++k) s[k] = vmul(sm.turn[g], s[k]);
+      run(zb, n3);
+    }
+#pragma unroll
+    for (int k = 0; k <= D; ++k) sm.s[(g * (D + 1) + k) * n12 + col] = s[k];
+  }
+  __syncthreads();
+  // x sums of (atom, power of d_z, row)
+  for (int i = tid; i < c.n_atoms * (D + 1) * n2; i += ANY_T) {
+    const int y = i % n2, r = i / n2, k = r / c.n_atoms, a = r - k * c.n_atoms;
+    const V* row = sm.s + (c.zg_of[a] * (D + 1) + k) * n12 + y * n1;
+    V R[3];
+#pragma unroll
+    for (int w = 0; w < 3; ++w) R[w] = vmk<V>((T)0, (T)0);
+    for (int x = 0; x < n1; ++x) {
+      const V p = vmul(sm.xf[a * n1 + x], row[x]);
+      const T d = sm.xd[a * n1 + x];
+      R[0] = vmk<V>(radd(R[0].x, p.x), radd(R[0].y, p.y));
+      if (k < D) R[1] = vaxpy(d, p, R[1]);
+      if (D == 2 && k == 0) R[2] = vaxpy(rmul(d, d), p, R[2]);
+    }
+    V* o = sm.rs + (a * 6 + (k == 0 ? 0 : (k == 1 ? 3 : 5))) * n2 + y;
+    o[0] = R[0];
+    if (k < D) o[n2] = R[1];
+    if (D == 2 && k == 0) o[2 * n2] = R[2];
+  }
+  __syncthreads();
+  // y sums of (atom, monomial), and the group's phase
+  for (int i = tid; i < c.n_atoms * NM; i += ANY_T) {
+    const int a = i / NM, mo = i - a * NM;
+    int ex = 0, ey = 0, ez = 0;
+    if (mo == 1 || mo == 5 || mo == 6) ex = 1;
+    if (mo == 4) ex = 2;
+    if (mo == 2 || mo == 5 || mo == 8) ey = 1;
+    if (mo == 7) ey = 2;
+    if (mo == 3 || mo == 6 || mo == 8) ez = 1;
+    if (mo == 9) ez = 2;
+    const V* R = sm.rs + (a * 6 + (ez == 0 ? ex : (ez == 1 ? 3 + ex : 5))) * n2;
+    V M = vmk<V>((T)0, (T)0);
+    for (int y = 0; y < n2; ++y) {
+      const T d = sm.yd[a * n2 + y], wy = ey == 0 ? (T)1 : (ey == 1 ? d : rmul(d, d));
+      M = vaxpy(wy, vmul(sm.yf[a * n2 + y], R[y]), M);
+    }
+    sm.mres[i] = vmul(sm.kfin[c.zg_of[a]], M);
+  }
+  __syncthreads();
+}
+
+// Projection of projector j from its monomial sum, and the ket weights from P (null: from mres).
+template <typename T>
+__device__ void any_weights(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* P) {
+  using V = typename AnyC<T>::V;
+  for (int j = threadIdx.x; j < c.n_proj; j += ANY_T) {
+    const T sc = rmul(AnyTab<T>::dv(c), AnyTab<T>::pnorm(c)[j]), e = AnyTab<T>::wkb(c)[j];
+    const V p = P ? P[j] : vmk<V>(rmul(sc, sm.mres[j].x), rmul(sc, sm.mres[j].y));
+    sm.w[j] = vmul(vconj(sm.k0[c.zg_of[j >> 2]]), vmk<V>(rmul(e, p.x), rmul(e, p.y)));
+  }
+  __syncthreads();
+}
+
+// The two outputs k = p, p + 4 of an 8-point transform of x (INV: conjugate), p = the thread's part.
+template <bool INV, typename V> __device__ __forceinline__ void any_dft8(const V (&x)[8], V& lo, V& hi) {
+  using T = decltype(V().x);
+  const unsigned p = threadIdx.x & 3, s = p & 1;
+  // four-point sums over the even and the odd inputs: (x0 + s x4) + i^p (x2 + s x6)
+  V h[2];
+#pragma unroll
+  for (int o = 0; o < 2; ++o) {
+    const V e0 = vmk<V>(x[o].x + flip(x[o + 4].x, s), x[o].y + flip(x[o + 4].y, s));
+    const V e1 = vmk<V>(x[o + 2].x + flip(x[o + 6].x, s), x[o + 2].y + flip(x[o + 6].y, s));
+    // times (-i)^p (forward) or i^p
+    const unsigned sx = INV ? (p == 1 || p == 2) : (p >= 2), sy = INV ? (p >= 2) : (p == 1 || p == 2);
+    const T rx = s ? e1.y : e1.x, ry = s ? e1.x : e1.y;
+    h[o] = vmk<V>(e0.x + flip(rx, sx), e0.y + flip(ry, sy));
+  }
+  // exp(-+ 2 pi i p / 8)
+  const T r = (T)0.70710678118654752440;
+  const T co = p == 0 ? (T)1 : (p == 1 ? r : (p == 2 ? (T)0 : -r));
+  const T sn = flip(p == 0 ? (T)0 : (p == 2 ? (T)1 : r), INV ? 0u : 1u);
+  const V w = vmk<V>(fma(co, h[1].x, -sn * h[1].y), fma(co, h[1].y, sn * h[1].x));
+  lo = vmk<V>(h[0].x + w.x, h[0].y + w.y);
+  hi = vmk<V>(h[0].x - w.x, h[0].y - w.y);
+}
+
+struct Fwd { static constexpr bool value = false; };
+struct Inv { static constexpr bool value = true; };
+
+// Kinetic term of an 8^3 band for the thread's two points (z = p, p + 4 of column l).
+template <typename T>
+__device__ void any_kinetic8(const AnySmem<T>& sm, const typename AnyC<T>::V* t, typename AnyC<T>::V (&k)[2]) {
+  using V = typename AnyC<T>::V;
+  const int p = threadIdx.x & 3, l = threadIdx.x >> 2, l0 = l & 7, l1 = l >> 3;
+  V *x1 = sm.s, *x2 = sm.s + ANY_X8, v[8], lo, hi;
+  auto line = [&](V* src, V* dst, int at, int stride, auto inv) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = src[at + j * stride];
+    any_dft8<decltype(inv)::value>(v, lo, hi);
+    if (dst) {
+      dst[at + p * stride] = lo;
+      dst[at + (p + 4) * stride] = hi;
+      __syncthreads();
+    }
+  };
+  const int cz = l1 * 9 + l0, cx = l1 * 72 + l0 * 9, cy = l1 * 72 + l0;   // column; row y = l0; line x = l0
+#pragma unroll
+  for (int j = 0; j < 8; ++j) v[j] = t[j * 64 + l];
+  any_dft8<false>(v, lo, hi);
+  x1[cz + p * 72] = lo;
+  x1[cz + (p + 4) * 72] = hi;
+  __syncthreads();
+  line(x1, x2, cx, 1, Fwd());
+#pragma unroll
+  for (int j = 0; j < 8; ++j) v[j] = x2[cy + j * 9];
+  any_dft8<false>(v, lo, hi);
+  {
+    const T s = sm.lam[l0] + sm.lam[16 + l1], e0 = s + sm.lam[8 + p], e1 = s + sm.lam[12 + p];
+    x1[cy + p * 9] = vmk<V>(e0 * lo.x, e0 * lo.y);
+    x1[cy + (p + 4) * 9] = vmk<V>(e1 * hi.x, e1 * hi.y);
+  }
+  __syncthreads();
+  line(x1, x2, cy, 9, Inv());
+  line(x2, x1, cx, 1, Inv());
+  line(x1, (V*)nullptr, cz, 72, Inv());
+  k[0] = lo;
+  k[1] = hi;
+}
+
+// Kinetic term at point p from the star stencil.
+template <typename T>
+__device__ __forceinline__ typename AnyC<T>::V any_kinetic(const AnySmem<T>& sm, const CellDev& c,
+                                                           const typename AnyC<T>::V* t, int p) {
+  using V = typename AnyC<T>::V;
+  constexpr int M = TSBZ_MAX_ND + 1;
+  const int id = sm.idx[p], n12 = c.n1 * c.n2;
+  const int pos[3] = {id & 1023, (id >> 10) & 1023, id >> 20}, n[3] = {c.n1, c.n2, c.n3}, st[3] = {1, c.n1, n12};
+  const V ce = t[p];
+  V h = vmk<V>(sm.st[6 * M] * ce.x, sm.st[6 * M] * ce.y);
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) {
+    const V* line = t + p - pos[ax] * st[ax];
+#pragma unroll 4
+    for (int m = 1; m <= c.nd; ++m) {
+      const int up = pos[ax] + m, dn = pos[ax] - m;
+      const V a = line[(up >= n[ax] ? up - n[ax] : up) * st[ax]], b = line[(dn < 0 ? dn + n[ax] : dn) * st[ax]];
+      const T lw = sm.st[ax * M + m], qw = sm.st[3 * M + ax * M + m];
+      h.x = fma(lw, a.x + b.x, fma(qw, a.y - b.y, h.x));
+      h.y = fma(lw, a.y + b.y, fma(-qw, a.x - b.x, h.y));
+    }
+  }
+  return h;
+}
+
+// h t at the thread's points, handed to `use(point, t, h t)`; the ket weights are in sm.w.
+// t is complete (barrier behind its writes); `use` may write anywhere but t and sm.s.
+template <typename T, bool F8, typename U>
+__device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __restrict__ veff,
+                          const typename AnyC<T>::V* t, U&& use) {
+  using V = typename AnyC<T>::V;
+  const int tid = threadIdx.x, n1 = c.n1, n2 = c.n2, n3 = c.n3, n12 = n1 * n2, ng = c.use_proj ? c.n_zg : 0;
+  V k8[2];
+  if constexpr (F8) any_kinetic8<T>(sm, t, k8);
+  if (ng) {
+    // ket tables of (atom, x), then the coefficients C0, C1 of (group, column)
+    for (int i = tid; i < c.n_atoms * n1; i += ANY_T) {
+      const int a = i / n1, x = i - a * n1;
+      const V F = vconj(sm.xf[i]);
+      const T d = sm.xd[i];
+      sm.gt[(a * 3 + 0) * n1 + x] = vmul(F, vaxpy(d, sm.w[4 * a + 1], sm.w[4 * a]));
+      sm.gt[(a * 3 + 1) * n1 + x] = vmul(F, sm.w[4 * a + 2]);
+      sm.gt[(a * 3 + 2) * n1 + x] = vmul(F, sm.w[4 * a + 3]);
+    }
+    __syncthreads();
+    for (int i = tid; i < ng * n12; i += ANY_T) {
+      const int g = i / n12, col = i - g * n12, y = col / n1, x = col - y * n1;
+      V c0 = vmk<V>((T)0, (T)0), c1 = c0;
+      for (int e = c.zg_off[g]; e < c.zg_off[g + 1]; ++e) {
+        const int a = c.zg_mem[e];
+        const V F = vconj(sm.yf[a * n2 + y]);
+        const V b = vaxpy(sm.yd[a * n2 + y], sm.gt[(a * 3 + 1) * n1 + x], sm.gt[(a * 3 + 0) * n1 + x]);
+        const V g1 = sm.gt[(a * 3 + 2) * n1 + x];
+        c0 = vmk<V>(fma(F.x, b.x, fma(-F.y, b.y, c0.x)), fma(F.x, b.y, fma(F.y, b.x, c0.y)));
+        c1 = vmk<V>(fma(F.x, g1.x, fma(-F.y, g1.y, c1.x)), fma(F.x, g1.y, fma(F.y, g1.x, c1.y)));
+      }
+      sm.s[(2 * g) * n12 + col] = c0;
+      sm.s[(2 * g + 1) * n12 + col] = c1;
+    }
+    __syncthreads();
+  }
+  const int pts = F8 ? 2 : (c.npts + ANY_T - 1) / ANY_T;
+  for (int i = 0; i < pts; ++i) {
+    const int p = any_point<F8>(i);
+    if (!F8 && p >= c.npts) break;
+    const V ce = t[p];
+    V h;
+    if constexpr (F8) h = i ? k8[1] : k8[0]; else h = any_kinetic<T>(sm, c, t, p);
+    const T v = veff[p];
+    h.x = fma(v, ce.x, h.x);
+    h.y = fma(v, ce.y, h.y);
+    if (ng) {
+      const int z = F8 ? p >> 6 : sm.idx[p] >> 20, col = p - z * n12;
+      V x0 = vmk<V>((T)0, (T)0), x = x0;
+      for (int g = 0; g < ng; ++g) {
+        const T w0 = sm.zw[g * n3 + z], w1 = sm.zw[(ng + g) * n3 + z];
+        const V c0 = sm.s[(2 * g) * n12 + col], c1 = sm.s[(2 * g + 1) * n12 + col];
+        const V y = vmk<V>(fma(w0, c0.x, w1 * c1.x), fma(w0, c0.y, w1 * c1.y));
+        if (z < sm.zb[g]) {
+          x = vmk<V>(x.x + y.x, x.y + y.y);
+        } else {   // past the group's jump
+          const V tn = sm.turn[g];
+          x = vmk<V>(fma(tn.x, y.x, fma(-tn.y, y.y, x.x)), fma(tn.x, y.y, fma(tn.y, y.x, x.y)));
+        }
+      }
+      const V f = sm.phi[z];   // conj(phi) x
+      h.x = fma(f.x, x.x, fma(f.y, x.y, h.x));
+      h.y = fma(f.x, x.y, fma(-f.y, x.x, h.y));
+    }
+    use(p, ce, h);
+  }
+}
+
+// Pa rows (a, c_x, c_y, c_z) of every projector from the second-order sums of t, and a to Pnext if given.
+template <typename T>
+__device__ void any_current(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* t,
+                            typename AnyC<T>::V* u, typename AnyC<T>::V* __restrict__ Pab,
+                            typename AnyC<T>::V* __restrict__ Pnext) {
+  using V = typename AnyC<T>::V;
+  any_project<T, 2>(sm, c, t, u);
+  for (int o = threadIdx.x; o < 4 * c.n_proj; o += ANY_T) {
+    const int j = o >> 2, s = o & 3, a = j >> 2, ty = j & 3;
+    int e[3] = {ty == 1, ty == 2, ty == 3};
+    if (s > 0) e[s - 1] += 1;
+    const T sc = rmul(AnyTab<T>::dv(c), AnyTab<T>::pnorm(c)[j]);
+    const V M = sm.mres[a * 10 + any_mono(e[0], e[1], e[2])];
+    const V v = vmk<V>(rmul(sc, M.x), rmul(sc, M.y));
+    Pab[4 * j + s] = v;
+    if (Pnext && s == 0) Pnext[j] = v;
+  }
+}
+
+// Unit and band of the CTA; false when the unit sits the step out.
+__device__ __forceinline__ bool any_open(const LaunchSet& L, int& u, int& b) {
+  b = blockIdx.x % L.cell.n_bands;
+  u = L.unit_ids[blockIdx.x / L.cell.n_bands];
+  return unit_active(L, u);
+}
+
+// One time step of every band (arguments as launch_step64).
+template <typename T, bool F8>
+__global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T>::V* __restrict__ psi,
+                                                    typename AnyC<T>::V* __restrict__ P,
+                                                    typename AnyC<T>::V* __restrict__ Pa, int fresh_p, int want_pa,
+                                                    int same_next) {
+  using V = typename AnyC<T>::V;
+  extern __shared__ __align__(16) unsigned char any_raw[];
+  const CellDev& c = L.cell;
+  int u, b;
+  if (!any_open(L, u, b)) return;
+  AnySmem<T> sm;
+  any_carve<T>(c, any_raw, sm);
+  const UnitDev U = L.units[u];
+  const SubDev S = L.subs[U.sub];
+  const T* veff = reinterpret_cast<const T*>(S.veff);
+  V* band = psi + U.psi_off + (long long)b * c.npts;
+  V* Pu = P + U.p_off + (long long)b * c.n_proj;
+  for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = sm.acc[p] = band[p];
+  any_setup<T, F8>(sm, c, L.q_half + 3 * u);
+  if (c.use_proj) any_tables<T>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
+  __syncthreads();
+  if (c.use_proj) {
+    if (fresh_p) any_project<T, 1>(sm, c, sm.a, sm.b);
+    any_weights<T>(sm, c, fresh_p ? nullptr : Pu);
+  }
+  V *t = sm.a, *o = sm.b;
+  const T dt = (T)(S.dt * L.dt_scale);
+  T coef = (T)1;
+#pragma unroll 1
+  for (int m = 1; m <= 4; ++m) {
+    coef *= dt / (T)m;
+    const T sg = m == 1 || m == 4 ? coef : -coef;   // psi += (-i)^m coef s_m
+    any_apply<T, F8>(sm, c, veff, t, [&](int p, V, V h) {
+      V a = sm.acc[p];
+      if (m & 1) {
+        a.x = fma(sg, h.y, a.x);
+        a.y = fma(-sg, h.x, a.y);
+      } else {
+        a.x = fma(sg, h.x, a.x);
+        a.y = fma(sg, h.y, a.y);
+      }
+      if (m < 4) {
+        sm.acc[p] = a;
+        o[p] = h;
+      } else {
+        o[p] = a;
+        band[p] = a;
+      }
+    });
+    V* s = t;
+    t = o;
+    o = s;
+    if (m < 4) {
+      if (c.use_proj) {
+        any_project<T, 1>(sm, c, t, o);
+        any_weights<T>(sm, c, nullptr);
+      } else {
+        __syncthreads();
+      }
+    }
+  }
+  if (!c.use_proj || !want_pa) return;
+  __syncthreads();
+  if (!same_next) any_tables<T>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
+  any_current<T>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
+}
+
+// Projections of the current outside a step.
+template <typename T>
+__global__ void __launch_bounds__(ANY_T) k_pa_any(LaunchSet L, const typename AnyC<T>::V* __restrict__ src,
+                                                  typename AnyC<T>::V* __restrict__ Pa) {
+  using V = typename AnyC<T>::V;
+  extern __shared__ __align__(16) unsigned char any_raw[];
+  const CellDev& c = L.cell;
+  int u, b;
+  if (!any_open(L, u, b)) return;
+  AnySmem<T> sm;
+  any_carve<T>(c, any_raw, sm);
+  const UnitDev U = L.units[u];
+  const V* band = src + U.psi_off + (long long)b * c.npts;
+  for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = band[p];
+  any_tables<T>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
+  any_current<T>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
+}
+
+// The ground-state solver's filter (see k_filter64).
+template <bool F8>
+__global__ void __launch_bounds__(ANY_T) k_filter_any(LaunchSet L, const double2* in, double2* out,
+                                                      const double* __restrict__ fa, const double* __restrict__ fb,
+                                                      int degree) {
+  extern __shared__ __align__(16) unsigned char any_raw[];
+  const CellDev& c = L.cell;
+  int u, b;
+  if (!any_open(L, u, b)) return;
+  AnySmem<double> sm;
+  any_carve<double>(c, any_raw, sm);
+  const UnitDev U = L.units[u];
+  const double* veff = reinterpret_cast<const double*>(L.subs[U.sub].veff);
+  const long long off = U.psi_off + (long long)b * c.npts;
+  for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = in[off + p];
+  any_setup<double, F8>(sm, c, L.q_half + 3 * u);
+  if (c.use_proj)
+    any_tables<double>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
+  __syncthreads();
+  double2 *t = sm.a, *o = sm.b;
+#pragma unroll 1
+  for (int j = 0; j < degree; ++j) {
+    if (c.use_proj) {
+      any_project<double, 1>(sm, c, t, o);
+      any_weights<double>(sm, c, nullptr);
+    }
+    const double* f = j == 0 ? fa : fb;
+    const double f0 = f[3 * u], f1 = f[3 * u + 1], f2 = j == 0 ? 0.0 : f[3 * u + 2];
+    any_apply<double, F8>(sm, c, veff, t, [&](int p, double2 ce, double2 h) {
+      double2 y = make_double2(fma(f0, h.x, f1 * ce.x), fma(f0, h.y, f1 * ce.y));
+      if (j > 0) {
+        const double2 v = sm.acc[p];
+        y.x = fma(f2, v.x, y.x);
+        y.y = fma(f2, v.y, y.y);
+      }
+      sm.acc[p] = ce;
+      o[p] = y;
+    });
+    double2* s = t;
+    t = o;
+    o = s;
+    __syncthreads();
+  }
+  for (int p = threadIdx.x; p < c.npts; p += ANY_T) out[off + p] = t[p];
+}
+
+template <typename T> size_t any_smem(const CellDev& c) {
+  AnySmem<T> m;
+  return any_carve<T>(c, nullptr, m);
+}
+
+template <typename K> void any_attr(K* k, size_t bytes) {
+  if (bytes > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <typename T> bool any_ok(const CellDev& c) {
+  return c.n_atoms <= ANY_NA && c.n1 < 1024 && c.n2 < 1024 && c.n3 < 1024 && any_smem<T>(c) <= ANY_MAX_SMEM;
+}
+
+// Variant 0, from ANY_MIN_ORB orbitals on; smaller runs keep the sequences of launches,
+// whose number per step is part of the launch accounting.
+template <typename T> bool any_taken(const LaunchSet& L) {
+  return L.variant == 0 && (long long)L.n_units * L.cell.n_bands >= ANY_MIN_ORB && any_ok<T>(L.cell);
+}
+
+}  // namespace
+
+template <typename T>
+bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
+                     void* stream) {
+  using V = typename AnyC<T>::V;
+  if (L.n_units == 0 || !any_taken<T>(L)) return false;
+  const size_t bytes = any_smem<T>(L.cell);
+  const unsigned grid = (unsigned)L.n_units * L.cell.n_bands;
+  auto go = [&](auto k) {
+    any_attr(k, bytes);
+    k<<<grid, ANY_T, bytes, (cudaStream_t)stream>>>(L, (V*)psi, (V*)P, (V*)Pa, fresh_p, want_pa, same_next);
+  };
+  if (any_fft8(L.cell)) go(k_step_any<T, true>); else go(k_step_any<T, false>);
+  return true;
+}
+
+template <typename T> bool launch_pa_any(const LaunchSet& L, const void* src, void* Pa, void* stream) {
+  using V = typename AnyC<T>::V;
+  if (L.n_units == 0 || !any_taken<T>(L) || !L.cell.use_proj) return false;
+  const size_t bytes = any_smem<T>(L.cell);
+  any_attr(k_pa_any<T>, bytes);
+  k_pa_any<T><<<(unsigned)L.n_units * L.cell.n_bands, ANY_T, bytes, (cudaStream_t)stream>>>(L, (const V*)src, (V*)Pa);
+  return true;
+}
+
+template bool launch_step_any<double>(const LaunchSet&, void*, void*, void*, int, int, int, void*);
+template bool launch_step_any<float>(const LaunchSet&, void*, void*, void*, int, int, int, void*);
+template bool launch_pa_any<double>(const LaunchSet&, const void*, void*, void*);
+template bool launch_pa_any<float>(const LaunchSet&, const void*, void*, void*);
+
+bool launch_filter_any(const LaunchSet& L, const void* in, void* out, const double* fa, const double* fb, int degree,
+                       void* stream) {
+  if (L.n_units == 0 || !any_ok<double>(L.cell)) return false;
+  const size_t bytes = any_smem<double>(L.cell);
+  auto go = [&](auto k) {
+    any_attr(k, bytes);
+    k<<<(unsigned)L.n_units * L.cell.n_bands, ANY_T, bytes, (cudaStream_t)stream>>>(
+        L, (const double2*)in, (double2*)out, fa, fb, degree);
+  };
+  if (any_fft8(L.cell)) go(k_filter_any<true>); else go(k_filter_any<false>);
+  return true;
+}

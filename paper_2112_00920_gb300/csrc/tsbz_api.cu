@@ -456,6 +456,14 @@ template <typename T> int run_field(tsbz_ctx* ctx, int mode) {
   return TSBZ_OK;
 }
 
+// Cells whose variant 0 is a whole step by launch_step64 or launch_step_any: in single
+// precision those without a kernel of their own (16^3 cells, 32-point rows).
+template <typename T> bool whole_step_cell(const tsbz_ctx* ctx, const HostCell& hc) {
+  const CellDev& c = hc.dev;
+  if (ctx->precision == TSBZ_FP64) return true;
+  return ctx->precision == TSBZ_FP32 && !(c.n1 == 16 && c.n2 == 16 && c.n3 == 16) && !slab_supported(c);
+}
+
 template <typename T> int run_observe(tsbz_ctx* ctx, int fin_mode) {
   for (auto& hc : ctx->cells) {
     if (hc.unit_ids.empty()) continue;
@@ -471,10 +479,12 @@ template <typename T> int run_observe(tsbz_ctx* ctx, int fin_mode) {
                           cell_field_const(ctx, hc);
       if (ctx->precision == TSBZ_FP32_TC)
         launch_bra_tc(L, ctx->psi, ctx->Pa, 1, ctx->stream);
+      else if (whole_step_cell<T>(ctx, hc) && ((ctx->precision == TSBZ_FP64 &&
+                                                launch_pa64(L, ctx->psi, ctx->Pa, ctx->stream)) ||
+                                               launch_pa_any<T>(L, ctx->psi, ctx->Pa, ctx->stream)))
+        ;
       else if (sep)
         launch_bra_sep(L, ctx->psi, ctx->Pa, 1, 1, ctx->stream);
-      else if (ctx->precision == TSBZ_FP64 && launch_pa64(L, ctx->psi, ctx->Pa, ctx->stream))
-        ;
       else if (ctx->precision == TSBZ_FP32 &&
                launch_bra_slab(L, ctx->psi, ctx->Pa, 1, 1, ctx->stream, p_next ? ctx->P : nullptr))
         wrote_p = p_next && hc.dev.use_proj;
@@ -556,6 +566,22 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
   for (auto& hc : ctx->cells) {
     if (hc.unit_ids.empty()) continue;
     LaunchSet L = make_set(ctx, hc);
+    if (whole_step_cell<T>(ctx, hc)) {
+      const bool carried = !fresh_p && ctx->p_next_valid && hc.p_by_obs;
+      const int same_next = want_pa && same_next_allowed && cell_field_const(ctx, hc) ? 1 : 0;
+      ev_start(ctx, FAM_STAGE);
+      const bool whole =
+          (ctx->precision == TSBZ_FP64 &&
+           launch_step64(L, ctx->psi, ctx->P, ctx->Pa, carried ? 0 : 1, want_pa ? 1 : 0, same_next, ctx->stream)) ||
+          launch_step_any<T>(L, ctx->psi, ctx->P, ctx->Pa, carried ? 0 : 1, want_pa ? 1 : 0, same_next, ctx->stream);
+      ev_stop(ctx);
+      if (whole) {
+        hc.pa_by_stage = want_pa;
+        hc.p_by_obs = same_next && hc.dev.use_proj;
+        ++ctx->launches;
+        continue;
+      }
+    }
     if (ctx->precision == TSBZ_FP32 && sep_supported(hc.dev)) {
       // Four fused stages; each leaves the projections of its t_m in P, and the
       // bulk-staged stage 4 those of psi(t_{n+1}) for the next step and of the
@@ -587,21 +613,7 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
       }
       continue;
     }
-    if (ctx->precision == TSBZ_FP64) {
-      // 8^3 and 16^3 grids: the whole step in one launch
-      const bool carried = !fresh_p && ctx->p_next_valid && hc.p_by_obs;
-      const bool same_next = want_pa && same_next_allowed && cell_field_const(ctx, hc);
-      ev_start(ctx, FAM_STAGE);
-      const bool whole = launch_step64(L, ctx->psi, ctx->P, ctx->Pa, carried ? 0 : 1, want_pa ? 1 : 0,
-                                       same_next ? 1 : 0, ctx->stream);
-      ev_stop(ctx);
-      hc.pa_by_stage = whole && want_pa;
-      if (whole) {
-        hc.p_by_obs = same_next && hc.dev.use_proj;
-        ++ctx->launches;
-        continue;
-      }
-    }
+    hc.pa_by_stage = false;
     // single precision on 32-point rows: variant 0 is the slab z-march stage, the
     // point-parallel stage takes the variants after it
     const bool slab = ctx->precision == TSBZ_FP32 && slab_supported(hc.dev);
@@ -822,8 +834,8 @@ int sync_and_check(tsbz_ctx* ctx) {
 //     stage with CUDA-core projections;
 //   point-parallel path (FP64, and FP32 on shapes without a z-march kernel):
 //     bands per staged projection chunk 8 (0), 4 (1), 16 (2, when its shared
-//     memory fits); FP64 on 8^3 and 16^3 grids takes the whole step in one
-//     launch as variant 0;
+//     memory fits); 16^3 grids in FP64 and small grids in either take the whole
+//     step in one launch as variant 0;
 //   FP32 on grids with 32-point rows (slab_supported): 0 slab z-march stage,
 //     then the point-parallel stage with 4 (1), 16 (2, when it fits) or 8 (3)
 //     bands per chunk;
@@ -1681,7 +1693,8 @@ int tsbz_ground_state(tsbz_ctx* ctx, int max_iter, double tol, int degree, doubl
   auto apply = [&](HostCell& hc, const double* filt, void* in, void* out, void* prev) {
     ctx->d_filt = filt;
     LaunchSet L = make_set(ctx, hc);
-    if (!prev && launch_filter64(L, in, out, filt, filt, 1, ctx->stream)) {
+    if (!prev && (launch_filter64(L, in, out, filt, filt, 1, ctx->stream) ||
+                  launch_filter_any(L, in, out, filt, filt, 1, ctx->stream))) {
       ++ctx->launches;
       return;
     }
@@ -1815,7 +1828,9 @@ int tsbz_ground_state(tsbz_ctx* ctx, int max_iter, double tol, int degree, doubl
     for (size_t i = 0; i < ctx->cells.size(); ++i) {
       HostCell& hc = ctx->cells[i];
       if (hc.unit_ids.empty()) continue;
-      if (launch_filter64(make_set(ctx, hc), buf[0], buf[degree % 3], dfa, dfb, degree, ctx->stream)) {
+      const LaunchSet L = make_set(ctx, hc);
+      if (launch_filter64(L, buf[0], buf[degree % 3], dfa, dfb, degree, ctx->stream) ||
+          launch_filter_any(L, buf[0], buf[degree % 3], dfa, dfb, degree, ctx->stream)) {
         whole[i] = 1;
         ++ctx->launches;
       } else {

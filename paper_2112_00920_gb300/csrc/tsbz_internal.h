@@ -232,17 +232,22 @@ bool launch_observe_slab(const LaunchSet& L, const void* psi, double* rho_part, 
 bool launch_bra_slab(const LaunchSet& L, const void* src, void* out, int with_d, int use_obs, void* stream,
                      void* pnext = nullptr);
 
-// Double precision on 8^3 and 16^3 grids (tsbz_step64.cu), variant 0 of such cells;
-// false (nothing launched) otherwise.  launch_step64: the whole time step; fresh_p:
+// Double precision on 16^3 grids (tsbz_step64.cu) and either precision on small grids
+// of any shape (tsbz_any.cu), variant 0 of such cells; false (nothing launched) otherwise.  launch_step64: the whole time step; fresh_p:
 // the projections of psi are formed first (else taken from P); want_pa: those of the
 // current go to Pa, and with same_next those of the next step to P.
-bool step64_supported(const CellDev& c);
 bool launch_step64(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
                    void* stream);
 bool launch_pa64(const LaunchSet& L, const void* src, void* Pa, void* stream);
+template <typename T>
+bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
+                     void* stream);
+template <typename T> bool launch_pa_any(const LaunchSet& L, const void* src, void* Pa, void* stream);
 // the whole Chebyshev recurrence of the ground-state solver (degree 1: fa h + fa1)
 bool launch_filter64(const LaunchSet& L, const void* in, void* out, const double* fa, const double* fb, int degree,
                      void* stream);
+bool launch_filter_any(const LaunchSet& L, const void* in, void* out, const double* fa, const double* fb, int degree,
+                       void* stream);
 
 bool sep_supported(const CellDev& c);
 int sep_variants(const CellDev& c);   // kernel variants of the single-precision path on this cell

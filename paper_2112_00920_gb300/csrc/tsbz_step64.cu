@@ -1,4 +1,4 @@
-// Double precision on 8^3 and 16^3 grids: h applied to a band that stays in
+// Double precision on 16^3 grids: h applied to a band that stays in
 // one CTA, for the whole time step (four Taylor stages, the projections of the
 // current) or the whole Chebyshev filter of the ground-state solver in one launch.
 //
@@ -24,8 +24,7 @@
 // busy (a warp instruction occupies it for 16 clocks).
 // Measured: 512 k-points x 16 bands at 16^3, 79.8 -> 42.4 ms per step, FP64 pipe
 // 82% busy at 133 operations per point and stage; 8 k-points x 16 bands 1.77 ->
-// 0.96 ms; at 8^3 (two warps per CTA, bound by the latency of their chains)
-// 16 orbitals 0.37 -> 0.24 ms.
+// 0.96 ms.
 #include <cuda_runtime.h>
 
 #include "tsbz_fft.cuh"
@@ -498,18 +497,10 @@ template <typename K> void s64_attr(K* k, size_t bytes) {
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <int N>
-void step64(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
-            cudaStream_t st) {
-  s64_attr(k_step64<N>, sizeof(S64Smem<N>));
-  k_step64<N><<<(unsigned)L.n_units * L.cell.n_bands, N * N, sizeof(S64Smem<N>), st>>>(
-      L, (double2*)psi, (double2*)P, (double2*)Pa, fresh_p, want_pa, same_next);
-}
-
 }  // namespace
 
-bool step64_supported(const CellDev& c) {
-  return c.n1 == c.n2 && c.n2 == c.n3 && (c.n1 == 8 || c.n1 == 16) && c.n_atoms <= S64_NA;
+static bool step64_supported(const CellDev& c) {
+  return c.n1 == 16 && c.n2 == 16 && c.n3 == 16 && c.n_atoms <= S64_NA;
 }
 
 // Variant 0 of such cells, from S64_MIN_ORB orbitals on.  Runs of fewer orbitals
@@ -522,38 +513,25 @@ static bool step64_taken(const LaunchSet& L) {
 bool launch_step64(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
                    void* stream) {
   if (L.n_units == 0 || !step64_taken(L)) return false;
-  if (L.cell.n1 == 16)
-    step64<16>(L, psi, P, Pa, fresh_p, want_pa, same_next, (cudaStream_t)stream);
-  else
-    step64<8>(L, psi, P, Pa, fresh_p, want_pa, same_next, (cudaStream_t)stream);
+  s64_attr(k_step64<16>, sizeof(S64Smem<16>));
+  k_step64<16><<<(unsigned)L.n_units * L.cell.n_bands, 256, sizeof(S64Smem<16>), (cudaStream_t)stream>>>(
+      L, (double2*)psi, (double2*)P, (double2*)Pa, fresh_p, want_pa, same_next);
   return true;
 }
 
 bool launch_pa64(const LaunchSet& L, const void* src, void* Pa, void* stream) {
   if (L.n_units == 0 || !step64_taken(L) || !L.cell.use_proj) return false;
-  const unsigned grid = (unsigned)L.n_units * L.cell.n_bands;
-  if (L.cell.n1 == 16) {
-    s64_attr(k_pa64<16>, sizeof(S64Smem<16>));
-    k_pa64<16><<<grid, 256, sizeof(S64Smem<16>), (cudaStream_t)stream>>>(L, (const double2*)src, (double2*)Pa);
-  } else {
-    s64_attr(k_pa64<8>, sizeof(S64Smem<8>));
-    k_pa64<8><<<grid, 64, sizeof(S64Smem<8>), (cudaStream_t)stream>>>(L, (const double2*)src, (double2*)Pa);
-  }
+  s64_attr(k_pa64<16>, sizeof(S64Smem<16>));
+  k_pa64<16><<<(unsigned)L.n_units * L.cell.n_bands, 256, sizeof(S64Smem<16>), (cudaStream_t)stream>>>(
+      L, (const double2*)src, (double2*)Pa);
   return true;
 }
 
 bool launch_filter64(const LaunchSet& L, const void* in, void* out, const double* fa, const double* fb, int degree,
                      void* stream) {
   if (L.n_units == 0 || !step64_supported(L.cell)) return false;
-  const unsigned grid = (unsigned)L.n_units * L.cell.n_bands;
-  if (L.cell.n1 == 16) {
-    s64_attr(k_filter64<16>, sizeof(S64Smem<16>));
-    k_filter64<16><<<grid, 256, sizeof(S64Smem<16>), (cudaStream_t)stream>>>(L, (const double2*)in, (double2*)out, fa,
-                                                                            fb, degree);
-  } else {
-    s64_attr(k_filter64<8>, sizeof(S64Smem<8>));
-    k_filter64<8><<<grid, 64, sizeof(S64Smem<8>), (cudaStream_t)stream>>>(L, (const double2*)in, (double2*)out, fa,
-                                                                          fb, degree);
-  }
+  s64_attr(k_filter64<16>, sizeof(S64Smem<16>));
+  k_filter64<16><<<(unsigned)L.n_units * L.cell.n_bands, 256, sizeof(S64Smem<16>), (cudaStream_t)stream>>>(
+      L, (const double2*)in, (double2*)out, fa, fb, degree);
   return true;
 }
