@@ -1668,16 +1668,18 @@ int tsbz_ground_state(tsbz_ctx* ctx, int max_iter, double tol, int degree, doubl
   if (rc) return rc;
   const size_t ns = ctx->subs.size();
   // scratch: Gram matrices, coefficients, bounds
-  void *dS = nullptr, *dH = nullptr, *dC = nullptr, *dW1 = nullptr, *dW2 = nullptr;
+  void *dS = nullptr, *dH = nullptr, *dC = nullptr, *dW1 = nullptr, *dW2 = nullptr, *dG = nullptr;
   double *dlam = nullptr, *dfa = nullptr, *dfb = nullptr, *dfc = nullptr;
   int* dbad = nullptr;
   const size_t mat = std::max<size_t>(max_mat, 1) * sizeof(double2);
   auto cleanup = [&]() {
-    for (void* p : {dS, dH, dC, dW1, dW2, (void*)dlam, (void*)dfa, (void*)dfb, (void*)dfc, (void*)dbad})
+    for (void* p : {dS, dH, dC, dW1, dW2, dG, (void*)dlam, (void*)dfa, (void*)dfb, (void*)dfc, (void*)dbad})
       dfree(ctx, p);
     ctx->d_filt = nullptr;
   };
-  if ((rc = dalloc(ctx, mat, &dS)) || (rc = dalloc(ctx, mat, &dH)) || (rc = dalloc(ctx, mat, &dC)) ||
+  size_t gram = 0;
+  for (auto& hc : ctx->cells) gram = std::max(gram, scf_gram_scratch(hc.dev, (int)hc.unit_ids.size()));
+  if ((rc = dalloc(ctx, gram, &dG)) || (rc = dalloc(ctx, mat, &dS)) || (rc = dalloc(ctx, mat, &dH)) || (rc = dalloc(ctx, mat, &dC)) ||
       (rc = dalloc(ctx, mat, &dW1)) || (rc = dalloc(ctx, mat, &dW2)) ||
       (rc = dalloc_t(ctx, (size_t)max_units, &dlam)) || (rc = dalloc_t(ctx, 3 * (size_t)ctx->n_units, &dfa)) ||
       (rc = dalloc_t(ctx, 3 * (size_t)ctx->n_units, &dfb)) || (rc = dalloc_t(ctx, 3 * (size_t)ctx->n_units, &dfc)) ||
@@ -1719,7 +1721,7 @@ int tsbz_ground_state(tsbz_ctx* ctx, int max_iter, double tol, int degree, doubl
       void* src = y;
       void* dst = hy;
       for (int pass = 0; pass < 3; ++pass) {
-        launch_scf_gram(L, src, nullptr, dS, nullptr, ctx->stream);
+        launch_scf_gram(L, src, nullptr, dS, nullptr, dG, ctx->stream);
         launch_scf_ortho(L.n_units, nb, pass == 0 ? shift_coef : 0.0, 0, dS, dH, dC, dW1, dW2, dlam, dbad,
                          ctx->stream);
         launch_scf_rotate(L, src, dC, dst, ctx->stream);
@@ -1728,9 +1730,9 @@ int tsbz_ground_state(tsbz_ctx* ctx, int max_iter, double tol, int degree, doubl
       // the orthonormal block is in `src` (= hy); h Q into `dst` (= y)
       apply(hc, dfc, src, dst, nullptr);
       L = make_set(ctx, hc);
-      launch_scf_gram(L, src, dst, dS, dH, ctx->stream);
+      launch_scf_gram(L, src, dst, dS, dH, dG, ctx->stream);
       launch_scf_ortho(L.n_units, nb, 0.0, 1, dS, dH, dC, dW1, dW2, dlam, dbad, ctx->stream);
-      ctx->launches += 11;
+      ctx->launches += 15;
       std::vector<double> lam(L.n_units);
       CK(cudaMemcpyAsync(lam.data(), dlam, sizeof(double) * lam.size(), cudaMemcpyDeviceToHost, ctx->stream));
       CK(cudaStreamSynchronize(ctx->stream));

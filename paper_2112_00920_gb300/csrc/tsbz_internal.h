@@ -208,7 +208,9 @@ void launch_stage_v(const LaunchSet& L, const void* tin, void* tout, void* psi, 
 // single-precision fused stage and projections (cells with at most 8 atoms, depth 8 or 16, n1 n2 <= 256)
 // Ground-state solver (tsbz_scf.cu).
 int scf_max_bands();
-void launch_scf_gram(const LaunchSet& L, const void* Y, const void* HY, void* S, void* H, void* stream);
+// G: scratch of scf_gram_scratch bytes (partial sums over point chunks)
+size_t scf_gram_scratch(const CellDev& c, int n_units);
+void launch_scf_gram(const LaunchSet& L, const void* Y, const void* HY, void* S, void* H, void* G, void* stream);
 // HY null: S only.  S, H, C, W1, W2: n_units n_b^2 complex each;
 // C = L^{-H} with S + shift_coef tr(S) I = L L^H; with want_lam, H is
 // replaced by L^{-1} H L^{-H} and lam receives its largest eigenvalue
