@@ -456,12 +456,29 @@ template <typename T> int run_field(tsbz_ctx* ctx, int mode) {
   return TSBZ_OK;
 }
 
-// Cells whose variant 0 is a whole step by launch_step64 or launch_step_any: in single
-// precision those without a kernel of their own (16^3 cells, 32-point rows).
-template <typename T> bool whole_step_cell(const tsbz_ctx* ctx, const HostCell& hc) {
+// The whole step of a cell by launch_step64 (FP64, 16^3), launch_step_fft32 (FP32, 32^3) or
+// launch_step_any (small grids; in single precision those without a kernel of their
+// own); false when the cell takes the launches per stage.  The 16^3 single-precision
+// cells have launch_step_fused.
+template <typename T>
+bool whole_step(tsbz_ctx* ctx, const HostCell& hc, const LaunchSet& L, int fresh_p, int want_pa, int same_next) {
   const CellDev& c = hc.dev;
-  if (ctx->precision == TSBZ_FP64) return true;
-  return ctx->precision == TSBZ_FP32 && !(c.n1 == 16 && c.n2 == 16 && c.n3 == 16) && !slab_supported(c);
+  const bool any = ctx->precision == TSBZ_FP64 || (!(c.n1 == 16 && c.n2 == 16 && c.n3 == 16) && !slab_supported(c));
+  if (ctx->precision == TSBZ_FP64 && launch_step64(L, ctx->psi, ctx->P, ctx->Pa, fresh_p, want_pa, same_next, ctx->stream))
+    return true;
+  if (ctx->precision == TSBZ_FP32 &&
+      launch_step_fft32(L, ctx->psi, ctx->P, ctx->Pa, fresh_p, want_pa, same_next, ctx->stream))
+    return true;
+  return any && launch_step_any<T>(L, ctx->psi, ctx->P, ctx->Pa, fresh_p, want_pa, same_next, ctx->stream);
+}
+
+// The current's projections of such cells outside a step.
+template <typename T> bool whole_pa(tsbz_ctx* ctx, const HostCell& hc, const LaunchSet& L) {
+  const CellDev& c = hc.dev;
+  const bool any = ctx->precision == TSBZ_FP64 || (!(c.n1 == 16 && c.n2 == 16 && c.n3 == 16) && !slab_supported(c));
+  if (ctx->precision == TSBZ_FP64 && launch_pa64(L, ctx->psi, ctx->Pa, ctx->stream)) return true;
+  if (ctx->precision == TSBZ_FP32 && launch_pa_fft32(L, ctx->psi, ctx->Pa, ctx->stream)) return true;
+  return any && launch_pa_any<T>(L, ctx->psi, ctx->Pa, ctx->stream);
 }
 
 template <typename T> int run_observe(tsbz_ctx* ctx, int fin_mode) {
@@ -479,9 +496,7 @@ template <typename T> int run_observe(tsbz_ctx* ctx, int fin_mode) {
                           cell_field_const(ctx, hc);
       if (ctx->precision == TSBZ_FP32_TC)
         launch_bra_tc(L, ctx->psi, ctx->Pa, 1, ctx->stream);
-      else if (whole_step_cell<T>(ctx, hc) && ((ctx->precision == TSBZ_FP64 &&
-                                                launch_pa64(L, ctx->psi, ctx->Pa, ctx->stream)) ||
-                                               launch_pa_any<T>(L, ctx->psi, ctx->Pa, ctx->stream)))
+      else if (whole_pa<T>(ctx, hc, L))
         ;
       else if (sep)
         launch_bra_sep(L, ctx->psi, ctx->Pa, 1, 1, ctx->stream);
@@ -566,14 +581,11 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
   for (auto& hc : ctx->cells) {
     if (hc.unit_ids.empty()) continue;
     LaunchSet L = make_set(ctx, hc);
-    if (whole_step_cell<T>(ctx, hc)) {
+    {
       const bool carried = !fresh_p && ctx->p_next_valid && hc.p_by_obs;
       const int same_next = want_pa && same_next_allowed && cell_field_const(ctx, hc) ? 1 : 0;
       ev_start(ctx, FAM_STAGE);
-      const bool whole =
-          (ctx->precision == TSBZ_FP64 &&
-           launch_step64(L, ctx->psi, ctx->P, ctx->Pa, carried ? 0 : 1, want_pa ? 1 : 0, same_next, ctx->stream)) ||
-          launch_step_any<T>(L, ctx->psi, ctx->P, ctx->Pa, carried ? 0 : 1, want_pa ? 1 : 0, same_next, ctx->stream);
+      const bool whole = whole_step<T>(ctx, hc, L, carried ? 0 : 1, want_pa ? 1 : 0, same_next);
       ev_stop(ctx);
       if (whole) {
         hc.pa_by_stage = want_pa;
@@ -1146,14 +1158,15 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
   }
   // z groups: atoms with bit-identical z rows of the factor tables
   const int nm_z = c.nmax;
-  auto same_z = [&](int a, int b) {
+  auto same_axis = [&](int a, int b, int ax) {
     for (int i = 0; i < nm_z; ++i) {
-      const size_t ia = (size_t)(a * 3 + 2) * nm_z + i, ib = (size_t)(b * 3 + 2) * nm_z + i;
+      const size_t ia = (size_t)(a * 3 + ax) * nm_z + i, ib = (size_t)(b * 3 + ax) * nm_z + i;
       if (g1f[ia] != g1f[ib] || d1f[ia] != d1f[ib]) return false;
       if (ctx->precision == TSBZ_FP64 && (g1[ia] != g1[ib] || d1[ia] != d1[ib])) return false;
     }
     return true;
   };
+  auto same_z = [&](int a, int b) { return same_axis(a, b, 2); };
   c.zs_n = 0;
   for (int i = 0; i <= 8; ++i) c.zs_off[i] = 0;
   for (int i = 0; i < 64; ++i) c.zs_mem[i] = 0;
@@ -1176,6 +1189,33 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
           if (grp[a] == g) c.zs_mem[k++] = a;
       }
       for (int g = c.zs_n; g <= 8; ++g) c.zs_off[g] = k;
+    }
+  }
+  // x and y classes alike
+  c.xc_n = c.yc_n = 0;
+  if (c.use_proj && d->n_atoms <= 64) {
+    int n[2] = {0, 0};
+    int* rep[2] = {c.xc_rep, c.yc_rep};
+    unsigned char* of[2] = {c.xc_of, c.yc_of};
+    bool fits = true;
+    for (int ax = 0; ax < 2; ++ax)
+      for (int a = 0; a < d->n_atoms && fits; ++a) {
+        int g = -1;
+        for (int k = 0; k < n[ax] && g < 0; ++k)
+          if (same_axis(a, rep[ax][k], ax)) g = k;
+        if (g < 0) {
+          if (n[ax] == 8) {
+            fits = false;
+            break;
+          }
+          g = n[ax]++;
+          rep[ax][g] = a;
+        }
+        of[ax][a] = (unsigned char)g;
+      }
+    if (fits) {
+      c.xc_n = n[0];
+      c.yc_n = n[1];
     }
   }
   c.n_zg = 0;

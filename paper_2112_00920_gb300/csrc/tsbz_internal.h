@@ -86,6 +86,11 @@ struct CellDev {
   int zs_n;
   int zs_off[9];      // members of group g: zs_mem[zs_off[g] .. zs_off[g + 1])
   int zs_mem[64];
+  // x and y classes of such cells: atoms with identical tables along the axis (at
+  // most 8 of each, else xc_n = yc_n = 0)
+  int xc_n, yc_n;
+  int xc_rep[8], yc_rep[8];   // first atom of a class
+  unsigned char xc_of[64], yc_of[64];
 };
 
 // Whether the finalize spreads one unit over a whole CTA (units with many
@@ -250,6 +255,12 @@ bool launch_filter64(const LaunchSet& L, const void* in, void* out, const double
                      void* stream);
 bool launch_filter_any(const LaunchSet& L, const void* in, void* out, const double* fa, const double* fb, int degree,
                        void* stream);
+
+// FP32 on 32^3 grids with at most 8 classes of atoms per axis (tsbz_step32c.cu), variant 0;
+// arguments as launch_step64.
+bool launch_step_fft32(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
+                       void* stream);
+bool launch_pa_fft32(const LaunchSet& L, const void* src, void* Pa, void* stream);
 
 bool sep_supported(const CellDev& c);
 int sep_variants(const CellDev& c);   // kernel variants of the single-precision path on this cell
