@@ -34,6 +34,7 @@ struct HostCell {
   double2* tw[3] = {nullptr, nullptr, nullptr};
   std::vector<int> unit_ids;
   int* d_unit_ids = nullptr;
+  void* images = nullptr;      // operand images (LaunchSet::images)
   std::vector<int> hxc_subs;   // non-frozen sub-simulations of this cell
   int* d_hxc_subs = nullptr;
   bool pa_by_stage = false;    // the last stage 4 also wrote P (next step) and Pa
@@ -222,6 +223,7 @@ LaunchSet make_set(tsbz_ctx* ctx, HostCell& hc) {
   L.qt_half = ctx->qt_half;
   L.variant = hc.variant;
   L.dt_scale = ctx->dt_scale;
+  L.images = hc.images;
   L.filt = ctx->d_filt;
   return L;
 }
@@ -396,6 +398,8 @@ int layout(tsbz_ctx* ctx) {
       CK(cudaMemcpyAsync(hc.d_unit_ids, hc.unit_ids.data(), sizeof(int) * hc.unit_ids.size(), cudaMemcpyHostToDevice,
                          ctx->stream));
     }
+    const size_t img = ctx->precision == TSBZ_FP32 ? step_fft32_images(hc.dev, (int)hc.unit_ids.size()) : 0;
+    if (img && (rc = dalloc(ctx, img, &hc.images))) return rc;
     if (!hc.hxc_subs.empty()) {
       if ((rc = dalloc_t(ctx, hc.hxc_subs.size(), &hc.d_hxc_subs))) return rc;
       CK(cudaMemcpyAsync(hc.d_hxc_subs, hc.hxc_subs.data(), sizeof(int) * hc.hxc_subs.size(),
@@ -451,6 +455,12 @@ template <typename T> int run_field(tsbz_ctx* ctx, int mode) {
     launch_field<T>(make_set(ctx, hc), keep ? TSBZ_FIELD_STEP_KEEP : mode, ctx->stream);
     hc.tables_step = mode == TSBZ_FIELD_STEP;
     ++ctx->launches;
+    if (hc.images && !keep) {
+      LaunchSet L = make_set(ctx, hc);
+      L.variant = 0;   // whatever the variant in force, so that a change of it finds them
+      launch_images_fft32(L, ctx->stream);
+      ++ctx->launches;
+    }
   }
   ev_stop(ctx);
   return TSBZ_OK;

@@ -165,6 +165,7 @@ struct LaunchSet {
   void* qt_half;          // [unit][4] in T: q_x, q_y, q_z, |q|^2 / 2 at t_n + dt/2
   int variant;            // kernel variant of this cell (0 = default; chosen by the autotuner)
   double dt_scale;        // the stage kernels advance by dt * dt_scale (1, or 1/2 in the ETRS half steps)
+  void* images;           // operand images of the 32^3 whole-step kernel (null if the cell has none)
   const double* filt;     // [unit][3] filter coefficients of the ground-state solver (stage m = 0), or null
 };
 
@@ -257,7 +258,10 @@ bool launch_filter_any(const LaunchSet& L, const void* in, void* out, const doub
                        void* stream);
 
 // FP32 on 32^3 grids with at most 8 classes of atoms per axis (tsbz_step32c.cu), variant 0;
-// arguments as launch_step64.
+// arguments as launch_step64.  The operand images of a cell (step_fft32_images bytes, 0 if
+// it does not qualify) are rebuilt after every field launch that rebuilds the phase tables.
+size_t step_fft32_images(const CellDev& c, int n_units);
+void launch_images_fft32(const LaunchSet& L, void* stream);
 bool launch_step_fft32(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
                        void* stream);
 bool launch_pa_fft32(const LaunchSet& L, const void* src, void* Pa, void* stream);

@@ -9,7 +9,7 @@
 // decimation step, then 16 points in registers); along y the star stencil runs on
 // the transformed rows, the neighbour CTAs' four rows on either side read through
 // distributed shared memory (the same volume as a transform's two exchanges,
-// with one cluster barrier instead of two).
+// with one exchange instead of two; the same barrier publishes the partial projections).
 // Projectors: z sums of the columns on tcgen05 (three-product TF32, A in tensor
 // memory), x sums per (atom, row) over the atom's box, y sums over the CTA's rows,
 // and the eight CTAs' partial sums added in rank order through distributed
@@ -17,6 +17,9 @@
 // tcgen05 under the line transforms.  Atoms whose x (y, z) tables are identical share
 // them: at most 8 classes per axis (a 2 x 2 x 2 diamond supercell has 8).
 // Taylor terms are s_m = h^m psi; (-i dt)^m / m! enters the sum only.
+// Measured: 8 k-points x 128 bands of the 64-atom cell, stages and projections 3.31 ->
+// 2.00 ms per step (36% of issue slots, the rest barriers and the latency of the
+// remote rows).
 // Every wait on an MMA is bounded; a CTA that gave up keeps taking part in the
 // cluster's barriers and reports at the end.
 // Tensor-memory columns: Taylor sum [0, 64), v_eff [64, 96), bra accumulator
@@ -44,6 +47,7 @@ constexpr int QA = 64;            // atom slots
 constexpr int QG = 8;             // z groups, x and y classes
 constexpr int Q_ACC = 0, Q_VEFF = 64, Q_BRA_D = 96, Q_OP = 128, Q_BRA2_D = 0;
 constexpr uint32_t Q_COLS = 256;
+constexpr size_t Q_IMG = 16384 + 16384 + 24576;   // B images of a unit: ket, first- and second-order bra
 
 struct QSmem {
   float2 b1[QBUF];                 // line buffers [row][z or k_z][x or k_x]
@@ -60,7 +64,8 @@ struct QSmem {
   int atom[QA];                    // atom of a slot (-1: none)
   unsigned char xc[QA], yc[QA], zg[QA];
   int xs[QG], xl[QG];              // x box of a class: start, length
-  unsigned long long mbar;
+  unsigned long long mbar;         // completion of the MMAs
+  unsigned long long mimg;         // arrival of the B images
   uint32_t tslot;
 };
 
@@ -124,6 +129,10 @@ __device__ __forceinline__ void q_st8(uint32_t taddr, const uint32_t (&r)[8]) {
       : "memory");
 }
 
+// The cluster's barrier in two halves (every thread of every CTA, alternating).
+__device__ __forceinline__ void q_arrive() { asm volatile("barrier.cluster.arrive.release;\n" ::: "memory"); }
+__device__ __forceinline__ void q_wait() { asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory"); }
+
 // Slots, classes and boxes of the cell; ends with a barrier.
 __device__ void q_cell(QSmem& sm, const CellDev& c) {
   const int tid = threadIdx.x;
@@ -155,45 +164,56 @@ __device__ __forceinline__ float2 q_zfactor(const CellDev& c, const float2* ph, 
 }
 
 // B of an order-D bra (N = 32 or 48): n = 2 q + c', q = (D + 1) g + k; K = 64:
-// kk = 32 h + 2 j + c for z = 2 j + h.  hi, then lo (N/8 * 2 KiB each).
+// kk = 32 h + 2 j + c for z = 2 j + h.  hi, then lo (N/8 * 2 KiB each).  A warp writes one
+// 8 x 16-byte core matrix (no bank conflicts).
 template <int D> __device__ void q_build_bra(unsigned char* bz, const CellDev& c, const float2* ph) {
   constexpr int NN = D == 1 ? 32 : 48, LO = NN / 8 * 2048;
-  for (int i = threadIdx.x; i < NN * 32; i += QT) {   // one (n pair's q, z, both components) entry pair
-    const int n = i >> 5, z = i & 31, q = n >> 1, cs = n & 1, g = q / (D + 1), k = q - g * (D + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 2
+  for (int m = warp; m < NN / 8 * 16; m += QT / 32) {
+    const int n = 8 * (m >> 4) + (lane >> 2), kk = 4 * (m & 15) + (lane & 3);
+    const int q = n >> 1, cs = n & 1, g = q / (D + 1), k = q - g * (D + 1), z = (kk & 30) + (kk >> 5), cu = kk & 1;
     float2 f = make_float2(0.f, 0.f);
     if (g < c.zs_n) f = q_zfactor(c, ph, g, z, k);
-    const int kk = 32 * (z & 1) + (z & ~1);   // j = z / 2: 2 j = z & ~1
-#pragma unroll
-    for (int cu = 0; cu < 2; ++cu) {
-      const float v = cs == 0 ? (cu == 0 ? f.x : -f.y) : (cu == 0 ? f.y : f.x);
-      uint32_t hi, lo;
-      q_split(v, hi, lo);
-      const int o = (n >> 3) * 2048 + ((kk + cu) >> 2) * 128 + (n & 7) * 16 + ((kk + cu) & 3) * 4;
-      *reinterpret_cast<uint32_t*>(bz + o) = hi;
-      *reinterpret_cast<uint32_t*>(bz + LO + o) = lo;
-    }
+    uint32_t hi, lo;
+    q_split(cs == 0 ? (cu == 0 ? f.x : -f.y) : (cu == 0 ? f.y : f.x), hi, lo);
+    *reinterpret_cast<uint32_t*>(bz + 128 * m + 4 * lane) = hi;
+    *reinterpret_cast<uint32_t*>(bz + LO + 128 * m + 4 * lane) = lo;
   }
 }
 
 // B of the ket: n = 2 (16 h' + j) + c for z = 2 j + h' (N = 64); K = 32: kk = 16 h + 8 part + i for
 // q = 8 h + i, part 0 the real, 1 the imaginary coefficient.
 __device__ void q_build_ket(unsigned char* bz, const CellDev& c, const float2* ph) {
-  for (int i = threadIdx.x; i < 16 * 32; i += QT) {
-    const int q = i >> 5, z = i & 31, g = q >> 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 2
+  for (int m = warp; m < 64; m += QT / 32) {
+    const int n = 8 * (m >> 3) + (lane >> 2), kk = 4 * (m & 7) + (lane & 3);
+    const int zi = n >> 1, cc = n & 1, z = 2 * (zi & 15) + (zi >> 4);
+    const int q = 8 * (kk >> 4) + (kk & 7), part = (kk >> 3) & 1, g = q >> 1;
     float2 f = make_float2(0.f, 0.f);
     if (g < c.zs_n) f = q_zfactor(c, ph, g, z, q & 1);
-    const int zi = 16 * (z & 1) + (z >> 1), k0 = 16 * (q >> 3) + (q & 7);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int part = e >> 1, cc = e & 1, n = 2 * zi + cc, kk = k0 + 8 * part;
-      const float v = part == 0 ? (cc ? f.y : f.x) : (cc ? f.x : -f.y);
-      uint32_t hi, lo;
-      q_split(v, hi, lo);
-      const int o = (n >> 3) * 1024 + (kk >> 2) * 128 + (n & 7) * 16 + (kk & 3) * 4;
-      *reinterpret_cast<uint32_t*>(bz + o) = hi;
-      *reinterpret_cast<uint32_t*>(bz + 8192 + o) = lo;
-    }
+    uint32_t hi, lo;
+    q_split(part == 0 ? (cc ? f.y : f.x) : (cc ? f.x : -f.y), hi, lo);
+    *reinterpret_cast<uint32_t*>(bz + 128 * m + 4 * lane) = hi;
+    *reinterpret_cast<uint32_t*>(bz + 8192 + 128 * m + 4 * lane) = lo;
   }
+}
+
+// The B matrices depend on the unit's tables only: one CTA per unit writes their images
+// after the field kernel rebuilt the tables (q_half for the stages, q_obs for the
+// current), and the step's CTAs fetch them by bulk copies.  Built in each of a
+// unit's 1024 CTAs they took 0.26 of 2.29 ms (128 bands).
+__global__ void __launch_bounds__(QT) k_images32(LaunchSet L, unsigned char* __restrict__ img) {
+  const CellDev& c = L.cell;
+  const int u = L.unit_ids[blockIdx.x];
+  if (!unit_active(L, u)) return;
+  unsigned char* o = img + (size_t)blockIdx.x * Q_IMG;
+  const float2* phh = (const float2*)L.ph_half + (long long)u * L.ph_stride;
+  const float2* pho = (const float2*)L.ph_obs + (long long)u * L.ph_stride;
+  if (blockIdx.y == 0) q_build_ket(o, c, phh);
+  if (blockIdx.y == 1) q_build_bra<1>(o + 16384, c, phh);
+  if (blockIdx.y == 2) q_build_bra<2>(o + 32768, c, pho);
 }
 
 // x factors of the classes, y factors on the CTA's rows, rows' slot masks; ends with a barrier.
@@ -246,29 +266,27 @@ __device__ __forceinline__ void q_stage(const float2 (&u)[16], const QState& x) 
   }
 }
 
-// z sums of the staged columns into zs[q][row][x]: MMAs (B in bz) and collection;
-// false when they did not complete.  Begins with a barrier (A staged, bz written and fenced), ends with one.
-template <int D>
-__device__ __forceinline__ bool q_zsums(QState& x, const unsigned char* bz, float2* zs) {
-  constexpr int NN = D == 1 ? 32 : 48, LO = NN / 8 * 2048, DC = D == 1 ? Q_BRA_D : Q_BRA2_D;
-  const int tid = threadIdx.x, warp = tid >> 5, h = warp >> 2, qd = warp & 3;
-  um_fence_before();
-  __syncthreads();
-  if (tid == 0) {
-    um_fence_after();
-    constexpr uint32_t idesc = um_idesc_tf32(128, NN);
-    const uint32_t b0 = bk_smem(bz), b1 = b0 + LO, d = x.tbase + DC;
+// The MMAs of an order-D bra (one thread, behind a barrier after q_stage and B's fenced writes).
+template <int D> __device__ __forceinline__ void q_issue_bra(const QState& x, const unsigned char* bz) {
+  constexpr int NN = D == 1 ? 32 : 48, LO = NN / 8 * 2048;
+  constexpr uint32_t idesc = um_idesc_tf32(128, NN);
+  um_fence_after();
+  const uint32_t b0 = bk_smem(bz), b1 = b0 + LO, d = x.tbase + (D == 1 ? Q_BRA_D : Q_BRA2_D);
 #pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-      const uint32_t a_hi = x.tbase + Q_OP + 64 * (ks >> 2) + 8 * (ks & 3), a_lo = a_hi + 32;
-      const uint64_t bh = um_sdesc(b0 + 256 * ks, 128, 2048), bl = um_sdesc(b1 + 256 * ks, 128, 2048);
-      um_mma_tf32_ts(d, a_lo, bh, idesc, ks > 0);
-      um_mma_tf32_ts(d, a_hi, bl, idesc, true);
-      um_mma_tf32_ts(d, a_hi, bh, idesc, true);
-    }
-    um_commit(x.bar);
+  for (int ks = 0; ks < 8; ++ks) {
+    const uint32_t a_hi = x.tbase + Q_OP + 64 * (ks >> 2) + 8 * (ks & 3), a_lo = a_hi + 32;
+    const uint64_t bh = um_sdesc(b0 + 256 * ks, 128, 2048), bl = um_sdesc(b1 + 256 * ks, 128, 2048);
+    um_mma_tf32_ts(d, a_lo, bh, idesc, ks > 0);
+    um_mma_tf32_ts(d, a_hi, bl, idesc, true);
+    um_mma_tf32_ts(d, a_hi, bh, idesc, true);
   }
-  const bool ok = q_poll(x);
+  um_commit(x.bar);
+}
+
+// The thread's share of its column's z sums into zs[q][row][x] (after q_poll).
+template <int D> __device__ __forceinline__ void q_collect(const QState& x, float2* zs) {
+  constexpr int DC = D == 1 ? Q_BRA_D : Q_BRA2_D;
+  const int tid = threadIdx.x, warp = tid >> 5, h = warp >> 2, qd = warp & 3;
   const int col = tid & 127, o = (col >> 5) * QP + (col & 31);
   if constexpr (D == 1) {
     float d[16];
@@ -286,9 +304,6 @@ __device__ __forceinline__ bool q_zsums(QState& x, const unsigned char* bz, floa
       zs[(8 + 4 * h + i) * QR * QP + o] =
           h ? make_float2(e[8 + 2 * i], e[9 + 2 * i]) : make_float2(e[2 * i], e[2 * i + 1]);
   }
-  um_fence_before();
-  __syncthreads();
-  return ok;
 }
 
 // The CTA's partial monomial sums of order <= D of slot tid / 4 over its rows: thread
@@ -361,12 +376,24 @@ __device__ __forceinline__ float2 q_total(cg::cluster_group& cl, float2* p, int 
 
 // Rows (a_j, c_jx, c_jy, c_jz) from the second-order pass of the staged columns into Pab
 // (and a_j into Pnext if given).  The CTA of rank r writes the slots 8 r .. 8 r + 7.
-__device__ bool q_current(QSmem& sm, cg::cluster_group& cl, QState& x, const CellDev& c, const float2* ph,
-                          float2* __restrict__ Pab, float2* __restrict__ Pnext) {
+// img: the unit's images; parity: of the copy's arrival.
+__device__ bool q_current(QSmem& sm, cg::cluster_group& cl, QState& x, const CellDev& c, const unsigned char* img,
+                          uint32_t parity, float2* __restrict__ Pab, float2* __restrict__ Pnext) {
   unsigned char* bz = reinterpret_cast<unsigned char*>(sm.b1);
-  q_build_bra<2>(bz, c, ph);
+  const uint32_t bar = bk_smem(&sm.mimg);
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  const bool ok = q_zsums<2>(x, bz, sm.b2);
+  um_fence_before();
+  __syncthreads();
+  bool ok = true;
+  if (threadIdx.x == 0) {
+    bk_mbar_expect_tx(bar, 24576);
+    bk_copy_g2s(bk_smem(bz), img + 32768, 24576, bar);
+    ok = bk_mbar_wait(bar, parity, BK_WAIT_POLLS);
+    q_issue_bra<2>(x, bz);
+  }
+  ok = q_poll(x) && ok;
+  q_collect<2>(x, sm.b2);
+  __syncthreads();
   q_moments<2>(sm, sm.b2, sm.tab);
   cl.sync();
   const int tid = threadIdx.x, s = (int)cl.block_rank() * 8 + (tid >> 4), o = tid & 15;
@@ -388,7 +415,10 @@ __device__ bool q_current(QSmem& sm, cg::cluster_group& cl, QState& x, const Cel
 
 __device__ __forceinline__ QState q_open(QSmem& sm) {
   if ((threadIdx.x >> 5) == 0) um_alloc(bk_smem(&sm.tslot), Q_COLS);
-  if (threadIdx.x == 0) bk_mbar_init(bk_smem(&sm.mbar), 1);
+  if (threadIdx.x == 0) {
+    bk_mbar_init(bk_smem(&sm.mbar), 1);
+    bk_mbar_init(bk_smem(&sm.mimg), 1);
+  }
   um_fence_before();
   __syncthreads();
   um_fence_after();
@@ -408,8 +438,8 @@ __device__ __forceinline__ void q_close(cg::cluster_group& cl, const QState& x, 
 
 // One time step of every band (arguments as launch_step64).
 __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
-    k_step_fft32(LaunchSet L, float2* __restrict__ psi, float2* __restrict__ P, float2* __restrict__ Pa, int fresh_p,
-                 int want_pa, int same_next) {
+    k_step_fft32(LaunchSet L, const unsigned char* __restrict__ images, float2* __restrict__ psi,
+                 float2* __restrict__ P, float2* __restrict__ Pa, int fresh_p, int want_pa, int same_next) {
   extern __shared__ __align__(128) unsigned char q_raw[];
   QSmem& sm = *reinterpret_cast<QSmem*>(q_raw);
   cg::cluster_group cl = cg::this_cluster();
@@ -427,7 +457,14 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
   float2* band = psi + U.psi_off + (long long)b * c.npts + at;
   const float2* ph = (const float2*)L.ph_half + (long long)u * L.ph_stride;
   const float* qt = reinterpret_cast<const float*>(L.qt_half) + 4 * u;
+  const unsigned char* img = images + (size_t)(orb / c.n_bands) * Q_IMG;
   QState x = q_open(sm);
+  if (tid == 0) {
+    const uint32_t bar = bk_smem(&sm.mimg);
+    bk_mbar_expect_tx(bar, 32768);
+    bk_copy_g2s(bk_smem(sm.bket), img, 16384, bar);
+    bk_copy_g2s(bk_smem(sm.bbra), img + 16384, 16384, bar);
+  }
   float2 t[16];
   {
     float v[16];
@@ -454,9 +491,6 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
   }
   q_cell(sm, c);
   q_tables(sm, c, ph, r0);
-  q_build_ket(sm.bket, c, ph);
-  q_build_bra<1>(sm.bbra, c, ph);
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   const int line = (ry * QN + ix) * QP;                  // as a line: row ry, plane (frequency) ix
   float2* c1 = sm.b1 + ry * QN * QP + ix;                // the column, planes QP apart
   float2* c2 = sm.b2 + ry * QN * QP + ix;
@@ -464,24 +498,43 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
   const float2* dn = cl.map_shared_rank(sm.b1, (rank + QC - 1) & (QC - 1));
   const float dt = (float)(S.dt * L.dt_scale);
   float coef = 1.f;
-  bool ok = true;
+  bool ok = bk_mbar_wait(bk_smem(&sm.mimg), 0, BK_WAIT_POLLS);
+  q_arrive();   // (this CTA's b1 is free)
 #pragma unroll 1
   for (int m = 1; m <= 4; ++m) {
-    // W of s_{m-1}: partial sums over the CTA's rows, added over the cluster
-    if (m > 1 || fresh_p) {
-      q_stage(t, x);
-      ok = q_zsums<1>(x, sm.bbra, sm.b2) && ok;
-      q_moments<1>(sm, sm.b2, sm.part);
-      cl.sync();   // also: every neighbour is done with this CTA's b1
-    } else {
+    const bool chain = m > 1 || fresh_p;   // projections of s_{m-1} from the column, else from P
+    float2 f[16];
+    if (chain) q_stage(t, x);
+    q_wait();   // the neighbours are done with this CTA's b1 and partial sums
+#pragma unroll
+    for (int j = 0; j < 16; ++j) c1[(2 * j + h) * QP] = t[j];
+    um_fence_before();
+    __syncthreads();
+    if (chain && tid == 0) q_issue_bra<1>(x, sm.bbra);
+    // forward along z under the z sums' MMAs
+    q_line<-1>(c1, QP, h, f);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) c2[(2 * i + h) * QP] = f[i];
+    __syncthreads();
+    if (chain) {
+      ok = q_poll(x) && ok;
+      q_collect<1>(x, sm.b1);
+      um_fence_before();
+      __syncthreads();
+      q_moments<1>(sm, sm.b1, sm.part);
       __syncthreads();
     }
+    // forward along x
+    q_line<-1>(sm.b2 + line, 1, h, f);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sm.b1[line + 2 * i + h] = f[i];
+    cl.sync();   // rows and partial sums of every CTA
     {
       const int s = tid >> 2, a = sm.atom[s], j = 4 * a + (tid & 3);
       float2 w = make_float2(0.f, 0.f);
       if (a >= 0) {
         float2 p;
-        if (m > 1 || fresh_p) {
+        if (chain) {
           const float2 M = q_total(cl, sm.part, tid);
           const float sc = __fmul_rn(c.dvf, c.pnormf[j]);
           p = make_float2(__fmul_rn(sc, M.x), __fmul_rn(sc, M.y));
@@ -491,7 +544,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
         const float e = c.wkbf[j];
         w = make_float2(e * p.x, e * p.y);
       }
-      sm.b2[tid] = w;   // (the z sums are consumed)
+      sm.b2[tid] = w;   // (the rows before the x transform are consumed)
     }
     __syncwarp();
     {
@@ -505,8 +558,6 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
       o[1] = q_mul(F, make_float2(wx.x, -wx.y));
       o[2] = q_mul(F, make_float2(wz.x, -wz.y));
     }
-#pragma unroll
-    for (int j = 0; j < 16; ++j) c1[(2 * j + h) * QP] = t[j];
     __syncthreads();
     {
       // the ket's A row of the column: groups 4 h .. 4 h + 3
@@ -541,14 +592,10 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
       q_st8(o + 16, rl);
       q_st8(o + 24, il);
     }
-    // forward along z, then the ket's MMAs under the transforms that follow
-    float2 f[16];
-    q_line<-1>(c1, QP, h, f);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) c2[(2 * i + h) * QP] = f[i];
     um_fence_before();
     __syncthreads();
     if (tid == 0) {
+      // the ket's MMAs, under the transforms that follow
       um_fence_after();
       constexpr uint32_t idesc = um_idesc_tf32(128, 32);
       const uint32_t b0 = bk_smem(sm.bket), b1 = b0 + 8192;
@@ -567,13 +614,15 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
       }
       um_commit(x.bar);
     }
-    // forward along x
-    q_line<-1>(sm.b2 + line, 1, h, f);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) sm.b1[line + 2 * i + h] = f[i];
-    cl.sync();
     // symbol along x and z, stencil along y: thread (k_x = lane, k_z = warp + 8 i), four rows
-#pragma unroll 1
+    float2 wl[4], wg[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      wl[e] = make_float2(sm.wl[e], sm.wl[e]);
+      wg[e] = make_float2(sm.wg[e], sm.wg[e]);
+    }
+    const float lx = sm.lx[lane];
+#pragma unroll 2
     for (int i = 0; i < 4; ++i) {
       const int kz = warp + 8 * i, o = kz * QP + lane;
       float2 w[12];
@@ -583,7 +632,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
         w[4 + r] = sm.b1[r * QN * QP + o];
         w[8 + r] = up[r * QN * QP + o];
       }
-      const float l = sm.lx[lane] + sm.lz[kz];
+      const float l = lx + sm.lz[kz];
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         float2 k = __fmul2_rn(make_float2(l, l), w[4 + r]);
@@ -591,12 +640,13 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
 #pragma unroll
         for (int e = 1; e <= 4; ++e) {
           const float2 a = w[4 + r + e], d = w[4 + r - e];
-          k = __ffma2_rn(make_float2(sm.wl[e - 1], sm.wl[e - 1]), fft_add(a, d), k);
-          g = __ffma2_rn(make_float2(sm.wg[e - 1], sm.wg[e - 1]), fft_sub(a, d), g);
+          k = __ffma2_rn(wl[e - 1], fft_add(a, d), k);
+          g = __ffma2_rn(wg[e - 1], fft_sub(a, d), g);
         }
         sm.b2[r * QN * QP + o] = make_float2(k.x + g.y, k.y - g.x);   // -i q grad
       }
     }
+    q_arrive();
     __syncthreads();
     // back along x (in place: the line's two threads sit in warps w and w + 4) and z
     q_line<1>(sm.b2 + line, 1, h, f);
@@ -647,21 +697,21 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
   }
 #pragma unroll
   for (int j = 0; j < 16; ++j) band[2 * j * QN * QN] = t[j];
+  q_wait();   // the neighbours are done with b1
   if (want_pa) {
     // a constant field leaves the step's tables in place (q_obs = q_half)
-    const float2* pho = (const float2*)L.ph_obs + (long long)u * L.ph_stride;
-    cl.sync();   // the neighbours are done with b1, this CTA with its tables
-    if (!same_next) q_tables(sm, c, pho, r0);
+    __syncthreads();   // this CTA is done with its tables
+    if (!same_next) q_tables(sm, c, (const float2*)L.ph_obs + (long long)u * L.ph_stride, r0);
     q_stage(t, x);
-    ok = q_current(sm, cl, x, c, same_next ? ph : pho, Pa + U.pa_off + 4LL * b * c.n_proj,
-                   same_next ? Pu : nullptr) && ok;
+    ok = q_current(sm, cl, x, c, img, 1, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr) && ok;
   }
   q_close(cl, x, ok, S.status);
 }
 
 // Projections of the current outside a step.
 __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
-    k_pa_fft32(LaunchSet L, const float2* __restrict__ src, float2* __restrict__ Pa) {
+    k_pa_fft32(LaunchSet L, const unsigned char* __restrict__ images, const float2* __restrict__ src,
+               float2* __restrict__ Pa) {
   extern __shared__ __align__(128) unsigned char q_raw[];
   QSmem& sm = *reinterpret_cast<QSmem*>(q_raw);
   cg::cluster_group cl = cg::this_cluster();
@@ -682,15 +732,16 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
   q_stage(t, x);
   q_cell(sm, c);
   q_tables(sm, c, ph, rank * QR);
-  const bool ok = q_current(sm, cl, x, c, ph, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
+  const bool ok = q_current(sm, cl, x, c, images + (size_t)(orb / c.n_bands) * Q_IMG, 0,
+                            Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
   q_close(cl, x, ok, L.subs[U.sub].status);
 }
 
-bool q_taken(const LaunchSet& L) {
-  const CellDev& c = L.cell;
-  return L.variant == 0 && c.n1 == QN && c.n2 == QN && c.n3 == QN && c.nd == 4 && c.use_proj && c.n_atoms <= QA &&
-         c.zs_n > 0 && c.zs_n <= QG && c.xc_n > 0 && c.yc_n > 0;
+bool q_cell_ok(const CellDev& c) {
+  return c.n1 == QN && c.n2 == QN && c.n3 == QN && c.nd == 4 && c.use_proj && c.n_atoms <= QA && c.zs_n > 0 &&
+         c.zs_n <= QG && c.xc_n > 0 && c.yc_n > 0;
 }
+bool q_taken(const LaunchSet& L) { return L.variant == 0 && L.images != nullptr && q_cell_ok(L.cell); }
 
 template <typename K> void q_attr(K* k) {
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(QSmem));
@@ -700,12 +751,19 @@ static_assert(sizeof(QSmem) <= 115712, "two CTAs per SM");
 
 }  // namespace
 
+size_t step_fft32_images(const CellDev& c, int n_units) { return q_cell_ok(c) ? Q_IMG * (size_t)n_units : 0; }
+
+void launch_images_fft32(const LaunchSet& L, void* stream) {
+  if (L.n_units == 0 || !q_taken(L)) return;
+  k_images32<<<dim3(L.n_units, 3), QT, 0, (cudaStream_t)stream>>>(L, (unsigned char*)L.images);
+}
+
 bool launch_step_fft32(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
                        void* stream) {
   if (L.n_units == 0 || !q_taken(L)) return false;
   q_attr(k_step_fft32);
   k_step_fft32<<<(unsigned)L.n_units * L.cell.n_bands * QC, QT, sizeof(QSmem), (cudaStream_t)stream>>>(
-      L, (float2*)psi, (float2*)P, (float2*)Pa, fresh_p, want_pa, same_next);
+      L, (const unsigned char*)L.images, (float2*)psi, (float2*)P, (float2*)Pa, fresh_p, want_pa, same_next);
   return true;
 }
 
@@ -713,6 +771,6 @@ bool launch_pa_fft32(const LaunchSet& L, const void* src, void* Pa, void* stream
   if (L.n_units == 0 || !q_taken(L)) return false;
   q_attr(k_pa_fft32);
   k_pa_fft32<<<(unsigned)L.n_units * L.cell.n_bands * QC, QT, sizeof(QSmem), (cudaStream_t)stream>>>(
-      L, (const float2*)src, (float2*)Pa);
+      L, (const unsigned char*)L.images, (const float2*)src, (float2*)Pa);
   return true;
 }
