@@ -173,9 +173,16 @@ bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int sam
     attr = true;
   }
   const unsigned grid = (unsigned)L.n_units * (unsigned)L.cell.n_bands;
-  if (fs_umma(L))
-    k_step_fft<<<grid, FX_NP, sizeof(FxSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P, (float2*)Pa,
-                                                                      same_next, want_pa);
+  if (fs_umma(L)) {
+    // bands per CTA: as many as leave 13 waves of CTAs (two per SM), so that the last
+    // one costs little.  65 536 orbitals: 6.91 (1 band), 6.57 (2), 6.38 (4), 6.32 ms (8);
+    // 16 384: 1.93, 1.89, 1.86, 1.92; 4096 (three launches a step): 1.27, 1.29, 1.30, 1.47.
+    int per = 1;
+    while (per < 8 && (long long)grid / (2 * per) >= 13 * 304) per *= 2;
+    const unsigned ctas = (unsigned)L.n_units * (unsigned)((L.cell.n_bands + per - 1) / per);
+    k_step_fft<<<ctas, FX_NP, sizeof(FxSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P, (float2*)Pa,
+                                                                      same_next, want_pa, per);
+  }
   else
     k_step_fused<4><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P, (float2*)Pa,
                                                                            same_next);

@@ -26,10 +26,10 @@
 // Each thread's row of A goes to tensor memory split into TF32 hi and lo (three
 // products, FP32 accumulate); B (hi, lo) sits in shared memory in the canonical
 // K-major layout; one thread issues the MMAs (M = 128 per half of the columns).
-// Tensor-memory columns of a CTA: bra accumulator [0, 64) (32 per half), v_eff in
-// the 16 columns behind a first-order accumulator, Taylor sum [64, 128), and
-// [128, 256), 64 per half, the bra's A (hi, lo 32 each) or the ket's A (hi, lo 16
-// each) and accumulator, whichever is live.
+// Tensor-memory columns of a CTA, 32 per half of the columns: [0, 64) the first-order
+// bra accumulator (16) and v_eff (16); [64, 128) the Taylor sum, and after it the
+// second-order accumulator; and [128, 256), 64 per half, the bra's A (hi, lo 32 each)
+// or the ket's A (hi, lo 16 each) and accumulator, whichever is live.
 #pragma once
 #include "tsbz_fft.cuh"
 #include "tsbz_fused.cuh"
@@ -46,21 +46,22 @@
 #define FX_BRA_D 0
 #define FX_VEFF 16
 #define FX_ACC 64
+#define FX_BRA2_D 64
 #define FX_BRA_A 128
 #define FX_KET_A 128
 #define FX_KET_D 160
 
 struct FxSmem {
   float2 buf[FX_N * FX_PL];          // line transforms; second-order z sums
-  float2 sums[2 * FX_G * FX_PL];     // first-order z sums; B of the second-order pass
+  float2 sums[2 * FX_G * FX_PL];     // first-order z sums
   unsigned char bket[4096];          // B of the ket (hi, lo)
   unsigned char bbra[4096];          // B of the first-order bra (hi, lo)
+  unsigned char bbra2[8192];         // B of the second-order bra (hi, lo)
   float4 zt[FX_G * FX_N];            // z factors per group (Re F, Im F, d, 0)
   float4 xt[FX_S * FX_N];            // x and y factors per slot
   float4 yt[FX_S * FX_N];
   float4 xpk[FX_S * FX_N * 3];       // d_x^w F_x as (Re, Re, Im, Im) pairs, w = 0..2
   float2 gt[FX_S * 3 * FX_N];        // ket column tables
-  float2 wt[4 * FX_S];               // W of the band at the start
   float psc[4 * FX_S];               // dV pn: projection from a monomial sum
   float wsc[4 * FX_S];               // pn E times that: W from a monomial sum
   float2 mres[FX_S * 10];            // monomial sums
@@ -124,19 +125,18 @@ __device__ __forceinline__ bool fx_poll(FxState& x) {
   return ok;
 }
 
-// Slots and scales of the cell (read after a barrier).
-__device__ __forceinline__ void fx_slots(FxSmem& sm, const CellDev& c) {
-  const int s = threadIdx.x;
-  if (s < FX_S) {
-    const int g = s >> 1, j = s & 1;
-    sm.atom[s] = g < c.n_zg && j < c.zg_off[g + 1] - c.zg_off[g] ? c.zg_mem[c.zg_off[g] + j] : -1;
-  }
+// Atom of a slot (-1: empty).
+__device__ __forceinline__ int fx_atom(const CellDev& c, int s) {
+  const int g = s >> 1, j = s & 1;
+  return g < c.n_zg && j < c.zg_off[g + 1] - c.zg_off[g] ? c.zg_mem[c.zg_off[g] + j] : -1;
 }
+// Slots and scales of the cell (read after a barrier).
 __device__ __forceinline__ void fx_scales(FxSmem& sm, const CellDev& c) {
   const int s = threadIdx.x;
   if (s < 4 * FX_S) {
-    const int a = sm.atom[s >> 2], j = 4 * a + (s & 3);
+    const int a = fx_atom(c, s >> 2), j = 4 * a + (s & 3);
     const float p = a < 0 ? 0.f : c.dvf * c.pnormf[j];
+    if ((s & 3) == 0) sm.atom[s >> 2] = a;
     sm.psc[s] = p;
     sm.wsc[s] = a < 0 ? 0.f : p * c.wkbf[j];
   }
@@ -145,7 +145,7 @@ __device__ __forceinline__ void fx_scales(FxSmem& sm, const CellDev& c) {
 // Factor tables of one phase table; read after a barrier.
 __device__ __forceinline__ void fx_tables(FxSmem& sm, const CellDev& c, const float2* ph) {
   const int tid = threadIdx.x, i = tid & (FX_N - 1), ax = (tid / FX_N) & 1, s = tid / (2 * FX_N);
-  const int a = sm.atom[s];
+  const int a = fx_atom(c, s);
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (a >= 0) {
     const int idx = (a * 3 + ax) * FX_N + i;
@@ -166,7 +166,7 @@ __device__ __forceinline__ void fx_tables(FxSmem& sm, const CellDev& c, const fl
     }
   }
   if (tid < FX_G * FX_N) {
-    const int z = tid & (FX_N - 1), a0 = sm.atom[2 * (tid / FX_N)];
+    const int z = tid & (FX_N - 1), a0 = fx_atom(c, 2 * (tid / FX_N));
     float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
     if (a0 >= 0) {
       const int idx = (a0 * 3 + 2) * FX_N + z;
@@ -241,7 +241,7 @@ template <int D> __device__ __forceinline__ void fx_issue_bra(const FxState& x, 
   const uint32_t b0 = bk_smem(bz), b1 = b0 + LO;
 #pragma unroll
   for (int hh = 0; hh < 2; ++hh) {
-    const uint32_t d = x.tbase + FX_BRA_D + 32 * hh;
+    const uint32_t d = x.tbase + (D == 1 ? FX_BRA_D : FX_BRA2_D) + 32 * hh;
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) {
       const uint32_t a_hi = x.tbase + FX_BRA_A + 64 * hh + 8 * ks, a_lo = a_hi + 32;
@@ -258,7 +258,7 @@ template <int D> __device__ __forceinline__ void fx_issue_bra(const FxState& x, 
 template <int D> __device__ __forceinline__ void fx_collect(const FxState& x, float2* zs) {
   const int tid = threadIdx.x, warp = tid >> 5, h = warp >> 2, qd = warp & 3;
   float2* o = zs + (tid / FX_N) * FX_ROW + (tid & (FX_N - 1));
-  const uint32_t at = um_addr(x.tbase, qd, FX_BRA_D + 32 * h);
+  const uint32_t at = um_addr(x.tbase, qd, (D == 1 ? FX_BRA_D : FX_BRA2_D) + 32 * h);
   if constexpr (D == 1) {
     float d[16];
     um_ld16(at, d);
@@ -384,11 +384,14 @@ __device__ __forceinline__ void fx_store_pa(FxSmem& sm, const float2* zs, float2
 }
 
 // A whole order-D pass over the staged column: z sums in zs (read after the
-// function); false when the MMAs did not complete.  bz: 4 D KiB.
+// function); false when the MMAs did not complete.  build: B is formed in bz here (else
+// it is there already, fenced).
 template <int D>
-__device__ __forceinline__ bool fx_pass(FxSmem& sm, FxState& x, unsigned char* bz, float2* zs) {
-  fx_build_bra<D>(sm, bz);
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+__device__ __forceinline__ bool fx_pass(FxSmem& sm, FxState& x, unsigned char* bz, float2* zs, bool build) {
+  if (build) {
+    fx_build_bra<D>(sm, bz);
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+  }
   um_fence_before();
   __syncthreads();
   if (threadIdx.x == 0) fx_issue_bra<D>(x, bz);
@@ -412,245 +415,280 @@ __device__ __forceinline__ void fx_ket_tables(FxSmem& sm, float2 ws, float2 wx, 
   }
 }
 
+// W of slot `warp` from the band's projections (lane t < 4 gets projector t), and the
+// ket tables from it (every lane of the warp).
+__device__ __forceinline__ float2 fx_load_w(const CellDev& c, const float2* __restrict__ Pu) {
+  const int lane = threadIdx.x & 31, a = fx_atom(c, threadIdx.x >> 5);
+  float2 w = make_float2(0.f, 0.f);
+  if (a >= 0 && lane < 4) {
+    const float2 p = Pu[4 * a + lane];
+    const float e = c.wkbf[4 * a + lane];
+    w = make_float2(e * p.x, e * p.y);
+  }
+  return w;
+}
+__device__ __forceinline__ void fx_ket_from_w(FxSmem& sm, float2 w) {
+  float2 v[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+    v[t] = make_float2(__shfl_sync(0xffffffffu, w.x, t), __shfl_sync(0xffffffffu, w.y, t));
+  fx_ket_tables(sm, v[0], v[1], v[2], v[3]);
+}
+
+// One CTA takes `per` bands of a unit in turn: under a constant field the unit's
+// tables and operand matrices, v_eff and the symbol serve them all, and the next
+// band is on its way to L2.  The set-up is a chain of dependent loads, about 1.0 ms
+// of the 6.9 ms launch with one band per CTA (65 536 orbitals).
 __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __restrict__ psi, float2* __restrict__ P,
-                                                       float2* __restrict__ Pa, int same_next, int want_pa) {
+                                                       float2* __restrict__ Pa, int same_next, int want_pa, int per) {
   constexpr int N = FX_N, NP = FX_NP, Q = 2 * FX_G;
   extern __shared__ __align__(128) unsigned char fs_raw[];
   FxSmem& sm = *reinterpret_cast<FxSmem*>(fs_raw);
   const CellDev& c = L.cell;
-  const int b = blockIdx.x % c.n_bands;
-  const int u = L.unit_ids[blockIdx.x / c.n_bands];
-  if (!unit_active(L, u)) return;
+  const int groups = (c.n_bands + per - 1) / per;
+  const int u = L.unit_ids[blockIdx.x / groups];
   const UnitDev U = L.units[u];
-  const SubDev S = L.subs[U.sub];
   const int tid = threadIdx.x, lo = tid & (N - 1), hi = tid / N;   // as a column: ix, iy
   const int warp = tid >> 5, h = warp >> 2, qd = warp & 3;
-  float2* Pu = P + U.p_off + (long long)b * c.n_proj;
-  float2* band = psi + U.psi_off + (long long)b * FX_PTS + tid;
-  fx_slots(sm, c);
-  FxState x = fx_open(sm);
+  const int b0 = (blockIdx.x % groups) * per, b1 = min(b0 + per, c.n_bands);
+  const long long off = (long long)u * L.ph_stride;
+  float2* band = psi + U.psi_off + (long long)b0 * FX_PTS + tid;
+  // every load of the set-up is issued before the first barrier
   float2 t[N];
+#pragma unroll
+  for (int z = 0; z < N; ++z) t[z] = band[z * NP];
+  const SubDev S = L.subs[U.sub];
+  if (*S.active == 0) return;
+  float2 w = fx_load_w(c, P + U.p_off + (long long)b0 * c.n_proj);
+  fx_tables(sm, c, (const float2*)L.ph_half + off);
+  fx_scales(sm, c);
+  if (tid < 3 * N) {
+    // kinetic symbol, the transforms' 1/N^3 folded in
+    const int ax = tid / N, k = tid - ax * N;
+    const float q = reinterpret_cast<const float*>(L.qt_half)[4 * u + ax];
+    const float* s = c.ksymf + 2 * ax * N;
+    sm.lam[tid] = fmaf(q, s[N + k], fmaf(0.5f * q, q, s[k])) * (1.f / (N * N * N));
+  }
+  FxState x = fx_open(sm);   // (and the barrier behind the tables)
   {
     float v[N];
     const float* veff = reinterpret_cast<const float*>(S.veff) + tid;
 #pragma unroll
-    for (int z = 0; z < N; ++z) {
-      t[z] = band[z * NP];
-      v[z] = veff[z * NP];
-    }
-    fx_tables(sm, c, (const float2*)L.ph_half + (long long)u * L.ph_stride);
-    fx_scales(sm, c);
+    for (int z = 0; z < N; ++z) v[z] = veff[z * NP];
     um_st16(um_addr(x.tbase, qd, FX_VEFF + 32 * h), reinterpret_cast<uint32_t(&)[16]>(v));
-    um_st32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(t));
   }
-  const float* qt = reinterpret_cast<const float*>(L.qt_half) + 4 * u;
-  if (tid < 3 * N) {
-    // kinetic symbol, the transforms' 1/N^3 folded in
-    const int ax = tid / N, k = tid - ax * N;
-    const float q = qt[ax];
-    const float* s = c.ksymf + 2 * ax * N;
-    sm.lam[tid] = fmaf(q, s[N + k], fmaf(0.5f * q, q, s[k])) * (1.f / (N * N * N));
-  } else if (tid >= 64 && tid < 64 + 4 * FX_S) {
-    const int j = tid - 64, a = sm.atom[j >> 2], i = 4 * a + (j & 3);
-    float2 w = make_float2(0.f, 0.f);
-    if (a >= 0) {
-      const float2 p = Pu[i];
-      const float e = c.wkbf[i];
-      w = make_float2(e * p.x, e * p.y);
-    }
-    sm.wt[j] = w;
-  }
-  __syncthreads();
   fx_build_ket(sm);
   fx_build_bra<1>(sm, sm.bbra);
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // both B's, issued behind later barriers
-  fx_ket_tables(sm, sm.wt[4 * warp], sm.wt[4 * warp + 1], sm.wt[4 * warp + 2], sm.wt[4 * warp + 3]);
+  const bool keep = same_next && per > 1;   // one second-order B for all bands
+  if (keep) fx_build_bra<2>(sm, sm.bbra2);
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // the B's, issued behind later barriers
   float2* colp = sm.buf + hi * FX_ROW + lo;            // the column: planes FX_PL apart
   float2* rowp = sm.buf + hi * FX_PL + lo * FX_ROW;    // row y = lo of plane z = hi
   float2* linp = sm.buf + hi * FX_PL + lo;             // line x = lo of plane z = hi
   const float dt = (float)(S.dt * L.dt_scale);
-  float coef = 1.f;
-  bool ok = true;
 #pragma unroll 1
-  for (int m = 1; m <= 4; ++m) {
-    float2 f[N];
+  for (int b = b0; b < b1; ++b, band += FX_PTS) {
+    float2* Pu = P + U.p_off + (long long)b * c.n_proj;
+    if (b > b0) {
 #pragma unroll
-    for (int z = 0; z < N; ++z) f[z] = t[z];
-    fft_line<N, -1>(f);
-#pragma unroll
-    for (int z = 0; z < N; ++z) colp[z * FX_PL] = f[z];
-    __syncthreads();
-    // forward along x and y, the symbol, back: within the half-warp's plane
-#pragma unroll
-    for (int k = 0; k < N; ++k) f[k] = rowp[k];
-    fft_line<N, -1>(f);
-#pragma unroll
-    for (int k = 0; k < N; ++k) rowp[k] = f[k];
-    __syncwarp();
-#pragma unroll
-    for (int y = 0; y < N; ++y) f[y] = linp[y * FX_ROW];
-    fft_line<N, -1>(f);
-    {
-      const float l0 = sm.lam[lo] + sm.lam[2 * N + hi];
-#pragma unroll
-      for (int y = 0; y < N; ++y) {
-        const float l = l0 + sm.lam[N + y];
-        f[y] = __fmul2_rn(make_float2(l, l), f[y]);
+      for (int z = 0; z < N; ++z) t[z] = band[z * NP];
+      w = fx_load_w(c, Pu);
+      __syncthreads();   // the last band's sums are consumed
+      if (!same_next) {
+        fx_tables(sm, c, (const float2*)L.ph_half + off);
+        __syncthreads();
+        fx_build_bra<1>(sm, sm.bbra);
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
       }
     }
-    fft_line<N, 1>(f);
-#pragma unroll
-    for (int y = 0; y < N; ++y) linp[y * FX_ROW] = f[y];
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < N; ++k) f[k] = rowp[k];
-    fft_line<N, 1>(f);
-#pragma unroll
-    for (int k = 0; k < N; ++k) rowp[k] = f[k];
-    if (m > 1) {
-      ok = ok && fx_poll(x);   // z sums of s_{m-1}
-      fx_collect<1>(x, sm.sums);
+    if (b + 1 < b1) {
+      const char* next = reinterpret_cast<const char*>(band - tid + FX_PTS) + 128 * tid;
+      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(next));
     }
-    if (!__syncthreads_and(ok)) {
-      if (m > 1) {
-        fx_bail(x, S.status);
-      } else {
-        fx_close(x);
-      }
-      return;
-    }
+    um_st32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(t));
+    fx_ket_from_w(sm, w);
+    float coef = 1.f;
+    bool ok = true;
+#pragma unroll 1
+    for (int m = 1; m <= 4; ++m) {
+      float2 f[N];
 #pragma unroll
-    for (int z = 0; z < N; ++z) f[z] = colp[z * FX_PL];
-    if (m > 1) {
-      float2 v[3], m2;
-      fx_moments<1>(sm, sm.sums, v, m2);
-      const float* sc = sm.wsc + 4 * warp;
-      fx_ket_tables(sm, make_float2(sc[0] * v[0].x, sc[0] * v[0].y), make_float2(sc[1] * v[1].x, sc[1] * v[1].y),
-                    make_float2(sc[2] * v[2].x, sc[2] * v[2].y), make_float2(sc[3] * v[0].x, sc[3] * v[0].y));
-    }
-    fft_line<N, 1>(f);   // the kinetic term of the column
-    __syncthreads();
-    {
-      // the ket's A row of the column
-      float2 av[Q];
+      for (int z = 0; z < N; ++z) f[z] = t[z];
+      fft_line<N, -1>(f);
 #pragma unroll
-      for (int q = 0; q < Q; ++q) av[q] = make_float2(0.f, 0.f);
+      for (int z = 0; z < N; ++z) colp[z * FX_PL] = f[z];
+      __syncthreads();
+      // forward along x and y, the symbol, back: within the half-warp's plane
 #pragma unroll
-      for (int s = 0; s < FX_S; ++s) {
-        const float4 fy = sm.yt[s * N + hi];
-        const float2 g0 = sm.gt[(s * 3 + 0) * N + lo], g1 = sm.gt[(s * 3 + 1) * N + lo];
-        const float2 g2 = sm.gt[(s * 3 + 2) * N + lo];
-        const float2 e = __ffma2_rn(make_float2(fy.z, fy.z), g1, g0);
-        float2& a0 = av[2 * (s >> 1)];
-        float2& a1 = av[2 * (s >> 1) + 1];
-        a0.x = fmaf(fy.x, e.x, fmaf(-fy.y, e.y, a0.x));
-        a0.y = fmaf(fy.x, e.y, fmaf(fy.y, e.x, a0.y));
-        a1.x = fmaf(fy.x, g2.x, fmaf(-fy.y, g2.y, a1.x));
-        a1.y = fmaf(fy.x, g2.y, fmaf(fy.y, g2.x, a1.y));
-      }
-      uint32_t ah[16], al[16];
+      for (int k = 0; k < N; ++k) f[k] = rowp[k];
+      fft_line<N, -1>(f);
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        fs_split(av[q].x, ah[q], al[q]);
-        fs_split(av[q].y, ah[Q + q], al[Q + q]);
-      }
-      um_st16(um_addr(x.tbase, qd, FX_KET_A + 64 * h), ah);
-      um_st16(um_addr(x.tbase, qd, FX_KET_A + 64 * h + 16), al);
-    }
-    um_fence_before();
-    __syncthreads();
-    if (tid == 0) {
-      um_fence_after();
-      constexpr uint32_t idesc = um_idesc_tf32(128, 32);
-      const uint32_t b0 = bk_smem(sm.bket), b1 = b0 + 2048;
+      for (int k = 0; k < N; ++k) rowp[k] = f[k];
+      __syncwarp();
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        const uint32_t d = x.tbase + FX_KET_D + 64 * hh;
+      for (int y = 0; y < N; ++y) f[y] = linp[y * FX_ROW];
+      fft_line<N, -1>(f);
+      {
+        const float l0 = sm.lam[lo] + sm.lam[2 * N + hi];
 #pragma unroll
-        for (int ks = 0; ks < 2; ++ks) {
-          const uint32_t a_hi = x.tbase + FX_KET_A + 64 * hh + 8 * ks, a_lo = a_hi + 16;
-          const uint64_t bh = um_sdesc(b0 + 256 * ks, 128, 512), bl = um_sdesc(b1 + 256 * ks, 128, 512);
-          um_mma_tf32_ts(d, a_lo, bh, idesc, ks > 0);
-          um_mma_tf32_ts(d, a_hi, bl, idesc, true);
-          um_mma_tf32_ts(d, a_hi, bh, idesc, true);
+        for (int y = 0; y < N; ++y) {
+          const float l = l0 + sm.lam[N + y];
+          f[y] = __fmul2_rn(make_float2(l, l), f[y]);
         }
       }
-      um_commit(x.bar);
-    }
-    // s_m = kinetic + v s_{m-1} + V_NL s_{m-1}
-    {
-      float v[16];
-      um_ld16(um_addr(x.tbase, qd, FX_VEFF + 32 * h), v);
+      fft_line<N, 1>(f);
 #pragma unroll
-      for (int z = 0; z < N; ++z) t[z] = __ffma2_rn(make_float2(v[z], v[z]), t[z], f[z]);
-    }
-    ok = fx_poll(x);
-    {
-      float d[32];
-      um_ld32(um_addr(x.tbase, qd, FX_KET_D + 64 * h), d);   // conj(V_NL s_{m-1})
+      for (int y = 0; y < N; ++y) linp[y * FX_ROW] = f[y];
+      __syncwarp();
 #pragma unroll
-      for (int z = 0; z < N; ++z) {
-        t[z].x += d[2 * z];
-        t[z].y -= d[2 * z + 1];
+      for (int k = 0; k < N; ++k) f[k] = rowp[k];
+      fft_line<N, 1>(f);
+#pragma unroll
+      for (int k = 0; k < N; ++k) rowp[k] = f[k];
+      if (m > 1) {
+        ok = ok && fx_poll(x);   // z sums of s_{m-1}
+        fx_collect<1>(x, sm.sums);
       }
-    }
-    if (m < 4) fx_stage(t, x);   // the bra's A
-    // psi += (-i)^m dt^m / m! s_m
-    coef *= dt / (float)m;
-    {
-      float2 a[N];
-      um_ld32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(a));
-      const float sg = m == 1 || m == 4 ? coef : -coef;
-      if (m & 1) {
+      if (!__syncthreads_and(ok)) {
+        if (m > 1) {
+          fx_bail(x, S.status);
+        } else {
+          fx_close(x);
+        }
+        return;
+      }
+#pragma unroll
+      for (int z = 0; z < N; ++z) f[z] = colp[z * FX_PL];
+      if (m > 1) {
+        float2 v[3], m2;
+        fx_moments<1>(sm, sm.sums, v, m2);
+        const float* sc = sm.wsc + 4 * warp;
+        fx_ket_tables(sm, make_float2(sc[0] * v[0].x, sc[0] * v[0].y), make_float2(sc[1] * v[1].x, sc[1] * v[1].y),
+                      make_float2(sc[2] * v[2].x, sc[2] * v[2].y), make_float2(sc[3] * v[0].x, sc[3] * v[0].y));
+      }
+      fft_line<N, 1>(f);   // the kinetic term of the column
+      __syncthreads();
+      {
+        // the ket's A row of the column
+        float2 av[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) av[q] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < FX_S; ++s) {
+          const float4 fy = sm.yt[s * N + hi];
+          const float2 g0 = sm.gt[(s * 3 + 0) * N + lo], g1 = sm.gt[(s * 3 + 1) * N + lo];
+          const float2 g2 = sm.gt[(s * 3 + 2) * N + lo];
+          const float2 e = __ffma2_rn(make_float2(fy.z, fy.z), g1, g0);
+          float2& a0 = av[2 * (s >> 1)];
+          float2& a1 = av[2 * (s >> 1) + 1];
+          a0.x = fmaf(fy.x, e.x, fmaf(-fy.y, e.y, a0.x));
+          a0.y = fmaf(fy.x, e.y, fmaf(fy.y, e.x, a0.y));
+          a1.x = fmaf(fy.x, g2.x, fmaf(-fy.y, g2.y, a1.x));
+          a1.y = fmaf(fy.x, g2.y, fmaf(fy.y, g2.x, a1.y));
+        }
+        uint32_t ah[16], al[16];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          fs_split(av[q].x, ah[q], al[q]);
+          fs_split(av[q].y, ah[Q + q], al[Q + q]);
+        }
+        um_st16(um_addr(x.tbase, qd, FX_KET_A + 64 * h), ah);
+        um_st16(um_addr(x.tbase, qd, FX_KET_A + 64 * h + 16), al);
+      }
+      um_fence_before();
+      __syncthreads();
+      if (tid == 0) {
+        um_fence_after();
+        constexpr uint32_t idesc = um_idesc_tf32(128, 32);
+        const uint32_t b0 = bk_smem(sm.bket), b1 = b0 + 2048;
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          const uint32_t d = x.tbase + FX_KET_D + 64 * hh;
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks) {
+            const uint32_t a_hi = x.tbase + FX_KET_A + 64 * hh + 8 * ks, a_lo = a_hi + 16;
+            const uint64_t bh = um_sdesc(b0 + 256 * ks, 128, 512), bl = um_sdesc(b1 + 256 * ks, 128, 512);
+            um_mma_tf32_ts(d, a_lo, bh, idesc, ks > 0);
+            um_mma_tf32_ts(d, a_hi, bl, idesc, true);
+            um_mma_tf32_ts(d, a_hi, bh, idesc, true);
+          }
+        }
+        um_commit(x.bar);
+      }
+      // s_m = kinetic + v s_{m-1} + V_NL s_{m-1}
+      {
+        float v[16];
+        um_ld16(um_addr(x.tbase, qd, FX_VEFF + 32 * h), v);
+#pragma unroll
+        for (int z = 0; z < N; ++z) t[z] = __ffma2_rn(make_float2(v[z], v[z]), t[z], f[z]);
+      }
+      ok = fx_poll(x);
+      {
+        float d[32];
+        um_ld32(um_addr(x.tbase, qd, FX_KET_D + 64 * h), d);   // conj(V_NL s_{m-1})
 #pragma unroll
         for (int z = 0; z < N; ++z) {
-          a[z].x = fmaf(sg, t[z].y, a[z].x);
-          a[z].y = fmaf(-sg, t[z].x, a[z].y);
+          t[z].x += d[2 * z];
+          t[z].y -= d[2 * z + 1];
         }
-      } else {
-#pragma unroll
-        for (int z = 0; z < N; ++z) a[z] = __ffma2_rn(make_float2(sg, sg), t[z], a[z]);
       }
-      if (m < 4) {
-        um_st32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(a));
-      } else {
+      if (m < 4) fx_stage(t, x);   // the bra's A
+      // psi += (-i)^m dt^m / m! s_m
+      coef *= dt / (float)m;
+      {
+        float2 a[N];
+        um_ld32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(a));
+        const float sg = m == 1 || m == 4 ? coef : -coef;
+        if (m & 1) {
 #pragma unroll
-        for (int z = 0; z < N; ++z) t[z] = a[z];
+          for (int z = 0; z < N; ++z) {
+            a[z].x = fmaf(sg, t[z].y, a[z].x);
+            a[z].y = fmaf(-sg, t[z].x, a[z].y);
+          }
+        } else {
+#pragma unroll
+          for (int z = 0; z < N; ++z) a[z] = __ffma2_rn(make_float2(sg, sg), t[z], a[z]);
+        }
+        if (m < 4) {
+          um_st32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(a));
+        } else {
+#pragma unroll
+          for (int z = 0; z < N; ++z) t[z] = a[z];
+        }
       }
+      um_fence_before();
+      if (!__syncthreads_and(ok)) {   // at m = 4: every buffer is free
+        fx_bail(x, S.status);
+        return;
+      }
+      if (m < 4 && tid == 0) fx_issue_bra<1>(x, sm.bbra);
     }
-    um_fence_before();
-    if (!__syncthreads_and(ok)) {   // at m = 4: every buffer is free
-      fx_bail(x, S.status);
-      return;
-    }
-    if (m < 4 && tid == 0) fx_issue_bra<1>(x, sm.bbra);
-  }
 #pragma unroll
-  for (int z = 0; z < N; ++z) band[z * NP] = t[z];
-  if (want_pa) {
-    // projections of the new psi: those of the next step (P, q of the next step) and of
-    // the current (Pa, q at t_{n+1}); a constant field makes both q's the step's own, so
-    // the tables stay and the next step's are the current's first-order sums
-    fx_stage(t, x);
-    const long long off = (long long)u * L.ph_stride;
-    bool done = true;
-    if (!same_next) {
-      fx_tables(sm, c, (const float2*)L.ph_next + off);
-      __syncthreads();
-      done = fx_pass<1>(sm, x, sm.bbra, sm.sums);
-      if (done) {
-        fx_store_p(sm, sm.sums, Pu);
+    for (int z = 0; z < N; ++z) band[z * NP] = t[z];
+    if (want_pa) {
+      // projections of the new psi: those of the next step (P, q of the next step) and of
+      // the current (Pa, q at t_{n+1}); a constant field makes both q's the step's own, so
+      // the tables stay and the next step's are the current's first-order sums
+      fx_stage(t, x);
+      bool done = true;
+      if (!same_next) {
+        fx_tables(sm, c, (const float2*)L.ph_next + off);
         __syncthreads();
-        fx_tables(sm, c, (const float2*)L.ph_obs + off);
-        __syncthreads();
+        done = fx_pass<1>(sm, x, sm.bbra, sm.sums, true);
+        if (done) {
+          fx_store_p(sm, sm.sums, Pu);
+          __syncthreads();
+          fx_tables(sm, c, (const float2*)L.ph_obs + off);
+          __syncthreads();
+        }
       }
+      done = done && fx_pass<2>(sm, x, sm.bbra2, sm.buf, !keep);
+      if (!done) {
+        fx_bail(x, S.status);
+        return;
+      }
+      fx_store_pa(sm, sm.buf, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
     }
-    done = done && fx_pass<2>(sm, x, reinterpret_cast<unsigned char*>(sm.sums), sm.buf);
-    if (!done) {
-      fx_bail(x, S.status);
-      return;
-    }
-    fx_store_pa(sm, sm.buf, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
   }
   fx_close(x);
 }
@@ -668,17 +706,16 @@ __global__ void __launch_bounds__(FX_NP, 2) k_project_fft(LaunchSet L, const flo
   const int u = L.unit_ids[blockIdx.x / c.n_bands];
   if (!unit_active(L, u)) return;
   const UnitDev U = L.units[u];
-  fx_slots(sm, c);
+  fx_scales(sm, c);
   FxState x = fx_open(sm);
   const float2* band = src + U.psi_off + (long long)b * FX_PTS + threadIdx.x;
   float2 t[FX_N];
 #pragma unroll
   for (int z = 0; z < FX_N; ++z) t[z] = band[z * FX_NP];
   fx_tables(sm, c, (const float2*)(PA ? L.ph_obs : L.ph_half) + (long long)u * L.ph_stride);
-  fx_scales(sm, c);
   fx_stage(t, x);
   __syncthreads();
-  if (!fx_pass<PA ? 2 : 1>(sm, x, reinterpret_cast<unsigned char*>(sm.sums), sm.buf)) {
+  if (!fx_pass<PA ? 2 : 1>(sm, x, sm.bbra2, sm.buf, true)) {
     fx_bail(x, L.subs[U.sub].status);
     return;
   }
