@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include "tsbz_internal.h"
+#include "tsbz_launch.cuh"
 
 namespace {
 
@@ -501,6 +502,7 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
                                                     typename AnyC<T>::V* __restrict__ P,
                                                     typename AnyC<T>::V* __restrict__ Pa, int fresh_p, int want_pa,
                                                     int same_next) {
+  step_enter();
   using V = typename AnyC<T>::V;
   extern __shared__ __align__(16) unsigned char any_raw[];
   const CellDev& c = L.cell;
@@ -657,7 +659,7 @@ bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh
   const unsigned grid = (unsigned)L.n_units * L.cell.n_bands;
   auto go = [&](auto k) {
     any_attr(k, bytes);
-    k<<<grid, ANY_T, bytes, (cudaStream_t)stream>>>(L, (V*)psi, (V*)P, (V*)Pa, fresh_p, want_pa, same_next);
+    step_launch(k, grid, ANY_T, bytes, stream, L, (V*)psi, (V*)P, (V*)Pa, fresh_p, want_pa, same_next);
   };
   if (any_fft8(L.cell)) go(k_step_any<T, true>); else go(k_step_any<T, false>);
   return true;

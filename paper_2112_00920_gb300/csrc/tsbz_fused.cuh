@@ -900,6 +900,7 @@ __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const f
                                                             double* __restrict__ rho_part,
                                                             double* __restrict__ jk_part,
                                                             double* __restrict__ nrm_part) {
+  step_enter();
   constexpr int ND = ZM_ND, N = FS_N, NP = FS_NP;
   extern __shared__ __align__(128) unsigned char fo_raw[];
   FoSmem& sm = *reinterpret_cast<FoSmem*>(fo_raw);

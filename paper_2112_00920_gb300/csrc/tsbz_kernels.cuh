@@ -21,6 +21,7 @@
 #include <math.h>
 #include "tsbz_fft.cuh"
 #include "tsbz_internal.h"
+#include "tsbz_launch.cuh"
 
 template <typename T> struct Cplx;
 template <> struct Cplx<double> { using type = double2; };
@@ -71,6 +72,7 @@ template <> struct Tab<float> {
 // ----------------------------------------------------------------------------
 template <typename T>
 __global__ void k_field(LaunchSet L, int mode) {
+  step_enter();
   using V = typename Cplx<T>::type;
   const int u = L.unit_ids[blockIdx.x];
   const UnitDev U = L.units[u];
@@ -731,6 +733,7 @@ template <typename T>
 __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename Cplx<T>::type* __restrict__ psi,
                                                      double* __restrict__ rho_part, double* __restrict__ jk_part,
                                                      double* __restrict__ nrm_part) {
+  step_enter();
   using V = typename Cplx<T>::type;
   __shared__ T red_n[TSBZ_BG][TSBZ_PT];
   __shared__ double red_j[3][TSBZ_PT / 32];
@@ -830,6 +833,7 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
     const double* __restrict__ q_obs, const typename Cplx<T>::type* __restrict__ Pa,
     const double* __restrict__ rho_part, const double* __restrict__ jk_part, const double* __restrict__ nrm_part,
     const int* __restrict__ mask, int mode) {
+  step_enter();
   using V = typename Cplx<T>::type;
   __shared__ double red[3][FIN_THREADS];
   __shared__ int last;
@@ -1147,6 +1151,7 @@ static __global__ void __launch_bounds__(HXC_THREADS) k_hxc_planes(const SubDev*
                                                                    const double2* __restrict__ tw2,
                                                                    const double2* __restrict__ tw3,
                                                                    double2* __restrict__ work) {
+  step_enter();
   extern __shared__ __align__(16) double2 hxc_sm[];
   const int n1 = c.n1, n2 = c.n2, n3 = c.n3, n13 = n1 * n3, ky = blockIdx.y;
   const SubDev S = subs[sub_ids[blockIdx.x]];
@@ -1185,6 +1190,7 @@ static __global__ void __launch_bounds__(HXC_THREADS) k_hxc_planes(const SubDev*
 template <typename T>
 __global__ void __launch_bounds__(64) k_hxc_sum(const SubDev* subs, const int* sub_ids, CellDev c,
                                                 const double2* __restrict__ tw2, const double2* __restrict__ work) {
+  step_enter();
   const int blocks = (c.npts + 63) / 64, sl = blockIdx.x / blocks;
   const int r = (blockIdx.x - sl * blocks) * 64 + threadIdx.x;
   if (r >= c.npts) return;
@@ -1264,7 +1270,7 @@ template <typename K> void stage_smem_attr(K* kernel, size_t bytes) {
 
 template <typename T> void launch_field(const LaunchSet& L, int mode, void* stream) {
   if (L.n_units == 0) return;
-  k_field<T><<<L.n_units, 128, 0, (cudaStream_t)stream>>>(L, mode);
+  step_launch(k_field<T>, L.n_units, 128, 0, stream, L, mode);
 }
 
 template <typename T>
@@ -1315,7 +1321,7 @@ void launch_observe(const LaunchSet& L, const void* psi, double* rho_part, doubl
   using V = typename Cplx<T>::type;
   if (L.n_units == 0) return;
   dim3 grid(L.cell.n_tiles, L.n_units, L.cell.n_bgroups);
-  k_observe<T><<<grid, TSBZ_PT, 0, (cudaStream_t)stream>>>(L, (const V*)psi, rho_part, jk_part, nrm_part);
+  step_launch(k_observe<T>, grid, TSBZ_PT, 0, stream, L, (const V*)psi, rho_part, jk_part, nrm_part);
 }
 
 template <typename T>
@@ -1326,8 +1332,8 @@ void launch_finalize_t(const SubDev* subs, int n_subs, const UnitDev* units, con
   if (n_subs == 0) return;
   // n_tiles (16 .. TSBZ_FIN_MAX_TILES) tiles per sub-simulation: density points, and units for the
   // current and the norms
-  k_finalize<T><<<dim3(n_subs, n_tiles), FIN_THREADS, 0, (cudaStream_t)stream>>>(subs, units, cells_dev, q_obs, (const V*)Pa,
-                                                                         rho_part, jk_part, nrm_part, mask, mode);
+  step_launch(k_finalize<T>, dim3(n_subs, n_tiles), FIN_THREADS, 0, stream, subs, units, cells_dev, q_obs,
+              (const V*)Pa, rho_part, jk_part, nrm_part, mask, mode);
 }
 
 template <typename T>
@@ -1343,9 +1349,10 @@ int launch_hxc_t(const SubDev* subs_dev, const int* sub_ids_dev, int n_subs, con
   if (c.poisson && (pow2 || total >= HXC_PLANES_MIN)) {
     const size_t sm = (size_t)2 * c.n1 * c.n3 * sizeof(double2);
     if (sm > 48 * 1024) cudaFuncSetAttribute(k_hxc_planes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_hxc_planes<<<dim3(n_subs, c.n2 / 2 + 1), HXC_THREADS, sm, st>>>(subs_dev, sub_ids_dev, c, tw[0], tw[1], tw[2],
-                                                                      wa);
-    k_hxc_sum<T><<<(unsigned)((long long)((c.npts + 63) / 64) * n_subs), 64, 0, st>>>(subs_dev, sub_ids_dev, c, tw[1], wa);
+    step_launch(k_hxc_planes, dim3(n_subs, c.n2 / 2 + 1), HXC_THREADS, sm, stream, subs_dev, sub_ids_dev, c, tw[0],
+                tw[1], tw[2], wa);
+    step_launch(k_hxc_sum<T>, (unsigned)((long long)((c.npts + 63) / 64) * n_subs), 64, 0, stream, subs_dev,
+                sub_ids_dev, c, tw[1], wa);
     return 2;
   }
   const int thr = 256;

@@ -1,5 +1,6 @@
 // Launchers of the single-precision fused stage and projection kernels.
 #include "tsbz_internal.h"
+#include "tsbz_launch.cuh"
 #include "tsbz_sep.cuh"
 #include "tsbz_fused.cuh"
 #include "tsbz_step32.cuh"
@@ -180,8 +181,8 @@ bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int sam
     int per = 1;
     while (per < 8 && (long long)grid / (2 * per) >= 13 * 304) per *= 2;
     const unsigned ctas = (unsigned)L.n_units * (unsigned)((L.cell.n_bands + per - 1) / per);
-    k_step_fft<<<ctas, FX_NP, sizeof(FxSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P, (float2*)Pa,
-                                                                      same_next, want_pa, per);
+    step_launch(k_step_fft, ctas, FX_NP, sizeof(FxSmem), stream, L, (float2*)psi, (float2*)P, (float2*)Pa, same_next,
+                want_pa, per);
   }
   else
     k_step_fused<4><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P, (float2*)Pa,
@@ -202,7 +203,7 @@ bool launch_observe_fused(const LaunchSet& L, const void* psi, double* rho_part,
     cudaFuncSetAttribute(k_observe_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FoSmem));
     attr = true;
   }
-  k_observe_fused<<<dim3(L.n_units, c.n_bgroups), FS_NP, sizeof(FoSmem), (cudaStream_t)stream>>>(L, (const float2*)psi, rho_part,
-                                                                              jk_part, nrm_part);
+  step_launch(k_observe_fused, dim3(L.n_units, c.n_bgroups), FS_NP, sizeof(FoSmem), stream, L, (const float2*)psi,
+              rho_part, jk_part, nrm_part);
   return true;
 }

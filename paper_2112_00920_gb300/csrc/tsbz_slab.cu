@@ -30,6 +30,7 @@
 #include "tsbz.h"
 #include "tsbz_bulk.cuh"
 #include "tsbz_internal.h"
+#include "tsbz_launch.cuh"
 #include "tsbz_zmarch.cuh"
 
 #define SL_N1 32                      // points per grid row
@@ -549,6 +550,7 @@ __device__ __forceinline__ uint32_t so_parity(long long q) { return (uint32_t)((
 __global__ void __launch_bounds__(SL_T, 3) k_observe_slab(LaunchSet L, const float2* __restrict__ psi,
                                                           double* __restrict__ rho_part, double* __restrict__ jk_part,
                                                           double* __restrict__ nrm_part) {
+  step_enter();
   constexpr int ND = SL_ND, NZ = SO_ZP, np = SO_ZP + SL_ND;
   extern __shared__ __align__(128) unsigned char soraw[];
   SoSmem& sm = *reinterpret_cast<SoSmem*>(soraw);
@@ -768,6 +770,6 @@ bool launch_observe_slab(const LaunchSet& L, const void* psi, double* rho_part, 
   const size_t smem = sizeof(SoSmem);
   cudaFuncSetAttribute(k_observe_slab, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const dim3 grid(c.n_bgroups * n_pt, L.n_units);
-  k_observe_slab<<<grid, SL_T, smem, (cudaStream_t)stream>>>(L, (const float2*)psi, rho_part, jk_part, nrm_part);
+  step_launch(k_observe_slab, grid, SL_T, smem, stream, L, (const float2*)psi, rho_part, jk_part, nrm_part);
   return true;
 }

@@ -441,6 +441,7 @@ __device__ __forceinline__ void fx_ket_from_w(FxSmem& sm, float2 w) {
 // of the 6.9 ms launch with one band per CTA (65 536 orbitals).
 __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __restrict__ psi, float2* __restrict__ P,
                                                        float2* __restrict__ Pa, int same_next, int want_pa, int per) {
+  step_enter();
   constexpr int N = FX_N, NP = FX_NP, Q = 2 * FX_G;
   extern __shared__ __align__(128) unsigned char fs_raw[];
   FxSmem& sm = *reinterpret_cast<FxSmem*>(fs_raw);

@@ -31,6 +31,7 @@
 #include "tsbz_bulk.cuh"
 #include "tsbz_fft.cuh"
 #include "tsbz_internal.h"
+#include "tsbz_launch.cuh"
 #include "tsbz_umma.cuh"
 
 namespace cg = cooperative_groups;
@@ -205,6 +206,7 @@ __device__ void q_build_ket(unsigned char* bz, const CellDev& c, const float2* p
 // current), and the step's CTAs fetch them by bulk copies.  Built in each of a
 // unit's 1024 CTAs they took 0.26 of 2.29 ms (128 bands).
 __global__ void __launch_bounds__(QT) k_images32(LaunchSet L, unsigned char* __restrict__ img) {
+  step_enter();
   const CellDev& c = L.cell;
   const int u = L.unit_ids[blockIdx.x];
   if (!unit_active(L, u)) return;
@@ -440,6 +442,7 @@ __device__ __forceinline__ void q_close(cg::cluster_group& cl, const QState& x, 
 __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
     k_step_fft32(LaunchSet L, const unsigned char* __restrict__ images, float2* __restrict__ psi,
                  float2* __restrict__ P, float2* __restrict__ Pa, int fresh_p, int want_pa, int same_next) {
+  step_enter();
   extern __shared__ __align__(128) unsigned char q_raw[];
   QSmem& sm = *reinterpret_cast<QSmem*>(q_raw);
   cg::cluster_group cl = cg::this_cluster();
@@ -755,15 +758,15 @@ size_t step_fft32_images(const CellDev& c, int n_units) { return q_cell_ok(c) ? 
 
 void launch_images_fft32(const LaunchSet& L, void* stream) {
   if (L.n_units == 0 || !q_taken(L)) return;
-  k_images32<<<dim3(L.n_units, 3), QT, 0, (cudaStream_t)stream>>>(L, (unsigned char*)L.images);
+  step_launch(k_images32, dim3(L.n_units, 3), QT, 0, stream, L, (unsigned char*)L.images);
 }
 
 bool launch_step_fft32(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
                        void* stream) {
   if (L.n_units == 0 || !q_taken(L)) return false;
   q_attr(k_step_fft32);
-  k_step_fft32<<<(unsigned)L.n_units * L.cell.n_bands * QC, QT, sizeof(QSmem), (cudaStream_t)stream>>>(
-      L, (const unsigned char*)L.images, (float2*)psi, (float2*)P, (float2*)Pa, fresh_p, want_pa, same_next);
+  step_launch(k_step_fft32, (unsigned)L.n_units * L.cell.n_bands * QC, QT, sizeof(QSmem), stream, L,
+              (const unsigned char*)L.images, (float2*)psi, (float2*)P, (float2*)Pa, fresh_p, want_pa, same_next);
   return true;
 }
 

@@ -29,6 +29,7 @@
 
 #include "tsbz_fft.cuh"
 #include "tsbz_internal.h"
+#include "tsbz_launch.cuh"
 
 namespace {
 
@@ -358,6 +359,7 @@ template <int N>
 __global__ void __launch_bounds__(N* N, 1) k_step64(LaunchSet L, double2* __restrict__ psi, double2* __restrict__ P,
                                                     double2* __restrict__ Pa, int fresh_p, int want_pa,
                                                     int same_next) {
+  step_enter();
   extern __shared__ __align__(16) unsigned char s64_raw[];
   S64Smem<N>& sm = *reinterpret_cast<S64Smem<N>*>(s64_raw);
   constexpr int NN = N * N;
@@ -514,8 +516,8 @@ bool launch_step64(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p
                    void* stream) {
   if (L.n_units == 0 || !step64_taken(L)) return false;
   s64_attr(k_step64<16>, sizeof(S64Smem<16>));
-  k_step64<16><<<(unsigned)L.n_units * L.cell.n_bands, 256, sizeof(S64Smem<16>), (cudaStream_t)stream>>>(
-      L, (double2*)psi, (double2*)P, (double2*)Pa, fresh_p, want_pa, same_next);
+  step_launch(k_step64<16>, (unsigned)L.n_units * L.cell.n_bands, 256, sizeof(S64Smem<16>), stream, L, (double2*)psi,
+              (double2*)P, (double2*)Pa, fresh_p, want_pa, same_next);
   return true;
 }
 
