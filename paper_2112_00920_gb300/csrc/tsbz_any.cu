@@ -221,16 +221,30 @@ __device__ void any_setup(const AnySmem<T>& sm, const CellDev& c, const double* 
   }
 }
 
+// Lanes that share one sum when `items` sums are formed by the CTA's threads (1 .. 8).
+__device__ __forceinline__ int any_share(int items) { return items * 8 <= ANY_T ? 8 : items * 4 <= ANY_T ? 4 : items * 2 <= ANY_T ? 2 : 1; }
+
+// Sum over `n` consecutive lanes (a power of two), the same in all of them.
+template <typename V> __device__ __forceinline__ V any_lane_sum(V v, int n) {
+  for (int off = 1; off < n; off <<= 1) {
+    v.x = radd(v.x, __shfl_xor_sync(0xffffffffu, v.x, off));
+    v.y = radd(v.y, __shfl_xor_sync(0xffffffffu, v.y, off));
+  }
+  return v;
+}
+
 // Monomial sums of order <= D of every atom into mres[a NM + mono] (see tsbz_step64.cu),
-// from the band in t; u is scratch of npts.  Begins and ends with a barrier.
-template <typename T, int D>
+// from the band in t; u is scratch of npts.  Begins and ends with a barrier.  Few sums
+// are shared by lanes (by the count of the second-order pass, so that both orders
+// share alike).
+template <typename T, int D, bool F8>
 __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* t,
                             typename AnyC<T>::V* u) {
   using V = typename AnyC<T>::V;
   constexpr int NM = D == 1 ? 4 : 10;
   const int tid = threadIdx.x, n1 = c.n1, n2 = c.n2, n3 = c.n3, n12 = n1 * n2, ng = c.n_zg;
   __syncthreads();
-  for (int p = tid; p < c.npts; p += ANY_T) u[p] = vmul(sm.phi[p / n12], t[p]);
+  for (int p = tid; p < c.npts; p += ANY_T) u[p] = vmul(sm.phi[F8 ? p >> 6 : sm.idx[p] >> 20], t[p]);
   __syncthreads();
   // z sums of (group, column)
   for (int i = tid; i < ng * n12; i += ANY_T) {
@@ -258,42 +272,57 @@ __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typena
   }
   __syncthreads();
   // x sums of (atom, power of d_z, row)
-  for (int i = tid; i < c.n_atoms * (D + 1) * n2; i += ANY_T) {
-    const int y = i % n2, r = i / n2, k = r / c.n_atoms, a = r - k * c.n_atoms;
-    const V* row = sm.s + (c.zg_of[a] * (D + 1) + k) * n12 + y * n1;
-    V R[3];
+  {
+    const int share = any_share(c.n_atoms * 3 * n2), sub = tid & (share - 1), items = c.n_atoms * (D + 1) * n2;
+    for (int i0 = 0; i0 < items; i0 += ANY_T / share) {
+      const int i = i0 + tid / share;
+      const bool in = i < items;
+      const int y = in ? i % n2 : 0, r = in ? i / n2 : 0, k = r / c.n_atoms, a = r - k * c.n_atoms;
+      const V* row = sm.s + (c.zg_of[a] * (D + 1) + k) * n12 + y * n1;
+      V R[3];
 #pragma unroll
-    for (int w = 0; w < 3; ++w) R[w] = vmk<V>((T)0, (T)0);
-    for (int x = 0; x < n1; ++x) {
-      const V p = vmul(sm.xf[a * n1 + x], row[x]);
-      const T d = sm.xd[a * n1 + x];
-      R[0] = vmk<V>(radd(R[0].x, p.x), radd(R[0].y, p.y));
-      if (k < D) R[1] = vaxpy(d, p, R[1]);
-      if (D == 2 && k == 0) R[2] = vaxpy(rmul(d, d), p, R[2]);
+      for (int w = 0; w < 3; ++w) R[w] = vmk<V>((T)0, (T)0);
+      for (int x = sub; in && x < n1; x += share) {
+        const V p = vmul(sm.xf[a * n1 + x], row[x]);
+        const T d = sm.xd[a * n1 + x];
+        R[0] = vmk<V>(radd(R[0].x, p.x), radd(R[0].y, p.y));
+        if (k < D) R[1] = vaxpy(d, p, R[1]);
+        if (D == 2 && k == 0) R[2] = vaxpy(rmul(d, d), p, R[2]);
+      }
+#pragma unroll
+      for (int w = 0; w <= D; ++w) R[w] = any_lane_sum(R[w], share);
+      if (in && sub == 0) {
+        V* o = sm.rs + (a * 6 + (k == 0 ? 0 : (k == 1 ? 3 : 5))) * n2 + y;
+        o[0] = R[0];
+        if (k < D) o[n2] = R[1];
+        if (D == 2 && k == 0) o[2 * n2] = R[2];
+      }
     }
-    V* o = sm.rs + (a * 6 + (k == 0 ? 0 : (k == 1 ? 3 : 5))) * n2 + y;
-    o[0] = R[0];
-    if (k < D) o[n2] = R[1];
-    if (D == 2 && k == 0) o[2 * n2] = R[2];
   }
   __syncthreads();
   // y sums of (atom, monomial), and the group's phase
-  for (int i = tid; i < c.n_atoms * NM; i += ANY_T) {
-    const int a = i / NM, mo = i - a * NM;
-    int ex = 0, ey = 0, ez = 0;
-    if (mo == 1 || mo == 5 || mo == 6) ex = 1;
-    if (mo == 4) ex = 2;
-    if (mo == 2 || mo == 5 || mo == 8) ey = 1;
-    if (mo == 7) ey = 2;
-    if (mo == 3 || mo == 6 || mo == 8) ez = 1;
-    if (mo == 9) ez = 2;
-    const V* R = sm.rs + (a * 6 + (ez == 0 ? ex : (ez == 1 ? 3 + ex : 5))) * n2;
-    V M = vmk<V>((T)0, (T)0);
-    for (int y = 0; y < n2; ++y) {
-      const T d = sm.yd[a * n2 + y], wy = ey == 0 ? (T)1 : (ey == 1 ? d : rmul(d, d));
-      M = vaxpy(wy, vmul(sm.yf[a * n2 + y], R[y]), M);
+  {
+    const int share = any_share(c.n_atoms * 10), sub = tid & (share - 1), items = c.n_atoms * NM;
+    for (int i0 = 0; i0 < items; i0 += ANY_T / share) {
+      const int i = i0 + tid / share;
+      const bool in = i < items;
+      const int a = in ? i / NM : 0, mo = in ? i - a * NM : 0;
+      int ex = 0, ey = 0, ez = 0;
+      if (mo == 1 || mo == 5 || mo == 6) ex = 1;
+      if (mo == 4) ex = 2;
+      if (mo == 2 || mo == 5 || mo == 8) ey = 1;
+      if (mo == 7) ey = 2;
+      if (mo == 3 || mo == 6 || mo == 8) ez = 1;
+      if (mo == 9) ez = 2;
+      const V* R = sm.rs + (a * 6 + (ez == 0 ? ex : (ez == 1 ? 3 + ex : 5))) * n2;
+      V M = vmk<V>((T)0, (T)0);
+      for (int y = sub; in && y < n2; y += share) {
+        const T d = sm.yd[a * n2 + y], wy = ey == 0 ? (T)1 : (ey == 1 ? d : rmul(d, d));
+        M = vaxpy(wy, vmul(sm.yf[a * n2 + y], R[y]), M);
+      }
+      M = any_lane_sum(M, share);
+      if (in && sub == 0) sm.mres[i] = vmul(sm.kfin[c.zg_of[a]], M);
     }
-    sm.mres[i] = vmul(sm.kfin[c.zg_of[a]], M);
   }
   __syncthreads();
 }
@@ -350,7 +379,7 @@ __device__ void any_kinetic8(const AnySmem<T>& sm, const typename AnyC<T>::V* t,
     if (dst) {
       dst[at + p * stride] = lo;
       dst[at + (p + 4) * stride] = hi;
-      __syncthreads();
+      __syncwarp();   // a plane's x and y lines belong to one warp
     }
   };
   const int cz = l1 * 9 + l0, cx = l1 * 72 + l0 * 9, cy = l1 * 72 + l0;   // column; row y = l0; line x = l0
@@ -369,9 +398,10 @@ __device__ void any_kinetic8(const AnySmem<T>& sm, const typename AnyC<T>::V* t,
     x1[cy + p * 9] = vmk<V>(e0 * lo.x, e0 * lo.y);
     x1[cy + (p + 4) * 9] = vmk<V>(e1 * hi.x, e1 * hi.y);
   }
-  __syncthreads();
+  __syncwarp();
   line(x1, x2, cy, 9, Inv());
   line(x2, x1, cx, 1, Inv());
+  __syncthreads();
   line(x1, (V*)nullptr, cz, 72, Inv());
   k[0] = lo;
   k[1] = hi;
@@ -471,12 +501,12 @@ __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __res
 }
 
 // Pa rows (a, c_x, c_y, c_z) of every projector from the second-order sums of t, and a to Pnext if given.
-template <typename T>
+template <typename T, bool F8>
 __device__ void any_current(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* t,
                             typename AnyC<T>::V* u, typename AnyC<T>::V* __restrict__ Pab,
                             typename AnyC<T>::V* __restrict__ Pnext) {
   using V = typename AnyC<T>::V;
-  any_project<T, 2>(sm, c, t, u);
+  any_project<T, 2, F8>(sm, c, t, u);
   for (int o = threadIdx.x; o < 4 * c.n_proj; o += ANY_T) {
     const int j = o >> 2, s = o & 3, a = j >> 2, ty = j & 3;
     int e[3] = {ty == 1, ty == 2, ty == 3};
@@ -520,7 +550,7 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
   if (c.use_proj) any_tables<T>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
   __syncthreads();
   if (c.use_proj) {
-    if (fresh_p) any_project<T, 1>(sm, c, sm.a, sm.b);
+    if (fresh_p) any_project<T, 1, F8>(sm, c, sm.a, sm.b);
     any_weights<T>(sm, c, fresh_p ? nullptr : Pu);
   }
   V *t = sm.a, *o = sm.b;
@@ -552,7 +582,7 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
     o = s;
     if (m < 4) {
       if (c.use_proj) {
-        any_project<T, 1>(sm, c, t, o);
+        any_project<T, 1, F8>(sm, c, t, o);
         any_weights<T>(sm, c, nullptr);
       } else {
         __syncthreads();
@@ -562,11 +592,11 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
   if (!c.use_proj || !want_pa) return;
   __syncthreads();
   if (!same_next) any_tables<T>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
-  any_current<T>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
+  any_current<T, F8>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
 }
 
 // Projections of the current outside a step.
-template <typename T>
+template <typename T, bool F8>
 __global__ void __launch_bounds__(ANY_T) k_pa_any(LaunchSet L, const typename AnyC<T>::V* __restrict__ src,
                                                   typename AnyC<T>::V* __restrict__ Pa) {
   using V = typename AnyC<T>::V;
@@ -579,8 +609,9 @@ __global__ void __launch_bounds__(ANY_T) k_pa_any(LaunchSet L, const typename An
   const UnitDev U = L.units[u];
   const V* band = src + U.psi_off + (long long)b * c.npts;
   for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = band[p];
+  any_setup<T, F8>(sm, c, L.q_obs + 3 * u);
   any_tables<T>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
-  any_current<T>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
+  any_current<T, F8>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
 }
 
 // The ground-state solver's filter (see k_filter64).
@@ -606,7 +637,7 @@ __global__ void __launch_bounds__(ANY_T) k_filter_any(LaunchSet L, const double2
 #pragma unroll 1
   for (int j = 0; j < degree; ++j) {
     if (c.use_proj) {
-      any_project<double, 1>(sm, c, t, o);
+      any_project<double, 1, F8>(sm, c, t, o);
       any_weights<double>(sm, c, nullptr);
     }
     const double* f = j == 0 ? fa : fb;
@@ -669,8 +700,11 @@ template <typename T> bool launch_pa_any(const LaunchSet& L, const void* src, vo
   using V = typename AnyC<T>::V;
   if (L.n_units == 0 || !any_taken<T>(L) || !L.cell.use_proj) return false;
   const size_t bytes = any_smem<T>(L.cell);
-  any_attr(k_pa_any<T>, bytes);
-  k_pa_any<T><<<(unsigned)L.n_units * L.cell.n_bands, ANY_T, bytes, (cudaStream_t)stream>>>(L, (const V*)src, (V*)Pa);
+  auto go = [&](auto k) {
+    any_attr(k, bytes);
+    k<<<(unsigned)L.n_units * L.cell.n_bands, ANY_T, bytes, (cudaStream_t)stream>>>(L, (const V*)src, (V*)Pa);
+  };
+  if (any_fft8(L.cell)) go(k_pa_any<T, true>); else go(k_pa_any<T, false>);
   return true;
 }
 
