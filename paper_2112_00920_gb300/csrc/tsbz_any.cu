@@ -148,42 +148,42 @@ template <bool F8> __device__ __forceinline__ int any_point(int i) {
 }
 
 // Projector factor tables of one q (phase table ph of the unit); read after a barrier.
-template <typename T>
+template <typename T, bool F8>
 __device__ void any_tables(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* ph, const double* q) {
   using V = typename AnyC<T>::V;
-  const int nm = c.nmax;
+  const int n1 = F8 ? 8 : c.n1, n2 = F8 ? 8 : c.n2, n3 = F8 ? 8 : c.n3, nm = F8 ? 8 : c.nmax;
   const T *g1 = AnyTab<T>::g1(c), *d1 = AnyTab<T>::d1(c);
-  for (int i = threadIdx.x; i < c.n_atoms * c.n1; i += ANY_T) {
-    const int a = i / c.n1, k = a * 3 * nm + i - a * c.n1;
+  for (int i = threadIdx.x; i < c.n_atoms * n1; i += ANY_T) {
+    const int a = i / n1, k = a * 3 * nm + i - a * n1;
     sm.xf[i] = vmk<V>(g1[k] * ph[k].x, g1[k] * ph[k].y);
     sm.xd[i] = d1[k];
   }
-  for (int i = threadIdx.x; i < c.n_atoms * c.n2; i += ANY_T) {
-    const int a = i / c.n2, k = (a * 3 + 1) * nm + i - a * c.n2;
+  for (int i = threadIdx.x; i < c.n_atoms * n2; i += ANY_T) {
+    const int a = i / n2, k = (a * 3 + 1) * nm + i - a * n2;
     sm.yf[i] = vmk<V>(g1[k] * ph[k].x, g1[k] * ph[k].y);
     sm.yd[i] = d1[k];
   }
-  for (int i = threadIdx.x; i < c.n_zg * c.n3; i += ANY_T) {
-    const int g = i / c.n3, k = (c.zg_rep[g] * 3 + 2) * nm + i - g * c.n3;
+  for (int i = threadIdx.x; i < c.n_zg * n3; i += ANY_T) {
+    const int g = i / n3, k = (c.zg_rep[g] * 3 + 2) * nm + i - g * n3;
     sm.zw[i] = g1[k];
-    sm.zw[c.n_zg * c.n3 + i] = g1[k] * d1[k];
-    sm.zw[2 * c.n_zg * c.n3 + i] = g1[k] * d1[k] * d1[k];
+    sm.zw[c.n_zg * n3 + i] = g1[k] * d1[k];
+    sm.zw[2 * c.n_zg * n3 + i] = g1[k] * d1[k] * d1[k];
   }
   // phases along z: of the planes, and of each group before and after its jump
-  for (int i = threadIdx.x; i < c.n3 + 2 * c.n_zg; i += ANY_T) {
-    const int g = (i - c.n3) >> 1, after = (i - c.n3) & 1;
-    const double z = i < c.n3 ? c.hz * i : c.zg_k0[g] - (after ? c.hz * c.n3 : 0.0);
+  for (int i = threadIdx.x; i < n3 + 2 * c.n_zg; i += ANY_T) {
+    const int g = (i - n3) >> 1, after = (i - n3) & 1;
+    const double z = i < n3 ? c.hz * i : c.zg_k0[g] - (after ? c.hz * n3 : 0.0);
     double sn, co;
     sincos(q[2] * z, &sn, &co);
     const V e = vmk<V>((T)co, (T)sn);
-    if (i < c.n3) {
+    if (i < n3) {
       sm.phi[i] = e;
     } else {
       if (!after) sm.k0[g] = e;
-      if (after == (c.zg_brk[g] < c.n3 ? 1 : 0)) sm.kfin[g] = e;
+      if (after == (c.zg_brk[g] < n3 ? 1 : 0)) sm.kfin[g] = e;
       if (after) {
         double s2, c2;
-        sincos(q[2] * (c.hz * c.n3), &s2, &c2);
+        sincos(q[2] * (c.hz * n3), &s2, &c2);
         sm.turn[g] = vmk<V>((T)c2, (T)s2);   // phase before over phase after
         sm.zb[g] = c.zg_brk[g];
       }
@@ -242,9 +242,10 @@ __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typena
                             typename AnyC<T>::V* u) {
   using V = typename AnyC<T>::V;
   constexpr int NM = D == 1 ? 4 : 10;
-  const int tid = threadIdx.x, n1 = c.n1, n2 = c.n2, n3 = c.n3, n12 = n1 * n2, ng = c.n_zg;
+  const int tid = threadIdx.x, n1 = F8 ? 8 : c.n1, n2 = F8 ? 8 : c.n2, n3 = F8 ? 8 : c.n3, n12 = n1 * n2, ng = c.n_zg;
+  const int npts = n12 * n3;
   __syncthreads();
-  for (int p = tid; p < c.npts; p += ANY_T) u[p] = vmul(sm.phi[F8 ? p >> 6 : sm.idx[p] >> 20], t[p]);
+  for (int p = tid; p < npts; p += ANY_T) u[p] = vmul(sm.phi[F8 ? p >> 6 : sm.idx[p] >> 20], t[p]);
   __syncthreads();
   // z sums of (group, column)
   for (int i = tid; i < ng * n12; i += ANY_T) {
@@ -438,7 +439,8 @@ template <typename T, bool F8, typename U>
 __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __restrict__ veff,
                           const typename AnyC<T>::V* t, U&& use) {
   using V = typename AnyC<T>::V;
-  const int tid = threadIdx.x, n1 = c.n1, n2 = c.n2, n3 = c.n3, n12 = n1 * n2, ng = c.use_proj ? c.n_zg : 0;
+  const int tid = threadIdx.x, n1 = F8 ? 8 : c.n1, n2 = F8 ? 8 : c.n2, n3 = F8 ? 8 : c.n3, n12 = n1 * n2;
+  const int ng = c.use_proj ? c.n_zg : 0;
   V k8[2];
   if constexpr (F8) any_kinetic8<T>(sm, t, k8);
   if (ng) {
@@ -469,6 +471,7 @@ __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __res
     __syncthreads();
   }
   const int pts = F8 ? 2 : (c.npts + ANY_T - 1) / ANY_T;
+#pragma unroll(F8 ? 2 : 1)
   for (int i = 0; i < pts; ++i) {
     const int p = any_point<F8>(i);
     if (!F8 && p >= c.npts) break;
@@ -547,7 +550,7 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
   V* Pu = P + U.p_off + (long long)b * c.n_proj;
   for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = sm.acc[p] = band[p];
   any_setup<T, F8>(sm, c, L.q_half + 3 * u);
-  if (c.use_proj) any_tables<T>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
+  if (c.use_proj) any_tables<T, F8>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
   __syncthreads();
   if (c.use_proj) {
     if (fresh_p) any_project<T, 1, F8>(sm, c, sm.a, sm.b);
@@ -591,7 +594,7 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
   }
   if (!c.use_proj || !want_pa) return;
   __syncthreads();
-  if (!same_next) any_tables<T>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
+  if (!same_next) any_tables<T, F8>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
   any_current<T, F8>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
 }
 
@@ -610,7 +613,7 @@ __global__ void __launch_bounds__(ANY_T) k_pa_any(LaunchSet L, const typename An
   const V* band = src + U.psi_off + (long long)b * c.npts;
   for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = band[p];
   any_setup<T, F8>(sm, c, L.q_obs + 3 * u);
-  any_tables<T>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
+  any_tables<T, F8>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
   any_current<T, F8>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
 }
 
@@ -631,7 +634,7 @@ __global__ void __launch_bounds__(ANY_T) k_filter_any(LaunchSet L, const double2
   for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = in[off + p];
   any_setup<double, F8>(sm, c, L.q_half + 3 * u);
   if (c.use_proj)
-    any_tables<double>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
+    any_tables<double, F8>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
   __syncthreads();
   double2 *t = sm.a, *o = sm.b;
 #pragma unroll 1

@@ -729,7 +729,9 @@ __global__ void __launch_bounds__(256, 4) k_stage_z(LaunchSet L, const typename 
 // so each point loads its forward neighbours only (the tile partials differ
 // from the gradient form's, their total does not).
 // ----------------------------------------------------------------------------
-template <typename T>
+// ND: the stencil half-width known at compile time (0: c.nd), so that all neighbours of
+// a point are loaded before the first is used.
+template <typename T, int ND>
 __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename Cplx<T>::type* __restrict__ psi,
                                                      double* __restrict__ rho_part, double* __restrict__ jk_part,
                                                      double* __restrict__ nrm_part) {
@@ -767,7 +769,8 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
       const V zero = cmk<V>((T)0, (T)0);
       V vx = zero, vy = zero, vz = zero;
       const int rowb = iz * n12 + iy * c.n1;
-      for (int mm = 1; mm <= c.nd; ++mm) {
+#pragma unroll
+      for (int mm = 1; mm <= (ND ? ND : c.nd); ++mm) {
         rfma(vx, gw[0][mm], tb[rowb + wrap_idx(ix + mm, c.n1)]);
         rfma(vy, gw[1][mm], tb[iz * n12 + wrap_idx(iy + mm, c.n2) * c.n1 + ix]);
         rfma(vz, gw[2][mm], tb[wrap_idx(iz + mm, c.n3) * n12 + iy * c.n1 + ix]);
@@ -1321,7 +1324,10 @@ void launch_observe(const LaunchSet& L, const void* psi, double* rho_part, doubl
   using V = typename Cplx<T>::type;
   if (L.n_units == 0) return;
   dim3 grid(L.cell.n_tiles, L.n_units, L.cell.n_bgroups);
-  step_launch(k_observe<T>, grid, TSBZ_PT, 0, stream, L, (const V*)psi, rho_part, jk_part, nrm_part);
+  if (L.cell.nd == 4)
+    step_launch(k_observe<T, 4>, grid, TSBZ_PT, 0, stream, L, (const V*)psi, rho_part, jk_part, nrm_part);
+  else
+    step_launch(k_observe<T, 0>, grid, TSBZ_PT, 0, stream, L, (const V*)psi, rho_part, jk_part, nrm_part);
 }
 
 template <typename T>
