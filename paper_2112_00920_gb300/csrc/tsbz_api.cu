@@ -230,9 +230,11 @@ LaunchSet make_set(tsbz_ctx* ctx, HostCell& hc) {
 
 // Point tiles and band groups of a cell's observation kernel.  With few units the
 // bands are split further, until about the CTAs that the GPU holds at once are
-// there (two per SM of the fused form, three of the slab form, and of the
-// point-parallel form two, each already a warp per quarter of an SM); not more,
-// which would begin a second wave (256 units: 116 us in one, 143 us in two).
+// there (two per SM of the fused form, and of the point-parallel form two, each
+// already a warp per quarter of an SM); not more, which would begin a second wave
+// (256 units: 116 us in one, 143 us in two).  The slab form, whose groups hold at
+// most 32 bands, goes to four waves of three CTAs per SM: 8 units of 128 bands took
+// two waves of 32 bands.
 void plan_observe(const tsbz_ctx* ctx, CellDev& c, long long n_units) {
   const bool single = ctx->precision == TSBZ_FP32;
   int tiles = c.n_tiles, most = TSBZ_BG, least = 1;
@@ -246,8 +248,8 @@ void plan_observe(const tsbz_ctx* ctx, CellDev& c, long long n_units) {
     return;
   } else if (single && observe_slab_tiles(c)) {
     tiles = observe_slab_tiles(c);
-    least = 2;
-    want = 456;
+    least = 4;
+    want = 4 * 456;
   }
   const long long groups = std::max<long long>(1, want / (n_units * tiles));
   const long long bg = (c.n_bands + groups - 1) / groups;

@@ -821,12 +821,13 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
 //    added in part order;
 //  - norms, current: tiles take units; a unit is shared by one warp, or by the
 //    whole CTA when its projections are many (fin_wide) or there are no more
-//    units than tiles.  Each thread adds its own bands, partials and projectors
+//    units than tiles, then by as many CTAs as there are tiles for it.  Each thread
+//    adds its own bands, partials and projectors
 //    of all its units; one reduction per CTA follows, and the CTA that finishes
 //    last adds the tiles' currents, writes J and advances the step.
 // Measured per step: 8 k-points at 16^3 31 -> 13 us (FP32), two subgrids of 512
-// k-points 155 -> 33 us, 64 of 64 k-points 109 -> 71 us; with one warp and 16 tiles
-// for each unit and a shuffle sum per band before.
+// k-points 155 -> 33 us, 64 of 64 k-points 109 -> 71 us, 8 k-points of the 64-atom cell
+// 80 -> 33 us; with one warp or CTA for each unit and a shuffle sum per band before.
 // ----------------------------------------------------------------------------
 #define FIN_THREADS 256
 
@@ -877,8 +878,10 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
                                                     (mode == TSBZ_FIN_J0MINUS || step == 0)));
   const int warp = tid >> 5, lane = tid & 31, n_warps = FIN_THREADS / 32;
   const bool wide = fin_wide(c) || n_k <= ntile;
-  const int u_first = wide ? tile : tile + ntile * warp, u_step = wide ? ntile : ntile * n_warps;
-  const int e_first = wide ? tid : lane, e_step = wide ? FIN_THREADS : 32;
+  const int share = wide ? max(1, ntile / n_k) : 1;   // CTAs of a unit
+  const int u_first = wide ? tile / share : tile + ntile * warp;
+  const int u_step = wide ? ntile / share + (share > 1 ? n_k : 0) : ntile * n_warps;   // (shared units: one each)
+  const int e_first = wide ? (tile % share) * FIN_THREADS + tid : lane, e_step = wide ? share * FIN_THREADS : 32;
   double v[3] = {0.0, 0.0, 0.0};   // this thread's share of sum occ <u|pi|u> / occ
   for (int kl = u_first; kl < n_k; kl += u_step) {
     const int u = S.unit0 + kl;
