@@ -30,10 +30,19 @@
 
 namespace {
 
-constexpr int ANY_T = 256;         // threads
 constexpr int ANY_NA = 8;          // atoms
 constexpr int ANY_MIN_ORB = 8;     // orbitals from which the whole-step form is taken
-constexpr size_t ANY_MAX_SMEM = 200 * 1024;
+constexpr size_t ANY_MAX_SMEM = 200 * 1024, ANY_WIDE_SMEM = 56 * 1024;
+
+// The form of a kernel: 8^3 grids with every size at compile time, or any grid with so many threads.
+struct Form8 {
+  static constexpr bool eight = true;
+  static constexpr int threads = 256;
+};
+template <int N> struct FormAny {
+  static constexpr bool eight = false;
+  static constexpr int threads = N;
+};
 
 __host__ __device__ __forceinline__ bool any_fft8(const CellDev& c) { return c.n1 == 8 && c.n2 == 8 && c.n3 == 8; }
 
@@ -143,34 +152,35 @@ __device__ __forceinline__ int any_mono(int i, int j, int k) {   // 000 100 010 
 }
 
 // Point i of the thread: in 8^3 cells the outputs z = p, p + 4 of column l (l = t / 4, p = t % 4).
-template <bool F8> __device__ __forceinline__ int any_point(int i) {
-  return F8 ? ((int)threadIdx.x & 3) * 64 + ((int)threadIdx.x >> 2) + 256 * i : (int)threadIdx.x + ANY_T * i;
+template <class F> __device__ __forceinline__ int any_point(int i) {
+  return F::eight ? ((int)threadIdx.x & 3) * 64 + ((int)threadIdx.x >> 2) + 256 * i : (int)threadIdx.x + F::threads * i;
 }
 
 // Projector factor tables of one q (phase table ph of the unit); read after a barrier.
-template <typename T, bool F8>
+template <typename T, class F>
 __device__ void any_tables(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* ph, const double* q) {
   using V = typename AnyC<T>::V;
-  const int n1 = F8 ? 8 : c.n1, n2 = F8 ? 8 : c.n2, n3 = F8 ? 8 : c.n3, nm = F8 ? 8 : c.nmax;
+  const int n1 = F::eight ? 8 : c.n1, n2 = F::eight ? 8 : c.n2, n3 = F::eight ? 8 : c.n3;
+  const int nm = F::eight ? 8 : c.nmax;
   const T *g1 = AnyTab<T>::g1(c), *d1 = AnyTab<T>::d1(c);
-  for (int i = threadIdx.x; i < c.n_atoms * n1; i += ANY_T) {
+  for (int i = threadIdx.x; i < c.n_atoms * n1; i += F::threads) {
     const int a = i / n1, k = a * 3 * nm + i - a * n1;
     sm.xf[i] = vmk<V>(g1[k] * ph[k].x, g1[k] * ph[k].y);
     sm.xd[i] = d1[k];
   }
-  for (int i = threadIdx.x; i < c.n_atoms * n2; i += ANY_T) {
+  for (int i = threadIdx.x; i < c.n_atoms * n2; i += F::threads) {
     const int a = i / n2, k = (a * 3 + 1) * nm + i - a * n2;
     sm.yf[i] = vmk<V>(g1[k] * ph[k].x, g1[k] * ph[k].y);
     sm.yd[i] = d1[k];
   }
-  for (int i = threadIdx.x; i < c.n_zg * n3; i += ANY_T) {
+  for (int i = threadIdx.x; i < c.n_zg * n3; i += F::threads) {
     const int g = i / n3, k = (c.zg_rep[g] * 3 + 2) * nm + i - g * n3;
     sm.zw[i] = g1[k];
     sm.zw[c.n_zg * n3 + i] = g1[k] * d1[k];
     sm.zw[2 * c.n_zg * n3 + i] = g1[k] * d1[k] * d1[k];
   }
   // phases along z: of the planes, and of each group before and after its jump
-  for (int i = threadIdx.x; i < n3 + 2 * c.n_zg; i += ANY_T) {
+  for (int i = threadIdx.x; i < n3 + 2 * c.n_zg; i += F::threads) {
     const int g = (i - n3) >> 1, after = (i - n3) & 1;
     const double z = i < n3 ? c.hz * i : c.zg_k0[g] - (after ? c.hz * n3 : 0.0);
     double sn, co;
@@ -192,10 +202,10 @@ __device__ void any_tables(const AnySmem<T>& sm, const CellDev& c, const typenam
 }
 
 // Stencil weights (or the symbol of 8^3 grids) of the step's q, and the points' coordinates.
-template <typename T, bool F8>
+template <typename T, class F>
 __device__ void any_setup(const AnySmem<T>& sm, const CellDev& c, const double* q) {
   const int tid = threadIdx.x;
-  if (F8) {
+  if (F::eight) {
     if (tid < 24) {
       const int ax = tid >> 3, k = tid & 7;
       const T* s = AnyTab<T>::ksym(c) + 2 * ax * 8;
@@ -214,7 +224,7 @@ __device__ void any_setup(const AnySmem<T>& sm, const CellDev& c, const double* 
       for (int ax = 0; ax < 3; ++ax) d -= 0.5 * c.lapw[ax][0];
       sm.st[6 * M] = (T)d;
     }
-    for (int p = tid; p < c.npts; p += ANY_T) {
+    for (int p = tid; p < c.npts; p += F::threads) {
       const int ix = p % c.n1, r = p / c.n1;
       sm.idx[p] = ix | (r % c.n2) << 10 | (r / c.n2) << 20;
     }
@@ -222,7 +232,9 @@ __device__ void any_setup(const AnySmem<T>& sm, const CellDev& c, const double* 
 }
 
 // Lanes that share one sum when `items` sums are formed by the CTA's threads (1 .. 8).
-__device__ __forceinline__ int any_share(int items) { return items * 8 <= ANY_T ? 8 : items * 4 <= ANY_T ? 4 : items * 2 <= ANY_T ? 2 : 1; }
+template <class F> __device__ __forceinline__ int any_share(int items) {
+  return items * 8 <= F::threads ? 8 : items * 4 <= F::threads ? 4 : items * 2 <= F::threads ? 2 : 1;
+}
 
 // Sum over `n` consecutive lanes (a power of two), the same in all of them.
 template <typename V> __device__ __forceinline__ V any_lane_sum(V v, int n) {
@@ -237,18 +249,19 @@ template <typename V> __device__ __forceinline__ V any_lane_sum(V v, int n) {
 // from the band in t; u is scratch of npts.  Begins and ends with a barrier.  Few sums
 // are shared by lanes (by the count of the second-order pass, so that both orders
 // share alike).
-template <typename T, int D, bool F8>
+template <typename T, int D, class F>
 __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* t,
                             typename AnyC<T>::V* u) {
   using V = typename AnyC<T>::V;
   constexpr int NM = D == 1 ? 4 : 10;
-  const int tid = threadIdx.x, n1 = F8 ? 8 : c.n1, n2 = F8 ? 8 : c.n2, n3 = F8 ? 8 : c.n3, n12 = n1 * n2, ng = c.n_zg;
+  const int tid = threadIdx.x;
+  const int n1 = F::eight ? 8 : c.n1, n2 = F::eight ? 8 : c.n2, n3 = F::eight ? 8 : c.n3, n12 = n1 * n2, ng = c.n_zg;
   const int npts = n12 * n3;
   __syncthreads();
-  for (int p = tid; p < npts; p += ANY_T) u[p] = vmul(sm.phi[F8 ? p >> 6 : sm.idx[p] >> 20], t[p]);
+  for (int p = tid; p < npts; p += F::threads) u[p] = vmul(sm.phi[F::eight ? p >> 6 : sm.idx[p] >> 20], t[p]);
   __syncthreads();
   // z sums of (group, column)
-  for (int i = tid; i < ng * n12; i += ANY_T) {
+  for (int i = tid; i < ng * n12; i += F::threads) {
     const int g = i / n12, col = i - g * n12, zb = sm.zb[g];
     const T* w = sm.zw + g * n3;
     V s[D + 1];
@@ -274,8 +287,8 @@ __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typena
   __syncthreads();
   // x sums of (atom, power of d_z, row)
   {
-    const int share = any_share(c.n_atoms * 3 * n2), sub = tid & (share - 1), items = c.n_atoms * (D + 1) * n2;
-    for (int i0 = 0; i0 < items; i0 += ANY_T / share) {
+    const int share = any_share<F>(c.n_atoms * 3 * n2), sub = tid & (share - 1), items = c.n_atoms * (D + 1) * n2;
+    for (int i0 = 0; i0 < items; i0 += F::threads / share) {
       const int i = i0 + tid / share;
       const bool in = i < items;
       const int y = in ? i % n2 : 0, r = in ? i / n2 : 0, k = r / c.n_atoms, a = r - k * c.n_atoms;
@@ -303,8 +316,8 @@ __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typena
   __syncthreads();
   // y sums of (atom, monomial), and the group's phase
   {
-    const int share = any_share(c.n_atoms * 10), sub = tid & (share - 1), items = c.n_atoms * NM;
-    for (int i0 = 0; i0 < items; i0 += ANY_T / share) {
+    const int share = any_share<F>(c.n_atoms * 10), sub = tid & (share - 1), items = c.n_atoms * NM;
+    for (int i0 = 0; i0 < items; i0 += F::threads / share) {
       const int i = i0 + tid / share;
       const bool in = i < items;
       const int a = in ? i / NM : 0, mo = in ? i - a * NM : 0;
@@ -329,10 +342,10 @@ __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typena
 }
 
 // Projection of projector j from its monomial sum, and the ket weights from P (null: from mres).
-template <typename T>
+template <typename T, class F>
 __device__ void any_weights(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* P) {
   using V = typename AnyC<T>::V;
-  for (int j = threadIdx.x; j < c.n_proj; j += ANY_T) {
+  for (int j = threadIdx.x; j < c.n_proj; j += F::threads) {
     const T sc = rmul(AnyTab<T>::dv(c), AnyTab<T>::pnorm(c)[j]), e = AnyTab<T>::wkb(c)[j];
     const V p = P ? P[j] : vmk<V>(rmul(sc, sm.mres[j].x), rmul(sc, sm.mres[j].y));
     sm.w[j] = vmul(vconj(sm.k0[c.zg_of[j >> 2]]), vmk<V>(rmul(e, p.x), rmul(e, p.y)));
@@ -435,54 +448,55 @@ __device__ __forceinline__ typename AnyC<T>::V any_kinetic(const AnySmem<T>& sm,
 
 // h t at the thread's points, handed to `use(point, t, h t)`; the ket weights are in sm.w.
 // t is complete (barrier behind its writes); `use` may write anywhere but t and sm.s.
-template <typename T, bool F8, typename U>
+template <typename T, class F, typename U>
 __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __restrict__ veff,
                           const typename AnyC<T>::V* t, U&& use) {
   using V = typename AnyC<T>::V;
-  const int tid = threadIdx.x, n1 = F8 ? 8 : c.n1, n2 = F8 ? 8 : c.n2, n3 = F8 ? 8 : c.n3, n12 = n1 * n2;
+  const int tid = threadIdx.x;
+  const int n1 = F::eight ? 8 : c.n1, n2 = F::eight ? 8 : c.n2, n3 = F::eight ? 8 : c.n3, n12 = n1 * n2;
   const int ng = c.use_proj ? c.n_zg : 0;
   V k8[2];
-  if constexpr (F8) any_kinetic8<T>(sm, t, k8);
+  if constexpr (F::eight) any_kinetic8<T>(sm, t, k8);
   if (ng) {
     // ket tables of (atom, x), then the coefficients C0, C1 of (group, column)
-    for (int i = tid; i < c.n_atoms * n1; i += ANY_T) {
+    for (int i = tid; i < c.n_atoms * n1; i += F::threads) {
       const int a = i / n1, x = i - a * n1;
-      const V F = vconj(sm.xf[i]);
+      const V cf = vconj(sm.xf[i]);
       const T d = sm.xd[i];
-      sm.gt[(a * 3 + 0) * n1 + x] = vmul(F, vaxpy(d, sm.w[4 * a + 1], sm.w[4 * a]));
-      sm.gt[(a * 3 + 1) * n1 + x] = vmul(F, sm.w[4 * a + 2]);
-      sm.gt[(a * 3 + 2) * n1 + x] = vmul(F, sm.w[4 * a + 3]);
+      sm.gt[(a * 3 + 0) * n1 + x] = vmul(cf, vaxpy(d, sm.w[4 * a + 1], sm.w[4 * a]));
+      sm.gt[(a * 3 + 1) * n1 + x] = vmul(cf, sm.w[4 * a + 2]);
+      sm.gt[(a * 3 + 2) * n1 + x] = vmul(cf, sm.w[4 * a + 3]);
     }
     __syncthreads();
-    for (int i = tid; i < ng * n12; i += ANY_T) {
+    for (int i = tid; i < ng * n12; i += F::threads) {
       const int g = i / n12, col = i - g * n12, y = col / n1, x = col - y * n1;
       V c0 = vmk<V>((T)0, (T)0), c1 = c0;
       for (int e = c.zg_off[g]; e < c.zg_off[g + 1]; ++e) {
         const int a = c.zg_mem[e];
-        const V F = vconj(sm.yf[a * n2 + y]);
+        const V cf = vconj(sm.yf[a * n2 + y]);
         const V b = vaxpy(sm.yd[a * n2 + y], sm.gt[(a * 3 + 1) * n1 + x], sm.gt[(a * 3 + 0) * n1 + x]);
         const V g1 = sm.gt[(a * 3 + 2) * n1 + x];
-        c0 = vmk<V>(fma(F.x, b.x, fma(-F.y, b.y, c0.x)), fma(F.x, b.y, fma(F.y, b.x, c0.y)));
-        c1 = vmk<V>(fma(F.x, g1.x, fma(-F.y, g1.y, c1.x)), fma(F.x, g1.y, fma(F.y, g1.x, c1.y)));
+        c0 = vmk<V>(fma(cf.x, b.x, fma(-cf.y, b.y, c0.x)), fma(cf.x, b.y, fma(cf.y, b.x, c0.y)));
+        c1 = vmk<V>(fma(cf.x, g1.x, fma(-cf.y, g1.y, c1.x)), fma(cf.x, g1.y, fma(cf.y, g1.x, c1.y)));
       }
       sm.s[(2 * g) * n12 + col] = c0;
       sm.s[(2 * g + 1) * n12 + col] = c1;
     }
     __syncthreads();
   }
-  const int pts = F8 ? 2 : (c.npts + ANY_T - 1) / ANY_T;
-#pragma unroll(F8 ? 2 : 1)
+  const int pts = F::eight ? 2 : (c.npts + F::threads - 1) / F::threads;
+#pragma unroll(F::eight ? 2 : 1)
   for (int i = 0; i < pts; ++i) {
-    const int p = any_point<F8>(i);
-    if (!F8 && p >= c.npts) break;
+    const int p = any_point<F>(i);
+    if (!F::eight && p >= c.npts) break;
     const V ce = t[p];
     V h;
-    if constexpr (F8) h = i ? k8[1] : k8[0]; else h = any_kinetic<T>(sm, c, t, p);
+    if constexpr (F::eight) h = i ? k8[1] : k8[0]; else h = any_kinetic<T>(sm, c, t, p);
     const T v = veff[p];
     h.x = fma(v, ce.x, h.x);
     h.y = fma(v, ce.y, h.y);
     if (ng) {
-      const int z = F8 ? p >> 6 : sm.idx[p] >> 20, col = p - z * n12;
+      const int z = F::eight ? p >> 6 : sm.idx[p] >> 20, col = p - z * n12;
       V x0 = vmk<V>((T)0, (T)0), x = x0;
       for (int g = 0; g < ng; ++g) {
         const T w0 = sm.zw[g * n3 + z], w1 = sm.zw[(ng + g) * n3 + z];
@@ -504,13 +518,13 @@ __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __res
 }
 
 // Pa rows (a, c_x, c_y, c_z) of every projector from the second-order sums of t, and a to Pnext if given.
-template <typename T, bool F8>
+template <typename T, class F>
 __device__ void any_current(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* t,
                             typename AnyC<T>::V* u, typename AnyC<T>::V* __restrict__ Pab,
                             typename AnyC<T>::V* __restrict__ Pnext) {
   using V = typename AnyC<T>::V;
-  any_project<T, 2, F8>(sm, c, t, u);
-  for (int o = threadIdx.x; o < 4 * c.n_proj; o += ANY_T) {
+  any_project<T, 2, F>(sm, c, t, u);
+  for (int o = threadIdx.x; o < 4 * c.n_proj; o += F::threads) {
     const int j = o >> 2, s = o & 3, a = j >> 2, ty = j & 3;
     int e[3] = {ty == 1, ty == 2, ty == 3};
     if (s > 0) e[s - 1] += 1;
@@ -530,8 +544,8 @@ __device__ __forceinline__ bool any_open(const LaunchSet& L, int& u, int& b) {
 }
 
 // One time step of every band (arguments as launch_step64).
-template <typename T, bool F8>
-__global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T>::V* __restrict__ psi,
+template <typename T, class F>
+__global__ void __launch_bounds__(F::threads) k_step_any(LaunchSet L, typename AnyC<T>::V* __restrict__ psi,
                                                     typename AnyC<T>::V* __restrict__ P,
                                                     typename AnyC<T>::V* __restrict__ Pa, int fresh_p, int want_pa,
                                                     int same_next) {
@@ -548,13 +562,13 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
   const T* veff = reinterpret_cast<const T*>(S.veff);
   V* band = psi + U.psi_off + (long long)b * c.npts;
   V* Pu = P + U.p_off + (long long)b * c.n_proj;
-  for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = sm.acc[p] = band[p];
-  any_setup<T, F8>(sm, c, L.q_half + 3 * u);
-  if (c.use_proj) any_tables<T, F8>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
+  for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = sm.acc[p] = band[p];
+  any_setup<T, F>(sm, c, L.q_half + 3 * u);
+  if (c.use_proj) any_tables<T, F>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
   __syncthreads();
   if (c.use_proj) {
-    if (fresh_p) any_project<T, 1, F8>(sm, c, sm.a, sm.b);
-    any_weights<T>(sm, c, fresh_p ? nullptr : Pu);
+    if (fresh_p) any_project<T, 1, F>(sm, c, sm.a, sm.b);
+    any_weights<T, F>(sm, c, fresh_p ? nullptr : Pu);
   }
   V *t = sm.a, *o = sm.b;
   const T dt = (T)(S.dt * L.dt_scale);
@@ -563,7 +577,7 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
   for (int m = 1; m <= 4; ++m) {
     coef *= dt / (T)m;
     const T sg = m == 1 || m == 4 ? coef : -coef;   // psi += (-i)^m coef s_m
-    any_apply<T, F8>(sm, c, veff, t, [&](int p, V, V h) {
+    any_apply<T, F>(sm, c, veff, t, [&](int p, V, V h) {
       V a = sm.acc[p];
       if (m & 1) {
         a.x = fma(sg, h.y, a.x);
@@ -585,8 +599,8 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
     o = s;
     if (m < 4) {
       if (c.use_proj) {
-        any_project<T, 1, F8>(sm, c, t, o);
-        any_weights<T>(sm, c, nullptr);
+        any_project<T, 1, F>(sm, c, t, o);
+        any_weights<T, F>(sm, c, nullptr);
       } else {
         __syncthreads();
       }
@@ -594,13 +608,13 @@ __global__ void __launch_bounds__(ANY_T) k_step_any(LaunchSet L, typename AnyC<T
   }
   if (!c.use_proj || !want_pa) return;
   __syncthreads();
-  if (!same_next) any_tables<T, F8>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
-  any_current<T, F8>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
+  if (!same_next) any_tables<T, F>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
+  any_current<T, F>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
 }
 
 // Projections of the current outside a step.
-template <typename T, bool F8>
-__global__ void __launch_bounds__(ANY_T) k_pa_any(LaunchSet L, const typename AnyC<T>::V* __restrict__ src,
+template <typename T, class F>
+__global__ void __launch_bounds__(F::threads) k_pa_any(LaunchSet L, const typename AnyC<T>::V* __restrict__ src,
                                                   typename AnyC<T>::V* __restrict__ Pa) {
   using V = typename AnyC<T>::V;
   extern __shared__ __align__(16) unsigned char any_raw[];
@@ -611,15 +625,15 @@ __global__ void __launch_bounds__(ANY_T) k_pa_any(LaunchSet L, const typename An
   any_carve<T>(c, any_raw, sm);
   const UnitDev U = L.units[u];
   const V* band = src + U.psi_off + (long long)b * c.npts;
-  for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = band[p];
-  any_setup<T, F8>(sm, c, L.q_obs + 3 * u);
-  any_tables<T, F8>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
-  any_current<T, F8>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
+  for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = band[p];
+  any_setup<T, F>(sm, c, L.q_obs + 3 * u);
+  any_tables<T, F>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
+  any_current<T, F>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
 }
 
 // The ground-state solver's filter (see k_filter64).
-template <bool F8>
-__global__ void __launch_bounds__(ANY_T) k_filter_any(LaunchSet L, const double2* in, double2* out,
+template <class F>
+__global__ void __launch_bounds__(F::threads) k_filter_any(LaunchSet L, const double2* in, double2* out,
                                                       const double* __restrict__ fa, const double* __restrict__ fb,
                                                       int degree) {
   extern __shared__ __align__(16) unsigned char any_raw[];
@@ -631,21 +645,21 @@ __global__ void __launch_bounds__(ANY_T) k_filter_any(LaunchSet L, const double2
   const UnitDev U = L.units[u];
   const double* veff = reinterpret_cast<const double*>(L.subs[U.sub].veff);
   const long long off = U.psi_off + (long long)b * c.npts;
-  for (int p = threadIdx.x; p < c.npts; p += ANY_T) sm.a[p] = in[off + p];
-  any_setup<double, F8>(sm, c, L.q_half + 3 * u);
+  for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = in[off + p];
+  any_setup<double, F>(sm, c, L.q_half + 3 * u);
   if (c.use_proj)
-    any_tables<double, F8>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
+    any_tables<double, F>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
   __syncthreads();
   double2 *t = sm.a, *o = sm.b;
 #pragma unroll 1
   for (int j = 0; j < degree; ++j) {
     if (c.use_proj) {
-      any_project<double, 1, F8>(sm, c, t, o);
-      any_weights<double>(sm, c, nullptr);
+      any_project<double, 1, F>(sm, c, t, o);
+      any_weights<double, F>(sm, c, nullptr);
     }
     const double* f = j == 0 ? fa : fb;
     const double f0 = f[3 * u], f1 = f[3 * u + 1], f2 = j == 0 ? 0.0 : f[3 * u + 2];
-    any_apply<double, F8>(sm, c, veff, t, [&](int p, double2 ce, double2 h) {
+    any_apply<double, F>(sm, c, veff, t, [&](int p, double2 ce, double2 h) {
       double2 y = make_double2(fma(f0, h.x, f1 * ce.x), fma(f0, h.y, f1 * ce.y));
       if (j > 0) {
         const double2 v = sm.acc[p];
@@ -660,7 +674,7 @@ __global__ void __launch_bounds__(ANY_T) k_filter_any(LaunchSet L, const double2
     o = s;
     __syncthreads();
   }
-  for (int p = threadIdx.x; p < c.npts; p += ANY_T) out[off + p] = t[p];
+  for (int p = threadIdx.x; p < c.npts; p += F::threads) out[off + p] = t[p];
 }
 
 template <typename T> size_t any_smem(const CellDev& c) {
@@ -682,6 +696,21 @@ template <typename T> bool any_taken(const LaunchSet& L) {
   return L.variant == 0 && (long long)L.n_units * L.cell.n_bands >= ANY_MIN_ORB && any_ok<T>(L.cell);
 }
 
+// The form of a cell's kernels (of the cell alone, so that every kernel of a run sums
+// alike).  In single precision a CTA that fewer than four fit an SM takes 512 threads:
+// the SM then holds 16 warps or more (10 steps of 768 k-points, 12 orbitals each:
+// 18^3 21.1 -> 16.3 ms, 17 x 13 x 15 9.06 -> 8.40, 16 x 16 x 8 5.46 -> 5.35; smaller
+// cells lose, 9 x 11 x 13 3.77 -> 4.12 ms).  In double 256 threads hold the FP64 pipe
+// full already and 512 only wait longer at the barriers (10 x 12 x 14, 81 k-points
+// 22.3 -> 23.1 ms).
+template <typename T, typename G> void any_form(const CellDev& c, size_t bytes, G&& go) {
+  if (any_fft8(c)) return go(Form8());
+  if constexpr (sizeof(T) == sizeof(float)) {
+    if (bytes > ANY_WIDE_SMEM) return go(FormAny<512>());
+  }
+  go(FormAny<256>());
+}
+
 }  // namespace
 
 template <typename T>
@@ -691,11 +720,12 @@ bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh
   if (L.n_units == 0 || !any_taken<T>(L)) return false;
   const size_t bytes = any_smem<T>(L.cell);
   const unsigned grid = (unsigned)L.n_units * L.cell.n_bands;
-  auto go = [&](auto k) {
-    any_attr(k, bytes);
-    step_launch(k, grid, ANY_T, bytes, stream, L, (V*)psi, (V*)P, (V*)Pa, fresh_p, want_pa, same_next);
-  };
-  if (any_fft8(L.cell)) go(k_step_any<T, true>); else go(k_step_any<T, false>);
+  any_form<T>(L.cell, bytes, [&](auto f) {
+    using F = decltype(f);
+    any_attr(k_step_any<T, F>, bytes);
+    step_launch(k_step_any<T, F>, grid, F::threads, bytes, stream, L, (V*)psi, (V*)P, (V*)Pa, fresh_p, want_pa,
+                same_next);
+  });
   return true;
 }
 
@@ -703,11 +733,12 @@ template <typename T> bool launch_pa_any(const LaunchSet& L, const void* src, vo
   using V = typename AnyC<T>::V;
   if (L.n_units == 0 || !any_taken<T>(L) || !L.cell.use_proj) return false;
   const size_t bytes = any_smem<T>(L.cell);
-  auto go = [&](auto k) {
-    any_attr(k, bytes);
-    k<<<(unsigned)L.n_units * L.cell.n_bands, ANY_T, bytes, (cudaStream_t)stream>>>(L, (const V*)src, (V*)Pa);
-  };
-  if (any_fft8(L.cell)) go(k_pa_any<T, true>); else go(k_pa_any<T, false>);
+  any_form<T>(L.cell, bytes, [&](auto f) {
+    using F = decltype(f);
+    any_attr(k_pa_any<T, F>, bytes);
+    k_pa_any<T, F><<<(unsigned)L.n_units * L.cell.n_bands, F::threads, bytes, (cudaStream_t)stream>>>(
+        L, (const V*)src, (V*)Pa);
+  });
   return true;
 }
 
@@ -720,11 +751,11 @@ bool launch_filter_any(const LaunchSet& L, const void* in, void* out, const doub
                        void* stream) {
   if (L.n_units == 0 || !any_ok<double>(L.cell)) return false;
   const size_t bytes = any_smem<double>(L.cell);
-  auto go = [&](auto k) {
-    any_attr(k, bytes);
-    k<<<(unsigned)L.n_units * L.cell.n_bands, ANY_T, bytes, (cudaStream_t)stream>>>(
+  any_form<double>(L.cell, bytes, [&](auto f) {
+    using F = decltype(f);
+    any_attr(k_filter_any<F>, bytes);
+    k_filter_any<F><<<(unsigned)L.n_units * L.cell.n_bands, F::threads, bytes, (cudaStream_t)stream>>>(
         L, (const double2*)in, (double2*)out, fa, fb, degree);
-  };
-  if (any_fft8(L.cell)) go(k_filter_any<true>); else go(k_filter_any<false>);
+  });
   return true;
 }

@@ -72,3 +72,17 @@ def test_step_any_restart_bitwise(case, precision):
     np.testing.assert_array_equal(P1.current(0)[0][3:], P2.current(0)[0][3:])
     P1.close()
     P2.close()
+
+
+@pytest.mark.parametrize("n,bands", [((13, 15, 12), 3), ((18, 18, 16), 2), ((16, 16, 8), 3)])
+def test_step_any_wide_vs_oracle(n, bands):
+    """Single-precision cells of which fewer than four fit an SM (CTAs of 512 threads)."""
+    from oracle import dynamics, kpoints
+    cell = _cell(n, bands)
+    s = random_subsim(cell, (2, 2, 1), (0.25, 0.5, 0.125), 0.04, 3, PULSE, seed=230 + n[0])
+    P, g = gpu_run(cell, [s], precision="fp32")
+    P.close()
+    k = kpoints.kpoints_cartesian(cell.a, s["mp"], s["shift"])
+    o = dynamics.propagate(cell, k, s["psi"], s["dt"], 3, dynamics.field_samples(PULSE, s["dt"], 3),
+                           ops=dynamics.Operators(cell), keep_state=False)
+    compare(g[0], o, FP32_J_TOL, FP32_RHO_TOL, FP32_NORM_TOL)
