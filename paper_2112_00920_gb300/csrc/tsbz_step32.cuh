@@ -518,7 +518,25 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
       fft_line<N, -1>(f);
 #pragma unroll
       for (int z = 0; z < N; ++z) colp[z * FX_PL] = f[z];
-      __syncthreads();
+      if (m > 1) {
+        ok = ok && fx_poll(x);   // z sums of s_{m-1}
+        fx_collect<1>(x, sm.sums);
+      }
+      if (!__syncthreads_and(ok)) {
+        if (m > 1) {
+          fx_bail(x, S.status);
+        } else {
+          fx_close(x);
+        }
+        return;
+      }
+      if (m > 1) {
+        float2 v[3], m2;
+        fx_moments<1>(sm, sm.sums, v, m2);
+        const float* sc = sm.wsc + 4 * warp;
+        fx_ket_tables(sm, make_float2(sc[0] * v[0].x, sc[0] * v[0].y), make_float2(sc[1] * v[1].x, sc[1] * v[1].y),
+                      make_float2(sc[2] * v[2].x, sc[2] * v[2].y), make_float2(sc[3] * v[0].x, sc[3] * v[0].y));
+      }
       // forward along x and y, the symbol, back: within the half-warp's plane
 #pragma unroll
       for (int k = 0; k < N; ++k) f[k] = rowp[k];
@@ -546,28 +564,6 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
       fft_line<N, 1>(f);
 #pragma unroll
       for (int k = 0; k < N; ++k) rowp[k] = f[k];
-      if (m > 1) {
-        ok = ok && fx_poll(x);   // z sums of s_{m-1}
-        fx_collect<1>(x, sm.sums);
-      }
-      if (!__syncthreads_and(ok)) {
-        if (m > 1) {
-          fx_bail(x, S.status);
-        } else {
-          fx_close(x);
-        }
-        return;
-      }
-#pragma unroll
-      for (int z = 0; z < N; ++z) f[z] = colp[z * FX_PL];
-      if (m > 1) {
-        float2 v[3], m2;
-        fx_moments<1>(sm, sm.sums, v, m2);
-        const float* sc = sm.wsc + 4 * warp;
-        fx_ket_tables(sm, make_float2(sc[0] * v[0].x, sc[0] * v[0].y), make_float2(sc[1] * v[1].x, sc[1] * v[1].y),
-                      make_float2(sc[2] * v[2].x, sc[2] * v[2].y), make_float2(sc[3] * v[0].x, sc[3] * v[0].y));
-      }
-      fft_line<N, 1>(f);   // the kinetic term of the column
       __syncthreads();
       {
         // the ket's A row of the column
@@ -616,6 +612,10 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
         }
         um_commit(x.bar);
       }
+      // the kinetic term of the column, under the ket's MMAs
+#pragma unroll
+      for (int z = 0; z < N; ++z) f[z] = colp[z * FX_PL];
+      fft_line<N, 1>(f);
       // s_m = kinetic + v s_{m-1} + V_NL s_{m-1}
       {
         float v[16];
