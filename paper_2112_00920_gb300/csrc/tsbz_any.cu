@@ -21,7 +21,7 @@
 // last one left (same q) or from fresh ones, bit for bit.
 // Measured per step, all four stages with their projections: 8^3, 16 orbitals in
 // double 298 -> 109 us, 512 orbitals in single 65 -> 46 us; 10 x 12 x 14, 324 orbitals
-// in single under a pulse 179 -> 78 us (before: two launches per stage and one for
+// in single under a pulse 179 -> 73 us (before: two launches per stage and one for
 // the current).
 #include <cuda_runtime.h>
 
@@ -158,7 +158,7 @@ template <class F> __device__ __forceinline__ int any_point(int i) {
 
 // Projector factor tables of one q (phase table ph of the unit); read after a barrier.
 template <typename T, class F>
-__device__ void any_tables(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* ph, const double* q) {
+__device__ void any_tables(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* ph) {
   using V = typename AnyC<T>::V;
   const int n1 = F::eight ? 8 : c.n1, n2 = F::eight ? 8 : c.n2, n3 = F::eight ? 8 : c.n3;
   const int nm = F::eight ? 8 : c.nmax;
@@ -179,24 +179,18 @@ __device__ void any_tables(const AnySmem<T>& sm, const CellDev& c, const typenam
     sm.zw[c.n_zg * n3 + i] = g1[k] * d1[k];
     sm.zw[2 * c.n_zg * n3 + i] = g1[k] * d1[k] * d1[k];
   }
-  // phases along z: of the planes, and of each group before and after its jump
-  for (int i = threadIdx.x; i < n3 + 2 * c.n_zg; i += F::threads) {
-    const int g = (i - n3) >> 1, after = (i - n3) & 1;
-    const double z = i < n3 ? c.hz * i : c.zg_k0[g] - (after ? c.hz * n3 : 0.0);
-    double sn, co;
-    sincos(q[2] * z, &sn, &co);
-    const V e = vmk<V>((T)co, (T)sn);
+  // phases along z (formed with the other tables, CellDev::ph_z): of the planes, of
+  // each group before its jump and at its end, and of the jump
+  const V* pz = ph + c.ph_z;
+  for (int i = threadIdx.x; i < n3 + c.n_zg; i += F::threads) {
     if (i < n3) {
-      sm.phi[i] = e;
+      sm.phi[i] = pz[i];
     } else {
-      if (!after) sm.k0[g] = e;
-      if (after == (c.zg_brk[g] < n3 ? 1 : 0)) sm.kfin[g] = e;
-      if (after) {
-        double s2, c2;
-        sincos(q[2] * (c.hz * n3), &s2, &c2);
-        sm.turn[g] = vmk<V>((T)c2, (T)s2);   // phase before over phase after
-        sm.zb[g] = c.zg_brk[g];
-      }
+      const int g = i - n3;
+      sm.k0[g] = pz[n3 + 2 * g];
+      sm.kfin[g] = pz[n3 + 2 * g + 1];
+      sm.turn[g] = pz[n3 + 2 * c.n_zg];   // phase before over phase after
+      sm.zb[g] = c.zg_brk[g];
     }
   }
 }
@@ -564,7 +558,7 @@ __global__ void __launch_bounds__(F::threads) k_step_any(LaunchSet L, typename A
   V* Pu = P + U.p_off + (long long)b * c.n_proj;
   for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = sm.acc[p] = band[p];
   any_setup<T, F>(sm, c, L.q_half + 3 * u);
-  if (c.use_proj) any_tables<T, F>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
+  if (c.use_proj) any_tables<T, F>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride);
   __syncthreads();
   if (c.use_proj) {
     if (fresh_p) any_project<T, 1, F>(sm, c, sm.a, sm.b);
@@ -608,7 +602,7 @@ __global__ void __launch_bounds__(F::threads) k_step_any(LaunchSet L, typename A
   }
   if (!c.use_proj || !want_pa) return;
   __syncthreads();
-  if (!same_next) any_tables<T, F>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
+  if (!same_next) any_tables<T, F>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride);
   any_current<T, F>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
 }
 
@@ -627,7 +621,7 @@ __global__ void __launch_bounds__(F::threads) k_pa_any(LaunchSet L, const typena
   const V* band = src + U.psi_off + (long long)b * c.npts;
   for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = band[p];
   any_setup<T, F>(sm, c, L.q_obs + 3 * u);
-  any_tables<T, F>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride, L.q_obs + 3 * u);
+  any_tables<T, F>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride);
   any_current<T, F>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
 }
 
@@ -648,7 +642,7 @@ __global__ void __launch_bounds__(F::threads) k_filter_any(LaunchSet L, const do
   for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = in[off + p];
   any_setup<double, F>(sm, c, L.q_half + 3 * u);
   if (c.use_proj)
-    any_tables<double, F>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
+    any_tables<double, F>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride);
   __syncthreads();
   double2 *t = sm.a, *o = sm.b;
 #pragma unroll 1
@@ -712,6 +706,10 @@ template <typename T, typename G> void any_form(const CellDev& c, size_t bytes, 
 }
 
 }  // namespace
+
+template <typename T> bool any_cell(const CellDev& c) { return any_ok<T>(c); }
+template bool any_cell<double>(const CellDev&);
+template bool any_cell<float>(const CellDev&);
 
 template <typename T>
 bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,

@@ -269,7 +269,8 @@ int layout(tsbz_ctx* ctx) {
   for (auto& hc : ctx->cells) {
     hc.unit_ids.clear();
     hc.hxc_subs.clear();
-    ph_stride = std::max<long long>(ph_stride, (long long)hc.dev.n_atoms * 3 * hc.dev.nmax);
+    ph_stride = std::max<long long>(ph_stride, (long long)hc.dev.n_atoms * 3 * hc.dev.nmax +
+                                                   (hc.dev.ph_z ? hc.dev.n3 + 2 * hc.dev.n_zg + 1 : 0));
   }
   {
     std::vector<long long> cell_units(ctx->cells.size(), 0);
@@ -1092,6 +1093,15 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
   std::vector<double> wkb(ekb.size(), 0.0);
   if (c.use_proj)
     for (int j = 0; j < c.n_proj; ++j) wkb[j] = hc.pnorm[j] * ekb[j];
+  // the phase tables' factors (k_field) follow d1
+  d1.resize((size_t)d->n_atoms * 3 * c.nmax);
+  for (int i = 0; i < 3 * d->n_atoms; ++i) {
+    const int ax = i % 3;
+    const double f = hc.atoms[i] - std::floor(hc.atoms[i]);
+    d1.push_back(-f * d->n[ax] * (d->a[ax] / d->n[ax]));
+  }
+  for (int ax = 0; ax < 3; ++ax) d1.push_back(d->a[ax] / d->n[ax]);
+  for (int ax = 0; ax < 3; ++ax) d1.push_back(d->a[ax]);
   auto to_f = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
   const std::vector<float> g1f = to_f(g1), d1f = to_f(d1), pnf = to_f(hc.pnorm), wkf = to_f(wkb), ekf = to_f(ekb);
   double *vl, *gg, *dd, *pn, *ek, *wk;
@@ -1267,6 +1277,9 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
     for (int z = 1; z < c.n3 && c.zg_brk[g] == c.n3; ++z)
       if (image(z) != image(0)) c.zg_brk[g] = z;
   }
+  c.ph_z = 0;
+  if (c.n_zg > 0 && (ctx->precision == TSBZ_FP64 ? any_cell<double>(c) : any_cell<float>(c)))
+    c.ph_z = d->n_atoms * 3 * c.nmax;
   {
     std::vector<double> ks(6 * (size_t)c.nmax, 0.0);
     for (int ax = 0; ax < 3; ++ax)

@@ -43,7 +43,9 @@ struct CellDev {
   float2 gradw2[3][TSBZ_MAX_ND + 1]; // (w, w) pairs of gradwf
   double gsq_scale[3];               // (2 pi / a_ax)
   const double* g1;     // [n_atoms][3][nmax] Gaussian factor exp(-d^2/(2 rc^2)), 0 outside the box
-  const double* d1;     // [n_atoms][3][nmax] minimum-image displacement, 0 outside the box
+  const double* d1;     // [n_atoms][3][nmax] minimum-image displacement, 0 outside the box; then, of each atom
+                        // and axis, the displacement of point 0 (atom folded into the cell), the steps h[3]
+                        // and the edges [3]
   const double* pnorm;  // [n_atoms][4]        N_s, N_px, N_py, N_pz
   const double* ekb;    // [n_proj]
   const double* wkb;    // [n_proj]            pnorm_j * E_j
@@ -73,6 +75,10 @@ struct CellDev {
   // z < zg_brk, one cell edge less from there on (zg_brk = n3: no jump)
   int zg_brk[8];
   double zg_k0[8];
+  // phases along z for the small-grid step (its groups), at this offset in a unit's phase
+  // tables: exp(i q z) of the n3 planes, of (zg_k0, that at the group's end) per group,
+  // and of the cell edge; 0: none
+  int ph_z;
   double hz;
   // kinetic symbol per axis: [3][2][nmax], row 0 the eigenvalues of -1/2 lap_FD on
   // exp(2 pi i k j / n), row 1 those of -i grad_FD (times q in h)
@@ -158,7 +164,7 @@ struct LaunchSet {
   const double* kcart;    // [unit][3]
   double* q_half;         // [unit][3]
   double* q_obs;          // [unit][3]
-  void* ph_half;          // [unit][n_atoms*3*nmax] complex T
+  void* ph_half;          // [unit][n_atoms*3*nmax, and CellDev::ph_z] complex T
   void* ph_obs;
   void* ph_next;          // q = k + A(t_{n+1} + dt/2): tables of the next step (null if unused)
   long long ph_stride;    // complex elements per unit
@@ -247,6 +253,8 @@ bool launch_bra_slab(const LaunchSet& L, const void* src, void* out, int with_d,
 bool launch_step64(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
                    void* stream);
 bool launch_pa64(const LaunchSet& L, const void* src, void* Pa, void* stream);
+template <typename T>
+bool any_cell(const CellDev& c);   // its orbitals fit the small-grid step
 template <typename T>
 bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
                      void* stream);

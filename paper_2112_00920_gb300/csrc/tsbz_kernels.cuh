@@ -68,10 +68,28 @@ template <> struct Tab<float> {
 };
 
 // ----------------------------------------------------------------------------
-// field: q vectors and phase tables of every unit (k-point) of one cell
+// field: q vectors and phase tables of every unit (k-point) of one cell: exp(i q d)
+// of every (atom, axis, point) at q_half, q_obs and, where the step's projections
+// need it, the next step's q_half.  Bound by the FP64 pipe: a sine and cosine is some
+// 80 double instructions, 64 clocks each on a quarter of an SM.  On a regular axis
+// d = h j + anchor - w edge (w = -1, 0, 1), so in single precision the phase is the
+// product of two or three double factors, 3 (nmax + 1 + atoms) sines and cosines
+// per q instead of 3 nmax atoms, rounded once (as before) at the end; and an axis
+// along which q does not change is formed once for the three tables.  1024 k-points
+// at 16^3 with 8 atoms under a pulse along z 72 -> 42 us, 8 of the 64-atom cell 24 -> 12.  In double the sines and
+// cosines stay one per entry.
+// Cells whose step is the small-grid kernel get the phases of its planes and groups
+// too (CellDev::ph_z), once per unit instead of in every band's CTA.
 // ----------------------------------------------------------------------------
+#define FIELD_THREADS 256
+
+// factors of one q (at most)
+__host__ __device__ inline int field_factors(const CellDev& c) {
+  return 3 * (c.nmax + 1 + c.n_atoms) + (c.ph_z ? 2 * c.n_zg : 0);
+}
+
 template <typename T>
-__global__ void k_field(LaunchSet L, int mode) {
+__global__ void k_field(LaunchSet L, int mode, int factored) {
   step_enter();
   using V = typename Cplx<T>::type;
   const int u = L.unit_ids[blockIdx.x];
@@ -114,30 +132,114 @@ __global__ void k_field(LaunchSet L, int mode) {
     reinterpret_cast<T*>(L.qt_half)[4 * u + 3] = (T)(0.5 * (qh[0] * qh[0] + qh[1] * qh[1] + qh[2] * qh[2]));
   // constant field: q and every phase table equal those of the previous step
   if (mode == TSBZ_FIELD_STEP_KEEP) return;
-  V* phh = (V*)L.ph_half + (long long)u * L.ph_stride;
-  V* pho = (V*)L.ph_obs + (long long)u * L.ph_stride;
-  const int tab = c.n_atoms * 3 * c.nmax;
-  for (int i = threadIdx.x; i < tab; i += blockDim.x) {
-    const int ax = (i / c.nmax) % 3;
-    const double d = c.d1[i];
-    double s, co;
-    sincos(qh[ax] * d, &s, &co);
-    phh[i] = cmk<V>((T)co, (T)s);
-    sincos(qo[ax] * d, &s, &co);
-    pho[i] = cmk<V>((T)co, (T)s);
-  }
+  V* out[3] = {(V*)L.ph_half + (long long)u * L.ph_stride, (V*)L.ph_obs + (long long)u * L.ph_stride, nullptr};
+  double qn[3] = {0.0, 0.0, 0.0};
   if (L.ph_next != nullptr && mode == TSBZ_FIELD_STEP) {
     // q_half of step n + 1, evaluated exactly as that step's field launch will
     const int step = *S.step;
     const int jh = 2 * step + 3, jo = 2 * step + 4;
-    double qn[3];
     for (int ax = 0; ax < 3; ++ax) qn[ax] = L.kcart[3 * u + ax] + (jo < S.n_field ? S.A[3 * jh + ax] : 0.0);
-    V* phn = (V*)L.ph_next + (long long)u * L.ph_stride;
+    out[2] = (V*)L.ph_next + (long long)u * L.ph_stride;
+  }
+  const int nm = c.nmax, tab = c.n_atoms * 3 * nm;
+  if (sizeof(T) == sizeof(float) && factored) {
+    // factors of (set, axis): steps [nmax], edge, anchors [n_atoms], and along z the groups' [2 n_zg]
+    extern __shared__ double2 field_f[];
+    __shared__ double qs[9];
+    __shared__ int first[10];   // of the factors of (set, axis); none where q is that of set 0
+    const int na = c.n_atoms, ng = c.ph_z ? 2 * c.n_zg : 0, sets = out[2] ? 3 : 2;
+    if (threadIdx.x < 3) {
+      qs[threadIdx.x] = qh[threadIdx.x];
+      qs[3 + threadIdx.x] = qo[threadIdx.x];
+      qs[6 + threadIdx.x] = qn[threadIdx.x];
+    }
+    if (threadIdx.x == 0) {
+      int at = 0;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        const int ax = k % 3;
+        first[k] = at;
+        if (k < 3 || (k < 6 && qo[ax] != qh[ax]) || (k >= 6 && out[2] && qn[ax] != qh[ax]))
+          at += nm + 1 + na + (ax == 2 ? ng : 0);
+      }
+      first[9] = at;
+    }
+    __syncthreads();
+    const double* d0 = c.d1 + tab;   // displacements of point 0 [n_atoms][3], steps [3], edges [3]
+    for (int i = threadIdx.x; i < first[9]; i += blockDim.x) {
+      int k = 0;
+      while (i >= first[k + 1]) ++k;
+      const int ax = k % 3, e = i - first[k], g = e - (nm + 1 + na);
+      double d = d0[3 * na + ax] * e;
+      if (e == nm) d = d0[3 * na + 3 + ax];
+      if (e > nm) d = d0[3 * (e - nm - 1) + ax];   // (past the anchors: replaced)
+      if (g >= 0) d = c.zg_k0[g >> 1] - ((g & 1) && c.zg_brk[g >> 1] < c.n3 ? c.hz * c.n3 : 0.0);
+      double sn, co;
+      sincos(qs[k] * d, &sn, &co);
+      field_f[i] = make_double2(co, sn);
+    }
+    __syncthreads();
     for (int i = threadIdx.x; i < tab; i += blockDim.x) {
-      const int ax = (i / c.nmax) % 3;
+      const int r = i / nm, j = i - r * nm, ax = r / na, a = r - ax * na, o = (3 * a + ax) * nm + j;
+      const float d = c.d1f[o], *f0 = c.d1f + tab;
+      const float w =
+          d == 0.f ? 0.f : rintf((f0[3 * na + ax] * j + f0[3 * a + ax] - d) / f0[3 * na + 3 + ax]);
+      V v0 = cmk<V>((T)1, (T)0);
+      for (int set = 0; set < sets; ++set) {
+        V v = v0;
+        if (d != 0.f && first[3 * set + ax + 1] > first[3 * set + ax]) {
+          const double2* f = field_f + first[3 * set + ax];
+          const double2 x = f[j], b = f[nm + 1 + a];
+          double2 z = make_double2(fma(x.x, b.x, -x.y * b.y), fma(x.x, b.y, x.y * b.x));
+          if (w != 0.f) {   // times exp(-i q w edge)
+            const double2 e = f[nm];
+            const double ey = w > 0.f ? -e.y : e.y;
+            z = make_double2(fma(z.x, e.x, -z.y * ey), fma(z.x, ey, z.y * e.x));
+          }
+          v = cmk<V>((T)z.x, (T)z.y);
+        }
+        if (set == 0) v0 = v;
+        out[set][o] = v;
+      }
+    }
+    if (c.ph_z) {
+      for (int i = threadIdx.x; i < c.n3 + ng + 1; i += blockDim.x) {
+        const int e = i < c.n3 ? i : (i < c.n3 + ng ? nm + 1 + na + i - c.n3 : nm);
+        for (int set = 0; set < 2; ++set) {
+          const int k = first[3 * set + 3] > first[3 * set + 2] ? 3 * set + 2 : 2;
+          const double2 z = field_f[first[k] + e];
+          out[set][c.ph_z + i] = cmk<V>((T)z.x, (T)z.y);
+        }
+      }
+    }
+    return;
+  }
+  for (int i = threadIdx.x; i < tab; i += blockDim.x) {
+    const int ax = (i / nm) % 3;
+    const double d = c.d1[i];
+    double s, co;
+    sincos(qh[ax] * d, &s, &co);
+    out[0][i] = cmk<V>((T)co, (T)s);
+    sincos(qo[ax] * d, &s, &co);
+    out[1][i] = cmk<V>((T)co, (T)s);
+    if (out[2]) {
+      sincos(qn[ax] * d, &s, &co);
+      out[2][i] = cmk<V>((T)co, (T)s);
+    }
+  }
+  if (c.ph_z) {
+    // phases along z of the planes; of each group before its jump and at its end; and of a cell edge
+    const int nz = c.n3 + 2 * c.n_zg + 1;
+    for (int i = threadIdx.x; i < nz; i += blockDim.x) {
+      const int r = i - c.n3, g = r >> 1;
+      double z = c.hz * i;
+      if (r >= 0) z = r == 2 * c.n_zg ? c.hz * c.n3 : c.zg_k0[g] - ((r & 1) && c.zg_brk[g] < c.n3 ? c.hz * c.n3 : 0.0);
       double s, co;
-      sincos(qn[ax] * c.d1[i], &s, &co);
-      phn[i] = cmk<V>((T)co, (T)s);
+      sincos(qh[2] * z, &s, &co);
+      const V v = cmk<V>((T)co, (T)s);
+      out[0][c.ph_z + i] = v;
+      if (qo[2] != qh[2]) sincos(qo[2] * z, &s, &co);
+      out[1][c.ph_z + i] = cmk<V>((T)co, (T)s);
     }
   }
 }
@@ -1276,7 +1378,9 @@ template <typename K> void stage_smem_attr(K* kernel, size_t bytes) {
 
 template <typename T> void launch_field(const LaunchSet& L, int mode, void* stream) {
   if (L.n_units == 0) return;
-  step_launch(k_field<T>, L.n_units, 128, 0, stream, L, mode);
+  const size_t bytes = sizeof(double2) * 3 * field_factors(L.cell);
+  const bool factored = sizeof(T) == sizeof(float) && bytes <= 44 * 1024;
+  step_launch(k_field<T>, L.n_units, FIELD_THREADS, factored ? bytes : 0, stream, L, mode, factored ? 1 : 0);
 }
 
 template <typename T>
