@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "tsbz_fft.cuh"
 #include "tsbz_sep.cuh"
 
 #define FS_N 16
@@ -869,6 +870,10 @@ __global__ void __launch_bounds__(FS_NP, 2) k_pa_fused(LaunchSet L, const float2
 // mbarrier completes when its band has landed, its "empty" mbarrier when all
 // warps are done with it; thread 0 refills a slot once it is empty, so warps
 // never meet at a CTA barrier between bands.
+// Bound by shared memory's bandwidth when every point read its eight forward
+// neighbours (9.25 reads a point, 78% of the wavefronts).  The current's sums run
+// over whole lines, so a thread takes a line along each axis in turn into registers:
+// three reads a point.  65 536 orbitals 590 -> 467 us, 16 384 174 -> 135 us.
 // Per column and plane it accumulates occ sum_b |u|^2 (rho; over bands as an
 // unevaluated float pair s + e updated by the error-free two-sum, which keeps
 // the sum to about 2^-44 relative, i.e. FP64-grade, without FP64 arithmetic),
@@ -894,6 +899,26 @@ struct FoSmem {
 // One arrival of the calling thread on a shared-memory mbarrier.
 __device__ __forceinline__ void fo_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+
+// Local current of one periodic line along an axis, in correlation form:
+// sum_r Re(u* (-i grad) u) = 2 sum_m w_m Im sum_r u*(r) u(r + m), which needs the forward
+// neighbours only.
+__device__ __forceinline__ float fo_line(const float2 (&u)[FS_N], const float (&w)[TSBZ_MAX_ND + 1]) {
+  constexpr int N = FS_N, ND = ZM_ND;
+  float2 cc[ND];
+#pragma unroll
+  for (int m = 0; m < ND; ++m) cc[m] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    const float2 t = make_float2(-u[r].y, u[r].x);   // Im(conj(u) v) = -u_i v_r + u_r v_i
+#pragma unroll
+    for (int m = 1; m <= ND; ++m) cc[m - 1] = __ffma2_rn(t, u[(r + m) & (N - 1)], cc[m - 1]);
+  }
+  float s = 0.f;
+#pragma unroll
+  for (int m = 1; m <= ND; ++m) s = __fmaf_rn(2.f * w[m], cc[m - 1].x + cc[m - 1].y, s);
+  return s;
 }
 
 __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const float2* __restrict__ psi,
@@ -929,9 +954,9 @@ __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const f
       bk_mbar_expect_tx(bk_smem(&sm.full[k]), FS_NPTS * (uint32_t)sizeof(float2));
       bk_copy_g2s(bk_smem(sm.buf[k]), src + (long long)k * FS_NPTS, FS_NPTS * sizeof(float2), bk_smem(&sm.full[k]));
     }
-  float rho[N], rho_e[N];
+  float2 rho[N / 2], rho_e[N / 2];   // planes (2 i, 2 i + 1)
 #pragma unroll
-  for (int z = 0; z < N; ++z) rho[z] = rho_e[z] = 0.f;
+  for (int z = 0; z < N / 2; ++z) rho[z] = rho_e[z] = make_float2(0.f, 0.f);
   float js[3] = {0.f, 0.f, 0.f}, je[3] = {0.f, 0.f, 0.f};   // current over bands: js + je per axis
   int issued = nb < FO_SLOTS ? nb : FO_SLOTS;   // bands whose copy thread 0 has issued
   for (int b = 0; b < nb; ++b) {
@@ -943,46 +968,29 @@ __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const f
       break;
     }
     const float2* tb = sm.buf[slot];
-    const float2* cz = tb + col;
-    // the current's local part in correlation form: on the periodic grid
-    // sum_r Re(u* (-i grad_ax) u) = 2 sum_m w_m Im sum_r u*(r) u(r + m e_ax),
-    // which needs the forward neighbours only
-    float2 qv[N + ND];
+    float2 ln[N];
+    // along x: row (y, z) = thread, from a point that differs between lanes (no bank conflicts;
+    // the periodic sums do not depend on where a line begins)
 #pragma unroll
-    for (int k = 0; k < ND; ++k) qv[k] = cz[k * NP];
+    for (int x = 0; x < N; ++x) ln[x] = tb[tid * N + ((x + tid) & (N - 1))];
+    const float bx = fo_line(ln, c.gradwf[0]);
+#pragma unroll
+    for (int y = 0; y < N; ++y) ln[y] = tb[iy * NP + y * N + ix];   // line (x, z = iy)
+    const float by = fo_line(ln, c.gradwf[1]);
+#pragma unroll
+    for (int z = 0; z < N; ++z) ln[z] = tb[z * NP + col];
+    const float bz = fo_line(ln, c.gradwf[2]);
     float nbs = 0.f;
-    float cx[ND], cy[ND], czs[ND];
 #pragma unroll
-    for (int mm = 0; mm < ND; ++mm) cx[mm] = cy[mm] = czs[mm] = 0.f;
-#pragma unroll
-    for (int z = 0; z < N; ++z) {
-      qv[z + ND] = cz[((z + ND) & (N - 1)) * NP];
-      const float2 ce = qv[z];
-#pragma unroll
-      for (int mm = 1; mm <= ND; ++mm) {
-        const float2 xu = tb[z * NP + iy * N + ((ix + mm) & (N - 1))];
-        const float2 yu = tb[z * NP + ((iy + mm) & (N - 1)) * N + ix];
-        const float2 zu = qv[z + mm];
-        // Im(conj(u) v) = u_r v_i - u_i v_r
-        cx[mm - 1] = __fmaf_rn(ce.x, xu.y, __fmaf_rn(-ce.y, xu.x, cx[mm - 1]));
-        cy[mm - 1] = __fmaf_rn(ce.x, yu.y, __fmaf_rn(-ce.y, yu.x, cy[mm - 1]));
-        czs[mm - 1] = __fmaf_rn(ce.x, zu.y, __fmaf_rn(-ce.y, zu.x, czs[mm - 1]));
-      }
-      const float n2v = ce.x * ce.x + ce.y * ce.y;
-      {
-        // two-sum: rho + n2v = t + err exactly
-        const float t = rho[z] + n2v, bb = t - rho[z];
-        rho_e[z] += (rho[z] - (t - bb)) + (n2v - bb);
-        rho[z] = t;
-      }
-      nbs += n2v;
-    }
-    float bx = 0.f, by = 0.f, bz = 0.f;
-#pragma unroll
-    for (int mm = 1; mm <= ND; ++mm) {
-      bx = __fmaf_rn(2.f * c.gradwf[0][mm], cx[mm - 1], bx);
-      by = __fmaf_rn(2.f * c.gradwf[1][mm], cy[mm - 1], by);
-      bz = __fmaf_rn(2.f * c.gradwf[2][mm], czs[mm - 1], bz);
+    for (int z = 0; z < N; z += 2) {
+      const float2 n2v = make_float2(ln[z].x * ln[z].x + ln[z].y * ln[z].y,
+                                     ln[z + 1].x * ln[z + 1].x + ln[z + 1].y * ln[z + 1].y);
+      // two-sum: rho + n2v = t + err exactly
+      const float2 t = fft_add(rho[z / 2], n2v), bb = fft_sub(t, rho[z / 2]);
+      rho_e[z / 2] = fft_add(rho_e[z / 2], fft_add(fft_sub(rho[z / 2], fft_sub(t, bb)), fft_sub(n2v, bb)));
+      rho[z / 2] = t;
+      nbs += n2v.x;
+      nbs += n2v.y;
     }
     {
       const float bv[3] = {bx, by, bz};
@@ -1021,8 +1029,10 @@ __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const f
     return;
   }
 #pragma unroll
-  for (int z = 0; z < N; ++z)
-    rho_part[U.rho_off + (long long)grp * FS_NPTS + z * NP + col] = c.occ * ((double)rho[z] + (double)rho_e[z]);
+  for (int z = 0; z < N; ++z) {
+    const float r = z & 1 ? rho[z / 2].y : rho[z / 2].x, e = z & 1 ? rho_e[z / 2].y : rho_e[z / 2].x;
+    rho_part[U.rho_off + (long long)grp * FS_NPTS + z * NP + col] = c.occ * ((double)r + (double)e);
+  }
   double jx = (double)js[0] + (double)je[0], jy = (double)js[1] + (double)je[1], jz = (double)js[2] + (double)je[2];
   for (int off = 16; off > 0; off >>= 1) {
     jx += __shfl_xor_sync(0xffffffffu, jx, off);
