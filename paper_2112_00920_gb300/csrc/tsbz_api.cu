@@ -290,6 +290,9 @@ int layout(tsbz_ctx* ctx) {
     HostCell& hc = ctx->cells[hs.cell];
     const CellDev& c = hc.dev;
     hs.unit0 = (int)units.size();
+    // the bulk copies of the observation and stage kernels start on 16-byte boundaries: an
+    // odd cell before must not shift these orbitals
+    psi_e = (psi_e + 15) / 16 * 16;
     for (int k = 0; k < hs.n_k; ++k) {
       UnitDev U;
       U.psi_off = psi_e;
