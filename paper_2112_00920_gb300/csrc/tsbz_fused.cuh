@@ -21,6 +21,7 @@
 #include <stdint.h>
 
 #include "tsbz_fft.cuh"
+#include "tsbz_line.cuh"
 #include "tsbz_sep.cuh"
 
 #define FS_N 16
@@ -901,26 +902,6 @@ __device__ __forceinline__ void fo_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
 
-// Local current of one periodic line along an axis, in correlation form:
-// sum_r Re(u* (-i grad) u) = 2 sum_m w_m Im sum_r u*(r) u(r + m), which needs the forward
-// neighbours only.
-__device__ __forceinline__ float fo_line(const float2 (&u)[FS_N], const float (&w)[TSBZ_MAX_ND + 1]) {
-  constexpr int N = FS_N, ND = ZM_ND;
-  float2 cc[ND];
-#pragma unroll
-  for (int m = 0; m < ND; ++m) cc[m] = make_float2(0.f, 0.f);
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-    const float2 t = make_float2(-u[r].y, u[r].x);   // Im(conj(u) v) = -u_i v_r + u_r v_i
-#pragma unroll
-    for (int m = 1; m <= ND; ++m) cc[m - 1] = __ffma2_rn(t, u[(r + m) & (N - 1)], cc[m - 1]);
-  }
-  float s = 0.f;
-#pragma unroll
-  for (int m = 1; m <= ND; ++m) s = __fmaf_rn(2.f * w[m], cc[m - 1].x + cc[m - 1].y, s);
-  return s;
-}
-
 __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const float2* __restrict__ psi,
                                                             double* __restrict__ rho_part,
                                                             double* __restrict__ jk_part,
@@ -973,13 +954,13 @@ __global__ void __launch_bounds__(FS_NP, 2) k_observe_fused(LaunchSet L, const f
     // the periodic sums do not depend on where a line begins)
 #pragma unroll
     for (int x = 0; x < N; ++x) ln[x] = tb[tid * N + ((x + tid) & (N - 1))];
-    const float bx = fo_line(ln, c.gradwf[0]);
+    const float bx = line_current(ln, c.gradwf[0]);
 #pragma unroll
     for (int y = 0; y < N; ++y) ln[y] = tb[iy * NP + y * N + ix];   // line (x, z = iy)
-    const float by = fo_line(ln, c.gradwf[1]);
+    const float by = line_current(ln, c.gradwf[1]);
 #pragma unroll
     for (int z = 0; z < N; ++z) ln[z] = tb[z * NP + col];
-    const float bz = fo_line(ln, c.gradwf[2]);
+    const float bz = line_current(ln, c.gradwf[2]);
     float nbs = 0.f;
 #pragma unroll
     for (int z = 0; z < N; z += 2) {
