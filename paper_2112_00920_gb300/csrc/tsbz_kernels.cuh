@@ -912,7 +912,7 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
 }
 
 // ----------------------------------------------------------------------------
-// finalize: n_tiles CTAs per sub-simulation.  rho (Eq. 3), norms, and the current
+// finalize: n_tiles CTAs per sub-simulation for the density and as many for the rest.  rho (Eq. 3), norms, and the current
 // J = -(1/(Omega N_k)) sum_k sum_b occ [ dV Re<u|-i grad u> + q |u|^2
 //                                        + 2 sum_j E_j Im(conj(c_j) a_j) ]   (Eqs. 5-6)
 // summed in a fixed order.  Bound by latency: a chain of FP64 instructions (64
@@ -927,9 +927,9 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
 //    adds its own bands, partials and projectors
 //    of all its units; one reduction per CTA follows, and the CTA that finishes
 //    last adds the tiles' currents, writes J and advances the step.
-// Measured per step: 8 k-points at 16^3 31 -> 13 us (FP32), two subgrids of 512
-// k-points 155 -> 33 us, 64 of 64 k-points 109 -> 71 us, 8 k-points of the 64-atom cell
-// 80 -> 33 us; with one warp or CTA for each unit and a shuffle sum per band before.
+// Measured per step: 8 k-points at 16^3 31 -> 12 us (FP32), two subgrids of 512
+// k-points 155 -> 24 us, 64 of 64 k-points 109 -> 68 us, 8 k-points of the 64-atom cell
+// 80 -> 27 us; with one warp or CTA for each unit and a shuffle sum per band before.
 // ----------------------------------------------------------------------------
 #define FIN_THREADS 256
 
@@ -947,9 +947,9 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
   const SubDev S = subs[s];
   if ((mode == TSBZ_FIN_STEP || mode == TSBZ_FIN_RHO) && !*S.active) return;   // budget spent: nothing of this step
   const CellDev& c = cells[S.cell];
-  const int tile = blockIdx.y, ntile = gridDim.y;
+  const int ntile = gridDim.y / 2, tile = blockIdx.y % ntile;
   const int npts = c.npts, ngrp = c.n_bgroups, n_k = S.n_k;
-  {
+  if ((int)blockIdx.y >= ntile) {
     const int chunk = (npts + ntile - 1) / ntile, r0 = tile * chunk, r1 = min(npts, r0 + chunk);
     // parts of the (unit, group) terms: the units of a sub-simulation are consecutive,
     // ngrp * npts doubles apart, so term i starts at i * npts
@@ -973,6 +973,7 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
       }
       if (part == 0 && r < r1) S.rho[r] = acc * S.inv_nk;
     }
+    return;
   }
   const int step = *S.step;
   const bool write_j = mode != TSBZ_FIN_RHO &&
@@ -1025,7 +1026,6 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
   }
   if (mode == TSBZ_FIN_RHO) return;   // no current, step unchanged
   // one warp per axis: the threads' shares, then, in the CTA that is last, the tiles'
-  __syncthreads();
 #pragma unroll
   for (int ax = 0; ax < 3; ++ax) red[ax][tid] = v[ax];
   __syncthreads();
@@ -1445,7 +1445,7 @@ void launch_finalize_t(const SubDev* subs, int n_subs, const UnitDev* units, con
   if (n_subs == 0) return;
   // n_tiles (16 .. TSBZ_FIN_MAX_TILES) tiles per sub-simulation: density points, and units for the
   // current and the norms
-  step_launch(k_finalize<T>, dim3(n_subs, n_tiles), FIN_THREADS, 0, stream, subs, units, cells_dev, q_obs,
+  step_launch(k_finalize<T>, dim3(n_subs, 2 * n_tiles), FIN_THREADS, 0, stream, subs, units, cells_dev, q_obs,
               (const V*)Pa, rho_part, jk_part, nrm_part, mask, mode);
 }
 
