@@ -23,10 +23,13 @@
 // double 298 -> 109 us, 512 orbitals in single 65 -> 46 us; 10 x 12 x 14, 324 orbitals
 // in single under a pulse 179 -> 73 us (before: two launches per stage and one for
 // the current).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "tsbz_internal.h"
 #include "tsbz_launch.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -35,14 +38,34 @@ constexpr int ANY_MIN_ORB = 8;     // orbitals from which the whole-step form is
 constexpr size_t ANY_MAX_SMEM = 200 * 1024, ANY_WIDE_SMEM = 56 * 1024;
 
 // The form of a kernel: 8^3 grids with every size at compile time, or any grid with so many threads.
+// ctas > 1: a cluster of so many CTAs shares a band (see k_step_any).
 struct Form8 {
   static constexpr bool eight = true;
-  static constexpr int threads = 256;
+  static constexpr int threads = 256, ctas = 1, proj0 = 0;
 };
 template <int N> struct FormAny {
   static constexpr bool eight = false;
-  static constexpr int threads = N;
+  static constexpr int threads = N, ctas = 1, proj0 = 0;
 };
+struct Form8Cluster {
+  static constexpr bool eight = true;
+  static constexpr int threads = 128, ctas = 4, proj0 = 64;   // threads 0 .. 63 transform meanwhile
+};
+template <int C> struct FormCluster {
+  static constexpr bool eight = false;
+  static constexpr int threads = 256, ctas = C, proj0 = 0;
+};
+
+// Rows of the CTA's share: all of them, or those of its rank in the cluster.
+template <class F> __device__ __forceinline__ int any_row0(int rank, int n2) { return rank * n2 / F::ctas; }
+// Barrier of the threads that project, proj0 and up.
+template <class F> __device__ __forceinline__ void any_sync() {
+  if constexpr (F::proj0 == 0)
+    __syncthreads();
+  else
+    asm volatile("bar.sync 1, %0;\n" ::"n"(F::threads - F::proj0) : "memory");
+}
+__device__ __forceinline__ int any_rank() { return (int)cg::this_cluster().block_rank(); }
 
 __host__ __device__ __forceinline__ bool any_fft8(const CellDev& c) { return c.n1 == 8 && c.n2 == 8 && c.n3 == 8; }
 
@@ -81,6 +104,7 @@ template <typename T> struct AnySmem {
   using V = typename AnyC<T>::V;
   V *a, *b, *acc;        // t_{m-1} / t_m (roles alternate), Taylor sum
   V* s;                  // z sums, ket coefficients per (group, column); line transforms (8^3)
+  V *xk, *xl, *part;     // clusters: all k_z planes of an 8^3 band, the CTA's two, the ranks' monomial sums
   V *rs, *gt, *xf, *yf, *phi, *w, *mres, *k0, *kfin, *turn;
   T *xd, *yd, *zw, *lam, *st;
   int *idx, *zb;
@@ -88,7 +112,8 @@ template <typename T> struct AnySmem {
 
 constexpr int ANY_X8 = 8 * 72;   // one 8^3 line buffer with rows of 9
 
-template <typename T> __host__ __device__ inline size_t any_carve(const CellDev& c, unsigned char* base, AnySmem<T>& m) {
+template <typename T>
+__host__ __device__ inline size_t any_carve(const CellDev& c, unsigned char* base, AnySmem<T>& m, int ctas = 1) {
   using V = typename AnyC<T>::V;
   size_t at = 0;
   auto take = [&](size_t bytes) {
@@ -120,6 +145,13 @@ template <typename T> __host__ __device__ inline size_t any_carve(const CellDev&
   m.st = (T*)take(sizeof(T) * (6 * (TSBZ_MAX_ND + 1) + 1));
   m.idx = (int*)take(sizeof(int) * c.npts);
   m.zb = (int*)take(sizeof(int) * ANY_NA);
+  if (ctas > 1) {
+    m.part = (V*)take(sizeof(V) * 10 * ANY_NA * ctas);
+    if (any_fft8(c)) {
+      m.xk = (V*)take(sizeof(V) * ANY_X8);
+      m.xl = (V*)take(sizeof(V) * ANY_X8 / 2);
+    }
+  }
   return at;
 }
 
@@ -227,7 +259,8 @@ __device__ void any_setup(const AnySmem<T>& sm, const CellDev& c, const double* 
 
 // Lanes that share one sum when `items` sums are formed by the CTA's threads (1 .. 8).
 template <class F> __device__ __forceinline__ int any_share(int items) {
-  return items * 8 <= F::threads ? 8 : items * 4 <= F::threads ? 4 : items * 2 <= F::threads ? 2 : 1;
+  constexpr int n = F::threads - F::proj0;
+  return items * 8 <= n ? 8 : items * 4 <= n ? 4 : items * 2 <= n ? 2 : 1;
 }
 
 // Sum over `n` consecutive lanes (a power of two), the same in all of them.
@@ -245,18 +278,27 @@ template <typename V> __device__ __forceinline__ V any_lane_sum(V v, int n) {
 // share alike).
 template <typename T, int D, class F>
 __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* t,
-                            typename AnyC<T>::V* u) {
+                            typename AnyC<T>::V* u, int rank = 0) {
   using V = typename AnyC<T>::V;
   constexpr int NM = D == 1 ? 4 : 10;
-  const int tid = threadIdx.x;
+  constexpr int NT = F::threads - F::proj0;
+  const int tid = (int)threadIdx.x - F::proj0;
   const int n1 = F::eight ? 8 : c.n1, n2 = F::eight ? 8 : c.n2, n3 = F::eight ? 8 : c.n3, n12 = n1 * n2, ng = c.n_zg;
   const int npts = n12 * n3;
-  __syncthreads();
-  for (int p = tid; p < npts; p += F::threads) u[p] = vmul(sm.phi[F::eight ? p >> 6 : sm.idx[p] >> 20], t[p]);
-  __syncthreads();
+  const int y0 = any_row0<F>(rank, n2), rows = any_row0<F>(rank + 1, n2) - y0, cols = rows * n1;
+  any_sync<F>();
+  if constexpr (F::ctas == 1) {
+    for (int p = tid; p < npts; p += NT) u[p] = vmul(sm.phi[F::eight ? p >> 6 : sm.idx[p] >> 20], t[p]);
+  } else {
+    for (int i = tid; i < cols * n3; i += NT) {
+      const int z = i / cols, p = z * n12 + y0 * n1 + i - z * cols;
+      u[p] = vmul(sm.phi[z], t[p]);
+    }
+  }
+  any_sync<F>();
   // z sums of (group, column)
-  for (int i = tid; i < ng * n12; i += F::threads) {
-    const int g = i / n12, col = i - g * n12, zb = sm.zb[g];
+  for (int i = tid; i < ng * cols; i += NT) {
+    const int g = i / cols, col = y0 * n1 + i - g * cols, zb = sm.zb[g];
     const T* w = sm.zw + g * n3;
     V s[D + 1];
 #pragma unroll
@@ -278,14 +320,14 @@ __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typena
 #pragma unroll
     for (int k = 0; k <= D; ++k) sm.s[(g * (D + 1) + k) * n12 + col] = s[k];
   }
-  __syncthreads();
+  any_sync<F>();
   // x sums of (atom, power of d_z, row)
   {
-    const int share = any_share<F>(c.n_atoms * 3 * n2), sub = tid & (share - 1), items = c.n_atoms * (D + 1) * n2;
-    for (int i0 = 0; i0 < items; i0 += F::threads / share) {
+    const int share = any_share<F>(c.n_atoms * 3 * rows), sub = tid & (share - 1), items = c.n_atoms * (D + 1) * rows;
+    for (int i0 = 0; i0 < items; i0 += NT / share) {
       const int i = i0 + tid / share;
       const bool in = i < items;
-      const int y = in ? i % n2 : 0, r = in ? i / n2 : 0, k = r / c.n_atoms, a = r - k * c.n_atoms;
+      const int y = y0 + (in ? i % rows : 0), r = in ? i / rows : 0, k = r / c.n_atoms, a = r - k * c.n_atoms;
       const V* row = sm.s + (c.zg_of[a] * (D + 1) + k) * n12 + y * n1;
       V R[3];
 #pragma unroll
@@ -307,11 +349,11 @@ __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typena
       }
     }
   }
-  __syncthreads();
+  any_sync<F>();
   // y sums of (atom, monomial), and the group's phase
   {
     const int share = any_share<F>(c.n_atoms * 10), sub = tid & (share - 1), items = c.n_atoms * NM;
-    for (int i0 = 0; i0 < items; i0 += F::threads / share) {
+    for (int i0 = 0; i0 < items; i0 += NT / share) {
       const int i = i0 + tid / share;
       const bool in = i < items;
       const int a = in ? i / NM : 0, mo = in ? i - a * NM : 0;
@@ -324,16 +366,39 @@ __device__ void any_project(const AnySmem<T>& sm, const CellDev& c, const typena
       if (mo == 9) ez = 2;
       const V* R = sm.rs + (a * 6 + (ez == 0 ? ex : (ez == 1 ? 3 + ex : 5))) * n2;
       V M = vmk<V>((T)0, (T)0);
-      for (int y = sub; in && y < n2; y += share) {
+      for (int y = y0 + sub; in && y < y0 + rows; y += share) {
         const T d = sm.yd[a * n2 + y], wy = ey == 0 ? (T)1 : (ey == 1 ? d : rmul(d, d));
         M = vaxpy(wy, vmul(sm.yf[a * n2 + y], R[y]), M);
       }
       M = any_lane_sum(M, share);
-      if (in && sub == 0) sm.mres[i] = vmul(sm.kfin[c.zg_of[a]], M);
+      if (!in || sub != 0) continue;
+      if constexpr (F::ctas == 1) {
+        sm.mres[i] = vmul(sm.kfin[c.zg_of[a]], M);
+      } else {
+        for (int r = 0; r < F::ctas; ++r)
+          cg::this_cluster().map_shared_rank(sm.part, r)[rank * 10 * ANY_NA + i] = M;
+      }
     }
+  }
+  if constexpr (F::ctas == 1) any_sync<F>();
+}
+
+// The monomial sums from the ranks' parts, in rank order (behind a barrier of the cluster).
+template <typename T, int D, class F> __device__ void any_total(const AnySmem<T>& sm, const CellDev& c) {
+  using V = typename AnyC<T>::V;
+  constexpr int NM = D == 1 ? 4 : 10;
+  for (int i = threadIdx.x; i < c.n_atoms * NM; i += F::threads) {
+    V M = sm.part[i];
+#pragma unroll
+    for (int r = 1; r < F::ctas; ++r) {
+      const V v = sm.part[r * 10 * ANY_NA + i];
+      M = vmk<V>(radd(M.x, v.x), radd(M.y, v.y));
+    }
+    sm.mres[i] = vmul(sm.kfin[c.zg_of[i / NM]], M);
   }
   __syncthreads();
 }
+
 
 // Projection of projector j from its monomial sum, and the ket weights from P (null: from mres).
 template <typename T, class F>
@@ -348,9 +413,10 @@ __device__ void any_weights(const AnySmem<T>& sm, const CellDev& c, const typena
 }
 
 // The two outputs k = p, p + 4 of an 8-point transform of x (INV: conjugate), p = the thread's part.
-template <bool INV, typename V> __device__ __forceinline__ void any_dft8(const V (&x)[8], V& lo, V& hi) {
+template <bool INV, typename V>
+__device__ __forceinline__ void any_dft8(const V (&x)[8], V& lo, V& hi, unsigned p = threadIdx.x & 3) {
   using T = decltype(V().x);
-  const unsigned p = threadIdx.x & 3, s = p & 1;
+  const unsigned s = p & 1;
   // four-point sums over the even and the odd inputs: (x0 + s x4) + i^p (x2 + s x6)
   V h[2];
 #pragma unroll
@@ -415,6 +481,60 @@ __device__ void any_kinetic8(const AnySmem<T>& sm, const typename AnyC<T>::V* t,
   k[1] = hi;
 }
 
+// The same in a cluster of four: CTA `rank` takes frequencies k_z = rank, rank + 4 through x and
+// y and hands the two planes to every CTA (before the cluster's barrier); behind it, the
+// inverse along z for the CTA's 16 columns.  Called by threads 0 .. 63.
+template <typename T> __device__ void any_planes8(const AnySmem<T>& sm, const typename AnyC<T>::V* t, int rank) {
+  using V = typename AnyC<T>::V;
+  const int tid = threadIdx.x, p = tid & 3, line = (tid >> 2) & 15, j = line >> 3, l = line & 7;
+  V *x1 = sm.xl, *x2 = sm.xl + 2 * 72, v[8], lo, hi;
+  const int cx = j * 72 + l * 9, cy = j * 72 + l;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = t[k * 64 + tid];
+  any_dft8<false>(v, lo, hi, (unsigned)rank);
+  x1[(tid >> 3) * 9 + (tid & 7)] = lo;
+  x1[72 + (tid >> 3) * 9 + (tid & 7)] = hi;
+  asm volatile("bar.sync 2, 64;\n" ::: "memory");
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = x1[cx + k];
+  any_dft8<false>(v, lo, hi);
+  x2[cx + p] = lo;
+  x2[cx + p + 4] = hi;
+  __syncwarp();   // a plane's x and y lines belong to one warp
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = x2[cy + k * 9];
+  any_dft8<false>(v, lo, hi);
+  {
+    const T s = sm.lam[l] + sm.lam[16 + rank + 4 * j], e0 = s + sm.lam[8 + p], e1 = s + sm.lam[12 + p];
+    x1[cy + p * 9] = vmk<V>(e0 * lo.x, e0 * lo.y);
+    x1[cy + (p + 4) * 9] = vmk<V>(e1 * hi.x, e1 * hi.y);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = x1[cy + k * 9];
+  any_dft8<true>(v, lo, hi);
+  x2[cy + p * 9] = lo;
+  x2[cy + (p + 4) * 9] = hi;
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = x2[cx + k];
+  any_dft8<true>(v, lo, hi);
+  for (int r = 0; r < Form8Cluster::ctas; ++r) {
+    V* o = cg::this_cluster().map_shared_rank(sm.xk, r) + (rank + 4 * j) * 72 + l * 9;
+    o[p] = lo;
+    o[p + 4] = hi;
+  }
+}
+template <typename T>
+__device__ void any_columns8(const AnySmem<T>& sm, int rank, typename AnyC<T>::V (&k)[2]) {
+  using V = typename AnyC<T>::V;
+  const int q = (threadIdx.x >> 2) & 15;   // of the CTA's columns: row 2 rank + q / 8, x = q % 8
+  V v[8];
+#pragma unroll
+  for (int z = 0; z < 8; ++z) v[z] = sm.xk[z * 72 + (2 * rank + (q >> 3)) * 9 + (q & 7)];
+  any_dft8<true>(v, k[0], k[1]);
+}
+
 // Kinetic term at point p from the star stencil.
 template <typename T>
 __device__ __forceinline__ typename AnyC<T>::V any_kinetic(const AnySmem<T>& sm, const CellDev& c,
@@ -444,13 +564,15 @@ __device__ __forceinline__ typename AnyC<T>::V any_kinetic(const AnySmem<T>& sm,
 // t is complete (barrier behind its writes); `use` may write anywhere but t and sm.s.
 template <typename T, class F, typename U>
 __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __restrict__ veff,
-                          const typename AnyC<T>::V* t, U&& use) {
+                          const typename AnyC<T>::V* t, U&& use, int rank = 0) {
   using V = typename AnyC<T>::V;
   const int tid = threadIdx.x;
   const int n1 = F::eight ? 8 : c.n1, n2 = F::eight ? 8 : c.n2, n3 = F::eight ? 8 : c.n3, n12 = n1 * n2;
   const int ng = c.use_proj ? c.n_zg : 0;
+  const int y0 = any_row0<F>(rank, n2), cols = (any_row0<F>(rank + 1, n2) - y0) * n1;
   V k8[2];
-  if constexpr (F::eight) any_kinetic8<T>(sm, t, k8);
+  if constexpr (F::eight && F::ctas == 1) any_kinetic8<T>(sm, t, k8);
+  if constexpr (F::eight && F::ctas > 1) any_columns8<T>(sm, rank, k8);
   if (ng) {
     // ket tables of (atom, x), then the coefficients C0, C1 of (group, column)
     for (int i = tid; i < c.n_atoms * n1; i += F::threads) {
@@ -462,8 +584,8 @@ __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __res
       sm.gt[(a * 3 + 2) * n1 + x] = vmul(cf, sm.w[4 * a + 3]);
     }
     __syncthreads();
-    for (int i = tid; i < ng * n12; i += F::threads) {
-      const int g = i / n12, col = i - g * n12, y = col / n1, x = col - y * n1;
+    for (int i = tid; i < ng * cols; i += F::threads) {
+      const int g = i / cols, col = y0 * n1 + i - g * cols, y = col / n1, x = col - y * n1;
       V c0 = vmk<V>((T)0, (T)0), c1 = c0;
       for (int e = c.zg_off[g]; e < c.zg_off[g + 1]; ++e) {
         const int a = c.zg_mem[e];
@@ -478,11 +600,20 @@ __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __res
     }
     __syncthreads();
   }
-  const int pts = F::eight ? 2 : (c.npts + F::threads - 1) / F::threads;
+  const int own = cols * n3, pts = F::eight ? 2 : (own + F::threads - 1) / F::threads;
 #pragma unroll(F::eight ? 2 : 1)
   for (int i = 0; i < pts; ++i) {
-    const int p = any_point<F>(i);
-    if (!F::eight && p >= c.npts) break;
+    int p = any_point<F>(i);
+    if constexpr (F::ctas == 1) {
+      if (!F::eight && p >= own) break;
+    } else if constexpr (F::eight) {
+      if (tid >= 64) break;
+      p = (tid & 3) * 64 + 16 * rank + (tid >> 2) + 256 * i;
+    } else {
+      if (p >= own) break;
+      const int z = p / cols;
+      p = z * n12 + y0 * n1 + p - z * cols;
+    }
     const V ce = t[p];
     V h;
     if constexpr (F::eight) h = i ? k8[1] : k8[0]; else h = any_kinetic<T>(sm, c, t, p);
@@ -515,9 +646,14 @@ __device__ void any_apply(const AnySmem<T>& sm, const CellDev& c, const T* __res
 template <typename T, class F>
 __device__ void any_current(const AnySmem<T>& sm, const CellDev& c, const typename AnyC<T>::V* t,
                             typename AnyC<T>::V* u, typename AnyC<T>::V* __restrict__ Pab,
-                            typename AnyC<T>::V* __restrict__ Pnext) {
+                            typename AnyC<T>::V* __restrict__ Pnext, int rank = 0) {
   using V = typename AnyC<T>::V;
-  any_project<T, 2, F>(sm, c, t, u);
+  if ((int)threadIdx.x >= F::proj0) any_project<T, 2, F>(sm, c, t, u, rank);
+  if constexpr (F::ctas > 1) {
+    cg::this_cluster().sync();
+    if (rank != 0) return;
+    any_total<T, 2, F>(sm, c);
+  }
   for (int o = threadIdx.x; o < 4 * c.n_proj; o += F::threads) {
     const int j = o >> 2, s = o & 3, a = j >> 2, ty = j & 3;
     int e[3] = {ty == 1, ty == 2, ty == 3};
@@ -531,26 +667,33 @@ __device__ void any_current(const AnySmem<T>& sm, const CellDev& c, const typena
 }
 
 // Unit and band of the CTA; false when the unit sits the step out.
-__device__ __forceinline__ bool any_open(const LaunchSet& L, int& u, int& b) {
-  b = blockIdx.x % L.cell.n_bands;
-  u = L.unit_ids[blockIdx.x / L.cell.n_bands];
+__device__ __forceinline__ bool any_open(const LaunchSet& L, int& u, int& b, int ctas = 1) {
+  const int orb = blockIdx.x / ctas;
+  b = orb % L.cell.n_bands;
+  u = L.unit_ids[orb / L.cell.n_bands];
   return unit_active(L, u);
 }
 
 // One time step of every band (arguments as launch_step64).
+//
+// With few orbitals in double one SM's FP64 pipe is the bound (8^3: 24 us a stage), so a
+// cluster of F::ctas CTAs shares a band by rows y.  Each CTA keeps the whole t_{m-1} and
+// forms its own rows of t_m, which it stores to every CTA; the projections' x and z sums
+// run over the CTA's rows and the ranks' sums are added in rank order; the 8^3 transform
+// splits by k_z between its two z passes.  Two barriers of the cluster a stage.
 template <typename T, class F>
-__global__ void __launch_bounds__(F::threads) k_step_any(LaunchSet L, typename AnyC<T>::V* __restrict__ psi,
-                                                    typename AnyC<T>::V* __restrict__ P,
-                                                    typename AnyC<T>::V* __restrict__ Pa, int fresh_p, int want_pa,
-                                                    int same_next) {
+__device__ __forceinline__ void any_step(const LaunchSet& L, typename AnyC<T>::V* __restrict__ psi,
+                                         typename AnyC<T>::V* __restrict__ P, typename AnyC<T>::V* __restrict__ Pa,
+                                         int fresh_p, int want_pa, int same_next) {
   step_enter();
   using V = typename AnyC<T>::V;
   extern __shared__ __align__(16) unsigned char any_raw[];
   const CellDev& c = L.cell;
   int u, b;
-  if (!any_open(L, u, b)) return;
+  if (!any_open(L, u, b, F::ctas)) return;   // the whole cluster
+  const int rank = F::ctas > 1 ? any_rank() : 0;
   AnySmem<T> sm;
-  any_carve<T>(c, any_raw, sm);
+  any_carve<T>(c, any_raw, sm, F::ctas);
   const UnitDev U = L.units[u];
   const SubDev S = L.subs[U.sub];
   const T* veff = reinterpret_cast<const T*>(S.veff);
@@ -559,8 +702,8 @@ __global__ void __launch_bounds__(F::threads) k_step_any(LaunchSet L, typename A
   for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = sm.acc[p] = band[p];
   any_setup<T, F>(sm, c, L.q_half + 3 * u);
   if (c.use_proj) any_tables<T, F>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride);
-  __syncthreads();
-  if (c.use_proj) {
+  if constexpr (F::ctas > 1) cg::this_cluster().sync(); else __syncthreads();
+  if (F::ctas == 1 && c.use_proj) {
     if (fresh_p) any_project<T, 1, F>(sm, c, sm.a, sm.b);
     any_weights<T, F>(sm, c, fresh_p ? nullptr : Pu);
   }
@@ -571,7 +714,17 @@ __global__ void __launch_bounds__(F::threads) k_step_any(LaunchSet L, typename A
   for (int m = 1; m <= 4; ++m) {
     coef *= dt / (T)m;
     const T sg = m == 1 || m == 4 ? coef : -coef;   // psi += (-i)^m coef s_m
-    any_apply<T, F>(sm, c, veff, t, [&](int p, V, V h) {
+    if constexpr (F::ctas > 1) {
+      const bool chain = c.use_proj && (m > 1 || fresh_p);   // projections of t, else from P
+      if constexpr (F::eight) {
+        if (threadIdx.x < F::proj0) any_planes8<T>(sm, t, rank);
+      }
+      if (chain && (int)threadIdx.x >= F::proj0) any_project<T, 1, F>(sm, c, t, o, rank);
+      cg::this_cluster().sync();
+      if (chain) any_total<T, 1, F>(sm, c);
+      if (c.use_proj) any_weights<T, F>(sm, c, chain ? nullptr : Pu);
+    }
+    auto use = [&](int p, V, V h) {
       V a = sm.acc[p];
       if (m & 1) {
         a.x = fma(sg, h.y, a.x);
@@ -582,16 +735,24 @@ __global__ void __launch_bounds__(F::threads) k_step_any(LaunchSet L, typename A
       }
       if (m < 4) {
         sm.acc[p] = a;
-        o[p] = h;
       } else {
-        o[p] = a;
+        h = a;
         band[p] = a;
       }
-    });
+      if constexpr (F::ctas == 1) {
+        o[p] = h;
+      } else {
+#pragma unroll
+        for (int r = 0; r < F::ctas; ++r) cg::this_cluster().map_shared_rank(o, r)[p] = h;
+      }
+    };
+    any_apply<T, F>(sm, c, veff, t, use, rank);
     V* s = t;
     t = o;
     o = s;
-    if (m < 4) {
+    if constexpr (F::ctas > 1) {
+      cg::this_cluster().sync();
+    } else if (m < 4) {
       if (c.use_proj) {
         any_project<T, 1, F>(sm, c, t, o);
         any_weights<T, F>(sm, c, nullptr);
@@ -603,7 +764,21 @@ __global__ void __launch_bounds__(F::threads) k_step_any(LaunchSet L, typename A
   if (!c.use_proj || !want_pa) return;
   __syncthreads();
   if (!same_next) any_tables<T, F>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride);
-  any_current<T, F>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr);
+  if constexpr (F::proj0 > 0) __syncthreads();   // (else the projection begins with it)
+  any_current<T, F>(sm, c, t, o, Pa + U.pa_off + 4LL * b * c.n_proj, same_next ? Pu : nullptr, rank);
+}
+
+template <typename T, class F>
+__global__ void __launch_bounds__(F::threads)
+    k_step_any(LaunchSet L, typename AnyC<T>::V* psi, typename AnyC<T>::V* P, typename AnyC<T>::V* Pa, int fresh_p,
+               int want_pa, int same_next) {
+  any_step<T, F>(L, psi, P, Pa, fresh_p, want_pa, same_next);
+}
+template <typename T, class F>
+__global__ void __cluster_dims__(F::ctas, 1, 1) __launch_bounds__(F::threads)
+    k_step_any_cluster(LaunchSet L, typename AnyC<T>::V* psi, typename AnyC<T>::V* P, typename AnyC<T>::V* Pa,
+                       int fresh_p, int want_pa, int same_next) {
+  any_step<T, F>(L, psi, P, Pa, fresh_p, want_pa, same_next);
 }
 
 // Projections of the current outside a step.
@@ -718,6 +893,26 @@ bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh
   if (L.n_units == 0 || !any_taken<T>(L)) return false;
   const size_t bytes = any_smem<T>(L.cell);
   const unsigned grid = (unsigned)L.n_units * L.cell.n_bands;
+  auto cluster = [&](auto f) {
+    using F = decltype(f);
+    AnySmem<T> m;
+    const size_t more = any_carve<T>(L.cell, nullptr, m, F::ctas);
+    any_attr(k_step_any_cluster<T, F>, more);
+    step_launch(k_step_any_cluster<T, F>, grid * F::ctas, F::threads, more, stream, L, (V*)psi, (V*)P, (V*)Pa, fresh_p,
+                want_pa, same_next);
+  };
+  // Double precision with few orbitals: clusters while their CTAs find an SM each (8^3,
+  // bound by latency more than by the pipe: two an SM).
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (any_fft8(L.cell) ? grid * 4 <= 304 : grid * 4 <= 152) {
+      if (any_fft8(L.cell)) cluster(Form8Cluster()); else cluster(FormCluster<4>());
+      return true;
+    }
+    if (!any_fft8(L.cell) && grid * 2 <= 152) {
+      cluster(FormCluster<2>());
+      return true;
+    }
+  }
   any_form<T>(L.cell, bytes, [&](auto f) {
     using F = decltype(f);
     any_attr(k_step_any<T, F>, bytes);
