@@ -800,17 +800,17 @@ __global__ void __launch_bounds__(F::threads) k_pa_any(LaunchSet L, const typena
   any_current<T, F>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
 }
 
-// The ground-state solver's filter (see k_filter64).
+// The ground-state solver's filter (see k_filter64); clusters as any_step.
 template <class F>
-__global__ void __launch_bounds__(F::threads) k_filter_any(LaunchSet L, const double2* in, double2* out,
-                                                      const double* __restrict__ fa, const double* __restrict__ fb,
-                                                      int degree) {
+__device__ __forceinline__ void any_filter(const LaunchSet& L, const double2* in, double2* out,
+                                           const double* __restrict__ fa, const double* __restrict__ fb, int degree) {
   extern __shared__ __align__(16) unsigned char any_raw[];
   const CellDev& c = L.cell;
   int u, b;
-  if (!any_open(L, u, b)) return;
+  if (!any_open(L, u, b, F::ctas)) return;
+  const int rank = F::ctas > 1 ? any_rank() : 0;
   AnySmem<double> sm;
-  any_carve<double>(c, any_raw, sm);
+  any_carve<double>(c, any_raw, sm, F::ctas);
   const UnitDev U = L.units[u];
   const double* veff = reinterpret_cast<const double*>(L.subs[U.sub].veff);
   const long long off = U.psi_off + (long long)b * c.npts;
@@ -818,17 +818,24 @@ __global__ void __launch_bounds__(F::threads) k_filter_any(LaunchSet L, const do
   any_setup<double, F>(sm, c, L.q_half + 3 * u);
   if (c.use_proj)
     any_tables<double, F>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride);
-  __syncthreads();
+  if constexpr (F::ctas > 1) cg::this_cluster().sync(); else __syncthreads();
   double2 *t = sm.a, *o = sm.b;
 #pragma unroll 1
   for (int j = 0; j < degree; ++j) {
-    if (c.use_proj) {
+    if constexpr (F::ctas > 1) {
+      if constexpr (F::eight) {
+        if (threadIdx.x < F::proj0) any_planes8<double>(sm, t, rank);
+      }
+      if (c.use_proj && (int)threadIdx.x >= F::proj0) any_project<double, 1, F>(sm, c, t, o, rank);
+      cg::this_cluster().sync();
+      if (c.use_proj) any_total<double, 1, F>(sm, c);
+    } else if (c.use_proj) {
       any_project<double, 1, F>(sm, c, t, o);
-      any_weights<double, F>(sm, c, nullptr);
     }
+    if (c.use_proj) any_weights<double, F>(sm, c, nullptr);
     const double* f = j == 0 ? fa : fb;
     const double f0 = f[3 * u], f1 = f[3 * u + 1], f2 = j == 0 ? 0.0 : f[3 * u + 2];
-    any_apply<double, F>(sm, c, veff, t, [&](int p, double2 ce, double2 h) {
+    auto use = [&](int p, double2 ce, double2 h) {
       double2 y = make_double2(fma(f0, h.x, f1 * ce.x), fma(f0, h.y, f1 * ce.y));
       if (j > 0) {
         const double2 v = sm.acc[p];
@@ -836,14 +843,31 @@ __global__ void __launch_bounds__(F::threads) k_filter_any(LaunchSet L, const do
         y.y = fma(f2, v.y, y.y);
       }
       sm.acc[p] = ce;
-      o[p] = y;
-    });
+      if constexpr (F::ctas == 1) {
+        o[p] = y;
+      } else {
+#pragma unroll
+        for (int r = 0; r < F::ctas; ++r) cg::this_cluster().map_shared_rank(o, r)[p] = y;
+      }
+    };
+    any_apply<double, F>(sm, c, veff, t, use, rank);
     double2* s = t;
     t = o;
     o = s;
-    __syncthreads();
+    if constexpr (F::ctas > 1) cg::this_cluster().sync(); else __syncthreads();
   }
-  for (int p = threadIdx.x; p < c.npts; p += F::threads) out[off + p] = t[p];
+  const int p0 = rank * c.npts / F::ctas, p1 = (rank + 1) * c.npts / F::ctas;
+  for (int p = p0 + threadIdx.x; p < p1; p += F::threads) out[off + p] = t[p];
+}
+template <class F>
+__global__ void __launch_bounds__(F::threads) k_filter_any(LaunchSet L, const double2* in, double2* out,
+                                                           const double* fa, const double* fb, int degree) {
+  any_filter<F>(L, in, out, fa, fb, degree);
+}
+template <class F>
+__global__ void __cluster_dims__(F::ctas, 1, 1) __launch_bounds__(F::threads)
+    k_filter_any_cluster(LaunchSet L, const double2* in, double2* out, const double* fa, const double* fb, int degree) {
+  any_filter<F>(L, in, out, fa, fb, degree);
 }
 
 template <typename T> size_t any_smem(const CellDev& c) {
@@ -863,6 +887,27 @@ template <typename T> bool any_ok(const CellDev& c) {
 // whose number per step is part of the launch accounting.
 template <typename T> bool any_taken(const LaunchSet& L) {
   return L.variant == 0 && (long long)L.n_units * L.cell.n_bands >= ANY_MIN_ORB && any_ok<T>(L.cell);
+}
+
+// Double precision with few orbitals takes clusters, while their CTAs find an SM each (8^3:
+// two an SM, it is bound by latency as much as by the pipe).  20 steps, one CTA a band
+// -> cluster: 8^3 with 8 atoms 16 orbitals 3.21 -> 2.29 ms, 64 3.25 -> 2.55 (128 3.31 -> 4.23, so
+// not); 10^3 32 orbitals 6.92 -> 4.28 (four CTAs), 64 6.96 -> 4.89 (two), 96 5.97 -> 6.12 (two, 2 atoms; so
+// not); 12^3 32 orbitals 10.1 -> 4.86.  Eight CTAs gain less than four (32 orbitals at 12^3
+// 8.68 against 4.58 ms with 2 atoms).  Single precision gains nothing (12^3, 32 orbitals 2.86 -> 2.78 ms; 8^3 loses).
+template <typename G> bool any_cluster(const LaunchSet& L, G&& go) {
+  const long long orb = (long long)L.n_units * L.cell.n_bands;
+  if (any_fft8(L.cell)) {
+    if (orb * Form8Cluster::ctas > 304) return false;
+    go(Form8Cluster());
+  } else if (orb * 4 <= 152) {
+    go(FormCluster<4>());
+  } else if (orb * 2 <= 152) {
+    go(FormCluster<2>());
+  } else {
+    return false;
+  }
+  return true;
 }
 
 // The form of a cell's kernels (of the cell alone, so that every kernel of a run sums
@@ -901,17 +946,8 @@ bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh
     step_launch(k_step_any_cluster<T, F>, grid * F::ctas, F::threads, more, stream, L, (V*)psi, (V*)P, (V*)Pa, fresh_p,
                 want_pa, same_next);
   };
-  // Double precision with few orbitals: clusters while their CTAs find an SM each (8^3,
-  // bound by latency more than by the pipe: two an SM).
   if constexpr (sizeof(T) == sizeof(double)) {
-    if (any_fft8(L.cell) ? grid * 4 <= 304 : grid * 4 <= 152) {
-      if (any_fft8(L.cell)) cluster(Form8Cluster()); else cluster(FormCluster<4>());
-      return true;
-    }
-    if (!any_fft8(L.cell) && grid * 2 <= 152) {
-      cluster(FormCluster<2>());
-      return true;
-    }
+    if (any_cluster(L, cluster)) return true;
   }
   any_form<T>(L.cell, bytes, [&](auto f) {
     using F = decltype(f);
@@ -944,6 +980,15 @@ bool launch_filter_any(const LaunchSet& L, const void* in, void* out, const doub
                        void* stream) {
   if (L.n_units == 0 || !any_ok<double>(L.cell)) return false;
   const size_t bytes = any_smem<double>(L.cell);
+  const bool done = any_cluster(L, [&](auto f) {
+    using F = decltype(f);
+    AnySmem<double> m;
+    const size_t more = any_carve<double>(L.cell, nullptr, m, F::ctas);
+    any_attr(k_filter_any_cluster<F>, more);
+    k_filter_any_cluster<F><<<(unsigned)L.n_units * L.cell.n_bands * F::ctas, F::threads, more, (cudaStream_t)stream>>>(
+        L, (const double2*)in, (double2*)out, fa, fb, degree);
+  });
+  if (done) return true;
   any_form<double>(L.cell, bytes, [&](auto f) {
     using F = decltype(f);
     any_attr(k_filter_any<F>, bytes);

@@ -54,3 +54,25 @@ def test_cluster_repeats_bitwise(case):
         P.close()
     for J, psi in out[1:]:
         assert np.array_equal(J, out[0][0]) and np.array_equal(psi, out[0][1])
+
+
+@pytest.mark.parametrize("n", [8, 10])
+def test_ground_state_cluster_equals_single(n):
+    """The solver's filter with a band per cluster (16 orbitals) and with a band per CTA (the
+    same sub-simulation six times): the converged densities agree to the solver's tolerance."""
+    from paper_2112_00920_gb300 import Propagator, shifted_kpoints
+    from oracle.cell import Grid
+    cell = W.cell_a_coarse(n=n)
+    start = W.random_orbitals(1, cell.n_bands, cell.n, Grid(cell).dv, seed=23)
+    rho = []
+    for copies in (1, 6):
+        P = Propagator("fp64")
+        cid = P.add_cell_spec(cell)
+        sids = [P.add_subsim(cid, shifted_kpoints(cell.a, (1, 1, 1), (0.25, 0.5, 0.125)), 0.08, 1) for _ in range(copies)]
+        for sid in sids:
+            P.load_ground_state(sid, start)
+        _, err = P.ground_state(max_iter=120, tol=1e-10)
+        assert err <= 1e-10
+        rho.append(P.density(sids[-1]))
+        P.close()
+    assert np.max(np.abs(rho[0] - rho[1])) <= 1e-8 * np.max(rho[1])
