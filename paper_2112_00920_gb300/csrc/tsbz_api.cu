@@ -615,7 +615,11 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
       // bulk-staged stage 4 those of psi(t_{n+1}) for the next step and of the
       // current (Pa).  The projections of psi are computed here only when P does
       // not hold them already (first step, or after the state or field changed).
-      if (fresh_p || !ctx->p_next_valid || !hc.pa_by_stage) {
+      // A step that must form them in any case (ETRS) does so from the band it has loaded,
+      // where its kernel can: three passes over psi less per ETRS step (4 subgrids of 64
+      // k-points: 1.87 -> 1.64 ms with the copy that the predictor no longer needs).
+      const bool in_step = fresh_p && step_forms_p(L);
+      if (!in_step && (fresh_p || !ctx->p_next_valid || !hc.pa_by_stage)) {
         ev_start(ctx, FAM_BRA);
         launch_bra_sep(L, ctx->psi, ctx->P, 0, 0, ctx->stream);
         ev_stop(ctx);
@@ -624,7 +628,7 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
       const int same_next = (same_next_allowed && cell_field_const(ctx, hc)) ? 1 : 0;
       ev_start(ctx, FAM_STAGE);
       const bool whole = launch_step_fused(L, ctx->psi, ctx->P, ctx->Pa, same_next, want_pa ? 1 : 0,
-                                           ctx->stream);
+                                           in_step ? 1 : 0, ctx->stream);
       ev_stop(ctx);
       if (whole) {
         hc.pa_by_stage = want_pa;
@@ -668,7 +672,7 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
 
 // Enforced-time-reversal-symmetry step: a Taylor-4 predictor gives rho~(t_{n+1})
 // and v~_eff; then psi(t_{n+1}) = T4(dt/2; A(t_{n+1}), v~_eff) T4(dt/2; A(t_n),
-// v_eff(t_n)) psi(t_n).  psi(t_n) and v_eff(t_n) are kept on the device.
+// v_eff(t_n)) psi(t_n).  The predictor runs on a copy of psi(t_n); v_eff(t_n) is kept on the device.
 template <typename T> int run_step_etrs(tsbz_ctx* ctx) {
   int rc;
   if (!ctx->psi_save && (rc = dalloc(ctx, ctx->psi_bytes, &ctx->psi_save))) return rc;
@@ -677,14 +681,17 @@ template <typename T> int run_step_etrs(tsbz_ctx* ctx) {
   launch_veff_keep_t<T>(ctx->d_subs, ctx->d_cells, ns, 0, ctx->stream);
   ++ctx->launches;
   // predictor: the Taylor-4 step, then rho~ and v~_eff (no current, step unchanged)
+  // on the copy, so that psi(t_n) needs not be brought back
   ctx->dt_scale = 1.0;
   run_field<T>(ctx, TSBZ_FIELD_STEP);
-  if ((rc = run_stages<T>(ctx, true, 0, false))) return rc;
-  run_observe<T>(ctx, TSBZ_FIN_RHO);
+  std::swap(ctx->psi, ctx->psi_save);
+  rc = run_stages<T>(ctx, true, 0, false);
+  if (!rc) run_observe<T>(ctx, TSBZ_FIN_RHO);
+  std::swap(ctx->psi, ctx->psi_save);
+  if (rc) return rc;
   run_hxc<T>(ctx);
   launch_veff_keep_t<T>(ctx->d_subs, ctx->d_cells, ns, 1, ctx->stream);   // v_eff(t_n) back, v~_eff kept
   ++ctx->launches;
-  CK(cudaMemcpyAsync(ctx->psi, ctx->psi_save, ctx->psi_bytes, cudaMemcpyDeviceToDevice, ctx->stream));
   // the two half steps
   ctx->dt_scale = 0.5;
   run_field<T>(ctx, TSBZ_FIELD_AT_NOW);

@@ -279,7 +279,9 @@ int sep_variants(const CellDev& c);   // kernel variants of the single-precision
 // The whole time step of every unit in one launch (16^3 cells with z groups,
 // variant 0); false when the cell takes the per-stage kernels.
 // want_pa: the projections of the current (and of the next step) follow from psi.
-bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int same_next, int want_pa, void* stream);
+bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int same_next, int want_pa, int fresh_p,
+                       void* stream);
+bool step_forms_p(const LaunchSet& L);   // launch_step_fused takes fresh_p (else P holds the projections of psi)
 void launch_bra_sep(const LaunchSet& L, const void* src, void* out, int with_d, int use_obs, void* stream);
 // stage 4 on the bulk-staged path also writes P (next step) and Pa; returns whether it did
 // same_next: the field is constant, so at m = 4 the next step's projections come from the current's sums

@@ -165,11 +165,15 @@ bool launch_stage_sep(const LaunchSet& L, const void* tin, void* tout, void* psi
   return false;
 }
 
-bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int same_next, int want_pa, void* stream) {
+bool step_forms_p(const LaunchSet& L) { return stage_kind(L) == 0 && fs_umma(L); }
+
+bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int same_next, int want_pa, int fresh_p,
+                       void* stream) {
   if (L.n_units == 0 || stage_kind(L) != 0) return false;
   static bool attr = false;
   if (!attr) {
-    fs_attr(k_step_fft, sizeof(FxSmem));
+    fs_attr(k_step_fft<false>, sizeof(FxSmem));
+    fs_attr(k_step_fft<true>, sizeof(FxSmem));
     fs_attr(k_step_fused<4>, sizeof(FsSmem));
     attr = true;
   }
@@ -181,8 +185,8 @@ bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int sam
     int per = 1;
     while (per < 8 && (long long)grid / (2 * per) >= 13 * 304) per *= 2;
     const unsigned ctas = (unsigned)L.n_units * (unsigned)((L.cell.n_bands + per - 1) / per);
-    step_launch(k_step_fft, ctas, FX_NP, sizeof(FxSmem), stream, L, (float2*)psi, (float2*)P, (float2*)Pa, same_next,
-                want_pa, per);
+    step_launch(fresh_p ? k_step_fft<true> : k_step_fft<false>, ctas, FX_NP, sizeof(FxSmem), stream, L, (float2*)psi,
+                (float2*)P, (float2*)Pa, same_next, want_pa, per);
   }
   else
     k_step_fused<4><<<grid, FS_NP, sizeof(FsSmem), (cudaStream_t)stream>>>(L, (float2*)psi, (float2*)P, (float2*)Pa,

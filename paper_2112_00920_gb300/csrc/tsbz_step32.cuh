@@ -439,6 +439,8 @@ __device__ __forceinline__ void fx_ket_from_w(FxSmem& sm, float2 w) {
 // tables and operand matrices, v_eff and the symbol serve them all, and the next
 // band is on its way to L2.  The set-up is a chain of dependent loads, about 1.0 ms
 // of the 6.9 ms launch with one band per CTA (65 536 orbitals).
+// FRESH: the projections of psi are formed from the band (else taken from P).
+template <bool FRESH>
 __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __restrict__ psi, float2* __restrict__ P,
                                                        float2* __restrict__ Pa, int same_next, int want_pa, int per) {
   step_enter();
@@ -507,30 +509,38 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
       asm volatile("prefetch.global.L2 [%0];\n" ::"l"(next));
     }
     um_st32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(t));
-    fx_ket_from_w(sm, w);
+    if (FRESH) {
+      fx_stage(t, x);
+      um_fence_before();
+      __syncthreads();
+      if (tid == 0) fx_issue_bra<1>(x, sm.bbra);
+    } else {
+      fx_ket_from_w(sm, w);
+    }
     float coef = 1.f;
     bool ok = true;
 #pragma unroll 1
     for (int m = 1; m <= 4; ++m) {
+      const bool chain = m > 1 || FRESH;
       float2 f[N];
 #pragma unroll
       for (int z = 0; z < N; ++z) f[z] = t[z];
       fft_line<N, -1>(f);
 #pragma unroll
       for (int z = 0; z < N; ++z) colp[z * FX_PL] = f[z];
-      if (m > 1) {
+      if (chain) {
         ok = ok && fx_poll(x);   // z sums of s_{m-1}
         fx_collect<1>(x, sm.sums);
       }
       if (!__syncthreads_and(ok)) {
-        if (m > 1) {
+        if (chain) {
           fx_bail(x, S.status);
         } else {
           fx_close(x);
         }
         return;
       }
-      if (m > 1) {
+      if (chain) {
         float2 v[3], m2;
         fx_moments<1>(sm, sm.sums, v, m2);
         const float* sc = sm.wsc + 4 * warp;
