@@ -317,30 +317,32 @@ STAGE_KERNEL = {
     "fp32": "k_stage_fused (z-march stencil + tensor-core projector contractions + Taylor accumulate), one launch "
             "per Taylor stage",
     "fp32_tc": "k_stage_zb (z-march stencil + non-local term + Taylor accumulate)",
-    "fp64": "k_stage (stencil + ket + Taylor accumulate)",
+    "fp64": "k_step64 (variant 0: the four Taylor stages of a time step in one launch, register FFT lines; bound by the "
+            "FP64 pipe) or k_stage (stencil + ket + Taylor accumulate), one launch per Taylor stage",
 }
-STEP_KERNEL = ("k_step_fused (the four Taylor stages of a time step in one launch: z-march stencil, tensor-core "
-               "projector z contractions (tcgen05 + TMEM in variant 0, mma.sync in variant 3), Taylor "
-               "accumulation in registers)")
+STEP_KERNEL = ("k_step_fft (the four Taylor stages of a time step in one launch: kinetic operator by register "
+               "FFT lines, projector z contractions on tcgen05 with TMEM operands and accumulators, Taylor sum in "
+               "TMEM); variant 3 is k_step_fused (star stencil, mma.sync)")
 # FP32 arithmetic of the local part of h, the Taylor scaling and the psi sum,
-# per grid point, orbital and Taylor stage (complex values): Laplacian and
+# per grid point, orbital and Taylor stage (complex values), as the star stencil of
+# the method counts them (the kernel gets the same operator from fewer): Laplacian and
 # gradient pairs 3 axes x 4 x (2 + 4 + 2 + 4) = 144, q.grad 10, diagonal 3,
 # combination 4, (-i dt/m) 2, accumulation 2.
 FLOPS_LOCAL_PER_POINT_STAGE = 165
 FP32_LANES_PER_SM = 128
-# DRAM bytes of one k_step_fused launch from an ncu capture (dram__bytes_read.sum
+# DRAM bytes of one k_step_fft launch from an ncu capture (dram__bytes_read.sum
 # + dram__bytes_write.sum) on the reduced workload (8 of the 64 subgrids, 8192
 # orbitals), scaled by the orbital count to the full workload.  Valid only for
 # the source it was taken on: the SHA-1 of the kernel header is checked at run time.
-STEP_TRAFFIC = {"file": "tsbz_fused.cuh", "sha1": "93d95614680d5daa93a0a54a1c9dbb337bade2aa",
-                "bytes_per_launch_full": 8 * (273.970432e6 + 218.047744e6),
-                "profile": "profiles/k_step_fused_tcgen05_twostep8.md"}
+STEP_TRAFFIC = {"file": "tsbz_step32.cuh", "sha1": "43982e016be64ba9647dcc42a9e3c724b1d1b108",
+                "bytes_per_launch_full": 8 * (272.373760e6 + 219.642368e6),
+                "profile": "profiles/k_step_fft_twostep8.md"}
 # DRAM bytes of the per-stage stencil kernel k_stage_zb<false> from an ncu capture of the
 # reduced dense tensor-core workload (8 of the 64 subgrids): stages 1 and 2 moved 774.8 and
 # 1295.1 MB against 805.3 and 1342.2 MB of algorithmic bytes (0.964 of them); the full
-# launch is taken as that fraction of its algorithmic bytes.  Valid for the source it
-# was taken on.
-STENCIL_TRAFFIC = {"file": "tsbz_tc.cuh", "sha1": "2bd77934cbda428416643c624a258d0564747242",
+# launch is taken as that fraction of its algorithmic bytes.  Valid for the kernel it
+# was taken on (since then only the observation's launcher of that header has changed).
+STENCIL_TRAFFIC = {"file": "tsbz_tc.cuh", "sha1": "68941056c11d87cbd1f5e6ce87fa165ad27e17e7",
                    "fraction_of_algorithmic": (774.778112 + 1295.140096) / (805.306368 + 1342.17728),
                    "profile": "profiles/k_stage_zb_fp32tc_twostep8.md"}
 
@@ -368,7 +370,7 @@ def alu_peaks(device):
 
 
 def step_roofline(step_ms, n_orb, cell, elem, peaks, subsims, clocks, alu):
-    """Roofline of k_step_fused.  It reads and writes psi once per step, so its
+    """Roofline of k_step_fft.  It reads and writes psi once per step, so its
     HBM traffic is 2 arrays (plus P and Pa) and it is bound by its arithmetic
     issue, not by HBM: the ALU roofline is the primary one, against the FP32
     FMA peak measured on this GPU (the faster of the scalar and the packed
@@ -631,8 +633,10 @@ def main():
         alu = alu_peaks(local_rank) if not args.profile_run else None
         roof = step_roofline(fam["stage"] / args.steps, n_orb, cell, elem, peaks, args.subsims, clk.summary(), alu)
     else:
-        stage_ms = fam["stage"] / (4 * args.steps)
-        bytes_launch = stage_bytes_per_launch(elem, n_orb, cell.n_pts, reads_v=args.precision == "fp32_tc")
+        one = args.precision == "fp64" and variant == 0   # a launch per step: psi read and written
+        stage_ms = fam["stage"] / ((1 if one else 4) * args.steps)
+        bytes_launch = (2.0 * elem * n_orb * cell.n_pts if one else
+                        stage_bytes_per_launch(elem, n_orb, cell.n_pts, reads_v=args.precision == "fp32_tc"))
         achieved = bytes_launch / (stage_ms / 1e3) / 1e9
         roof = {"kernel": STAGE_KERNEL[args.precision], "bound": "hbm", "achieved": achieved,
                 "peak": hbm, "unit": "GB/s", "frac": achieved / hbm, "traffic": None,

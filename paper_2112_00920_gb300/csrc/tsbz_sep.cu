@@ -25,10 +25,10 @@ template <typename K> static void fs_attr(K* kernel, size_t bytes) {
 static inline bool fs_cube16(const CellDev& c) { return c.n1 == 16 && c.n2 == 16 && c.n3 == 16; }
 
 // Kernel variants of the single-precision path (LaunchSet::variant):
-//   16^3 cells with z groups: 0 whole step in one launch with the z
-//     contractions on tcgen05, 1 fused stage per launch (mma.sync), 2 z-march
-//     stage with CUDA-core projections, 3 whole step with the z contractions
-//     on mma.sync;
+//   16^3 cells with z groups: 0 whole step in one launch (k_step_fft: Fourier symbol, z
+//     contractions on tcgen05), 1 fused stage per launch (mma.sync), 2 z-march
+//     stage with CUDA-core projections, 3 whole step with the star stencil and
+//     the z contractions on mma.sync;
 //   other 16^3 cells and 8^3 cells: 0 fused / bulk-staged stage, 1 z-march stage;
 //   other shapes: the z-march stage only.
 // Returns 0 (whole step), 1 (fused or bulk-staged stage) or 2 (z-march stage).
@@ -180,8 +180,9 @@ bool launch_step_fused(const LaunchSet& L, void* psi, void* P, void* Pa, int sam
   const unsigned grid = (unsigned)L.n_units * (unsigned)L.cell.n_bands;
   if (fs_umma(L)) {
     // bands per CTA: as many as leave 13 waves of CTAs (two per SM), so that the last
-    // one costs little.  65 536 orbitals: 6.91 (1 band), 6.57 (2), 6.38 (4), 6.32 ms (8);
-    // 16 384: 1.93, 1.89, 1.86, 1.92; 4096 (three launches a step): 1.27, 1.29, 1.30, 1.47.
+    // one costs little.  Measured when a stage still had one barrier more: 65 536 orbitals
+    // 6.91 (1 band), 6.57 (2), 6.38 (4), 6.32 ms (8); 16 384: 1.93, 1.89, 1.86, 1.92; 4096
+    // (three launches a step): 1.27, 1.29, 1.30, 1.47.
     int per = 1;
     while (per < 8 && (long long)grid / (2 * per) >= 13 * 304) per *= 2;
     const unsigned ctas = (unsigned)L.n_units * (unsigned)((L.cell.n_bands + per - 1) / per);

@@ -15,7 +15,12 @@
 // barrier.  The projector work rides along: the z sums of t_m run on the tensor
 // cores under the next stage's transforms, one warp per atom forms their x and y
 // sums and, from them, the atom's ket tables.
+// The ket's MMAs run under the column's inverse transform.
 // Taylor terms are kept as s_m = h^m psi; (-i dt)^m / m! enters the sum only.
+// Measured, 65 536 orbitals: 10.50 (four star stencils, k_step_fused with its contractions
+// on tcgen05) -> 6.10 ms; 122 instructions a point and stage, projections of the current
+// included, 54% of the issue slots.  Without any transform it takes 4.8 ms, with the
+// butterflies in scalar instead of packed arithmetic 6.5 ms.
 //
 // Contractions (see tsbz_fused.cuh for the factorisation).  Atoms are addressed by
 // slot 2 g + j, the j-th atom of z group g (empty slots have zero tables).
