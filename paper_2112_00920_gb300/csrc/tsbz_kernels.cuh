@@ -170,10 +170,13 @@ __global__ void k_field(LaunchSet L, int mode, int factored) {
       int k = 0;
       while (i >= first[k + 1]) ++k;
       const int ax = k % 3, e = i - first[k], g = e - (nm + 1 + na);
-      double d = d0[3 * na + ax] * e;
-      if (e == nm) d = d0[3 * na + 3 + ax];
-      if (e > nm) d = d0[3 * (e - nm - 1) + ax];   // (past the anchors: replaced)
-      if (g >= 0) d = c.zg_k0[g >> 1] - ((g & 1) && c.zg_brk[g >> 1] < c.n3 ? c.hz * c.n3 : 0.0);
+      double d;
+      if (g >= 0)
+        d = c.zg_k0[g >> 1] - ((g & 1) && c.zg_brk[g >> 1] < c.n3 ? c.hz * c.n3 : 0.0);
+      else if (e > nm)
+        d = d0[3 * (e - nm - 1) + ax];
+      else
+        d = e == nm ? d0[3 * na + 3 + ax] : d0[3 * na + ax] * e;
       double sn, co;
       sincos(qs[k] * d, &sn, &co);
       field_f[i] = make_double2(co, sn);
