@@ -1,6 +1,6 @@
 // Small grids of any shape: the whole time step of a band (or the whole
 // Chebyshev recurrence of the ground-state solver) in one CTA and one launch, in
-// double or single precision.
+// double or single precision; with few orbitals in double in a cluster of CTAs.
 //
 // What bounds such runs is latency: a step of nine to twelve launches, each a
 // few CTAs that wait on dependent loads, and in double precision the FP64
@@ -9,7 +9,7 @@
 // contraction is spread over all eight warps as independent items, and the next
 // launch is the observation.
 //  - Kinetic operator: the star stencil from shared memory, or on 8^3 grids its
-//    Fourier symbol (ANY_FFT8): four threads per line, each forming the outputs k and
+//    Fourier symbol (Form8): four threads per line, each forming the outputs k and
 //    k + 4 of an 8-point transform (20 operations), 6 passes.
 //  - Projectors: the phase e^{i q z} is taken off once per point, so the z sums are
 //    real per (z group, column); then x sums per (atom, power, row), y sums per
@@ -20,7 +20,7 @@
 // same rounded operations, so a step may start from the projections that the
 // last one left (same q) or from fresh ones, bit for bit.
 // Measured per step, all four stages with their projections: 8^3, 16 orbitals in
-// double 298 -> 109 us, 512 orbitals in single 65 -> 46 us; 10 x 12 x 14, 324 orbitals
+// double 298 -> 64 us (96 with a CTA per band), 512 orbitals in single 65 -> 41 us; 10 x 12 x 14, 324 orbitals
 // in single under a pulse 179 -> 73 us (before: two launches per stage and one for
 // the current).
 #include <cooperative_groups.h>

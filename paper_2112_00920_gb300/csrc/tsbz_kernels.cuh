@@ -1169,8 +1169,8 @@ __global__ void k_hxc_final(const SubDev* subs, const int* sub_ids, int n_subs, 
 // transform each, then R1 threads with R2 points each (44 instructions deep
 // at N = 16; 148 for one thread per line).  Axes of 2 .. 32 points that are
 // powers of two go this way, others by plain sums, one output per thread.
-// Measured per step (both launches): one 16^3 grid 127 -> 29 us, 64 of them
-// 144 -> 62 us, 8^3 33 -> 21 us, 32^3 145 -> 86 us, two 10 x 12 x 14 78 -> 36 us
+// Measured per step (both launches): one 16^3 grid 127 -> 25 us, 64 of them
+// 144 -> 60 us, 8^3 33 -> 19 us, 32^3 145 -> 83 us, two 10 x 12 x 14 78 -> 33 us
 // (before: the whole grid in one CTA, or one launch per axis).
 // ----------------------------------------------------------------------------
 #define HXC_THREADS 128
