@@ -264,7 +264,10 @@ LaunchSet make_set(tsbz_ctx* ctx, HostCell& hc) {
 // already a warp per quarter of an SM); not more, which would begin a second wave
 // (256 units: 116 us in one, 143 us in two).  The slab form, whose groups hold at
 // most 32 bands, goes to four waves of three CTAs per SM: 8 units of 128 bands took
-// two waves of 32 bands.
+// two waves of 32 bands.  Its line form (32^3) streams a group's bands without a barrier,
+// so it wants long groups, whose partial densities cost less: two waves of two CTAs
+// per SM (8 units of 128 bands: observation and finalize 103 + 19 us, with three times
+// the groups 119 + 27, with six times 150 + 47).
 void plan_observe(const tsbz_ctx* ctx, CellDev& c, long long n_units) {
   const bool single = ctx->precision == TSBZ_FP32;
   int tiles = c.n_tiles, most = TSBZ_BG, least = 1;
@@ -279,7 +282,7 @@ void plan_observe(const tsbz_ctx* ctx, CellDev& c, long long n_units) {
   } else if (single && observe_slab_tiles(c)) {
     tiles = observe_slab_tiles(c);
     least = 4;
-    want = 4 * 456;
+    want = c.n2 == 32 && c.n3 == 32 ? 608 : 4 * 456;
   }
   const long long groups = std::max<long long>(1, want / (n_units * tiles));
   const long long bg = (c.n_bands + groups - 1) / groups;

@@ -932,7 +932,7 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
 //    last adds the tiles' currents, writes J and advances the step.
 // Measured per step: 8 k-points at 16^3 31 -> 12 us (FP32), two subgrids of 512
 // k-points 155 -> 24 us, 64 of 64 k-points 109 -> 68 us, 8 k-points of the 64-atom cell
-// 80 -> 27 us; with one warp or CTA for each unit and a shuffle sum per band before.
+// 80 -> 19 us; with one warp or CTA for each unit and a shuffle sum per band before.
 // ----------------------------------------------------------------------------
 #define FIN_THREADS 256
 

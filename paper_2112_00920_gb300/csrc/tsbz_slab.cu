@@ -699,7 +699,7 @@ __global__ void __launch_bounds__(SL_T, 3) k_observe_slab(LaunchSet L, const flo
 // Every point is read from shared memory three times instead of nine and from L2
 // twice instead of 2.25 times (the tiles of a band run side by side, so DRAM sees it
 // about once), and the barrier per plane is gone: 8 units of 128 bands of the 64-atom
-// cell 226 -> 119 us per step (the copy floor is 40 us).
+// cell 226 -> 103 us per step (the copy floor is 40 us).
 // Outputs as k_observe_slab, whose tile count it has (16).
 #define LO_N 32
 #define LO_T 224
