@@ -875,10 +875,6 @@ template <typename T> size_t any_smem(const CellDev& c) {
   return any_carve<T>(c, nullptr, m);
 }
 
-template <typename K> void any_attr(K* k, size_t bytes) {
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename T> bool any_ok(const CellDev& c) {
   return c.n_atoms <= ANY_NA && c.n1 < 1024 && c.n2 < 1024 && c.n3 < 1024 && any_smem<T>(c) <= ANY_MAX_SMEM;
 }
@@ -942,7 +938,7 @@ bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh
     using F = decltype(f);
     AnySmem<T> m;
     const size_t more = any_carve<T>(L.cell, nullptr, m, F::ctas);
-    any_attr(k_step_any_cluster<T, F>, more);
+    smem_limit<k_step_any_cluster<T, F>>(more);
     step_launch(k_step_any_cluster<T, F>, grid * F::ctas, F::threads, more, stream, L, (V*)psi, (V*)P, (V*)Pa, fresh_p,
                 want_pa, same_next);
   };
@@ -951,7 +947,7 @@ bool launch_step_any(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh
   }
   any_form<T>(L.cell, bytes, [&](auto f) {
     using F = decltype(f);
-    any_attr(k_step_any<T, F>, bytes);
+    smem_limit<k_step_any<T, F>>(bytes);
     step_launch(k_step_any<T, F>, grid, F::threads, bytes, stream, L, (V*)psi, (V*)P, (V*)Pa, fresh_p, want_pa,
                 same_next);
   });
@@ -964,7 +960,7 @@ template <typename T> bool launch_pa_any(const LaunchSet& L, const void* src, vo
   const size_t bytes = any_smem<T>(L.cell);
   any_form<T>(L.cell, bytes, [&](auto f) {
     using F = decltype(f);
-    any_attr(k_pa_any<T, F>, bytes);
+    smem_limit<k_pa_any<T, F>>(bytes);
     k_pa_any<T, F><<<(unsigned)L.n_units * L.cell.n_bands, F::threads, bytes, (cudaStream_t)stream>>>(
         L, (const V*)src, (V*)Pa);
   });
@@ -984,14 +980,14 @@ bool launch_filter_any(const LaunchSet& L, const void* in, void* out, const doub
     using F = decltype(f);
     AnySmem<double> m;
     const size_t more = any_carve<double>(L.cell, nullptr, m, F::ctas);
-    any_attr(k_filter_any_cluster<F>, more);
+    smem_limit<k_filter_any_cluster<F>>(more);
     k_filter_any_cluster<F><<<(unsigned)L.n_units * L.cell.n_bands * F::ctas, F::threads, more, (cudaStream_t)stream>>>(
         L, (const double2*)in, (double2*)out, fa, fb, degree);
   });
   if (done) return true;
   any_form<double>(L.cell, bytes, [&](auto f) {
     using F = decltype(f);
-    any_attr(k_filter_any<F>, bytes);
+    smem_limit<k_filter_any<F>>(bytes);
     k_filter_any<F><<<(unsigned)L.n_units * L.cell.n_bands, F::threads, bytes, (cudaStream_t)stream>>>(
         L, (const double2*)in, (double2*)out, fa, fb, degree);
   });

@@ -700,6 +700,7 @@ template <typename T> int run_stages(tsbz_ctx* ctx, bool fresh_p, int same_next_
       ++ctx->launches;
     }
   }
+  CK(cudaPeekAtLastError());   // a refused launch ends the step here
   return TSBZ_OK;
 }
 

@@ -1374,11 +1374,6 @@ __global__ void k_convert_out(const typename Cplx<T>::type* __restrict__ src, do
 // ----------------------------------------------------------------------------
 // launchers
 // ----------------------------------------------------------------------------
-// Dynamic shared memory above the 48 KiB default needs the kernel's opt-in.
-template <typename K> void stage_smem_attr(K* kernel, size_t bytes) {
-  if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename T> void launch_field(const LaunchSet& L, int mode, void* stream) {
   if (L.n_units == 0) return;
   const size_t bytes = sizeof(double2) * 3 * field_factors(L.cell);
@@ -1417,13 +1412,13 @@ void launch_stage(const LaunchSet& L, const void* tin, void* tout, void* psi, co
   const size_t sm = (size_t)bc * (L.cell.n_proj > 0 ? L.cell.n_proj : 1) * sizeof(V);
   cudaStream_t st = (cudaStream_t)stream;
   if (bc == 4) {
-    stage_smem_attr(k_stage<T, 4>, sm);
+    smem_limit<k_stage<T, 4>>(sm);
     k_stage<T, 4><<<grid, TSBZ_PT, sm, st>>>(L, (const V*)tin, (V*)tout, (V*)psi, (const V*)P, m);
   } else if (bc == 16) {
-    stage_smem_attr(k_stage<T, 16>, sm);
+    smem_limit<k_stage<T, 16>>(sm);
     k_stage<T, 16><<<grid, TSBZ_PT, sm, st>>>(L, (const V*)tin, (V*)tout, (V*)psi, (const V*)P, m);
   } else {
-    stage_smem_attr(k_stage<T, 8>, sm);
+    smem_limit<k_stage<T, 8>>(sm);
     k_stage<T, 8><<<grid, TSBZ_PT, sm, st>>>(L, (const V*)tin, (V*)tout, (V*)psi, (const V*)P, m);
   }
 }
@@ -1464,7 +1459,7 @@ int launch_hxc_t(const SubDev* subs_dev, const int* sub_ids_dev, int n_subs, con
   const bool pow2 = hxc_pow2(c.n1) && hxc_pow2(c.n2) && hxc_pow2(c.n3);
   if (c.poisson && (pow2 || total >= HXC_PLANES_MIN)) {
     const size_t sm = (size_t)2 * c.n1 * c.n3 * sizeof(double2);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_hxc_planes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    smem_limit<k_hxc_planes>(sm);
     step_launch(k_hxc_planes, dim3(n_subs, c.n2 / 2 + 1), HXC_THREADS, sm, stream, subs_dev, sub_ids_dev, c, tw[0],
                 tw[1], tw[2], wa);
     step_launch(k_hxc_sum<T>, (unsigned)((long long)((c.npts + 63) / 64) * n_subs), 64, 0, stream, subs_dev,

@@ -14,6 +14,21 @@ __device__ __forceinline__ void step_enter() {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 
+// Dynamic shared memory above 48 KB, for a kernel whose need differs from cell to cell.
+// The limit belongs to the kernel, not to a context or a thread, so every launch sets
+// it to the same value, the most that a block can have: a limit set to what one cell needs
+// was lowered by a context with a smaller cell between another thread's call and its
+// launch, which was then refused.
+template <auto kernel> inline void smem_limit(size_t bytes) {
+  if (bytes <= 48 * 1024) return;
+  static const int most = [] {
+    cudaFuncAttributes a = {};
+    cudaFuncGetAttributes(&a, kernel);
+    return 227 * 1024 - (int)a.sharedSizeBytes;
+  }();
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 template <typename... K, typename... A>
 inline void step_launch(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, void* stream, A... args) {
   cudaLaunchAttribute at[1];

@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include "tsbz_internal.h"
+#include "tsbz_launch.cuh"
 
 #define SCF_MAXB 256   // bands a unit may have in the ground-state solver
 #define SCF_T 16       // band tile edge of the Gram kernel
@@ -402,8 +403,7 @@ void launch_scf_rotate(const LaunchSet& L, const void* Y, const void* C, void* Y
   if (L.n_units == 0) return;
   const int nb = L.cell.n_bands;
   const size_t smem = sizeof(double2) * (size_t)nb * SCF_RB;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_scf_rotate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  smem_limit<k_scf_rotate>(smem);
   dim3 grid(L.n_units, (nb + SCF_RB - 1) / SCF_RB, (L.cell.npts + 127) / 128);
   k_scf_rotate<<<grid, 128, smem, (cudaStream_t)stream>>>(L, (const double2*)Y, (const double2*)C, (double2*)Yout);
 }
