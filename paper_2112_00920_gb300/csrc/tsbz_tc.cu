@@ -70,7 +70,10 @@ void launch_stage_v(const LaunchSet& L, const void* tin, void* tout, void* psi, 
                                                                       (float2*)psi, (const float2*)V, m);
 }
 
-bool observe_zf_ok(const CellDev& c) { return c.n3 == 16 && c.n1 <= 16 && c.n2 <= 16 && c.n_bgroups == 1; }
+// (k_observe_zf sums TC_ND neighbours a side: wider stencils would lose their outer weights)
+bool observe_zf_ok(const CellDev& c) {
+  return c.nd == TC_ND && c.n3 == 16 && c.n1 <= 16 && c.n2 <= 16 && c.n_bgroups == 1;
+}
 
 bool launch_observe_zf(const LaunchSet& L, const void* psi, double* rho_part, double* jk_part, double* nrm_part,
                        void* stream) {
