@@ -35,7 +35,6 @@ namespace {
 
 constexpr int S64_NA = 8;        // atoms of a cell
 constexpr int S64_GC = 4;        // z groups of one pass over a column
-constexpr int S64_MIN_ORB = 8;   // orbitals from which the whole-step form is taken
 
 template <int N> struct S64Smem {
   static constexpr int NN = N * N, NP = N * N * N;
@@ -505,11 +504,26 @@ static bool step64_supported(const CellDev& c) {
   return c.n1 == 16 && c.n2 == 16 && c.n3 == 16 && c.n_atoms <= S64_NA;
 }
 
-// Variant 0 of such cells, from S64_MIN_ORB orbitals on.  Runs of fewer orbitals
-// keep the point-parallel sequence, whose point tiles occupy more SMs than the
-// few bands would, and whose launches per step are fixed by the launch accounting.
+// Variant 0 of such cells, where it is the quicker form.  One CTA holds a band, so up to 152
+// orbitals cost what one does, while the point-parallel sequence spreads few bands of
+// many k-points over every SM: its projections cost by the bands of a unit (a CTA takes
+// up to 8), its stages by the rounds of 32 point tiles per unit and the bands.  Both sides
+// as fitted to times of a whole step (us; 1 .. 64 k-points times 1 .. 16 bands, no, 1, 2, 4 and 8
+// atoms in 1 .. 8 z groups, within 8%; sequence against one launch):
+// 8 atoms on 4 planes: 8 x 1 433 / 772, 8 x 4 714 / 782, 8 x 6 947 / 787, 16 x 1 676 / 778,
+// 16 x 2 810 / 783, 24 x 1 989 / 782, 1 x 6 762 / 772, 1 x 8 913 / 775; 8 atoms on 8 planes: 8 x 6
+// 973 / 1003, 1 x 16 1211 / 994; without projectors: 1 x 8 219 / 489, 8 x 16 640 / 527, 64 x 1 343 / 511.
+// The filter of the ground-state solver is chosen alike (an application of h, 2 atoms, 1 x 4
+// 84 / 154, 24 x 2 130 / 154, 1 x 16 194 / 154).
+static bool step64_quicker(const CellDev& c, int n_units) {
+  const long long b = c.n_bands, n = (32LL * n_units + 151) / 152, waves = (n_units * b + 151) / 152;
+  if (!c.use_proj) return 60 + 2 * n + 18 * n * b >= 50 + 440 * waves;
+  const long long whole =
+      440 + 138 + 38 * (c.n_zg - 1) + 8 * (c.n_atoms - c.n_zg) + (c.n_zg > S64_GC ? 65 : 0);
+  return 146 + n * (2 + 12 * c.n_atoms) + 64 * (b < 8 ? b : 8) + 35 * n * b / 2 >= 50 + whole * waves;
+}
 static bool step64_taken(const LaunchSet& L) {
-  return L.variant == 0 && step64_supported(L.cell) && (long long)L.n_units * L.cell.n_bands >= S64_MIN_ORB;
+  return L.variant == 0 && step64_supported(L.cell) && step64_quicker(L.cell, L.n_units);
 }
 
 bool launch_step64(const LaunchSet& L, void* psi, void* P, void* Pa, int fresh_p, int want_pa, int same_next,
@@ -531,7 +545,7 @@ bool launch_pa64(const LaunchSet& L, const void* src, void* Pa, void* stream) {
 
 bool launch_filter64(const LaunchSet& L, const void* in, void* out, const double* fa, const double* fb, int degree,
                      void* stream) {
-  if (L.n_units == 0 || !step64_supported(L.cell)) return false;
+  if (L.n_units == 0 || !step64_supported(L.cell) || !step64_quicker(L.cell, L.n_units)) return false;
   s64_attr(k_filter64<16>, sizeof(S64Smem<16>));
   k_filter64<16><<<(unsigned)L.n_units * L.cell.n_bands, 256, sizeof(S64Smem<16>), (cudaStream_t)stream>>>(
       L, (const double2*)in, (double2*)out, fa, fb, degree);
