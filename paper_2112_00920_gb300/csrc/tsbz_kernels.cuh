@@ -1174,12 +1174,29 @@ __global__ void k_hxc_final(const SubDev* subs, const int* sub_ids, int n_subs, 
 // (before: the whole grid in one CTA, or one launch per axis).
 // ----------------------------------------------------------------------------
 #define HXC_THREADS 128
-// Points in all from which sizes that are no power of two take the planes.  The
-// nine small launches lose everywhere (78 against 36 us at 3360 points); they stay
-// below this line because the launches of such a step are part of the accounting.
+// Points in all from which sizes that are no power of two may take the planes.  The
+// nine launches are slower below this line too (one 10^3 grid 48 against 16 us, one 10 x 12 x 14 56
+// against 25); they stay there because callers rely on the number of launches of a small run's step.
 #define HXC_PLANES_MIN 2048
 
 __host__ __device__ inline bool hxc_pow2(int n) { return n == 2 || n == 4 || n == 8 || n == 16 || n == 32; }
+
+// Whether the planes are the quicker way for sizes that are no power of two up to 32.  An
+// axis that is summed plainly costs 8 n products per point of a plane (four there and four back), on the
+// n2 / 2 + 1 SMs that hold a plane; the launches over all points spread such sums over the GPU,
+// but take a chain of n per axis.  Both in FP64 products of one SM (4 a ns), fitted to
+// 161 sizes (10^3 .. 80^3, flat and long cells, 1 .. 64 sub-simulations; the worst choice is
+// 3% slower).  us, launches over all points / planes: 24^3 86 / 83, 36^3 190 / 247 (two of them
+// 278 / 252), 48^3 361 / 527 (two 691 / 543), 64^3 1055 / 1230, 80^3 2579 / 2420, 64 x 16 x 64
+// 249 / 1026 (eight 1581 / 1071), 16 x 64 x 16 102 / 39, 100 x 10 x 10 116 / 221, 10 x 100 x 10 120 / 38.
+inline bool hxc_planes_quicker(const CellDev& c, int n_subs) {
+  const long long n13 = (long long)c.n1 * c.n3, total = (long long)n_subs * c.npts, n = c.n1 + c.n2 + c.n3;
+  const long long plane = n13 * (c.n2 + (hxc_pow2(c.n1) ? 0 : 8 * c.n1) + (hxc_pow2(c.n3) ? 0 : 8 * c.n3));
+  const long long rounds = ((long long)n_subs * (c.n2 / 2 + 1) + 151) / 152;
+  const long long planes = 60000 + rounds * plane + total * c.n2 / 152;
+  const long long chain = 88000 + 3200 * n, spread = 160000 + total * n / 12;
+  return planes <= (chain > spread ? chain : spread);
+}
 
 // Transform of `lines` lines of R1 R2 values `stride` apart, from w to `other`
 // (both swapped); line l starts at (l / inner) * outer + l % inner.
@@ -1454,10 +1471,10 @@ int launch_hxc_t(const SubDev* subs_dev, const int* sub_ids_dev, int n_subs, con
   cudaStream_t st = (cudaStream_t)stream;
   const long long total = (long long)n_subs * c.npts;
   // by frequency planes on power-of-two grids and, from HXC_PLANES_MIN points in
-  // all on, every other size whose planes fit; the sequence of nine launches
-  // below stays for smaller and larger ones
+  // all on, every other size whose planes fit and are quicker; the sequence of nine launches
+  // below stays for the others
   const bool pow2 = hxc_pow2(c.n1) && hxc_pow2(c.n2) && hxc_pow2(c.n3);
-  if (c.poisson && (pow2 || total >= HXC_PLANES_MIN)) {
+  if (c.poisson && (pow2 || (total >= HXC_PLANES_MIN && hxc_planes_quicker(c, n_subs)))) {
     const size_t sm = (size_t)2 * c.n1 * c.n3 * sizeof(double2);
     smem_limit<k_hxc_planes>(sm);
     step_launch(k_hxc_planes, dim3(n_subs, c.n2 / 2 + 1), HXC_THREADS, sm, stream, subs_dev, sub_ids_dev, c, tw[0],
