@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(256) k_scf_gram_sum(int nb, double dv, const d
 // W1; s = shift_coef tr S), Li = L^{-1} (one column per thread, in W2) and
 // C = L^{-H}; when want_lam is set, also A = L^{-1} Hs L^{-H} over Hs (T =
 // Hs L^{-H} in W1 first) and its largest eigenvalue by power iteration on
-// A + shift (Gershgorin shift so that A + shift is positive semidefinite).
+// A + shift (Gershgorin shift, and a little more, so that A + shift is positive definite: a
+// multiple of the identity, as one band has, would leave a zero matrix to iterate with).
 // The matrices live in global memory (they stay in L2); every sum runs in a
 // fixed order.  status bit 4: S + s I not positive definite.
 __global__ void __launch_bounds__(SCF_OT) k_scf_ortho(int nb, double shift_coef, int want_lam,
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(SCF_OT) k_scf_ortho(int nb, double shift_coef,
   if (tid == 0) {
     double lo = red[0][0];
     for (int i = 1; i < min(nb, nt); ++i) lo = fmin(lo, red[0][i]);
-    sc[0] = -lo;
+    sc[0] = -lo + 1e-6 * (1.0 + fabs(lo));
   }
   __syncthreads();
   const double shift = sc[0];
