@@ -988,18 +988,36 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
   const int u_first = wide ? tile / share : tile + ntile * warp;
   const int u_step = wide ? ntile / share + (share > 1 ? n_k : 0) : ntile * n_warps;   // (shared units: one each)
   const int e_first = wide ? (tile % share) * FIN_THREADS + tid : lane, e_step = wide ? share * FIN_THREADS : 32;
+  // norms: a thread per band, or a warp whose lanes share the band's point tiles, by the length of
+  // the chain of sums (lengths in sums; a warp's five exchanges count 16)
+  const int nt = c.n_otiles, rows = e_step / 32;
+  const bool lanes = (c.n_bands + rows - 1) / rows * ((nt + 31) / 32 + 16) < (c.n_bands + e_step - 1) / e_step * nt;
   double v[3] = {0.0, 0.0, 0.0};   // this thread's share of sum occ <u|pi|u> / occ
   for (int kl = u_first; kl < n_k; kl += u_step) {
     const int u = S.unit0 + kl;
     const UnitDev U = units[u];
     double nsum = 0.0, jk[3] = {0.0, 0.0, 0.0};
-    for (int b = e_first; b < c.n_bands; b += e_step) {
-      double nb = 0.0;
+    if (lanes) {
+      for (int b = e_first / 32; b < c.n_bands; b += rows) {
+        double nb = 0.0;
+#pragma unroll 4
+        for (int t = lane; t < nt; t += 32) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
+        for (int off = 16; off > 0; off >>= 1) nb += __shfl_xor_sync(0xffffffffu, nb, off);
+        if (lane == 0) {
+          nb *= c.dv;
+          S.norms[kl * c.n_bands + b] = nb;
+          nsum += nb;
+        }
+      }
+    } else {
+      for (int b = e_first; b < c.n_bands; b += e_step) {
+        double nb = 0.0;
 #pragma unroll 8
-      for (int t = 0; t < c.n_otiles; ++t) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
-      nb *= c.dv;
-      S.norms[kl * c.n_bands + b] = nb;
-      nsum += nb;
+        for (int t = 0; t < nt; ++t) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
+        nb *= c.dv;
+        S.norms[kl * c.n_bands + b] = nb;
+        nsum += nb;
+      }
     }
     for (int i = e_first; i < c.n_otiles * ngrp; i += e_step)
 #pragma unroll
