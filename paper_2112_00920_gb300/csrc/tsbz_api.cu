@@ -114,6 +114,7 @@ struct tsbz_ctx {
   const double* d_filt = nullptr;  // ground-state solver: filter coefficients per unit (stage m = 0)
   double* d_jtile = nullptr; // per sub-simulation: [TSBZ_FIN_MAX_TILES][3] partial currents of the finalize
   int fin_tiles = 16;        // CTAs per sub-simulation of the finalize
+  int fin_otiles = 0;        // most point tiles of a cell's observation
   int* d_jcount = nullptr;   // per sub-simulation: finalize tiles done
   double2* work_a = nullptr;
   double2* work_b = nullptr;
@@ -318,6 +319,8 @@ int layout(tsbz_ctx* ctx) {
   for (size_t s = 0; s < ctx->subs.size(); ++s)
     if (fin_wide(ctx->cells[ctx->subs[s].cell].dev)) fin_units = std::max(fin_units, ctx->subs[s].n_k);
   ctx->fin_tiles = std::min(TSBZ_FIN_MAX_TILES, fin_units);
+  ctx->fin_otiles = 0;
+  for (auto& hs : ctx->subs) ctx->fin_otiles = std::max(ctx->fin_otiles, ctx->cells[hs.cell].dev.n_otiles);
   for (size_t s = 0; s < ctx->subs.size(); ++s) {
     HostSub& hs = ctx->subs[s];
     HostCell& hc = ctx->cells[hs.cell];
@@ -571,7 +574,7 @@ template <typename T> int run_observe(tsbz_ctx* ctx, int fin_mode) {
   ev_start(ctx, FAM_FIN);
   launch_finalize_t<T>(ctx->d_subs, (int)ctx->subs.size(), ctx->d_units, ctx->d_cells, ctx->q_obs, ctx->Pa,
                        ctx->rho_part, ctx->jk_part, ctx->nrm_part, ctx->d_mask, fin_mode, ctx->fin_tiles,
-                       ctx->stream);
+                       ctx->fin_otiles, ctx->stream);
   ev_stop(ctx);
   ++ctx->launches;
   return TSBZ_OK;

@@ -202,7 +202,8 @@ void launch_observe(const LaunchSet& L, const void* psi, double* rho_part, doubl
 template <typename T>
 void launch_finalize_t(const SubDev* subs, int n_subs, const UnitDev* units, const CellDev* cells_dev,
                        const double* q_obs, const void* Pa, const double* rho_part, const double* jk_part,
-                       const double* nrm_part, const int* mask, int mode, int n_tiles, void* stream);
+                       const double* nrm_part, const int* mask, int mode, int n_tiles, int most_otiles,
+                       void* stream);
 template <typename T>
 int launch_hxc_t(const SubDev* subs_dev, const int* sub_ids_dev, int n_subs, const CellDev& c, double2* wa,
                  double2* wb, double2* const tw[3], void* stream);

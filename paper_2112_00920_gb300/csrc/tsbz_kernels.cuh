@@ -936,7 +936,9 @@ __global__ void __launch_bounds__(TSBZ_PT) k_observe(LaunchSet L, const typename
 // ----------------------------------------------------------------------------
 #define FIN_THREADS 256
 
-template <typename T>
+// LANES: some cell has so many point tiles that a band's norm may be shared by a warp (the launcher
+// decides; without that form the kernel keeps its 64 registers).
+template <typename T, bool LANES>
 __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
     const SubDev* __restrict__ subs, const UnitDev* __restrict__ units, const CellDev* __restrict__ cells,
     const double* __restrict__ q_obs, const typename Cplx<T>::type* __restrict__ Pa,
@@ -990,18 +992,19 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
   const int e_first = wide ? (tile % share) * FIN_THREADS + tid : lane, e_step = wide ? share * FIN_THREADS : 32;
   // norms: a thread per band, or a warp whose lanes share the band's point tiles, by the length of
   // the chain of sums (lengths in sums; a warp's five exchanges count 16)
-  const int nt = c.n_otiles, rows = e_step / 32;
-  const bool lanes = (c.n_bands + rows - 1) / rows * ((nt + 31) / 32 + 16) < (c.n_bands + e_step - 1) / e_step * nt;
+  const int rows = e_step / 32;
+  const bool lanes = LANES && (c.n_bands + rows - 1) / rows * ((c.n_otiles + 31) / 32 + 16) <
+                                  (c.n_bands + e_step - 1) / e_step * c.n_otiles;
   double v[3] = {0.0, 0.0, 0.0};   // this thread's share of sum occ <u|pi|u> / occ
   for (int kl = u_first; kl < n_k; kl += u_step) {
     const int u = S.unit0 + kl;
     const UnitDev U = units[u];
     double nsum = 0.0, jk[3] = {0.0, 0.0, 0.0};
-    if (lanes) {
+    if (LANES && lanes) {
       for (int b = e_first / 32; b < c.n_bands; b += rows) {
         double nb = 0.0;
 #pragma unroll 4
-        for (int t = lane; t < nt; t += 32) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
+        for (int t = lane; t < c.n_otiles; t += 32) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
         for (int off = 16; off > 0; off >>= 1) nb += __shfl_xor_sync(0xffffffffu, nb, off);
         if (lane == 0) {
           nb *= c.dv;
@@ -1013,7 +1016,7 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finalize(
       for (int b = e_first; b < c.n_bands; b += e_step) {
         double nb = 0.0;
 #pragma unroll 8
-        for (int t = 0; t < nt; ++t) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
+        for (int t = 0; t < c.n_otiles; ++t) nb += nrm_part[U.nrm_off + (long long)t * c.n_bands + b];
         nb *= c.dv;
         S.norms[kl * c.n_bands + b] = nb;
         nsum += nb;
@@ -1473,13 +1476,15 @@ void launch_observe(const LaunchSet& L, const void* psi, double* rho_part, doubl
 template <typename T>
 void launch_finalize_t(const SubDev* subs, int n_subs, const UnitDev* units, const CellDev* cells_dev,
                        const double* q_obs, const void* Pa, const double* rho_part, const double* jk_part,
-                       const double* nrm_part, const int* mask, int mode, int n_tiles, void* stream) {
+                       const double* nrm_part, const int* mask, int mode, int n_tiles, int most_otiles,
+                       void* stream) {
   using V = typename Cplx<T>::type;
   if (n_subs == 0) return;
   // n_tiles (16 .. TSBZ_FIN_MAX_TILES) tiles per sub-simulation: density points, and units for the
   // current and the norms
-  step_launch(k_finalize<T>, dim3(n_subs, 2 * n_tiles), FIN_THREADS, 0, stream, subs, units, cells_dev, q_obs,
-              (const V*)Pa, rho_part, jk_part, nrm_part, mask, mode);
+  // (a warp is not taken below 18 point tiles, see `lanes`)
+  step_launch(most_otiles < 18 ? k_finalize<T, false> : k_finalize<T, true>, dim3(n_subs, 2 * n_tiles), FIN_THREADS, 0,
+              stream, subs, units, cells_dev, q_obs, (const V*)Pa, rho_part, jk_part, nrm_part, mask, mode);
 }
 
 template <typename T>
