@@ -253,8 +253,10 @@ template <int D> __device__ __forceinline__ void fx_issue_bra(const FxState& x, 
       const uint64_t bh = um_sdesc(b0 + 256 * ks, 128, 1024), bl = um_sdesc(b1 + 256 * ks, 128, 1024);
       um_mma_tf32_ts(d, a_lo, bh, idesc, ks > 0);
       um_mma_tf32_ts(d, a_hi, bl, idesc, true);
-      um_mma_tf32_ts(d, a_hi, bh, idesc, true);
     }
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)   // the large products last (see um_mma_tf32_ts)
+      um_mma_tf32_ts(d, x.tbase + FX_BRA_A + 64 * hh + 8 * ks, um_sdesc(b0 + 256 * ks, 128, 1024), idesc, true);
   }
   um_commit(x.bar);
 }
@@ -622,8 +624,10 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
             const uint64_t bh = um_sdesc(b0 + 256 * ks, 128, 512), bl = um_sdesc(b1 + 256 * ks, 128, 512);
             um_mma_tf32_ts(d, a_lo, bh, idesc, ks > 0);
             um_mma_tf32_ts(d, a_hi, bl, idesc, true);
-            um_mma_tf32_ts(d, a_hi, bh, idesc, true);
           }
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks)
+            um_mma_tf32_ts(d, x.tbase + FX_KET_A + 64 * hh + 8 * ks, um_sdesc(b0 + 256 * ks, 128, 512), idesc, true);
         }
         um_commit(x.bar);
       }

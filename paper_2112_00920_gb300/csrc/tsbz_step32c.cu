@@ -22,9 +22,10 @@
 // remote rows).
 // Every wait on an MMA is bounded; a CTA that gave up keeps taking part in the
 // cluster's barriers and reports at the end.
-// Tensor-memory columns: Taylor sum [0, 64), v_eff [64, 96), bra accumulator
-// [96, 128), and [128, 256), 64 per thread half: the bra's A (hi, lo 32 each), or the
-// ket's A (hi, lo 16 each) and accumulator.  The second-order bra accumulates in [0, 48).
+// Tensor-memory columns: Taylor sum [0, 64), v_eff [64, 96), bra accumulator of the large
+// products [96, 128), and [128, 256): the bra's A (three parts) and its accumulator of
+// the small products, or the ket's A (hi, lo) and accumulators.  The second-order bra
+// accumulates in [0, 96).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -46,15 +47,17 @@ constexpr int QP = 33;            // row pitch (float2): no bank conflicts along
 constexpr int QBUF = QR * QN * QP;
 constexpr int QA = 64;            // atom slots
 constexpr int QG = 8;             // z groups, x and y classes
-constexpr int Q_ACC = 0, Q_VEFF = 64, Q_BRA_D = 96, Q_OP = 128, Q_BRA2_D = 0;
+constexpr int Q_ACC = 0, Q_VEFF = 64, Q_OP = 128;
+constexpr int Q_BRA_D = 96, Q_BRA_S = 208, Q_BRA2_D = 0, Q_BRA2_S = 48;   // accumulators of large and small products
 constexpr uint32_t Q_COLS = 256;
-constexpr size_t Q_IMG = 16384 + 16384 + 24576;   // B images of a unit: ket, first- and second-order bra
+constexpr int Q_KET_B = 16384, Q_BRA_B = 12288, Q_BRA2_B = 18432;
+constexpr size_t Q_IMG = Q_KET_B + Q_BRA_B + Q_BRA2_B;   // B images of a unit: ket, first- and second-order bra
 
 struct QSmem {
   float2 b1[QBUF];                 // line buffers [row][z or k_z][x or k_x]
   float2 b2[QBUF];
-  unsigned char bket[16384];       // B of the ket (hi, lo)
-  unsigned char bbra[16384];       // B of the first-order bra (hi, lo)
+  unsigned char bket[Q_KET_B];     // B of the ket (hi, lo)
+  unsigned char bbra[Q_BRA_B];     // B of the first-order bra (three parts)
   float4 xt[QG * QN];              // x factors per class (Re F, Im F, d, 0)
   float4 yt[QG * QR];              // y factors per class on the CTA's rows
   float2 tab[QA * QR * 3];         // ket tables per (slot, row); second-order partial sums
@@ -165,21 +168,21 @@ __device__ __forceinline__ float2 q_zfactor(const CellDev& c, const float2* ph, 
 }
 
 // B of an order-D bra (N = 32 or 48): n = 2 q + c', q = (D + 1) g + k; K = 64:
-// kk = 32 h + 2 j + c for z = 2 j + h.  hi, then lo (N/8 * 2 KiB each).  A warp writes one
-// 8 x 16-byte core matrix (no bank conflicts).
+// kk = 32 h + 2 j + c for z = 2 j + h.  Three parts (um_split3), N/8 KiB each.  A warp writes one
+// 8 x 16-byte core matrix (no bank conflicts), a lane both components of a plane.
 template <int D> __device__ void q_build_bra(unsigned char* bz, const CellDev& c, const float2* ph) {
-  constexpr int NN = D == 1 ? 32 : 48, LO = NN / 8 * 2048;
+  constexpr int NN = D == 1 ? 32 : 48, PART = NN / 8 * 1024;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll 2
-  for (int m = warp; m < NN / 8 * 16; m += QT / 32) {
-    const int n = 8 * (m >> 4) + (lane >> 2), kk = 4 * (m & 15) + (lane & 3);
-    const int q = n >> 1, cs = n & 1, g = q / (D + 1), k = q - g * (D + 1), z = (kk & 30) + (kk >> 5), cu = kk & 1;
+  for (int m = warp; m < NN / 8 * 8; m += QT / 32) {
+    const int n = 8 * (m >> 3) + (lane >> 2), kk = 8 * (m & 7) + 2 * (lane & 3);
+    const int q = n >> 1, g = q / (D + 1), k = q - g * (D + 1), z = (kk & 30) + (kk >> 5);
     float2 f = make_float2(0.f, 0.f);
     if (g < c.zs_n) f = q_zfactor(c, ph, g, z, k);
-    uint32_t hi, lo;
-    q_split(cs == 0 ? (cu == 0 ? f.x : -f.y) : (cu == 0 ? f.y : f.x), hi, lo);
-    *reinterpret_cast<uint32_t*>(bz + 128 * m + 4 * lane) = hi;
-    *reinterpret_cast<uint32_t*>(bz + LO + 128 * m + 4 * lane) = lo;
+    uint32_t r[3];
+    um_split3((n & 1) == 0 ? make_float2(f.x, -f.y) : make_float2(f.y, f.x), r);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) *reinterpret_cast<uint32_t*>(bz + PART * i + 128 * m + 4 * lane) = r[i];
   }
 }
 
@@ -214,8 +217,8 @@ __global__ void __launch_bounds__(QT) k_images32(LaunchSet L, unsigned char* __r
   const float2* phh = (const float2*)L.ph_half + (long long)u * L.ph_stride;
   const float2* pho = (const float2*)L.ph_obs + (long long)u * L.ph_stride;
   if (blockIdx.y == 0) q_build_ket(o, c, phh);
-  if (blockIdx.y == 1) q_build_bra<1>(o + 16384, c, phh);
-  if (blockIdx.y == 2) q_build_bra<2>(o + 32768, c, pho);
+  if (blockIdx.y == 1) q_build_bra<1>(o + Q_KET_B, c, phh);
+  if (blockIdx.y == 2) q_build_bra<2>(o + Q_KET_B + Q_BRA_B, c, pho);
 }
 
 // x factors of the classes, y factors on the CTA's rows, rows' slot masks; ends with a barrier.
@@ -252,59 +255,69 @@ __device__ void q_tables(QSmem& sm, const CellDev& c, const float2* ph, int r0) 
   __syncthreads();
 }
 
+// Tensor-memory columns of a thread half's operands, one or the other live: the bra's A, 16 words
+// per part, and the ket's A and accumulator.  The next stage's bra is written while the other
+// half may still read its ket accumulator, so neither half's columns meet the other's.
+__host__ __device__ constexpr int q_bra_a(int h, int part) { return part < 2 ? Q_OP + 32 * h + 16 * part : Q_OP + 64 + 48 * h; }
+__host__ __device__ constexpr int q_ket_a(int h) { return Q_OP + 32 * h; }
+__host__ __device__ constexpr int q_ket_d(int h) { return Q_OP + 64 + 32 * h; }
+
 // The column's planes as a row of the bra's A.
 __device__ __forceinline__ void q_stage(const float2 (&u)[16], const QState& x) {
   const int warp = threadIdx.x >> 5, h = warp >> 2, qd = warp & 3;
+  uint32_t p[3][16];
 #pragma unroll
-  for (int kk = 0; kk < 2; ++kk) {
-    uint32_t hi[16], lo[16];
+  for (int j = 0; j < 16; ++j) {
+    uint32_t r[3];
+    um_split3(u[j], r);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      q_split(u[8 * kk + j].x, hi[2 * j], lo[2 * j]);
-      q_split(u[8 * kk + j].y, hi[2 * j + 1], lo[2 * j + 1]);
-    }
-    um_st16(um_addr(x.tbase, qd, Q_OP + 64 * h + 16 * kk), hi);
-    um_st16(um_addr(x.tbase, qd, Q_OP + 64 * h + 32 + 16 * kk), lo);
+    for (int i = 0; i < 3; ++i) p[i][j] = r[i];
   }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) um_st16(um_addr(x.tbase, qd, q_bra_a(h, i)), p[i]);
 }
 
-// The MMAs of an order-D bra (one thread, behind a barrier after q_stage and B's fenced writes).
+// The MMAs of an order-D bra (one thread, behind a barrier after q_stage and B's fenced writes):
+// the products of the first parts by themselves, the five next ones (down to 2^-18) in an
+// accumulator of their own; what is left out is below 2^-26.
 template <int D> __device__ __forceinline__ void q_issue_bra(const QState& x, const unsigned char* bz) {
-  constexpr int NN = D == 1 ? 32 : 48, LO = NN / 8 * 2048;
-  constexpr uint32_t idesc = um_idesc_tf32(128, NN);
+  constexpr int NN = D == 1 ? 32 : 48, PART = NN / 8 * 1024;
+  constexpr uint32_t idesc = um_idesc_bf16(128, NN);
   um_fence_after();
-  const uint32_t b0 = bk_smem(bz), b1 = b0 + LO, d = x.tbase + (D == 1 ? Q_BRA_D : Q_BRA2_D);
+  const uint32_t b = bk_smem(bz);
+  const uint32_t d0 = x.tbase + (D == 1 ? Q_BRA_D : Q_BRA2_D), d1 = x.tbase + (D == 1 ? Q_BRA_S : Q_BRA2_S);
+  // (part of A, part of B), the smallest products first
+  constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
 #pragma unroll
-  for (int ks = 0; ks < 8; ++ks) {
-    const uint32_t a_hi = x.tbase + Q_OP + 64 * (ks >> 2) + 8 * (ks & 3), a_lo = a_hi + 32;
-    const uint64_t bh = um_sdesc(b0 + 256 * ks, 128, 2048), bl = um_sdesc(b1 + 256 * ks, 128, 2048);
-    um_mma_tf32_ts(d, a_lo, bh, idesc, ks > 0);
-    um_mma_tf32_ts(d, a_hi, bl, idesc, true);
-    um_mma_tf32_ts(d, a_hi, bh, idesc, true);
-  }
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+      um_mma_bf16_ts(i < 5 ? d1 : d0, x.tbase + q_bra_a(ks >> 1, pa[i]) + 8 * (ks & 1),
+                     um_sdesc(b + PART * pb[i] + 256 * ks, 128, 1024), idesc, ks > 0 || (i > 0 && i < 5));
   um_commit(x.bar);
 }
 
 // The thread's share of its column's z sums into zs[q][row][x] (after q_poll).
 template <int D> __device__ __forceinline__ void q_collect(const QState& x, float2* zs) {
-  constexpr int DC = D == 1 ? Q_BRA_D : Q_BRA2_D;
+  constexpr int DC = D == 1 ? Q_BRA_D : Q_BRA2_D, DS = D == 1 ? Q_BRA_S : Q_BRA2_S;
   const int tid = threadIdx.x, warp = tid >> 5, h = warp >> 2, qd = warp & 3;
   const int col = tid & 127, o = (col >> 5) * QP + (col & 31);
-  if constexpr (D == 1) {
-    float d[16];
-    um_ld16(um_addr(x.tbase, qd, DC + 16 * h), d);   // q = 8 h ..
+  float d[16], e[16];
+  um_ld16(um_addr(x.tbase, qd, DC + (D == 1 ? 16 : 32) * h), d);   // q = 8 h .. (D = 2: 16 h ..)
+  um_ld16(um_addr(x.tbase, qd, DS + (D == 1 ? 16 : 32) * h), e);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) zs[(8 * h + i) * QR * QP + o] = make_float2(d[2 * i], d[2 * i + 1]);
-  } else {
-    float d[16], e[16];
-    um_ld16(um_addr(x.tbase, qd, DC + 32 * h), d);   // q = 16 h ..
-    um_ld16(um_addr(x.tbase, qd, DC + 16), e);       // q = 8 .. 15, four for each half
+  for (int i = 0; i < 8; ++i)
+    zs[((D == 1 ? 8 : 16) * h + i) * QR * QP + o] =
+        make_float2(__fadd_rn(d[2 * i], e[2 * i]), __fadd_rn(d[2 * i + 1], e[2 * i + 1]));
+  if constexpr (D == 2) {
+    um_ld16(um_addr(x.tbase, qd, DC + 16), d);   // q = 8 .. 15, four for each half
+    um_ld16(um_addr(x.tbase, qd, DS + 16), e);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) zs[(16 * h + i) * QR * QP + o] = make_float2(d[2 * i], d[2 * i + 1]);
+    for (int i = 0; i < 16; ++i) d[i] = __fadd_rn(d[i], e[i]);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       zs[(8 + 4 * h + i) * QR * QP + o] =
-          h ? make_float2(e[8 + 2 * i], e[9 + 2 * i]) : make_float2(e[2 * i], e[2 * i + 1]);
+          h ? make_float2(d[8 + 2 * i], d[9 + 2 * i]) : make_float2(d[2 * i], d[2 * i + 1]);
   }
 }
 
@@ -388,8 +401,8 @@ __device__ bool q_current(QSmem& sm, cg::cluster_group& cl, QState& x, const Cel
   __syncthreads();
   bool ok = true;
   if (threadIdx.x == 0) {
-    bk_mbar_expect_tx(bar, 24576);
-    bk_copy_g2s(bk_smem(bz), img + 32768, 24576, bar);
+    bk_mbar_expect_tx(bar, Q_BRA2_B);
+    bk_copy_g2s(bk_smem(bz), img + Q_KET_B + Q_BRA_B, Q_BRA2_B, bar);
     ok = bk_mbar_wait(bar, parity, BK_WAIT_POLLS);
     q_issue_bra<2>(x, bz);
   }
@@ -464,9 +477,9 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
   QState x = q_open(sm);
   if (tid == 0) {
     const uint32_t bar = bk_smem(&sm.mimg);
-    bk_mbar_expect_tx(bar, 32768);
-    bk_copy_g2s(bk_smem(sm.bket), img, 16384, bar);
-    bk_copy_g2s(bk_smem(sm.bbra), img + 16384, 16384, bar);
+    bk_mbar_expect_tx(bar, Q_KET_B + Q_BRA_B);
+    bk_copy_g2s(bk_smem(sm.bket), img, Q_KET_B, bar);
+    bk_copy_g2s(bk_smem(sm.bbra), img + Q_KET_B, Q_BRA_B, bar);
   }
   float2 t[16];
   {
@@ -589,7 +602,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
         q_split(av[i].x, rh[i], rl[i]);
         q_split(av[i].y, ih[i], il[i]);
       }
-      const uint32_t o = um_addr(x.tbase, qd, Q_OP + 64 * h);
+      const uint32_t o = um_addr(x.tbase, qd, q_ket_a(h));
       q_st8(o, rh);
       q_st8(o + 8, ih);
       q_st8(o + 16, rl);
@@ -604,15 +617,19 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
       const uint32_t b0 = bk_smem(sm.bket), b1 = b0 + 8192;
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {   // planes of half hh
-        const uint32_t d = x.tbase + Q_OP + 64 * hh + 32;
+        const uint32_t d = x.tbase + q_ket_d(hh);
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
-          const uint32_t a_hi = x.tbase + Q_OP + 64 * (ks >> 1) + 8 * (ks & 1), a_lo = a_hi + 16;
+          const uint32_t a_hi = x.tbase + q_ket_a(ks >> 1) + 8 * (ks & 1), a_lo = a_hi + 16;
           const uint64_t bh = um_sdesc(b0 + 4096 * hh + 256 * ks, 128, 1024);
           const uint64_t bl = um_sdesc(b1 + 4096 * hh + 256 * ks, 128, 1024);
           um_mma_tf32_ts(d, a_lo, bh, idesc, ks > 0);
           um_mma_tf32_ts(d, a_hi, bl, idesc, true);
-          um_mma_tf32_ts(d, a_hi, bh, idesc, true);
+        }
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {   // the large products last
+          const uint32_t a_hi = x.tbase + q_ket_a(ks >> 1) + 8 * (ks & 1);
+          um_mma_tf32_ts(d, a_hi, um_sdesc(b0 + 4096 * hh + 256 * ks, 128, 1024), idesc, true);
         }
       }
       um_commit(x.bar);
@@ -667,7 +684,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
     ok = q_poll(x) && ok;
     {
       float d[32];
-      um_ld32(um_addr(x.tbase, qd, Q_OP + 64 * h + 32), d);   // conj(V_NL s_{m-1})
+      um_ld32(um_addr(x.tbase, qd, q_ket_d(h)), d);   // conj(V_NL s_{m-1})
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         t[j].x += d[2 * j];

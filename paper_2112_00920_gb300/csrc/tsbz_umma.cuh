@@ -63,7 +63,18 @@ __host__ __device__ constexpr uint32_t um_idesc_tf32(int m, int n) {
          | ((uint32_t)(m >> 4) << 24);   // M
 }
 
+// The same of kind::f16 with A and B in bfloat16 (16-bit cells: two along K per
+// 32-bit word of tensor or shared memory, the lower half first; K = 16).
+__host__ __device__ constexpr uint32_t um_idesc_bf16(int m, int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+
 // ---- MMA -----------------------------------------------------------------------
+// Rounding: the sum of an MMA's products and its accumulator is cut off (toward zero) at
+// 24 bits, on average 3e-8 of it per MMA that adds to a sum of full size (measured: K = 16
+// of positive numbers in three-product TF32, six such MMAs -1.0e-7, with the two small
+// products' MMAs before the large one's -6.6e-8).  So small products come first, and a
+// sum of many K steps keeps its large products in an accumulator of their own.
 // D[tmem] (+)= A[tmem] B[smem]^T: M x N x 8 (TF32), issued by one thread.
 __device__ __forceinline__ void um_mma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
                                                bool accumulate) {
@@ -72,6 +83,26 @@ __device__ __forceinline__ void um_mma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem,
       " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
       : "memory");
+}
+
+// The same in bfloat16 (um_idesc_bf16): M x N x 16.
+__device__ __forceinline__ void um_mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                               bool accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
+      : "memory");
+}
+
+// A float is the sum of three bfloat16 numbers (8 bits each, 24 in all), each the rounded
+// rest of the ones before.  Two floats at once: word i holds part i of both, x in the lower half.
+__device__ __forceinline__ void um_split3(float2 v, uint32_t (&r)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;\n" : "=r"(r[i]) : "f"(v.y), "f"(v.x));
+    v = __fadd2_rn(v, make_float2(-__uint_as_float(r[i] << 16), -__uint_as_float(r[i] & 0xffff0000u)));
+  }
 }
 
 // Arrive once on the mbarrier when every MMA issued so far by this thread has
