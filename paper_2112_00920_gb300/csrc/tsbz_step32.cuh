@@ -16,7 +16,8 @@
 // cores under the next stage's transforms, one warp per atom forms their x and y
 // sums and, from them, the atom's ket tables.
 // The ket's MMAs run under the column's inverse transform.
-// Taylor terms are kept as s_m = h^m psi; (-i dt)^m / m! enters the sum only.
+// Taylor terms are kept as s_m = dt h^m psi; the rest of (-i dt)^m / m! enters the sum only,
+// psi's increment (see tsbz_any.cu).
 // Measured, 65 536 orbitals: 10.50 (four star stencils, k_step_fused with its contractions
 // on tcgen05) -> 6.10 ms; 122 instructions a point and stage, projections of the current
 // included, 54% of the issue slots.  Without any transform it takes 4.8 ms, with the
@@ -515,7 +516,6 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
       const char* next = reinterpret_cast<const char*>(band - tid + FX_PTS) + 128 * tid;
       asm volatile("prefetch.global.L2 [%0];\n" ::"l"(next));
     }
-    um_st32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(t));
     if (FRESH) {
       fx_stage(t, x);
       um_fence_before();
@@ -652,28 +652,38 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
           t[z].y -= d[2 * z + 1];
         }
       }
+      if (m == 1) {
+#pragma unroll
+        for (int z = 0; z < N; ++z) t[z] = __fmul2_rn(make_float2(dt, dt), t[z]);
+      } else {
+        coef *= dt / (float)m;
+      }
       if (m < 4) fx_stage(t, x);   // the bra's A
-      // psi += (-i)^m dt^m / m! s_m
-      coef *= dt / (float)m;
+      // the increment of psi: (-i)^m coef s_m summed over m
       {
         float2 a[N];
-        um_ld32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(a));
-        const float sg = m == 1 || m == 4 ? coef : -coef;
-        if (m & 1) {
+        if (m == 1) {
 #pragma unroll
-          for (int z = 0; z < N; ++z) {
-            a[z].x = fmaf(sg, t[z].y, a[z].x);
-            a[z].y = fmaf(-sg, t[z].x, a[z].y);
-          }
+          for (int z = 0; z < N; ++z) a[z] = make_float2(t[z].y, -t[z].x);
         } else {
+          um_ld32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(a));
+          const float sg = m == 4 ? coef : -coef;
+          if (m == 3) {
 #pragma unroll
-          for (int z = 0; z < N; ++z) a[z] = __ffma2_rn(make_float2(sg, sg), t[z], a[z]);
+            for (int z = 0; z < N; ++z) {
+              a[z].x = fmaf(sg, t[z].y, a[z].x);
+              a[z].y = fmaf(-sg, t[z].x, a[z].y);
+            }
+          } else {
+#pragma unroll
+            for (int z = 0; z < N; ++z) a[z] = __ffma2_rn(make_float2(sg, sg), t[z], a[z]);
+          }
         }
         if (m < 4) {
           um_st32(um_addr(x.tbase, qd, FX_ACC + 32 * h), reinterpret_cast<float(&)[32]>(a));
         } else {
 #pragma unroll
-          for (int z = 0; z < N; ++z) t[z] = a[z];
+          for (int z = 0; z < N; ++z) t[z] = fft_add(band[z * NP], a[z]);
         }
       }
       um_fence_before();

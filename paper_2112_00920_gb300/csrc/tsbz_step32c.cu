@@ -16,7 +16,9 @@
 // shared memory.  The ket goes back the same way, its contraction along z on
 // tcgen05 under the line transforms.  Atoms whose x (y, z) tables are identical share
 // them: at most 8 classes per axis (a 2 x 2 x 2 diamond supercell has 8).
-// Taylor terms are s_m = h^m psi; (-i dt)^m / m! enters the sum only.
+// Taylor terms are s_m = dt h^m psi; the rest of (-i dt)^m / m! enters the sum only (see
+// tsbz_any.cu; psi stays in the sum here: adding it last spilled, 2.00 -> 2.08 ms, and
+// gained nothing on so many points).
 // Measured: 8 k-points x 128 bands of the 64-atom cell, stages and projections 3.31 ->
 // 2.00 ms per step (36% of issue slots, the rest barriers and the latency of the
 // remote rows).
@@ -691,9 +693,14 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
         t[j].y -= d[2 * j + 1];
       }
     }
-    coef *= dt / (float)m;
+    if (m == 1) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) t[j] = __fmul2_rn(make_float2(dt, dt), t[j]);
+    } else {
+      coef *= dt / (float)m;
+    }
     {
-      // psi += (-i)^m dt^m / m! s_m
+      // psi += (-i)^m coef s_m
       float2 a[16];
       um_ld32(um_addr(x.tbase, qd, Q_ACC + 32 * h), reinterpret_cast<float(&)[32]>(a));
       const float sg = m == 1 || m == 4 ? coef : -coef;

@@ -15,8 +15,8 @@
 //    per group: the running sums are turned by e^{i q L} there).  22 operations
 //    a point for the sums (bra) and 20 for the ket with four groups; the box
 //    and point forms took 111 and 84.
-//  - The Taylor terms are kept as s_m = h^m psi; (-i dt)^m / m! enters only the
-//    sum, which lives in shared memory.
+//  - The Taylor terms are kept as s_m = dt h^m psi; the rest of (-i dt)^m / m! enters only
+//    the sum, psi's increment, which lives in shared memory (see tsbz_any.cu).
 // One CTA per (unit, band), one thread per (x, y) column holding its N values
 // along z in registers; the line transforms along x and y go through one
 // shared buffer with the x index turned by y (no bank conflicts).  At 16^3 the
@@ -382,32 +382,39 @@ __global__ void __launch_bounds__(N* N, 1) k_step64(LaunchSet L, double2* __rest
     if (fresh_p) s64_project<N, 1>(sm, c, t);
     s64_weights<N>(sm, c, fresh_p ? nullptr : Pu);
   }
-#pragma unroll
-  for (int z = 0; z < N; ++z) sm.acc[z * NN + tid] = t[z];
   const double dt = S.dt * L.dt_scale;
   double coef = 1.0;
 #pragma unroll 1
   for (int m = 1; m <= 4; ++m) {
     s64_apply<N>(sm, c, veff, t, f);
-    coef *= dt / (double)m;
-    // psi += (-i)^m coef s_m
-    const double sx = (m & 1) ? 0.0 : (m == 2 ? -coef : coef), sy = (m & 1) ? (m == 1 ? coef : -coef) : 0.0;
+    // the increment of psi: (-i)^m coef s_m summed over m
+    if (m == 1) {
 #pragma unroll
-    for (int z = 0; z < N; ++z) {
-      double2 a = sm.acc[z * NN + tid];
-      if (m & 1) {
-        a.x = fma(sy, f[z].y, a.x);
-        a.y = fma(-sy, f[z].x, a.y);
-      } else {
-        a.x = fma(sx, f[z].x, a.x);
-        a.y = fma(sx, f[z].y, a.y);
+      for (int z = 0; z < N; ++z) {
+        t[z] = make_double2(dt * f[z].x, dt * f[z].y);
+        sm.acc[z * NN + tid] = make_double2(t[z].y, -t[z].x);
       }
-      if (m < 4) {
-        sm.acc[z * NN + tid] = a;
-        t[z] = f[z];
-      } else {
-        t[z] = a;
-        band[z * NN] = a;
+    } else {
+      coef *= dt / (double)m;
+      const double sx = m == 2 ? -coef : coef;
+#pragma unroll
+      for (int z = 0; z < N; ++z) {
+        double2 a = sm.acc[z * NN + tid];
+        if (m == 3) {
+          a.x = fma(-coef, f[z].y, a.x);
+          a.y = fma(coef, f[z].x, a.y);
+        } else {
+          a.x = fma(sx, f[z].x, a.x);
+          a.y = fma(sx, f[z].y, a.y);
+        }
+        if (m < 4) {
+          sm.acc[z * NN + tid] = a;
+          t[z] = f[z];
+        } else {
+          const double2 u0 = band[z * NN];
+          t[z] = make_double2(u0.x + a.x, u0.y + a.y);
+          band[z * NN] = t[z];
+        }
       }
     }
     if (m < 4 && c.use_proj) {
