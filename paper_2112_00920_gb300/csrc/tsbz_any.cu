@@ -32,6 +32,7 @@
 
 #include "tsbz_internal.h"
 #include "tsbz_launch.cuh"
+#include "tsbz_symbol.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -110,7 +111,8 @@ template <typename T> struct AnySmem {
   V* s;                  // z sums, ket coefficients per (group, column); line transforms (8^3)
   V *xk, *xl, *part;     // clusters: all k_z planes of an 8^3 band, the CTA's two, the ranks' monomial sums
   V *rs, *gt, *xf, *yf, *phi, *w, *mres, *k0, *kfin, *turn;
-  T *xd, *yd, *zw, *lam, *st;
+  T *xd, *yd, *zw, *lam3, *st;
+  Symbol<T>* lam;
   int *idx, *zb;
 };
 
@@ -145,7 +147,10 @@ __host__ __device__ inline size_t any_carve(const CellDev& c, unsigned char* bas
   m.xd = (T*)take(sizeof(T) * na * c.n1);
   m.yd = (T*)take(sizeof(T) * na * c.n2);
   m.zw = (T*)take(sizeof(T) * 3 * ng * c.n3);
-  m.lam = (T*)take(sizeof(T) * 3 * 8);
+  if (any_fft8(c)) {
+    m.lam = (Symbol<T>*)take(sizeof(Symbol<T>) * 3 * 8);
+    m.lam3 = (T*)take(sizeof(T) * 512);   // the symbol at (k_z, k_y, k_x)
+  }
   m.st = (T*)take(sizeof(T) * (6 * (TSBZ_MAX_ND + 1) + 1));
   m.idx = (int*)take(sizeof(int) * c.npts);
   m.zb = (int*)take(sizeof(int) * ANY_NA);
@@ -165,7 +170,6 @@ template <> struct AnyTab<double> {
   static __device__ const double* d1(const CellDev& c) { return c.d1; }
   static __device__ const double* pnorm(const CellDev& c) { return c.pnorm; }
   static __device__ const double* wkb(const CellDev& c) { return c.wkb; }
-  static __device__ const double* ksym(const CellDev& c) { return c.ksym; }
   static __device__ double dv(const CellDev& c) { return c.dv; }
 };
 template <> struct AnyTab<float> {
@@ -173,7 +177,6 @@ template <> struct AnyTab<float> {
   static __device__ const float* d1(const CellDev& c) { return c.d1f; }
   static __device__ const float* pnorm(const CellDev& c) { return c.pnormf; }
   static __device__ const float* wkb(const CellDev& c) { return c.wkbf; }
-  static __device__ const float* ksym(const CellDev& c) { return c.ksymf; }
   static __device__ float dv(const CellDev& c) { return c.dvf; }
 };
 
@@ -233,15 +236,13 @@ __device__ void any_tables(const AnySmem<T>& sm, const CellDev& c, const typenam
 
 // Stencil weights (or the symbol of 8^3 grids) of the step's q, and the points' coordinates.
 template <typename T, class F>
-__device__ void any_setup(const AnySmem<T>& sm, const CellDev& c, const double* q) {
+__device__ void any_setup(const AnySmem<T>& sm, const CellDev& c, const LaunchSet& L, int u, const double* q) {
   const int tid = threadIdx.x;
   if (F::eight) {
-    if (tid < 24) {
-      const int ax = tid >> 3, k = tid & 7;
-      const T* s = AnyTab<T>::ksym(c) + 2 * ax * 8;
-      const T qa = (T)q[ax];
-      sm.lam[tid] = rfm(qa, s[8 + k], rfm((T)0.5 * qa, qa, s[k])) * (T)(1.0 / 512.0);
-    }
+    if (tid < 24) sm.lam[tid] = symbol_unit<T>(L, u)[tid];
+    __syncthreads();
+    const Symbol<T> xy = symbol_add(sm.lam[tid & 7], sm.lam[8 + ((tid >> 3) & 7)]);
+    for (int p = tid; p < 512; p += F::threads) sm.lam3[p] = symbol_value(symbol_add(xy, sm.lam[16 + (p >> 6)]));
   } else {
     constexpr int M = TSBZ_MAX_ND + 1;
     if (tid < 3 * M) {
@@ -472,7 +473,7 @@ __device__ void any_kinetic8(const AnySmem<T>& sm, const typename AnyC<T>::V* t,
   for (int j = 0; j < 8; ++j) v[j] = x2[cy + j * 9];
   any_dft8<false>(v, lo, hi);
   {
-    const T s = sm.lam[l0] + sm.lam[16 + l1], e0 = s + sm.lam[8 + p], e1 = s + sm.lam[12 + p];
+    const T *e = sm.lam3 + l1 * 64 + p * 8 + l0, e0 = e[0], e1 = e[32];
     x1[cy + p * 9] = vmk<V>(e0 * lo.x, e0 * lo.y);
     x1[cy + (p + 4) * 9] = vmk<V>(e1 * hi.x, e1 * hi.y);
   }
@@ -509,7 +510,7 @@ template <typename T> __device__ void any_planes8(const AnySmem<T>& sm, const ty
   for (int k = 0; k < 8; ++k) v[k] = x2[cy + k * 9];
   any_dft8<false>(v, lo, hi);
   {
-    const T s = sm.lam[l] + sm.lam[16 + rank + 4 * j], e0 = s + sm.lam[8 + p], e1 = s + sm.lam[12 + p];
+    const T *e = sm.lam3 + (rank + 4 * j) * 64 + p * 8 + l, e0 = e[0], e1 = e[32];
     x1[cy + p * 9] = vmk<V>(e0 * lo.x, e0 * lo.y);
     x1[cy + (p + 4) * 9] = vmk<V>(e1 * hi.x, e1 * hi.y);
   }
@@ -703,8 +704,8 @@ __device__ __forceinline__ void any_step(const LaunchSet& L, typename AnyC<T>::V
   const T* veff = reinterpret_cast<const T*>(S.veff);
   V* band = psi + U.psi_off + (long long)b * c.npts;
   V* Pu = P + U.p_off + (long long)b * c.n_proj;
-  for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = sm.acc[p] = band[p];
-  any_setup<T, F>(sm, c, L.q_half + 3 * u);
+  for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = band[p];
+  any_setup<T, F>(sm, c, L, u, L.q_half + 3 * u);
   if (c.use_proj) any_tables<T, F>(sm, c, (const V*)L.ph_half + (long long)u * L.ph_stride);
   if constexpr (F::ctas > 1) cg::this_cluster().sync(); else __syncthreads();
   if (F::ctas == 1 && c.use_proj) {
@@ -809,7 +810,7 @@ __global__ void __launch_bounds__(F::threads) k_pa_any(LaunchSet L, const typena
   const UnitDev U = L.units[u];
   const V* band = src + U.psi_off + (long long)b * c.npts;
   for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = band[p];
-  any_setup<T, F>(sm, c, L.q_obs + 3 * u);
+  any_setup<T, F>(sm, c, L, u, L.q_obs + 3 * u);
   any_tables<T, F>(sm, c, (const V*)L.ph_obs + (long long)u * L.ph_stride);
   any_current<T, F>(sm, c, sm.a, sm.b, Pa + U.pa_off + 4LL * b * c.n_proj, nullptr);
 }
@@ -829,7 +830,7 @@ __device__ __forceinline__ void any_filter(const LaunchSet& L, const double2* in
   const double* veff = reinterpret_cast<const double*>(L.subs[U.sub].veff);
   const long long off = U.psi_off + (long long)b * c.npts;
   for (int p = threadIdx.x; p < c.npts; p += F::threads) sm.a[p] = in[off + p];
-  any_setup<double, F>(sm, c, L.q_half + 3 * u);
+  any_setup<double, F>(sm, c, L, u, L.q_half + 3 * u);
   if (c.use_proj)
     any_tables<double, F>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride);
   if constexpr (F::ctas > 1) cg::this_cluster().sync(); else __syncthreads();

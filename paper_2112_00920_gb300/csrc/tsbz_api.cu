@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <complex>
 #include <cstring>
 #include <new>
 #include <string>
@@ -23,8 +24,10 @@
 
 #include "tsbz.h"
 #include "tsbz_host.h"
+#include "tsbz_fft.cuh"
 #include "tsbz_internal.h"
 #include "tsbz_bulk.cuh"
+#include "tsbz_symbol.cuh"
 
 namespace {
 
@@ -101,6 +104,8 @@ struct tsbz_ctx {
   double* q_obs = nullptr;
   double* kcart = nullptr;
   void* qt_half = nullptr;
+  void* symbols = nullptr;   // kinetic symbol of every unit (LaunchSet::symbols)
+  long long symbol_stride = 0;
   UnitDev* d_units = nullptr;
   SubDev* d_subs = nullptr;
   CellDev* d_cells = nullptr;
@@ -252,6 +257,8 @@ LaunchSet make_set(tsbz_ctx* ctx, HostCell& hc) {
   L.ph_next = ctx->ph_next;
   L.ph_stride = ctx->ph_stride;
   L.qt_half = ctx->qt_half;
+  L.symbols = ctx->symbols;
+  L.symbol_stride = ctx->symbol_stride;
   L.variant = hc.variant;
   L.dt_scale = ctx->dt_scale;
   L.images = hc.images;
@@ -375,6 +382,11 @@ int layout(tsbz_ctx* ctx) {
   if ((rc = dalloc_t(ctx, 3 * ctx->n_units, &ctx->q_obs))) return rc;
   if ((rc = dalloc_t(ctx, 3 * ctx->n_units, &ctx->kcart))) return rc;
   if ((rc = dalloc(ctx, 4 * ctx->n_units * (ctx->precision == TSBZ_FP64 ? 8 : 4), &ctx->qt_half))) return rc;
+  for (auto& hc : ctx->cells)
+    if (!hc.unit_ids.empty() && hc.dev.kscale != 0.0)
+      ctx->symbol_stride = std::max<long long>(ctx->symbol_stride, 3LL * hc.dev.nmax);
+  const size_t sym = ctx->precision == TSBZ_FP64 ? sizeof(Symbol<double>) : sizeof(Symbol<float>);
+  if ((rc = dalloc(ctx, sym * ctx->symbol_stride * ctx->n_units, &ctx->symbols))) return rc;
   if ((rc = dalloc_t(ctx, ctx->n_units, &ctx->d_units))) return rc;
   if ((rc = dalloc_t(ctx, ctx->subs.size(), &ctx->d_subs))) return rc;
   if ((rc = dalloc_t(ctx, ctx->cells.size(), &ctx->d_cells))) return rc;
@@ -1023,6 +1035,63 @@ __global__ void k_selftest_wait(int polls, int deliver, int* status) {
   if (!__syncthreads_and(ok) && threadIdx.x == 0) atomicOr(status, BK_STATUS_TIMEOUT);
 }
 
+// Twiddle exp(2 pi i m / 32), m = 0..15, as fft_butterfly applies it with its constants in T.
+template <typename T> std::complex<double> line_twiddle(int m, int sign) {
+  if (m == 0) return 1.0;
+  if (m == 8) return {0.0, (double)sign};
+  const double c = fft_cos32(m), s = sign * fft_sin32(m);
+  const bool by_c = m <= 4 || m >= 12;
+  const double r = (T)(by_c ? s / c : c / s), f = (T)(by_c ? c : s);
+  return by_c ? std::complex<double>(f, f * r) : std::complex<double>(f * r, f);
+}
+
+// fft_line (and any_dft8) without the rounding of the data; 32 points as q_line forms them.
+template <typename T> std::vector<std::complex<double>> line_transform(const std::vector<std::complex<double>>& x, int sign) {
+  const int n = (int)x.size(), h = n / 2;
+  if (n == 1) return x;
+  std::vector<std::complex<double>> a(h), b(h), out(n);
+  if (n == 32) {
+    for (int j = 0; j < h; ++j) {
+      a[j] = x[j] + x[j + h];
+      b[j] = (x[j] - x[j + h]) * std::complex<double>((T)fft_cos32(j), (T)(sign * fft_sin32(j)));
+    }
+    a = line_transform<T>(a, sign);
+    b = line_transform<T>(b, sign);
+    for (int j = 0; j < h; ++j) {
+      out[2 * j] = a[j];
+      out[2 * j + 1] = b[j];
+    }
+    return out;
+  }
+  for (int j = 0; j < h; ++j) {
+    a[j] = x[2 * j];
+    b[j] = x[2 * j + 1];
+  }
+  a = line_transform<T>(a, sign);
+  b = line_transform<T>(b, sign);
+  for (int j = 0; j < h; ++j) {
+    const std::complex<double> p = line_twiddle<T>(j * (32 / n), sign) * b[j];
+    out[j] = a[j] + p;
+    out[j + h] = a[j] - p;
+  }
+  return out;
+}
+
+// What a plane wave of each frequency comes back as from the line's transforms forward and back, less 1.
+template <typename T> std::vector<double> line_gain(int n) {
+  std::vector<double> g(n, 0.0);
+  if (n != 8 && n != 16 && n != 32) return g;
+  for (int k = 0; k < n; ++k) {
+    std::vector<std::complex<double>> w(n);
+    for (int j = 0; j < n; ++j) w[j] = std::polar(1.0, 2.0 * 3.14159265358979323846 * ((j * k) % n) / n);
+    const std::vector<std::complex<double>> back = line_transform<T>(line_transform<T>(w, -1), 1);
+    double sum = 0.0;
+    for (int j = 0; j < n; ++j) sum += std::real(std::conj(w[j]) * (back[j] / (double)n - w[j]));
+    g[k] = sum / n;
+  }
+  return g;
+}
+
 // A captured step holds the kernels of the variants it was captured with.
 void drop_step_graph(tsbz_ctx* ctx) {
   if (ctx->step_graph) {
@@ -1314,7 +1383,25 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
         ks[(2 * ax + 1) * (size_t)c.nmax + k] = grd;
       }
     up.add(ks, &c.ksym);
-    up.add(to_f(ks), &c.ksymf);
+    std::vector<double> kg(3 * (size_t)c.nmax, 0.0);
+    for (int ax = 0; ax < 3; ++ax) {
+      const std::vector<double> g = ctx->precision == TSBZ_FP64 ? line_gain<double>(nn[ax]) : line_gain<float>(nn[ax]);
+      std::copy(g.begin(), g.end(), kg.begin() + (size_t)ax * c.nmax);
+    }
+    up.add(kg, &c.kgain);
+    // cells whose step may take a Fourier form: 8^3, 16^3, and in single precision 32^3 (transforms along two axes)
+    c.kscale = c.n1 == c.n2 && c.n2 == c.n3 &&
+                       (c.n1 == 8 || c.n1 == 16 || (c.n1 == 32 && ctx->precision == TSBZ_FP32))
+                   ? 1.0 / (c.n1 == 32 ? c.n1 * c.n1 : c.npts)
+                   : 0.0;
+    double top = 8.0;   // (hartree, of the terms with q)
+    for (int ax = 0; ax < 3; ++ax) {
+      double m = 0.0;
+      for (int k = 0; k < nn[ax]; ++k) m = std::max(m, std::fabs(ks[(2 * ax) * (size_t)c.nmax + k]));
+      top += m;
+    }
+    c.kquant = std::ldexp(1.0, std::ilogb(top) + 1 - (ctx->precision == TSBZ_FP64 ? 52 : 23));
+    c.kquant_inv = 1.0 / c.kquant;
   }
   c.poisson = nullptr;
   if (c.n1 * c.n3 <= TSBZ_HXC_MAX_PLANE) {

@@ -83,7 +83,11 @@ struct CellDev {
   // kinetic symbol per axis: [3][2][nmax], row 0 the eigenvalues of -1/2 lap_FD on
   // exp(2 pi i k j / n), row 1 those of -i grad_FD (times q in h)
   const double* ksym;
-  const float* ksymf;
+  // [3][nmax]: what the line transforms of 8, 16 and 32 points of the context's precision do to
+  // a frequency, forward and back, less 1 (0 for other lengths; see tsbz_symbol.cuh)
+  const double* kgain;
+  double kscale;        // normalisation of the transforms that a step takes (a power of two; 0: no Fourier form)
+  double kquant, kquant_inv;   // a power of two whose multiples sum over the axes without rounding, and its inverse
   // 4 pi / (G^2 n_pts) (0 at G = 0), [n2 / 2 + 1][n3][n1]; null when an x-z plane is
   // too large for the v_Hxc kernels that work plane by plane
   const double* poisson;
@@ -169,6 +173,8 @@ struct LaunchSet {
   void* ph_next;          // q = k + A(t_{n+1} + dt/2): tables of the next step (null if unused)
   long long ph_stride;    // complex elements per unit
   void* qt_half;          // [unit][4] in T: q_x, q_y, q_z, |q|^2 / 2 at t_n + dt/2
+  void* symbols;          // [unit][symbol_stride] kinetic symbol per axis at t_n + dt/2 (Symbol<T>, tsbz_symbol.cuh)
+  long long symbol_stride;
   int variant;            // kernel variant of this cell (0 = default; chosen by the autotuner)
   double dt_scale;        // the stage kernels advance by dt * dt_scale (1, or 1/2 in the ETRS half steps)
   void* images;           // operand images of the 32^3 whole-step kernel (null if the cell has none)

@@ -22,6 +22,7 @@
 #include "tsbz_fft.cuh"
 #include "tsbz_internal.h"
 #include "tsbz_launch.cuh"
+#include "tsbz_symbol.cuh"
 
 template <typename T> struct Cplx;
 template <> struct Cplx<double> { using type = double2; };
@@ -132,6 +133,10 @@ __global__ void k_field(LaunchSet L, int mode, int factored) {
     reinterpret_cast<T*>(L.qt_half)[4 * u + 3] = (T)(0.5 * (qh[0] * qh[0] + qh[1] * qh[1] + qh[2] * qh[2]));
   // constant field: q and every phase table equal those of the previous step
   if (mode == TSBZ_FIELD_STEP_KEEP) return;
+  if (c.kscale != 0.0) {
+    Symbol<T>* sy = (Symbol<T>*)L.symbols + (long long)u * L.symbol_stride;
+    for (int i = threadIdx.x; i < 3 * c.nmax; i += blockDim.x) sy[i] = symbol_axis<T>(c, qh, i / c.nmax, i % c.nmax);
+  }
   V* out[3] = {(V*)L.ph_half + (long long)u * L.ph_stride, (V*)L.ph_obs + (long long)u * L.ph_stride, nullptr};
   double qn[3] = {0.0, 0.0, 0.0};
   if (L.ph_next != nullptr && mode == TSBZ_FIELD_STEP) {

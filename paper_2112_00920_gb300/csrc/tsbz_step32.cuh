@@ -5,7 +5,7 @@
 // What bounds it: instruction issue at 16 warps per SM (128 registers, two CTAs);
 // HBM sees psi once.  The star stencil needs 16 in-plane loads a point and
 // stage; the periodic grid's discrete Fourier basis diagonalises it (real symbol,
-// one number per axis, CellDev::ksymf), so six 16-point line transforms in
+// one number per axis, CellDev::ksym), so six 16-point line transforms in
 // registers replace it with 8 shared accesses and about 50 instructions a point.
 // One thread per (x, y) column.  The column of t stays in registers from one stage
 // to the next; the Taylor sum, v_eff and the tensor-core operands live in tensor
@@ -39,6 +39,7 @@
 #pragma once
 #include "tsbz_fft.cuh"
 #include "tsbz_fused.cuh"
+#include "tsbz_symbol.cuh"
 #include "tsbz_umma.cuh"
 
 #define FX_N 16
@@ -71,7 +72,8 @@ struct FxSmem {
   float psc[4 * FX_S];               // dV pn: projection from a monomial sum
   float wsc[4 * FX_S];               // pn E times that: W from a monomial sum
   float2 mres[FX_S * 10];            // monomial sums
-  float lam[3 * FX_N];               // kinetic symbol per axis and frequency
+  Symbol<float> lam[3 * FX_N];       // kinetic symbol per axis and frequency
+  float4 lam3[4 * FX_NP];            // and of the thread's line (k_x, k_z) at k_y = 4 i .. 4 i + 3
   int atom[FX_S];                    // atom of a slot (-1: empty)
   unsigned long long mbar;           // completion of the MMAs (one phase per commit)
   uint32_t tslot;
@@ -473,13 +475,7 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
   float2 w = fx_load_w(c, P + U.p_off + (long long)b0 * c.n_proj);
   fx_tables(sm, c, (const float2*)L.ph_half + off);
   fx_scales(sm, c);
-  if (tid < 3 * N) {
-    // kinetic symbol, the transforms' 1/N^3 folded in
-    const int ax = tid / N, k = tid - ax * N;
-    const float q = reinterpret_cast<const float*>(L.qt_half)[4 * u + ax];
-    const float* s = c.ksymf + 2 * ax * N;
-    sm.lam[tid] = fmaf(q, s[N + k], fmaf(0.5f * q, q, s[k])) * (1.f / (N * N * N));
-  }
+  if (tid < 3 * N) sm.lam[tid] = symbol_unit<float>(L, u)[tid];
   FxState x = fx_open(sm);   // (and the barrier behind the tables)
   {
     float v[N];
@@ -487,6 +483,16 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
 #pragma unroll
     for (int z = 0; z < N; ++z) v[z] = veff[z * NP];
     um_st16(um_addr(x.tbase, qd, FX_VEFF + 32 * h), reinterpret_cast<uint32_t(&)[16]>(v));
+  }
+  {
+    const Symbol<float> xz = symbol_add(sm.lam[lo], sm.lam[2 * N + hi]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = symbol_value(symbol_add(xz, sm.lam[N + 4 * i + k]));
+      sm.lam3[i * NP + tid] = make_float4(v[0], v[1], v[2], v[3]);
+    }
   }
   fx_build_ket(sm);
   fx_build_bra<1>(sm, sm.bbra);
@@ -565,11 +571,13 @@ __global__ void __launch_bounds__(FX_NP, 2) k_step_fft(LaunchSet L, float2* __re
       for (int y = 0; y < N; ++y) f[y] = linp[y * FX_ROW];
       fft_line<N, -1>(f);
       {
-        const float l0 = sm.lam[lo] + sm.lam[2 * N + hi];
 #pragma unroll
-        for (int y = 0; y < N; ++y) {
-          const float l = l0 + sm.lam[N + y];
-          f[y] = __fmul2_rn(make_float2(l, l), f[y]);
+        for (int i = 0; i < 4; ++i) {
+          const float4 l = sm.lam3[i * NP + tid];
+          f[4 * i] = __fmul2_rn(make_float2(l.x, l.x), f[4 * i]);
+          f[4 * i + 1] = __fmul2_rn(make_float2(l.y, l.y), f[4 * i + 1]);
+          f[4 * i + 2] = __fmul2_rn(make_float2(l.z, l.z), f[4 * i + 2]);
+          f[4 * i + 3] = __fmul2_rn(make_float2(l.w, l.w), f[4 * i + 3]);
         }
       }
       fft_line<N, 1>(f);

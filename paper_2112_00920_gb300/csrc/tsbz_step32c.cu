@@ -35,6 +35,7 @@
 #include "tsbz_fft.cuh"
 #include "tsbz_internal.h"
 #include "tsbz_launch.cuh"
+#include "tsbz_symbol.cuh"
 #include "tsbz_umma.cuh"
 
 namespace cg = cooperative_groups;
@@ -64,8 +65,8 @@ struct QSmem {
   float4 yt[QG * QR];              // y factors per class on the CTA's rows
   float2 tab[QA * QR * 3];         // ket tables per (slot, row); second-order partial sums
   float2 part[QA * 4];             // this CTA's partial monomial sums
-  float lx[QN], lz[QN];            // kinetic symbol along x and z
-  float wl[4], wg[4];              // stencil along y, transforms' 1/N^2 folded in
+  Symbol<float> lx[QN], lz[QN];    // kinetic symbol along x and z
+  float wl[4], wg[4], wd;          // stencil along y and its diagonal, transforms' 1/N^2 folded in
   unsigned long long ymask[QR];    // slots whose y factor is non-zero on the row
   int atom[QA];                    // atom of a slot (-1: none)
   unsigned char xc[QA], yc[QA], zg[QA];
@@ -498,14 +499,12 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
   constexpr float inv = 1.f / (QN * QN);
   if (tid < 64) {
     const int ax = tid < 32 ? 0 : 2, k = tid & 31;
-    const float q = qt[ax];
-    const float* s = c.ksymf + 2 * ax * QN;
-    float l = fmaf(q, s[QN + k], fmaf(0.5f * q, q, s[k])) * inv;
-    if (ax == 0) l += fmaf(0.5f * qt[1], qt[1], c.hlapf[1][0]) * inv;   // the y axis' diagonal
-    (ax == 0 ? sm.lx : sm.lz)[k] = l;
+    (ax == 0 ? sm.lx : sm.lz)[k] = symbol_unit<float>(L, u)[ax * QN + k];
   } else if (tid < 68) {
     sm.wl[tid - 64] = c.hlapf[1][tid - 63] * inv;
     sm.wg[tid - 64] = qt[1] * c.gradwf[1][tid - 63] * inv;
+  } else if (tid == 68) {
+    sm.wd = fmaf(0.5f * qt[1], qt[1], c.hlapf[1][0]) * inv;
   }
   q_cell(sm, c);
   q_tables(sm, c, ph, r0);
@@ -643,7 +642,9 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
       wl[e] = make_float2(sm.wl[e], sm.wl[e]);
       wg[e] = make_float2(sm.wg[e], sm.wg[e]);
     }
-    const float lx = sm.lx[lane];
+    // (the diagonal stays apart: added to the symbol it would round that of long waves at its own size)
+    const Symbol<float> lx = sm.lx[lane];
+    const float2 wd = make_float2(sm.wd, sm.wd);
 #pragma unroll 2
     for (int i = 0; i < 4; ++i) {
       const int kz = warp + 8 * i, o = kz * QP + lane;
@@ -654,10 +655,10 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QT, 2)
         w[4 + r] = sm.b1[r * QN * QP + o];
         w[8 + r] = up[r * QN * QP + o];
       }
-      const float l = lx + sm.lz[kz];
+      const float l = symbol_value(symbol_add(lx, sm.lz[kz]));
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        float2 k = __fmul2_rn(make_float2(l, l), w[4 + r]);
+        float2 k = __ffma2_rn(wd, w[4 + r], __fmul2_rn(make_float2(l, l), w[4 + r]));
         float2 g = make_float2(0.f, 0.f);
 #pragma unroll
         for (int e = 1; e <= 4; ++e) {

@@ -30,6 +30,7 @@
 #include "tsbz_fft.cuh"
 #include "tsbz_internal.h"
 #include "tsbz_launch.cuh"
+#include "tsbz_symbol.cuh"
 
 namespace {
 
@@ -51,7 +52,8 @@ template <int N> struct S64Smem {
   double2 gt[S64_NA * 3 * N];               // ket column tables
   double2 w[4 * S64_NA];                    // conj(k0) pn E P
   double2 mres[S64_NA * 10];                // monomial sums
-  double lam[3][N];                         // kinetic symbol, 1/N^3 folded in
+  Symbol<double> lam[3][N];                 // kinetic symbol per axis, 1/N^3 folded in
+  double lam3[N][NN];                       // and of line (k_x, k_z) at k_y
 };
 
 __device__ __forceinline__ double2 z_mul(double2 a, double2 b) {
@@ -108,13 +110,13 @@ __device__ void s64_tables(S64Smem<N>& sm, const CellDev& c, const double2* ph, 
   }
 }
 
-// Kinetic symbol per axis and frequency at the step's q.
-template <int N> __device__ void s64_symbol(S64Smem<N>& sm, const CellDev& c, const double* q) {
-  for (int i = threadIdx.x; i < 3 * N; i += blockDim.x) {
-    const int ax = i / N, k = i - ax * N;
-    const double* s = c.ksym + 2 * ax * c.nmax;
-    sm.lam[ax][k] = (s[k] + q[ax] * s[c.nmax + k] + 0.5 * q[ax] * q[ax]) / (double)(N * N * N);
-  }
+// Kinetic symbol of the unit (barrier inside; lam3 is read by the thread that wrote it).
+template <int N> __device__ void s64_symbol(S64Smem<N>& sm, const LaunchSet& L, int u) {
+  if (threadIdx.x < 3 * N) sm.lam[threadIdx.x / N][threadIdx.x % N] = symbol_unit<double>(L, u)[threadIdx.x];
+  __syncthreads();
+  const Symbol<double> xz = symbol_add(sm.lam[0][threadIdx.x % N], sm.lam[2][threadIdx.x / N]);
+#pragma unroll 4
+  for (int y = 0; y < N; ++y) sm.lam3[y][threadIdx.x] = symbol_value(symbol_add(xz, sm.lam[1][y]));
 }
 
 // Monomial sums M_a(i, j, k) = sum_r F_x F_y F_z d_x^i d_y^j d_z^k t(r), i + j + k <= D,
@@ -260,10 +262,9 @@ __device__ void s64_apply(S64Smem<N>& sm, const CellDev& c, const double* __rest
 #pragma unroll
     for (int y = 0; y < N; ++y) f[y] = pl[y * N + (lo ^ y)];
     fft_line<N, -1>(f);
-    const double l0 = sm.lam[0][lo] + sm.lam[2][hi];
 #pragma unroll
     for (int y = 0; y < N; ++y) {
-      const double l = l0 + sm.lam[1][y];
+      const double l = sm.lam3[y][tid];
       f[y].x *= l;
       f[y].y *= l;
     }
@@ -375,7 +376,7 @@ __global__ void __launch_bounds__(N* N, 1) k_step64(LaunchSet L, double2* __rest
   double2 t[N], f[N];
 #pragma unroll
   for (int z = 0; z < N; ++z) t[z] = band[z * NN];
-  s64_symbol<N>(sm, c, L.q_half + 3 * u);
+  s64_symbol<N>(sm, L, u);
   if (c.use_proj) s64_tables<N>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
   __syncthreads();
   if (c.use_proj) {
@@ -472,7 +473,7 @@ __global__ void __launch_bounds__(N* N, 1) k_filter64(LaunchSet L, const double2
   double2 t[N], f[N];
 #pragma unroll
   for (int z = 0; z < N; ++z) t[z] = in[off + z * NN];
-  s64_symbol<N>(sm, c, L.q_half + 3 * u);
+  s64_symbol<N>(sm, L, u);
   if (c.use_proj) s64_tables<N>(sm, c, (const double2*)L.ph_half + (long long)u * L.ph_stride, L.q_half + 3 * u);
   __syncthreads();
 #pragma unroll 1
