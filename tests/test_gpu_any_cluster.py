@@ -76,3 +76,21 @@ def test_ground_state_cluster_equals_single(n):
         rho.append(P.density(sids[-1]))
         P.close()
     assert np.max(np.abs(rho[0] - rho[1])) <= 1e-8 * np.max(rho[1])
+
+
+@pytest.mark.parametrize("case", [0, 3, 4])
+@pytest.mark.parametrize("field", [PULSE, W.Kick(k0=0.01)])
+def test_cluster_restart_bitwise(case, field):
+    cell, mp, nd = _cell(case)
+    s = random_subsim(cell, mp, (0.25, 0.5, 0.125), 0.04, 4, field, seed=280 + case)
+    P1, _ = gpu_run(cell, [s], precision="fp64", fd_nd=nd, steps=2)
+    mid, step = P1.get_state(0)
+    P1.propagate(2)
+    P2, _ = gpu_run(cell, [s], precision="fp64", fd_nd=nd, steps=0)
+    P2.load_state(0, mid, step)
+    P2.propagate(2)
+    assert np.array_equal(P1.get_state(0)[0], P2.get_state(0)[0])
+    assert np.array_equal(P1.density(0), P2.density(0))
+    assert np.array_equal(P1.current(0)[0][3:], P2.current(0)[0][3:])
+    P1.close()
+    P2.close()
