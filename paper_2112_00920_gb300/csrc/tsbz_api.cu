@@ -914,14 +914,14 @@ int sync_and_check(tsbz_ctx* ctx) {
 }
 
 // Kernel variants a cell can run (the autotuner's search space):
-//   FP32 on 16^3 / 8^3 cells: 0 fused tensor-core / bulk-staged stage, 1 z-march
-//     stage with CUDA-core projections;
+//   FP32 on 16^3 / 8^3 cells: see sep_variants (8^3 cells from 8 orbitals on take the
+//     whole step in one launch as variant 0);
 //   point-parallel path (FP64, and FP32 on shapes without a z-march kernel):
 //     bands per staged projection chunk 8 (0), 4 (1), 16 (2, when its shared
 //     memory fits); 16^3 grids in FP64 and small grids in either take the whole
 //     step in one launch as variant 0;
-//   FP32 on grids with 32-point rows (slab_supported): 0 slab z-march stage,
-//     then the point-parallel stage with 4 (1), 16 (2, when it fits) or 8 (3)
+//   FP32 on grids with 32-point rows (slab_supported): 0 slab z-march stage (32^3 with at
+//     most 8 classes of atoms per axis: the whole step), then the point-parallel stage with 4 (1), 16 (2, when it fits) or 8 (3)
 //     bands per chunk;
 //   FP32_TC on 16^3 grids: stage with the band of t bulk-staged in shared
 //     memory and V, psi read per plane (0) or bulk-staged too (1), z-march
@@ -1077,19 +1077,25 @@ template <typename T> std::vector<std::complex<double>> line_transform(const std
   return out;
 }
 
-// What a plane wave of each frequency comes back as from the line's transforms forward and back, less 1.
-template <typename T> std::vector<double> line_gain(int n) {
-  std::vector<double> g(n, 0.0);
-  if (n != 8 && n != 16 && n != 32) return g;
-  for (int k = 0; k < n; ++k) {
-    std::vector<std::complex<double>> w(n);
-    for (int j = 0; j < n; ++j) w[j] = std::polar(1.0, 2.0 * 3.14159265358979323846 * ((j * k) % n) / n);
-    const std::vector<std::complex<double>> back = line_transform<T>(line_transform<T>(w, -1), 1);
-    double sum = 0.0;
-    for (int j = 0; j < n; ++j) sum += std::real(std::conj(w[j]) * (back[j] / (double)n - w[j]));
-    g[k] = sum / n;
-  }
-  return g;
+// What a plane wave of each frequency comes back as from the line's transforms forward and back,
+// less 1 (formed once: 0.1 ms).
+template <typename T, int N> const std::vector<double>& line_gain() {
+  static const std::vector<double> gain = [] {
+    std::vector<double> g(N);
+    for (int k = 0; k < N; ++k) {
+      std::vector<std::complex<double>> w(N);
+      for (int j = 0; j < N; ++j) w[j] = std::polar(1.0, 2.0 * 3.14159265358979323846 * ((j * k) % N) / N);
+      const std::vector<std::complex<double>> back = line_transform<T>(line_transform<T>(w, -1), 1);
+      double sum = 0.0;
+      for (int j = 0; j < N; ++j) sum += std::real(std::conj(w[j]) * (back[j] / (double)N - w[j]));
+      g[k] = sum / N;
+    }
+    return g;
+  }();
+  return gain;
+}
+template <typename T> const std::vector<double>& line_gain(int n) {   // n = 8, 16 or 32
+  return n == 8 ? line_gain<T, 8>() : n == 16 ? line_gain<T, 16>() : line_gain<T, 32>();
 }
 
 // A captured step holds the kernels of the variants it was captured with.
@@ -1383,17 +1389,17 @@ int tsbz_init_cell(tsbz_ctx* ctx, const tsbz_cell_desc* d, int* cell_id) {
         ks[(2 * ax + 1) * (size_t)c.nmax + k] = grd;
       }
     up.add(ks, &c.ksym);
-    std::vector<double> kg(3 * (size_t)c.nmax, 0.0);
-    for (int ax = 0; ax < 3; ++ax) {
-      const std::vector<double> g = ctx->precision == TSBZ_FP64 ? line_gain<double>(nn[ax]) : line_gain<float>(nn[ax]);
-      std::copy(g.begin(), g.end(), kg.begin() + (size_t)ax * c.nmax);
-    }
-    up.add(kg, &c.kgain);
     // cells whose step may take a Fourier form: 8^3, 16^3, and in single precision 32^3 (transforms along two axes)
     c.kscale = c.n1 == c.n2 && c.n2 == c.n3 &&
                        (c.n1 == 8 || c.n1 == 16 || (c.n1 == 32 && ctx->precision == TSBZ_FP32))
                    ? 1.0 / (c.n1 == 32 ? c.n1 * c.n1 : c.npts)
                    : 0.0;
+    std::vector<double> kg(3 * (size_t)c.nmax, 0.0);
+    if (c.kscale != 0.0) {
+      const std::vector<double>& g = ctx->precision == TSBZ_FP64 ? line_gain<double>(c.n1) : line_gain<float>(c.n1);
+      for (int ax = 0; ax < 3; ++ax) std::copy(g.begin(), g.end(), kg.begin() + (size_t)ax * c.nmax);
+    }
+    up.add(kg, &c.kgain);
     double top = 8.0;   // (hartree, of the terms with q)
     for (int ax = 0; ax < 3; ++ax) {
       double m = 0.0;

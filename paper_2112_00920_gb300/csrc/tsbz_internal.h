@@ -83,8 +83,8 @@ struct CellDev {
   // kinetic symbol per axis: [3][2][nmax], row 0 the eigenvalues of -1/2 lap_FD on
   // exp(2 pi i k j / n), row 1 those of -i grad_FD (times q in h)
   const double* ksym;
-  // [3][nmax]: what the line transforms of 8, 16 and 32 points of the context's precision do to
-  // a frequency, forward and back, less 1 (0 for other lengths; see tsbz_symbol.cuh)
+  // [3][nmax]: what the line transforms of the context's precision do to a frequency, forward
+  // and back, less 1 (0 where the step takes no Fourier form; see tsbz_symbol.cuh)
   const double* kgain;
   double kscale;        // normalisation of the transforms that a step takes (a power of two; 0: no Fourier form)
   double kquant, kquant_inv;   // a power of two whose multiples sum over the axes without rounding, and its inverse
