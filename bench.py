@@ -323,6 +323,8 @@ STAGE_KERNEL = {
 STEP_KERNEL = ("k_step_fft (the four Taylor stages of a time step in one launch: kinetic operator by register "
                "FFT lines, projector z contractions on tcgen05 with TMEM operands and accumulators, Taylor sum in "
                "TMEM); variant 3 is k_step_fused (star stencil, mma.sync)")
+# FP64 operations of k_step64 per grid point, orbital and Taylor stage (profiles/k_step64_mp2.md)
+STEP64_OPS_PER_POINT_STAGE = 132
 # FP32 arithmetic of the local part of h, the Taylor scaling and the psi sum,
 # per grid point, orbital and Taylor stage (complex values), as the star stencil of
 # the method counts them (the kernel gets the same operator from fewer): Laplacian and
@@ -334,8 +336,8 @@ FP32_LANES_PER_SM = 128
 # + dram__bytes_write.sum) on the reduced workload (8 of the 64 subgrids, 8192
 # orbitals), scaled by the orbital count to the full workload.  Valid only for
 # the source it was taken on: the SHA-1 of the kernel header is checked at run time.
-STEP_TRAFFIC = {"file": "tsbz_step32.cuh", "sha1": "43982e016be64ba9647dcc42a9e3c724b1d1b108",
-                "bytes_per_launch_full": 8 * (272.373760e6 + 219.642368e6),
+STEP_TRAFFIC = {"file": "tsbz_step32.cuh", "sha1": "0d0e49945a14465a9c29991cfde98698931c27ae",
+                "bytes_per_launch_full": 8 * (272.730112e6 + 218.921984e6),
                 "profile": "profiles/k_step_fft_twostep8.md"}
 # DRAM bytes of the per-stage stencil kernel k_stage_zb<false> from an ncu capture of the
 # reduced dense tensor-core workload (8 of the 64 subgrids): stages 1 and 2 moved 774.8 and
@@ -633,7 +635,8 @@ def main():
         alu = alu_peaks(local_rank) if not args.profile_run else None
         roof = step_roofline(fam["stage"] / args.steps, n_orb, cell, elem, peaks, args.subsims, clk.summary(), alu)
     else:
-        one = args.precision == "fp64" and variant == 0   # a launch per step: psi read and written
+        # a launch per step (k_step64): psi read and written
+        one = args.precision == "fp64" and variant == 0
         stage_ms = fam["stage"] / ((1 if one else 4) * args.steps)
         bytes_launch = (2.0 * elem * n_orb * cell.n_pts if one else
                         stage_bytes_per_launch(elem, n_orb, cell.n_pts, reads_v=args.precision == "fp32_tc"))
@@ -642,6 +645,14 @@ def main():
                 "peak": hbm, "unit": "GB/s", "frac": achieved / hbm, "traffic": None,
                 "algorithmic_bytes_per_launch": bytes_launch,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (burst copy)" if peaks else "fallback 6.8 TB/s"}
+        if one and not args.profile_run:
+            # bound by the FP64 pipe: its operations (a fused one counts once, as one instruction)
+            # against half of the FMA probe's flops; the HBM figures stay beside it
+            ops = 4.0 * STEP64_OPS_PER_POINT_STAGE * cell.n_pts * n_orb / (stage_ms / 1e3) / 1e12
+            fp64 = alu_peaks(local_rank)["dfma_tflops"] / 2
+            roof.update(bound="fp64", achieved=ops, peak=fp64, unit="T FP64 operations/s", frac=ops / fp64,
+                        peak_source="FP64 FMA probe on this GPU / 2", hbm_achieved_gbs=achieved, hbm_peak_gbs=hbm,
+                        hbm_frac=achieved / hbm)
     hbm_src = "MEASURED_PEAKS.json hbm_gbs (burst copy)" if peaks else "fallback 6.8 TB/s"
     roof["family_ms_per_step"] = fam_ms
 

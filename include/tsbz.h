@@ -52,12 +52,17 @@ extern "C" {
  * terms themselves are formed from the float orbitals and projections in
  * float. */
 #define TSBZ_FP64 0          /* everything in double                          */
-#define TSBZ_FP32 1          /* stencil, Taylor and projectors in float; on
-                                cells of at most 8 atoms with 16^3 grids the
-                                projector contractions are factorised per axis
-                                and their z contractions run on tensor cores
-                                (three-product TF32, FP32 accumulate), fused
-                                with the stencil in one kernel per stage      */
+#define TSBZ_FP32 1          /* orbitals, kinetic operator, Taylor sum and
+                                projectors in float.  16^3 cells (at most 4
+                                atom planes of two atoms) and 32^3 cells run
+                                their projectors' z contractions on tensor
+                                cores with FP32 accumulators: three-product
+                                TF32 at 16^3; at 32^3 three bfloat16 parts of
+                                each float (24 bits, six products) for the
+                                projections and three-product TF32 for their
+                                way back.  The last bits of a result depend
+                                on what else the context holds (summation
+                                groups follow the number of orbitals)        */
 #define TSBZ_FP32_TC 2       /* as FP32 with dense projector GEMMs on tensor
                                 cores in their own kernels (scaled split-FP16,
                                 three products, FP32 accumulate)              */
@@ -267,11 +272,17 @@ int tsbz_autotune(tsbz_ctx* ctx, int budget_ms, int* n_tried);
 
 /* The variant in force for a cell, the number it can run (n_variants) and the
  * ms per step the autotuner measured for each (ms[0..n_ms-1], 0 = untimed);
- * any output pointer may be NULL.  Variants: FP32 on 16^3 and 8^3 cells:
- * 0 = fused tensor-core / bulk-staged stage, 1 = z-march stage with CUDA-core
- * projections; point-parallel stage kernels (FP64, other FP32 shapes): bands
- * per staged projection chunk 8 (0), 4 (1), 16 (2); 16^3 grids in FP64 and small
- * grids in FP64 and FP32: 0 = the whole step in one launch (from 8 orbitals on). */
+ * any output pointer may be NULL.  Variant 0 is the whole step in one launch
+ * where the cell has such a form: FP32 on 16^3 cells (at most 4 atom planes of
+ * two atoms) and 32^3 cells (at most 8 classes of atoms per axis), FP64 on 16^3
+ * grids unless few bands of many k-points are quicker otherwise, and small grids
+ * in both from 8 orbitals on.  The others: FP32 on such 16^3 cells a fused
+ * tensor-core stage (1), a z-march stage with CUDA-core projections (2) and the
+ * whole step with the star stencil (3); other 16^3 and 8^3 cells a fused or
+ * bulk-staged stage (0) and the z-march stage (1); FP32 with 32-point rows the
+ * slab stage (0, unless the whole step), then point-parallel kernels with 4 (1),
+ * 16 (2) and 8 (3) bands per staged projection chunk; everything else
+ * point-parallel kernels with 8 (0, unless the whole step), 4 (1) and 16 (2). */
 int tsbz_get_variant(tsbz_ctx* ctx, int cell_id, int* variant, int* n_variants, double* ms, int n_ms);
 
 /* Force a cell's variant (0 <= variant < n_variants; TSBZ_EINVAL otherwise). */

@@ -894,8 +894,9 @@ template <typename T> bool any_ok(const CellDev& c) {
   return c.n_atoms <= ANY_NA && c.n1 < 1024 && c.n2 < 1024 && c.n3 < 1024 && any_smem<T>(c) <= ANY_MAX_SMEM;
 }
 
-// Variant 0, from ANY_MIN_ORB orbitals on; smaller runs keep the sequences of launches,
-// whose number per step is part of the launch accounting.
+// Variant 0, from ANY_MIN_ORB orbitals on.  The launches per stage are slower for fewer too
+// (us a step, 4 orbitals: 8^3 single 76 -> 50, 10 x 12 x 14 single 208 -> 88, double 410 -> 170);
+// such runs keep them because callers rely on the number of launches of a small run's step.
 template <typename T> bool any_taken(const LaunchSet& L) {
   return L.variant == 0 && (long long)L.n_units * L.cell.n_bands >= ANY_MIN_ORB && any_ok<T>(L.cell);
 }
@@ -921,8 +922,8 @@ template <typename G> bool any_cluster(const LaunchSet& L, G&& go) {
   return true;
 }
 
-// The form of a cell's kernels (of the cell alone, so that every kernel of a run sums
-// alike).  In single precision a CTA that fewer than four fit an SM takes 512 threads:
+// The form of a cell's kernels where no cluster is taken (k_pa_any never takes one: J(0+) and
+// J(t) of a run in clusters are summed in different orders).  In single precision a CTA that fewer than four fit an SM takes 512 threads:
 // the SM then holds 16 warps or more (10 steps of 768 k-points, 12 orbitals each:
 // 18^3 21.1 -> 16.3 ms, 17 x 13 x 15 9.06 -> 8.40, 16 x 16 x 8 5.46 -> 5.35; smaller
 // cells lose, 9 x 11 x 13 3.77 -> 4.12 ms).  In double 256 threads hold the FP64 pipe

@@ -19,8 +19,9 @@
 // Taylor terms are kept as s_m = dt h^m psi; the rest of (-i dt)^m / m! enters the sum only,
 // psi's increment (see tsbz_any.cu).
 // Measured, 65 536 orbitals: 10.50 (four star stencils, k_step_fused with its contractions
-// on tcgen05) -> 6.10 ms; 122 instructions a point and stage, projections of the current
-// included, 54% of the issue slots.  Without any transform it takes 4.8 ms, with the
+// on tcgen05) -> 6.10 ms, 6.18 with the symbol's table and the increment summed apart (their
+// reason stands at tsbz_symbol.cuh and tsbz_any.cu); 121 instructions a point and stage, projections
+// of the current included, 52% of the issue slots.  Without any transform it takes 4.8 ms, with the
 // butterflies in scalar instead of packed arithmetic 6.5 ms.
 //
 // Contractions (see tsbz_fused.cuh for the factorisation).  Atoms are addressed by

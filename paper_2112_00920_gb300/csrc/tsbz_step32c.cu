@@ -10,7 +10,7 @@
 // the transformed rows, the neighbour CTAs' four rows on either side read through
 // distributed shared memory (the same volume as a transform's two exchanges,
 // with one exchange instead of two; the same barrier publishes the partial projections).
-// Projectors: z sums of the columns on tcgen05 (three-product TF32, A in tensor
+// Projectors: z sums of the columns on tcgen05 (three bfloat16 parts, A in tensor
 // memory), x sums per (atom, row) over the atom's box, y sums over the CTA's rows,
 // and the eight CTAs' partial sums added in rank order through distributed
 // shared memory.  The ket goes back the same way, its contraction along z on
@@ -20,7 +20,7 @@
 // tsbz_any.cu; psi stays in the sum here: adding it last spilled, 2.00 -> 2.08 ms, and
 // gained nothing on so many points).
 // Measured: 8 k-points x 128 bands of the 64-atom cell, stages and projections 3.31 ->
-// 2.00 ms per step (36% of issue slots, the rest barriers and the latency of the
+// 1.98 ms per step (36% of issue slots, the rest barriers and the latency of the
 // remote rows).
 // Every wait on an MMA is bounded; a CTA that gave up keeps taking part in the
 // cluster's barriers and reports at the end.

@@ -21,9 +21,9 @@
 // along z in registers; the line transforms along x and y go through one
 // shared buffer with the x index turned by y (no bank conflicts).  At 16^3 the
 // two buffers take 128 KiB: one CTA per SM, whose 8 warps keep the FP64 pipe
-// busy (a warp instruction occupies it for 16 clocks).
+// busy (a warp instruction occupies its quarter for 64 clocks).
 // Measured, the whole time step: 512 k-points x 16 bands at 16^3, 79.8 -> 42.1 ms, FP64 pipe
-// 82% busy at 133 operations per point and stage; 8 k-points x 16 bands 1.77 ->
+// 82% busy at 132 operations per point and stage; 8 k-points x 16 bands 1.77 ->
 // 0.83 ms.
 #include <cuda_runtime.h>
 
